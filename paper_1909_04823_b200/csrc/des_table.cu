@@ -336,20 +336,69 @@ extern "C" des_status_t des_table_export(des_table_t* t, uint64_t* d_keys, uint8
   return DES_OK;
 }
 
-__global__ void read_rows_kernel(const uint32_t* __restrict__ grows, long long n, int k, int stride,
-                                 unsigned long long total_rows, const float* __restrict__ W,
-                                 const float* __restrict__ A, float* emb, float* lin, float* acc_emb, float* acc_lin) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t g = grows[i];
-  bool ok = g != DES_ROW_NONE && g < total_rows;
-  for (int c = 0; c < k; ++c) {
-    if (emb) emb[i * k + c] = ok ? W[(size_t)g * stride + c] : 0.f;
-    if (acc_emb) acc_emb[i * k + c] = (ok && A) ? A[(size_t)g * stride + c] : 0.f;
+// Rows in and out of the table.  Both directions are bound by memory: every listed row is a random
+// (k + 4) * 4-byte read or write on the table's side and a dense one on the caller's.  G lanes take a row, one
+// 16-byte column each (V = float4; lane 0 also the tail), ROWS_U rows of a group in flight; the dense side of a warp is then
+// contiguous.  (One thread per row, walking its columns 4 bytes at a time, re-read every 32-byte sector eight
+// times: 1.6 M rows of k = 64 with state took 2.23 ms.)  V = float serves dense arrays that are not
+// 16-byte aligned.
+#define ROWS_U 4
+__device__ __forceinline__ void rows_zero(float& v) { v = 0.f; }
+__device__ __forceinline__ void rows_zero(float4& v) { v = make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ float rows_sq(float v) { return v * v; }
+__device__ __forceinline__ float rows_sq(const float4& v) { return v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w; }
+
+template <int G, typename V>
+__global__ void __launch_bounds__(256) read_rows_kernel(const uint32_t* __restrict__ grows, long long n, int k, int stride,
+                                                        unsigned long long total_rows, const float* __restrict__ W,
+                                                        const float* __restrict__ A, float* __restrict__ emb,
+                                                        float* __restrict__ lin, float* __restrict__ acc_emb,
+                                                        float* __restrict__ acc_lin) {
+  constexpr int VW = sizeof(V) / 4;
+  const int C = k / VW, lane = threadIdx.x % G;
+  // a warp's groups take neighbouring rows, its ROWS_U rounds too
+  const long long i0 = ((long long)blockIdx.x * 256 + (threadIdx.x & ~31)) / G * ROWS_U + (threadIdx.x & 31) / G;
+  uint32_t g[ROWS_U];
+#pragma unroll
+  for (int q = 0; q < ROWS_U; ++q) {
+    const long long i = i0 + q * (32 / G);
+    g[q] = i < n ? __ldg(grows + i) : DES_ROW_NONE;
+    if (g[q] >= total_rows) g[q] = DES_ROW_NONE;
   }
-  if (lin) lin[i] = ok ? W[(size_t)g * stride + k] : 0.f;
-  if (acc_lin) acc_lin[i] = (ok && A) ? A[(size_t)g * stride + k] : 0.f;
+  for (int c = lane; c < C; c += G) {
+    V w[ROWS_U], a[ROWS_U];
+#pragma unroll
+    for (int q = 0; q < ROWS_U; ++q) {
+      rows_zero(w[q]); rows_zero(a[q]);
+      if (g[q] != DES_ROW_NONE) {
+        if (emb) w[q] = __ldg(reinterpret_cast<const V*>(W + (size_t)g[q] * stride) + c);
+        if (acc_emb && A) a[q] = __ldg(reinterpret_cast<const V*>(A + (size_t)g[q] * stride) + c);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < ROWS_U; ++q) {
+      const long long i = i0 + q * (32 / G);
+      if (i >= n) continue;
+      if (emb) __stcs(reinterpret_cast<V*>(emb + i * k) + c, w[q]);
+      if (acc_emb) __stcs(reinterpret_cast<V*>(acc_emb + i * k) + c, a[q]);
+    }
+  }
+  if (lane == 0) {
+#pragma unroll
+    for (int q = 0; q < ROWS_U; ++q) {
+      const long long i = i0 + q * (32 / G);
+      if (i >= n) continue;
+      const bool ok = g[q] != DES_ROW_NONE;
+      if (lin) lin[i] = ok ? W[(size_t)g[q] * stride + k] : 0.f;
+      if (acc_lin) acc_lin[i] = (ok && A) ? A[(size_t)g[q] * stride + k] : 0.f;
+    }
+  }
 }
+
+static bool rows_vec(const void* a, const void* b) { return ((((uintptr_t)a) | ((uintptr_t)b)) & 15) == 0; }
+// lanes per row: the power of two that covers its 16-byte columns (k <= 64: at most 16)
+static int rows_group(int k) { int G = 1; while (G < k / 4) G <<= 1; return G; }
+static unsigned rows_grid(int64_t n, int G) { const int64_t per = 256 / G * ROWS_U; return (unsigned)((n + per - 1) / per); }
 
 extern "C" des_status_t des_table_read_rows(des_table_t* t, const uint32_t* d_global_rows, int64_t n, float* d_emb,
                                             float* d_lin, float* d_acc_emb, float* d_acc_lin, void* stream) {
@@ -357,29 +406,44 @@ extern "C" des_status_t des_table_read_rows(des_table_t* t, const uint32_t* d_gl
   if (n == 0) return DES_OK;                 // nothing to do, whatever the pointers
   if (!d_global_rows) return DES_ERR_INVALID_ARG;
   des_api_begin(t, (cudaStream_t)stream);
-  read_rows_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-      d_global_rows, n, t->k, t->stride, t->total_rows, t->W, t->A, d_emb, d_lin, d_acc_emb, d_acc_lin);
+  const int G = rows_group((int)t->k);
+#define RR(GG, VV) read_rows_kernel<GG, VV><<<rows_grid(n, GG), 256, 0, (cudaStream_t)stream>>>(                       \
+      d_global_rows, n, t->k, t->stride, t->total_rows, t->W, t->A, d_emb, d_lin, d_acc_emb, d_acc_lin)
+  if (!rows_vec(d_emb, d_acc_emb)) RR(16, float);
+  else switch (G) { case 1: RR(1, float4); break; case 2: RR(2, float4); break; case 4: RR(4, float4); break;
+                    case 8: RR(8, float4); break; default: RR(16, float4); }
+#undef RR
   DES_LAUNCH_CHECK(t, "read_rows_kernel");
   return DES_OK;
 }
 
-__global__ void write_rows_kernel(const uint32_t* __restrict__ grows, long long n, int k, int stride,
-                                  unsigned long long total_rows, float* W, float* A, const float* __restrict__ emb,
-                                  const float* __restrict__ lin, const float* __restrict__ acc_emb,
-                                  const float* __restrict__ acc_lin) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  uint32_t g = grows[i];
-  if (g == DES_ROW_NONE || g >= total_rows) return;
+template <int G, typename V>
+__global__ void __launch_bounds__(256) write_rows_kernel(const uint32_t* __restrict__ grows, long long n, int k, int stride,
+                                                         unsigned long long total_rows, float* W, float* A,
+                                                         const float* __restrict__ emb, const float* __restrict__ lin,
+                                                         const float* __restrict__ acc_emb, const float* __restrict__ acc_lin) {
+  constexpr int VW = sizeof(V) / 4;
+  const int C = k / VW, lane = threadIdx.x % G;
+  const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) / G;
+  uint32_t g = i < n ? __ldg(grows + i) : DES_ROW_NONE;
+  if (g >= total_rows) g = DES_ROW_NONE;
+  const bool ok = g != DES_ROW_NONE;
+  float* w = W + (ok ? (size_t)g * stride : 0);
   float n2 = 0.f;
-  for (int c = 0; c < k; ++c) {
-    if (emb) W[(size_t)g * stride + c] = emb[i * k + c];
-    if (acc_emb && A) A[(size_t)g * stride + c] = acc_emb[i * k + c];
-    const float v = W[(size_t)g * stride + c];
-    n2 += v * v;
-  }
-  W[(size_t)g * stride + k + 1] = n2;
-  if (lin) W[(size_t)g * stride + k] = lin[i];
+  if (ok)
+    for (int c = lane; c < C; c += G) {
+      V v;
+      if (emb) { v = __ldg(reinterpret_cast<const V*>(emb + i * k) + c); reinterpret_cast<V*>(w)[c] = v; }
+      else v = reinterpret_cast<const V*>(w)[c];
+      if (acc_emb && A)
+        reinterpret_cast<V*>(A + (size_t)g * stride)[c] = __ldg(reinterpret_cast<const V*>(acc_emb + i * k) + c);
+      n2 += rows_sq(v);
+    }
+#pragma unroll
+  for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);   // |v|^2, cached in the row's tail
+  if (!ok || lane) return;
+  w[k + 1] = n2;
+  if (lin) w[k] = lin[i];
   if (acc_lin && A) A[(size_t)g * stride + k] = acc_lin[i];
 }
 
@@ -390,8 +454,13 @@ extern "C" des_status_t des_table_write_rows(des_table_t* t, const uint32_t* d_g
   if (n == 0) return DES_OK;                 // nothing to do, whatever the pointers
   if (!d_global_rows) return DES_ERR_INVALID_ARG;
   des_api_begin(t, (cudaStream_t)stream);
-  write_rows_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-      d_global_rows, n, t->k, t->stride, t->total_rows, t->W, t->A, d_emb, d_lin, d_acc_emb, d_acc_lin);
+  const int G = rows_group((int)t->k);
+#define WR(GG, VV) write_rows_kernel<GG, VV><<<(unsigned)((n * GG + 255) / 256), 256, 0, (cudaStream_t)stream>>>(      \
+      d_global_rows, n, t->k, t->stride, t->total_rows, t->W, t->A, d_emb, d_lin, d_acc_emb, d_acc_lin)
+  if (!rows_vec(d_emb, d_acc_emb)) WR(16, float);
+  else switch (G) { case 1: WR(1, float4); break; case 2: WR(2, float4); break; case 4: WR(4, float4); break;
+                    case 8: WR(8, float4); break; default: WR(16, float4); }
+#undef WR
   DES_LAUNCH_CHECK(t, "write_rows_kernel");
   return DES_OK;
 }
