@@ -15,7 +15,7 @@ def test_rows_round_trip(k, n, shift):
     t = D.Table(3, 2, k, optimizer=D.OPT_ADAGRAD, max_rows=3000, max_nnz=4096, max_batch=2048)
     try:
         ids = torch.arange(1, n + 1, dtype=torch.int64, device="cuda")
-        off = torch.arange(2 * n + 1, dtype=torch.int64, device="cuda").clamp_(max=n)
+        off = (torch.arange(2 * n + 1, dtype=torch.int64, device="cuda") + 1) // 2      # one id per sample
         db = D.DeviceBatch(off, ids, None, n)
         t.find_or_insert(db)
         rows = db.uniq_rows[:n].clone()
