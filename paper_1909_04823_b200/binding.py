@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libdes.so — argument marshalling only.
+"""Thin binding of libdes.so — argument marshalling only: the calls of a step through the native extension
+_marshal (csrc/des_py.cpp), the others through ctypes.
 
 Every step of the path runs in the library's CUDA kernels; torch is used for
 device memory and streams.  If the library cannot be loaded this module raises:
@@ -96,6 +97,7 @@ class des_grads_t(C.Structure):
 
 _lib = None
 _lib_debug = None
+_native = {}                  # library path -> its handle in the marshalling extension
 _use_debug = False
 
 
@@ -126,6 +128,16 @@ def load():
     if _lib is None:
         _lib = _declare(C.CDLL(_build.build()))
     return _lib
+
+
+def native():
+    """(the marshalling extension, its handle of the library that load() returns)"""
+    path = lib_path()
+    if path not in _native:
+        load()
+        from . import _marshal
+        _native[path] = (_marshal, _marshal.open(path))
+    return _native[path]
 
 
 def _declare(L):
@@ -237,6 +249,7 @@ class Table:
         if not torch.cuda.is_available():
             raise RuntimeError("paper_1909_04823_b200 needs a CUDA device; there is no CPU path")
         self.L = load()
+        self.N, self._lib = native()
         self.S, self.F, self.k, self.H = num_shards, num_fields, emb_dim, hidden
         self.partition, self.max_nnz, self.max_batch = partition, int(max_nnz), int(max_batch)
         self.stride = emb_dim + 4
@@ -283,45 +296,30 @@ class Table:
 
     # -- the five calls of the path -------------------------------------------
     def find_or_insert(self, batch: DeviceBatch, insert: bool = True):
-        cb = batch.c()
-        self._check(self.L.des_find_or_insert(self.h, C.byref(cb), 1 if insert else 0, _stream()),
-                    "des_find_or_insert")
+        self._check(self.N.find_or_insert(self._lib, self.h.value, batch, insert), "des_find_or_insert")
 
     def forward_partials(self, ops, batch, part_small=None, pooled=None, part_pooled=None, part_dense=None):
-        cb = batch.c()
-        p = des_partials_t(_ptr(part_small), _ptr(pooled), _ptr(part_pooled), _ptr(part_dense))
-        self._check(self.L.des_forward_partials(self.h, ops, C.byref(cb), C.byref(p), _stream()),
+        self._check(self.N.forward_partials(self._lib, self.h.value, ops, batch, part_small, pooled, part_pooled, part_dense),
                     "des_forward_partials")
 
     def aggregate(self, ops, batch, part_small=None, pooled=None, part_pooled=None, part_dense=None,
                   out_small=None, out_pooled=None, Z=None):
-        cb = batch.c()
-        p = des_partials_t(_ptr(part_small), _ptr(pooled), _ptr(part_pooled), _ptr(part_dense))
-        o = des_outputs_t(_ptr(out_small), _ptr(out_pooled if out_pooled is not None else pooled), _ptr(Z))
-        self._check(self.L.des_aggregate(self.h, ops, C.byref(cb), C.byref(p), C.byref(o), _stream()),
-                    "des_aggregate")
+        self._check(self.N.aggregate(self._lib, self.h.value, ops, batch, part_small, pooled, part_pooled, part_dense,
+                                     out_small, out_pooled if out_pooled is not None else pooled, Z), "des_aggregate")
 
     def forward_fused(self, ops, batch, part_small=None, pooled=None, out_small=None, Z=None):
-        cb = batch.c()
-        p = des_partials_t(_ptr(part_small), _ptr(pooled), None, None)
-        o = des_outputs_t(_ptr(out_small), _ptr(pooled), _ptr(Z))
-        self._check(self.L.des_forward_fused(self.h, ops, C.byref(cb), C.byref(p), C.byref(o), _stream()),
+        self._check(self.N.forward_fused(self._lib, self.h.value, ops, batch, part_small, pooled, out_small, Z),
                     "des_forward_fused")
 
     def backward_update(self, ops, batch, out_small=None, pooled=None, Z=None, gL=None, gF=None, gE=None,
                         gZ=None, gE_work=None):
-        cb = batch.c()
-        o = des_outputs_t(_ptr(out_small), _ptr(pooled), _ptr(Z))
-        g = des_grads_t(_ptr(gL), _ptr(gF), _ptr(gE), _ptr(gZ), _ptr(gE_work))
-        self._check(self.L.des_backward_update(self.h, ops, C.byref(cb), C.byref(o), C.byref(g), _stream()),
-                    "des_backward_update")
+        self._check(self.N.backward_update(self._lib, self.h.value, ops, batch, out_small, pooled, Z, gL, gF, gE, gZ,
+                                           gE_work), "des_backward_update")
 
     def step_host(self, ops, batch_size, nnz, h_offsets, h_ids, h_vals, h_out_small, d_pooled=None, d_Z=None,
                   gL=None, gF=None, gE=None, gZ=None, gE_work=None):
-        g = des_grads_t(_ptr(gL), _ptr(gF), _ptr(gE), _ptr(gZ), _ptr(gE_work))
-        self._check(self.L.des_step_host(self.h, ops, batch_size, nnz, _ptr(h_offsets), _ptr(h_ids),
-                                         _ptr(h_vals), C.byref(g), _ptr(d_pooled), _ptr(d_Z),
-                                         _ptr(h_out_small), _stream()), "des_step_host")
+        self._check(self.N.step_host(self._lib, self.h.value, ops, batch_size, nnz, h_offsets, h_ids, h_vals, h_out_small,
+                                     d_pooled, d_Z, gL, gF, gE, gZ, gE_work), "des_step_host")
 
     # -- (+) across processes -----------------------------------------------------------
     def rank_partial(self, batch_size: int, part_small: torch.Tensor, rank_part: torch.Tensor):
@@ -335,15 +333,13 @@ class Table:
     def step_host_submit(self, ops, batch_size, nnz, h_offsets, h_ids, h_vals, h_out_small, d_pooled=None, d_Z=None,
                          gL=None, gF=None, gE=None, gZ=None, gE_work=None) -> int:
         """Pipelined des_step_host: returns a ticket for step_host_wait."""
-        g = des_grads_t(_ptr(gL), _ptr(gF), _ptr(gE), _ptr(gZ), _ptr(gE_work))
-        ticket = C.c_int32(-1)
-        self._check(self.L.des_step_host_submit(self.h, ops, batch_size, nnz, _ptr(h_offsets), _ptr(h_ids),
-                                                _ptr(h_vals), C.byref(g), _ptr(d_pooled), _ptr(d_Z),
-                                                _ptr(h_out_small), _stream(), C.byref(ticket)), "des_step_host_submit")
-        return int(ticket.value)
+        code, ticket = self.N.step_host_submit(self._lib, self.h.value, ops, batch_size, nnz, h_offsets, h_ids, h_vals,
+                                               h_out_small, d_pooled, d_Z, gL, gF, gE, gZ, gE_work)
+        self._check(code, "des_step_host_submit")
+        return ticket
 
     def step_host_wait(self, ticket: int):
-        self._check(self.L.des_step_host_wait(self.h, ticket), "des_step_host_wait")
+        self._check(self.N.step_host_wait(self._lib, self.h.value, ticket), "des_step_host_wait")
 
     # -- first dense layer ----------------------------------------------------------
     def dense1_set(self, W1: torch.Tensor):
@@ -352,8 +348,8 @@ class Table:
         torch.cuda.current_stream().synchronize()
 
     def dense1_get(self) -> torch.Tensor:
-        W1 = torch.empty((self.F * self.k, self.H), dtype=torch.float32, device="cuda")
-        self._check(self.L.des_dense1_get(self.h, _ptr(W1), _stream()), "des_dense1_get")
+        code, W1 = self.N.dense1_get(self._lib, self.h.value, self.F * self.k, self.H)
+        self._check(code, "des_dense1_get")
         return W1
 
     # -- inspection -------------------------------------------------------------------
@@ -376,12 +372,9 @@ class Table:
     def head(self, ops, batch_size, hc, out_small=None, pooled=None, Z=None, xdense=None, y=None, logit=None, loss=None,
              gL=None, gF=None, gE=None, gZ=None):
         """hc: dict(b0, c_lr, c_fm, u, b1, q, d) with device tensors (or None) for the vectors."""
-        h = des_head_t(float(hc["b0"]), float(hc["c_lr"]), float(hc["c_fm"]), _ptr(hc.get("u")), _ptr(hc.get("b1")),
-                       _ptr(hc.get("q")), _ptr(hc.get("d")), 0 if hc.get("d") is None else int(hc["d"].numel()))
-        o = des_outputs_t(_ptr(out_small), _ptr(pooled), _ptr(Z))
-        g = des_head_grads_t(_ptr(gL), _ptr(gF), _ptr(gE), _ptr(gZ))
-        self._check(self.L.des_head(self.h, ops, int(batch_size), C.byref(h), C.byref(o), _ptr(xdense), _ptr(y),
-                                    _ptr(logit), _ptr(loss), C.byref(g), _stream()), "des_head")
+        self._check(self.N.head(self._lib, self.h.value, ops, batch_size, hc["b0"], hc["c_lr"], hc["c_fm"], hc.get("u"),
+                                hc.get("b1"), hc.get("q"), hc.get("d"), out_small, pooled, Z, xdense, y, logit, loss, gL, gF,
+                                gE, gZ), "des_head")
 
     def evict_keys(self, keys: torch.Tensor) -> int:
         """keys: int64 / uint64 device tensor of ids to remove.  Returns the number of rows removed."""
@@ -450,20 +443,12 @@ class Table:
         torch.cuda.current_stream().synchronize()
 
     def read_rows(self, global_rows: torch.Tensor):
-        n = int(global_rows.numel())
-        dev = "cuda"
-        emb = torch.empty((n, self.k), dtype=torch.float32, device=dev)
-        lin = torch.empty(n, dtype=torch.float32, device=dev)
-        ae = torch.empty((n, self.k), dtype=torch.float32, device=dev)
-        al = torch.empty(n, dtype=torch.float32, device=dev)
-        self._check(self.L.des_table_read_rows(self.h, _ptr(global_rows), n, _ptr(emb), _ptr(lin), _ptr(ae),
-                                               _ptr(al), _stream()), "des_table_read_rows")
+        code, emb, lin, ae, al = self.N.read_rows(self._lib, self.h.value, global_rows, self.k)
+        self._check(code, "des_table_read_rows")
         return dict(emb=emb, lin=lin, acc_emb=ae, acc_lin=al)
 
     def write_rows(self, global_rows: torch.Tensor, emb=None, lin=None, acc_emb=None, acc_lin=None):
-        n = int(global_rows.numel())
-        self._check(self.L.des_table_write_rows(self.h, _ptr(global_rows), n, _ptr(emb), _ptr(lin), _ptr(acc_emb),
-                                                _ptr(acc_lin), _stream()), "des_table_write_rows")
+        self._check(self.N.write_rows(self._lib, self.h.value, global_rows, emb, lin, acc_emb, acc_lin), "des_table_write_rows")
 
     def profile_enable(self, on: bool = True):
         self._check(self.L.des_profile_enable(self.h, 1 if on else 0), "des_profile_enable")
@@ -516,23 +501,17 @@ def _check_free(code, where):
 def cross_forward(x0: torch.Tensor, x: torch.Tensor, w: torch.Tensor, b: torch.Tensor, num_shards: int,
                   want_part: bool = False):
     """-> (y [B][d], P [B], part [S][B] or None)"""
-    B, d = x.shape
-    y = torch.empty_like(x)
-    P = torch.empty(B, dtype=torch.float32, device=x.device)
-    part = torch.empty((num_shards, B), dtype=torch.float32, device=x.device) if want_part else None
-    _check_free(load().des_cross_forward(B, d, num_shards, _ptr(x0), _ptr(x), _ptr(w), _ptr(b), _ptr(part), _ptr(P),
-                                        _ptr(y), _stream()), "des_cross_forward")
+    N, lib = native()
+    code, y, P, part = N.cross_forward(lib, x0, x, w, b, num_shards, want_part)
+    _check_free(code, "des_cross_forward")
     return y, P, part
 
 
 def cross_backward(x0, x, w, P, gY):
     """-> (gx0, gx [B][d], gw, gb [d])"""
-    B, d = x.shape
-    gx0 = torch.empty_like(x); gx = torch.empty_like(x)
-    gw = torch.empty(d, dtype=torch.float32, device=x.device); gb = torch.empty_like(gw)
-    ws = torch.empty(int(load().des_cross_workspace_floats(B, d)), dtype=torch.float32, device=x.device)
-    _check_free(load().des_cross_backward(B, d, _ptr(x0), _ptr(x), _ptr(w), _ptr(P), _ptr(gY), _ptr(gx0), _ptr(gx),
-                                         _ptr(gw), _ptr(gb), _ptr(ws), _stream()), "des_cross_backward")
+    N, lib = native()
+    code, gx0, gx, gw, gb = N.cross_backward(lib, x0, x, w, P, gY)
+    _check_free(code, "des_cross_backward")
     return gx0, gx, gw, gb
 
 

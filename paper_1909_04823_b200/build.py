@@ -7,7 +7,8 @@ Two libraries come out of the same sources:
                    memory out of range (the stand-in for a memory checker), and test-only hooks exist.
 Every translation unit is compiled to an object of its own (kept under build/, rebuilt only when the
 source or a header it includes is newer), so a change to one kernel file recompiles that file only; the
-tensor-core GEMM units, which take longest, are shared by both libraries."""
+tensor-core GEMM units, which take longest, are shared by both libraries.
+Beside them _marshal.so, the Python extension that hands tensors to the C ABI (host code only)."""
 from __future__ import annotations
 
 import glob
@@ -23,6 +24,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libdes.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
+MARSHAL_SRC = os.path.join(CSRC, "des_py.cpp")
 LIB_DEBUG = os.path.join(HERE, "libdes_debug.so")
 
 
@@ -86,7 +89,37 @@ def needs_build(debug: bool = False) -> bool:
     return _stale(lib, deps)
 
 
+def _marshal_stale():
+    return _stale(MARSHAL, [MARSHAL_SRC, os.path.join(ROOT, "include", "des.h"), __file__])
+
+
+def build_marshal(force: bool = False) -> str:
+    """The argument-marshalling extension, with the host compiler against torch's headers."""
+    if not force and not _marshal_stale():
+        return MARSHAL
+    import fcntl
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension as ext
+    os.makedirs(OBJ, exist_ok=True)
+    with open(os.path.join(OBJ, ".lock"), "w") as lock:
+        fcntl.flock(lock, fcntl.LOCK_EX)
+        if not force and not _marshal_stale():
+            return MARSHAL
+        tmp = MARSHAL + ".tmp"
+        subprocess.check_call(
+            [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-o", tmp, MARSHAL_SRC,
+             "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(ROOT, "include"),
+             "-I", sysconfig.get_paths()["include"], "-I", "/usr/local/cuda/include"]
+            + [x for d in ext.include_paths() for x in ("-isystem", d)]
+            + [x for d in ext.library_paths() for x in ("-L" + d, "-Wl,-rpath," + d)]
+            + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python", "-ldl"])
+        os.replace(tmp, MARSHAL)
+    return MARSHAL
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
+    build_marshal(force)
     lib = LIB_DEBUG if debug else LIB
     if not force and not needs_build(debug):
         return lib
