@@ -3,20 +3,35 @@
 // update; a table that can only grow fits no memory for long, so keys can be removed here: by list, or by
 // age (rows carry the table's clock value of their insertion / last update).
 //
-// A maintenance operation, not part of the training step: it synchronises, allocates its temporaries
-// (4 bytes per row, 16 bytes per surviving key of the shards it touches) and frees them again.
-//   mark      every row to go gets fate = GONE (by probing the listed keys, or by comparing age stamps)
-//   count     rows to go per shard -> the shard's new size m
-//   pair      the freed rows below m (ascending) are paired with the surviving rows at or beyond m
-//             (ascending): one block per shard walks the shard's rows in order
-//   move      the surviving row's weights and state are copied into the freed row; fate = new row + 1
-//   collect   the slots of the touched shards are read once: (key, new row) of every surviving key
-//   clear + reinsert   the touched shards' slot regions are emptied and the survivors put back, so that
-//             linear probing never meets a deleted slot (no tombstones; the probe of the step is untouched)
+// A maintenance operation, not part of the training step: it synchronises on entry and once at the end.
+//   mark      a bit per row to go (by probing the listed keys, or by comparing age stamps), the counts per
+//             shard, and the list of the slots concerned
+//   pair      the freed rows below a shard's new size m (ascending) are paired with the surviving rows at or
+//             beyond m (ascending): one block per shard walks the shard's bits in order
+//   move      the surviving row's weights and state are copied into the freed row
+//   starts + repair   linear probing must never meet a deleted slot, and there are no tombstones: the run of
+//             occupied slots around a removed key is put back in order by one thread.  Runs are disjoint
+//             and short (a handful of slots at load 0.5), so this costs per removed key, not per key of the table
+//             (emptying and refilling the shards' regions, which remains for a region without a single empty
+//             slot, took 107 us for 0.25 M of 1.25 M keys; this takes 25 us and its cost does not
+//             grow with the table).
+//   relabel   survivors that changed rows get their new row number (one pass over the slots, only when any did)
+// The host learns the outcome with one copy at the end; nothing in between waits for it, and the temporaries
+// stay with the table unless they are large (allocating and freeing them took 1.8 ms a call).
 // Every loop is bounded (probes by the region size); a full region raises the sticky status word.
 #include "des_internal.cuh"
 
-#define FATE_GONE 0xFFFFFFFFu
+#define EV_NONE 0xFFFFFFFFu
+#define EV_KEEP_BYTES (64ull << 20)                    // temporaries up to this size stay allocated with the table
+
+struct EvictCtl {                                      // zero at the start of a call
+  uint32_t gone[DES_MAX_SHARDS];                       // rows to go
+  uint32_t pairs[DES_MAX_SHARDS];                      // rows that move
+  uint32_t n_list;                                     // slots of keys to go
+  uint32_t owned[DES_MAX_SHARDS];                      // a run of the shard has found its start (see ev_full)
+  uint32_t any_pairs;
+  uint32_t n_live;                                     // (rebuild only)
+};
 
 struct __align__(16) LiveKey { unsigned long long key; uint32_t row, shard; };
 
@@ -26,107 +41,168 @@ __device__ __forceinline__ int shard_of_pos(const unsigned long long* __restrict
   return lo;
 }
 
-// by list: one thread per (key, candidate shard); HASH: the key's own shard, FIELD: any shard may hold it
-__global__ void __launch_bounds__(256) evict_mark_keys_kernel(const unsigned long long* __restrict__ keys, long long n, int S,
-                                                             int partition, uint32_t mod_M, uint32_t mod_two32,
-                                                             const Slot* __restrict__ slots, const DevMeta* __restrict__ meta,
-                                                             uint32_t* __restrict__ fate) {
-  const long long per = partition == DES_PART_HASH ? 1 : S;
+// the rows' bits: shard s starts a word of its own at word row_base[s] / 32 + s
+__device__ __forceinline__ unsigned long long ev_word0(const DevMeta* __restrict__ meta, int s) {
+  return (meta->row_base[s] >> 5) + (unsigned long long)s;
+}
+__device__ __forceinline__ bool ev_gone(const uint32_t* __restrict__ bits, const DevMeta* __restrict__ meta, int s, uint32_t row) {
+  return (bits[ev_word0(meta, s) + (row >> 5)] >> (row & 31)) & 1u;
+}
+__device__ __forceinline__ uint32_t ev_append(uint32_t* counter, bool want) {   // whole warp; position for the lanes that want
+  const unsigned m = __ballot_sync(0xFFFFFFFFu, want);
+  const int lane = threadIdx.x & 31;
+  uint32_t base = 0;
+  if (m && lane == __ffs(m) - 1) base = atomicAdd(counter, __popc(m));
+  base = __shfl_sync(0xFFFFFFFFu, base, m ? __ffs(m) - 1 : 0);
+  return base + __popc(m & ((1u << lane) - 1u));
+}
+
+// A shard that loses keys has a run that starts behind an empty slot — unless its region has no empty slot at all.
+// Whole block.
+__device__ __forceinline__ bool ev_full(const EvictCtl* ctl, int S) {
+  bool full = false;
+  for (int s = threadIdx.x; s < S; s += blockDim.x) full |= ctl->gone[s] && !ctl->owned[s];
+  return __syncthreads_or(full);
+}
+
+// by list: one thread per key (HASH: the key's own shard; FIELD: thread (key, shard) looks in every shard)
+__global__ void __launch_bounds__(256) evict_mark_keys_kernel(const unsigned long long* __restrict__ keys, long long n,
+                                                              int S, int partition, uint32_t mod_M, uint32_t mod_two32,
+                                                              const Slot* __restrict__ slots, const DevMeta* __restrict__ meta,
+                                                              uint32_t* __restrict__ bits, uint32_t* __restrict__ list,
+                                                              EvictCtl* ctl) {
+  __shared__ uint32_t cnt[DES_MAX_SHARDS];
+  for (int i = threadIdx.x; i < S; i += 256) cnt[i] = 0;
+  __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * per) return;
-  const unsigned long long key = keys[i / per];
-  if (key == DES_KEY_EMPTY) return;
-  const unsigned long long h = des_mix64(key);
-  const uint32_t s = partition == DES_PART_HASH ? des_mod_small(h, (uint32_t)S, mod_M, mod_two32) : (uint32_t)(i % per);
-  const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cnt = hi - lo;
-  uint32_t cur = des_slot_home(h, lo, cnt);
-  for (uint32_t probe = 0; probe < cnt; ++probe) {
-    const Slot sl = slots[cur];
-    if (sl.key == key) {
-      if (sl.row != DES_ROW_NONE && sl.row < meta->n_rows[s]) fate[meta->row_base[s] + sl.row] = FATE_GONE;
-      return;
+  const long long per = partition == DES_PART_HASH ? 1 : S;
+  uint32_t slot = EV_NONE;
+  if (i < n * per) {
+    const unsigned long long key = keys[i / per];
+    const unsigned long long h = des_mix64(key);
+    const uint32_t s = partition == DES_PART_HASH ? des_mod_small(h, (uint32_t)S, mod_M, mod_two32) : (uint32_t)(i % per);
+    const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cap = hi - lo;
+    uint32_t cur = des_slot_home(h, lo, cap);
+    for (uint32_t probe = 0; key != DES_KEY_EMPTY && probe < cap; ++probe) {
+      const Slot sl = slots[cur];
+      if (sl.key == key) {
+        if (sl.row != DES_ROW_NONE && sl.row < meta->n_rows[s]) {
+          const uint32_t bit = 1u << (sl.row & 31);
+          if (!(atomicOr(bits + ev_word0(meta, s) + (sl.row >> 5), bit) & bit)) {   // (a key listed twice goes once)
+            slot = cur;
+            atomicAdd(&cnt[s], 1u);
+          }
+        }
+        break;
+      }
+      if (sl.key == DES_KEY_EMPTY) break;
+      cur = cur + 1 == hi ? lo : cur + 1;
     }
-    if (sl.key == DES_KEY_EMPTY) return;
-    cur = cur + 1 == hi ? lo : cur + 1;
+  }
+  const uint32_t at = ev_append(&ctl->n_list, slot != EV_NONE);
+  if (slot != EV_NONE) list[at] = slot;
+  __syncthreads();
+  for (int s = threadIdx.x; s < S; s += 256) if (cnt[s]) atomicAdd(&ctl->gone[s], cnt[s]);
+}
+
+// by age: one warp per word of 32 rows
+__global__ void __launch_bounds__(256) evict_mark_stale_kernel(const float* __restrict__ W, int k, int stride, int S,
+                                                              unsigned long long n_words, uint32_t min_clock,
+                                                              const DevMeta* __restrict__ meta, uint32_t* __restrict__ bits,
+                                                              EvictCtl* ctl) {
+  const unsigned long long w = (unsigned long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w >= n_words) return;                            // whole warp
+  int lo = 0, hi = S;                                  // the shard whose words hold w
+  while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (ev_word0(meta, mid) <= w) lo = mid; else hi = mid; }
+  const int lane = threadIdx.x & 31;
+  const unsigned long long row = (w - ev_word0(meta, lo)) * 32 + lane;
+  const bool dead = row < meta->n_rows[lo] && __float_as_uint(W[(meta->row_base[lo] + row) * stride + k + 2]) < min_clock;
+  const unsigned m = __ballot_sync(0xFFFFFFFFu, dead);
+  if (lane == 0 && m) { bits[w] = m; atomicAdd(&ctl->gone[lo], __popc(m)); }
+}
+
+// by age: the slots of the marked rows
+__global__ void __launch_bounds__(256) evict_list_kernel(const Slot* __restrict__ slots, unsigned long long total_slots, int S,
+                                                        const DevMeta* __restrict__ meta, const uint32_t* __restrict__ bits,
+                                                        uint32_t* __restrict__ list, EvictCtl* ctl) {
+  const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
+  const unsigned long long i0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned long long rounds = (total_slots + st - 1) / st;       // whole warps
+  for (unsigned long long r = 0; r < rounds; ++r) {
+    const unsigned long long i = i0 + r * st;
+    bool dead = false;
+    if (i < total_slots) {
+      const Slot sl = slots[i];
+      if (sl.key != DES_KEY_EMPTY && sl.row != DES_ROW_NONE) dead = ev_gone(bits, meta, shard_of_pos(meta->slot_base, S, i), sl.row);
+    }
+    const uint32_t at = ev_append(&ctl->n_list, dead);
+    if (dead) list[at] = (uint32_t)i;
   }
 }
 
-// by age: one thread per row
-__global__ void __launch_bounds__(256) evict_mark_stale_kernel(const float* __restrict__ W, int k, int stride, int S,
-                                                              unsigned long long total_rows, uint32_t min_clock,
-                                                              const DevMeta* __restrict__ meta, uint32_t* __restrict__ fate) {
-  const unsigned long long g = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= total_rows) return;
-  const int s = shard_of_pos(meta->row_base, S, g);
-  if (g - meta->row_base[s] >= meta->n_rows[s]) return;
-  if (__float_as_uint(W[g * stride + k + 2]) < min_clock) fate[g] = FATE_GONE;
+// where shard s's lists of freed and moving rows start: each shard needs at most min(rows to go, rows that stay)
+__device__ __forceinline__ unsigned long long ev_list_off(const DevMeta* __restrict__ meta, const EvictCtl* ctl, int s) {
+  unsigned long long off = 0;
+  for (int i = 0; i < s; ++i) off += min(ctl->gone[i], meta->n_rows[i] - ctl->gone[i]);
+  return off;
 }
 
-// one block per shard: rows to go
-__global__ void __launch_bounds__(1024) evict_count_kernel(const uint32_t* __restrict__ fate, const DevMeta* __restrict__ meta,
-                                                           uint32_t* __restrict__ gone) {
-  __shared__ uint32_t total;
-  const int s = blockIdx.x;
-  if (threadIdx.x == 0) total = 0;
-  __syncthreads();
-  const uint32_t n = meta->n_rows[s];
-  const unsigned long long base = meta->row_base[s];
-  uint32_t c = 0;
-  for (uint32_t r = threadIdx.x; r < n; r += blockDim.x) c += fate[base + r] == FATE_GONE;
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, d);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&total, c);
-  __syncthreads();
-  if (threadIdx.x == 0) gone[s] = total;
-}
-
-// one block per shard walks its rows in ascending order, 1024 at a time: freed rows below the new size and
-// surviving rows at or beyond it, each list in ascending order (list_off[s] = where the shard's lists start)
-__global__ void __launch_bounds__(1024) evict_pair_kernel(const uint32_t* __restrict__ fate, const DevMeta* __restrict__ meta,
-                                                          const uint32_t* __restrict__ gone,
-                                                          const unsigned long long* __restrict__ list_off,
-                                                          uint32_t* __restrict__ holes, uint32_t* __restrict__ movers,
-                                                          uint32_t* __restrict__ n_pairs) {
+// one block per shard walks its bits in ascending order, 1024 words at a time: freed rows below the new size and
+// surviving rows at or beyond it, each list in ascending order
+__global__ void __launch_bounds__(1024) evict_pair_kernel(const uint32_t* __restrict__ bits, const DevMeta* __restrict__ meta,
+                                                          EvictCtl* ctl, uint32_t* __restrict__ holes,
+                                                          uint32_t* __restrict__ movers) {
   __shared__ uint32_t wh[32], wm[32], carry_h, carry_m;
   const int s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t e = gone[s];
-  if (e == 0) { if (threadIdx.x == 0) n_pairs[s] = 0; return; }
+  const uint32_t e = ctl->gone[s];
+  if (e == 0) return;
   const uint32_t n = meta->n_rows[s], m = n - e;
-  const unsigned long long base = meta->row_base[s], off = list_off[s];
+  const uint32_t* b = bits + ev_word0(meta, s);
+  const unsigned long long off = ev_list_off(meta, ctl, s);
   if (threadIdx.x == 0) { carry_h = 0; carry_m = 0; }
   __syncthreads();
-  const unsigned lt = (1u << lane) - 1u;
-  for (uint32_t chunk = 0; chunk < n; chunk += 1024) {
-    const uint32_t r = chunk + threadIdx.x;
-    const bool dead = r < n && fate[base + r] == FATE_GONE;
-    const bool is_hole = dead && r < m, is_mover = !dead && r >= m && r < n;
-    const unsigned bh = __ballot_sync(0xFFFFFFFFu, is_hole), bm = __ballot_sync(0xFFFFFFFFu, is_mover);
-    if (lane == 0) { wh[warp] = __popc(bh); wm[warp] = __popc(bm); }
+  const uint32_t nw = (n + 31) / 32;
+  auto below = [](uint32_t w, uint32_t x) { return x <= w * 32 ? 0u : x >= w * 32 + 32 ? 0xFFFFFFFFu : (1u << (x - w * 32)) - 1u; };
+  for (uint32_t chunk = 0; chunk < nw; chunk += 1024) {
+    const uint32_t w = chunk + threadIdx.x;
+    uint32_t hb = 0, mb = 0;                            // bits: freed rows below m; surviving rows in [m, n)
+    if (w < nw) {
+      const uint32_t v = b[w], bm = below(w, m);
+      hb = v & bm;
+      mb = ~v & ~bm & below(w, n);
+    }
+    uint32_t ih = __popc(hb), im = __popc(mb);
+    const uint32_t ch = ih, cm = im;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, ih, d), y = __shfl_up_sync(0xFFFFFFFFu, im, d);
+      if (lane >= d) { ih += x; im += y; }
+    }
+    if (lane == 31) { wh[warp] = ih; wm[warp] = im; }
     __syncthreads();
     uint32_t ph = carry_h, pm = carry_m;
-    for (int w2 = 0; w2 < warp; ++w2) { ph += wh[w2]; pm += wm[w2]; }
-    if (is_hole) holes[off + ph + __popc(bh & lt)] = r;
-    if (is_mover) movers[off + pm + __popc(bm & lt)] = r;
+    for (int i = 0; i < warp; ++i) { ph += wh[i]; pm += wm[i]; }
+    unsigned long long oh = off + ph + ih - ch, om = off + pm + im - cm;
+    for (; hb; hb &= hb - 1) holes[oh++] = w * 32 + __ffs(hb) - 1;
+    for (; mb; mb &= mb - 1) movers[om++] = w * 32 + __ffs(mb) - 1;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t th = 0, tm = 0;
-      for (int w2 = 0; w2 < 32; ++w2) { th += wh[w2]; tm += wm[w2]; }
-      carry_h += th; carry_m += tm;
-    }
+    if (threadIdx.x == 1023) { carry_h = ph + ih; carry_m = pm + im; }
     __syncthreads();
   }
-  if (threadIdx.x == 0) n_pairs[s] = carry_h;          // (= carry_m: as many freed rows below m as survivors beyond it)
+  if (threadIdx.x == 0) {                               // (as many freed rows below m as survivors beyond it)
+    ctl->pairs[s] = carry_h;
+    if (carry_h) ctl->any_pairs = 1u;
+  }
 }
 
 // one warp per pair: the surviving row's weights and state move into the freed row
-__global__ void __launch_bounds__(256) evict_move_kernel(const DevMeta* __restrict__ meta,
-                                                         const unsigned long long* __restrict__ list_off,
+__global__ void __launch_bounds__(256) evict_move_kernel(const DevMeta* __restrict__ meta, const EvictCtl* ctl,
                                                          const uint32_t* __restrict__ holes, const uint32_t* __restrict__ movers,
-                                                         const uint32_t* __restrict__ n_pairs, int stride, float* W, float* A,
-                                                         float* A2, uint32_t* __restrict__ fate) {
+                                                         int stride, float* W, float* A, float* A2) {
   const int s = blockIdx.y, lane = threadIdx.x & 31;
-  const uint32_t np = n_pairs[s];
-  const unsigned long long base = meta->row_base[s], off = list_off[s];
+  const uint32_t np = ctl->pairs[s];
+  if (np == 0) return;
+  const unsigned long long base = meta->row_base[s], off = ev_list_off(meta, ctl, s);
   for (uint32_t i = blockIdx.x * 8 + (threadIdx.x >> 5); i < np; i += gridDim.x * 8) {
     const unsigned long long to = base + holes[off + i], from = base + movers[off + i];
     for (int c = lane; c < stride; c += 32) {
@@ -134,46 +210,127 @@ __global__ void __launch_bounds__(256) evict_move_kernel(const DevMeta* __restri
       if (A) A[to * stride + c] = A[from * stride + c];
       if (A2) A2[to * stride + c] = A2[from * stride + c];
     }
-    if (lane == 0) fate[from] = holes[off + i] + 1u;
   }
 }
 
-// every slot of a touched shard: the surviving keys with their (possibly new) rows
+// list[i]: a removed key's slot -> the first slot of the run of occupied slots it lies in, or EV_NONE when another
+// removed key of the same run comes before it (that one repairs the run).  Reads only.
+__global__ void __launch_bounds__(256) evict_starts_kernel(const Slot* __restrict__ slots, int S, const DevMeta* __restrict__ meta,
+                                                          const uint32_t* __restrict__ bits, const uint32_t* __restrict__ list,
+                                                          uint32_t* __restrict__ starts, EvictCtl* ctl) {
+  const uint32_t n = ctl->n_list;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    uint32_t cur = list[i];
+    const int s = shard_of_pos(meta->slot_base, S, cur);
+    const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cap = hi - lo;
+    uint32_t start = EV_NONE;
+    for (uint32_t step = 1; step < cap; ++step) {
+      const uint32_t prev = cur == lo ? hi - 1 : cur - 1;
+      const Slot sl = slots[prev];
+      if (sl.key == DES_KEY_EMPTY) { start = cur; break; }
+      if (sl.row != DES_ROW_NONE && ev_gone(bits, meta, s, sl.row)) break;
+      cur = prev;
+    }
+    starts[i] = start;
+    if (start != EV_NONE && !ctl->owned[s]) ctl->owned[s] = 1u;
+  }
+}
+
+// Slots of a run are taken out one after the other and, unless removed, put back from their home slot: everything
+// between the home and the slot just emptied has been through this, so a key never lands behind where it was,
+// and the result is what inserting the survivors in that order gives.  Keys without a row (their insert
+// met a full shard) are dropped on the way.
+__global__ void __launch_bounds__(128) evict_repair_kernel(Slot* slots, int S, const DevMeta* __restrict__ meta,
+                                                          const uint32_t* __restrict__ bits, const uint32_t* __restrict__ starts,
+                                                          const EvictCtl* ctl) {
+  if (ev_full(ctl, S)) return;
+  const uint32_t n = ctl->n_list;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    uint32_t cur = starts[i];
+    if (cur == EV_NONE) continue;
+    const int s = shard_of_pos(meta->slot_base, S, cur);
+    const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cap = hi - lo;
+    Slot empty; empty.key = DES_KEY_EMPTY; empty.row = DES_ROW_NONE; empty.first_occ = DES_ROW_NONE;
+    for (uint32_t step = 0; step < cap; ++step) {
+      const Slot sl = slots[cur];
+      if (sl.key == DES_KEY_EMPTY) break;               // the run's end
+      if (sl.row == DES_ROW_NONE || ev_gone(bits, meta, s, sl.row)) {
+        slots[cur] = empty;
+      } else {
+        uint32_t at = des_slot_home(des_mix64(sl.key), lo, cap);
+        for (uint32_t p = 0; p < cap && at != cur && slots[at].key != DES_KEY_EMPTY; ++p) at = at + 1 == hi ? lo : at + 1;
+        if (at != cur) { slots[at] = sl; slots[cur] = empty; }
+      }
+      cur = cur + 1 == hi ? lo : cur + 1;
+    }
+  }
+}
+
+// survivors that changed rows
+__global__ void __launch_bounds__(256) evict_relabel_kernel(Slot* slots, unsigned long long total_slots, int S,
+                                                           const DevMeta* __restrict__ meta, const EvictCtl* ctl,
+                                                           const uint32_t* __restrict__ holes, const uint32_t* __restrict__ movers) {
+  if (!ctl->any_pairs || ev_full(ctl, S)) return;
+  __shared__ unsigned long long off[DES_MAX_SHARDS];
+  for (int s = threadIdx.x; s < S; s += blockDim.x) off[s] = ev_list_off(meta, ctl, s);
+  __syncthreads();
+  unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
+  for (; i < total_slots; i += st) {
+    const Slot sl = slots[i];
+    if (sl.key == DES_KEY_EMPTY || sl.row == DES_ROW_NONE) continue;
+    const int s = shard_of_pos(meta->slot_base, S, i);
+    if (sl.row < meta->n_rows[s] - ctl->gone[s] || !ctl->pairs[s]) continue;
+    const uint32_t* mv = movers + off[s];
+    uint32_t a = 0, b = ctl->pairs[s];                  // mv[a] <= row < mv[b]: the row is in the list
+    while (b - a > 1) { const uint32_t mid = (a + b) >> 1; if (mv[mid] <= sl.row) a = mid; else b = mid; }
+    slots[i].row = holes[off[s] + a];
+  }
+}
+
+__global__ void evict_finish_kernel(DevMeta* meta, const EvictCtl* ctl, int S) {
+  if ((int)threadIdx.x < S) meta->n_rows[threadIdx.x] -= ctl->gone[threadIdx.x];
+}
+
+// A region without a single empty slot (only keys whose insert failed can fill it up): the survivors of the shards
+// that lose a key are collected, the regions emptied, the survivors put back.  Runs before evict_finish_kernel.
 __global__ void __launch_bounds__(256) evict_collect_kernel(const Slot* __restrict__ slots, unsigned long long total_slots,
-                                                            int S, const DevMeta* __restrict__ meta,
-                                                            const uint32_t* __restrict__ gone, const uint32_t* __restrict__ fate,
-                                                            LiveKey* __restrict__ live, unsigned long long* __restrict__ n_live) {
+                                                            int S, const DevMeta* __restrict__ meta, EvictCtl* ctl,
+                                                            const uint32_t* __restrict__ bits, const uint32_t* __restrict__ holes,
+                                                            const uint32_t* __restrict__ movers, LiveKey* __restrict__ live) {
   unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
   for (; i < total_slots; i += st) {
     const int s = shard_of_pos(meta->slot_base, S, i);
-    if (gone[s] == 0) continue;
+    if (ctl->gone[s] == 0) continue;
     const Slot sl = slots[i];
-    if (sl.key == DES_KEY_EMPTY || sl.row == DES_ROW_NONE) continue;
-    const uint32_t f = fate[meta->row_base[s] + sl.row];
-    if (f == FATE_GONE) continue;
-    LiveKey lk; lk.key = sl.key; lk.row = f ? f - 1u : sl.row; lk.shard = (uint32_t)s;
-    live[atomicAdd(n_live, 1ull)] = lk;
+    if (sl.key == DES_KEY_EMPTY || sl.row == DES_ROW_NONE || ev_gone(bits, meta, s, sl.row)) continue;
+    LiveKey lk; lk.key = sl.key; lk.row = sl.row; lk.shard = (uint32_t)s;
+    if (sl.row >= meta->n_rows[s] - ctl->gone[s]) {
+      const unsigned long long off = ev_list_off(meta, ctl, s);
+      uint32_t a = 0, b = ctl->pairs[s];
+      while (b - a > 1) { const uint32_t mid = (a + b) >> 1; if (movers[off + mid] <= sl.row) a = mid; else b = mid; }
+      lk.row = holes[off + a];
+    }
+    live[atomicAdd(&ctl->n_live, 1u)] = lk;
   }
 }
 
 __global__ void __launch_bounds__(256) evict_clear_kernel(Slot* slots, unsigned long long total_slots, int S,
-                                                          const DevMeta* __restrict__ meta, const uint32_t* __restrict__ gone) {
+                                                          const DevMeta* __restrict__ meta, const EvictCtl* ctl) {
   unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
   for (; i < total_slots; i += st) {
-    if (gone[shard_of_pos(meta->slot_base, S, i)] == 0) continue;
+    if (ctl->gone[shard_of_pos(meta->slot_base, S, i)] == 0) continue;
     Slot e; e.key = DES_KEY_EMPTY; e.row = DES_ROW_NONE; e.first_occ = DES_ROW_NONE;
     slots[i] = e;
   }
 }
 
 __global__ void __launch_bounds__(256) evict_reinsert_kernel(Slot* slots, DevMeta* meta, const LiveKey* __restrict__ live,
-                                                             const unsigned long long* __restrict__ n_live) {
-  const unsigned long long n = *n_live;
-  unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
-  for (; i < n; i += st) {
+                                                             const EvictCtl* ctl) {
+  const uint32_t n = ctl->n_live;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const LiveKey lk = live[i];
     const uint32_t lo = (uint32_t)meta->slot_base[lk.shard], hi = (uint32_t)meta->slot_base[lk.shard + 1], cnt = hi - lo;
     uint32_t cur = des_slot_home(des_mix64(lk.key), lo, cnt);
@@ -189,10 +346,6 @@ __global__ void __launch_bounds__(256) evict_reinsert_kernel(Slot* slots, DevMet
   }
 }
 
-__global__ void evict_finish_kernel(DevMeta* meta, const uint32_t* __restrict__ gone, int S) {
-  if ((int)threadIdx.x < S) meta->n_rows[threadIdx.x] -= gone[threadIdx.x];
-}
-
 static des_status_t evict_run(des_table_t* t, const uint64_t* d_keys, int64_t n, uint64_t min_clock, int by_age,
                               uint64_t* h_n_evicted) {
   if (h_n_evicted) *h_n_evicted = 0;
@@ -202,75 +355,82 @@ static des_status_t evict_run(des_table_t* t, const uint64_t* d_keys, int64_t n,
   DES_CUDA(cudaDeviceSynchronize());
   t->tag_valid = 0;                                    // rows move: whatever was derived from a batch is stale
   des_api_begin(t, 0);
+  if (!by_age && n == 0) return DES_OK;
   const int S = (int)t->S;
-  uint32_t *fate = nullptr, *gone = nullptr, *n_pairs = nullptr, *holes = nullptr, *movers = nullptr;
-  unsigned long long *list_off = nullptr, *n_live = nullptr;
+  // temporaries: [ctl | bits] cleared per call, then the lists
+  const uint64_t n_words = t->total_rows / 32 + S + 1;
+  const uint64_t per = t->cfg.partition == DES_PART_HASH ? 1 : S;
+  const uint64_t most = by_age || (uint64_t)n * per > t->total_rows ? t->total_rows : (uint64_t)n * per;   // rows to go
+  const uint64_t most_pairs = most < t->total_rows / 2 + 1 ? most : t->total_rows / 2 + 1;
+  const size_t clear = ((sizeof(EvictCtl) + n_words * 4) + 255) / 256 * 256;
+  const size_t bytes = clear + (2 * most + 2 * most_pairs) * 4;
+  unsigned char* ws = (unsigned char*)t->evict_ws;
+  if (bytes > t->evict_ws_bytes) {
+    cudaFree(ws);
+    t->evict_ws = nullptr; t->evict_ws_bytes = 0;
+    ws = nullptr;
+    if (cudaMalloc(&ws, bytes) != cudaSuccess) { cudaGetLastError(); return DES_ERR_CUDA; }
+    if (bytes <= EV_KEEP_BYTES) { t->evict_ws = ws; t->evict_ws_bytes = bytes; }
+  }
   LiveKey* live = nullptr;
-  des_status_t rc = DES_OK;
-  uint32_t h_gone[DES_MAX_SHARDS];
-  unsigned long long h_off[DES_MAX_SHARDS + 1], total_gone = 0, survivors = 0;
-  uint64_t h_rows[DES_MAX_SHARDS];
   auto bail = [&](des_status_t code) {
-    cudaDeviceSynchronize();
-    cudaFree(fate); cudaFree(gone); cudaFree(n_pairs); cudaFree(holes); cudaFree(movers); cudaFree(list_off);
-    cudaFree(n_live); cudaFree(live);
-    if (code == DES_ERR_CUDA) cudaGetLastError();
+    if (code != DES_OK) { cudaDeviceSynchronize(); cudaGetLastError(); }
+    if ((void*)ws != t->evict_ws) cudaFree(ws);
+    cudaFree(live);
     return code;
   };
 #define EV_CUDA(x) do { if ((x) != cudaSuccess) return bail(DES_ERR_CUDA); } while (0)
 #define EV_LAUNCH(name) do { if (des_prof_mark(t, name, 1)) return bail(DES_ERR_CUDA); } while (0)
-  EV_CUDA(cudaMalloc(&fate, (t->total_rows + 1) * 4));
-  EV_CUDA(cudaMalloc(&gone, DES_MAX_SHARDS * 4));
-  EV_CUDA(cudaMalloc(&n_pairs, DES_MAX_SHARDS * 4));
-  EV_CUDA(cudaMalloc(&list_off, (DES_MAX_SHARDS + 1) * 8));
-  EV_CUDA(cudaMalloc(&n_live, 8));
-  EV_CUDA(cudaMemset(fate, 0, (t->total_rows + 1) * 4));
-  EV_CUDA(cudaMemset(n_live, 0, 8));
+  EvictCtl* ctl = (EvictCtl*)ws;
+  uint32_t* bits = (uint32_t*)(ws + sizeof(EvictCtl));
+  uint32_t *list = (uint32_t*)(ws + clear), *starts = list + most, *holes = starts + most, *movers = holes + most_pairs;
+  const unsigned wide = (unsigned)(t->sm_count * 8);
+  EV_CUDA(cudaMemsetAsync(ws, 0, clear, 0));
   if (by_age) {
-    const unsigned long long rows = t->total_rows;
     const uint32_t mc = min_clock > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)min_clock;
-    evict_mark_stale_kernel<<<(unsigned)((rows + 255) / 256), 256>>>(t->W, (int)t->k, (int)t->stride, S, rows, mc, t->meta, fate);
+    evict_mark_stale_kernel<<<(unsigned)((n_words + 7) / 8), 256>>>(t->W, (int)t->k, (int)t->stride, S, n_words, mc, t->meta, bits, ctl);
     EV_LAUNCH("evict_mark_stale_kernel");
-  } else if (n > 0) {
+    evict_list_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, bits, list, ctl);
+    EV_LAUNCH("evict_list_kernel");
+  } else {
     uint32_t M, two32;
     des_mod_consts(t->S, &M, &two32);
-    const long long threads = n * (t->cfg.partition == DES_PART_HASH ? 1 : S);
-    evict_mark_keys_kernel<<<(unsigned)((threads + 255) / 256), 256>>>((const unsigned long long*)d_keys, n, S,
-                                                                      (int)t->cfg.partition, M, two32, t->slots, t->meta, fate);
+    evict_mark_keys_kernel<<<(unsigned)((n * per + 255) / 256), 256>>>((const unsigned long long*)d_keys, n, S,
+                                                                      (int)t->cfg.partition, M, two32, t->slots, t->meta, bits, list, ctl);
     EV_LAUNCH("evict_mark_keys_kernel");
   }
-  evict_count_kernel<<<S, 1024>>>(fate, t->meta, gone);
-  EV_LAUNCH("evict_count_kernel");
-  EV_CUDA(cudaMemcpy(h_gone, gone, S * 4, cudaMemcpyDeviceToHost));
-  if ((rc = des_table_size(t, h_rows)) != DES_OK) return bail(rc);
-  for (int s = 0; s < S; ++s) {
-    h_off[s] = total_gone;
-    total_gone += h_gone[s];
-    if (h_gone[s]) survivors += h_rows[s] - h_gone[s];
-  }
-  h_off[S] = total_gone;
-  if (total_gone == 0) return bail(DES_OK);
-  EV_CUDA(cudaMemcpy(list_off, h_off, (S + 1) * 8, cudaMemcpyHostToDevice));
-  EV_CUDA(cudaMalloc(&holes, total_gone * 4));
-  EV_CUDA(cudaMalloc(&movers, total_gone * 4));
-  EV_CUDA(cudaMalloc(&live, (survivors + 1) * sizeof(LiveKey)));
-  evict_pair_kernel<<<S, 1024>>>(fate, t->meta, gone, list_off, holes, movers, n_pairs);
+  evict_pair_kernel<<<S, 1024>>>(bits, t->meta, ctl, holes, movers);
   EV_LAUNCH("evict_pair_kernel");
-  evict_move_kernel<<<dim3((unsigned)(t->sm_count * 4), (unsigned)S), 256>>>(t->meta, list_off, holes, movers, n_pairs,
-                                                                             (int)t->stride, t->W, t->A, t->A2, fate);
+  evict_move_kernel<<<dim3((unsigned)((t->sm_count * 8 + S - 1) / S), (unsigned)S), 256>>>(t->meta, ctl, holes, movers,
+                                                                                         (int)t->stride, t->W, t->A, t->A2);
   EV_LAUNCH("evict_move_kernel");
-  evict_collect_kernel<<<t->sm_count * 8, 256>>>(t->slots, t->total_slots, S, t->meta, gone, fate, live, n_live);
-  EV_LAUNCH("evict_collect_kernel");
-  evict_clear_kernel<<<t->sm_count * 8, 256>>>(t->slots, t->total_slots, S, t->meta, gone);
-  EV_LAUNCH("evict_clear_kernel");
-  evict_reinsert_kernel<<<t->sm_count * 8, 256>>>(t->slots, t->meta, live, n_live);
-  EV_LAUNCH("evict_reinsert_kernel");
-  evict_finish_kernel<<<1, DES_MAX_SHARDS>>>(t->meta, gone, S);
+  evict_starts_kernel<<<wide, 256>>>(t->slots, S, t->meta, bits, list, starts, ctl);
+  EV_LAUNCH("evict_starts_kernel");
+  evict_repair_kernel<<<wide * 2, 128>>>(t->slots, S, t->meta, bits, starts, ctl);
+  EV_LAUNCH("evict_repair_kernel");
+  evict_relabel_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl, holes, movers);
+  EV_LAUNCH("evict_relabel_kernel");
+  EvictCtl h;
+  EV_CUDA(cudaMemcpy(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost));
+  bool full = false;
+  for (int s = 0; s < S; ++s) full |= h.gone[s] && !h.owned[s];
+  if (full) {
+    EV_CUDA(cudaMalloc(&live, (t->total_rows + 1) * sizeof(LiveKey)));
+    evict_collect_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl, bits, holes, movers, live);
+    EV_LAUNCH("evict_collect_kernel");
+    evict_clear_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl);
+    EV_LAUNCH("evict_clear_kernel");
+    evict_reinsert_kernel<<<wide, 256>>>(t->slots, t->meta, live, ctl);
+    EV_LAUNCH("evict_reinsert_kernel");
+  }
+  evict_finish_kernel<<<1, DES_MAX_SHARDS>>>(t->meta, ctl, S);
   EV_LAUNCH("evict_finish_kernel");
   EV_CUDA(cudaDeviceSynchronize());
 #undef EV_CUDA
 #undef EV_LAUNCH
-  if (h_n_evicted) *h_n_evicted = total_gone;
+  uint64_t total = 0;
+  for (int s = 0; s < S; ++s) total += h.gone[s];
+  if (h_n_evicted) *h_n_evicted = total;
   return bail(DES_OK);
 }
 

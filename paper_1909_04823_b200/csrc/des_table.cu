@@ -106,6 +106,7 @@ extern "C" des_status_t des_table_destroy(des_table_t* t) {
                   t->W1, t->accW1, t->W1b, t->gW1_part, t->pooled_b, t->gZ_b, t->gemm_ws, t->st_offsets[0], t->st_ids[0], t->st_vals[0], t->st_offsets[1], t->st_ids[1], t->st_vals[1], t->st_rows,
                   t->st_shards, t->st_uidx, t->st_uniq_rows, t->st_n_uniq, t->st_part_small, t->st_out_small};
   for (void* p : ptrs) dfree(t->cfg, p);
+  cudaFree(t->evict_ws);
   if (t->st_copy_stream) {
     cudaStreamDestroy(t->st_copy_stream);
     for (int s = 0; s < 2; ++s) { if (t->st_copied[s]) cudaEventDestroy(t->st_copied[s]); if (t->st_done[s]) cudaEventDestroy(t->st_done[s]); }
