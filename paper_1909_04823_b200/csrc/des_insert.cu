@@ -2,30 +2,26 @@
 // including shard routing (Section 5, "Large-scale Sparse Features": weights of
 // field f live on node f mod N; Section 4.2: any balanced partition).
 //
-// One call = nine short kernels, none of which waits on another thread; the table's slots are read
-// once per occurrence by the probe and once more by flag_count, and written only for new keys:
+// One call = four kernels, none of which waits on another thread; the table's slots are read
+// once per occurrence by the probe and once more by flag_count, and written only for new keys.  (At the sizes of
+// a small or ordinary batch the call is bound by launches and by the latency of each kernel's own
+// dependent loads, not by bytes; nine kernels took 20 us of GPU time and as much again in gaps at 10 k
+// occurrences.)
 //   probe_claim   every occurrence finds its key's slot in the owning shard's
 //                 region (linear probing) or claims an empty one with a 64-bit
 //                 CAS; the slot remembers the smallest occurrence index.
 //   flag_count    occurrence j is the FIRST of its key iff the slot remembers j,
-//                 and the key is NEW iff its slot has no row yet; per-block
-//                 counts of firsts and of new keys per shard.  Leaves the
+//                 and the key is NEW iff its slot has no row yet; counts of firsts and of new keys per
+//                 shard, per tile of IB occurrences and per SUP_TILES tiles.  Leaves the
 //                 slot's row and the first occurrence's index per occurrence.
-//   scan          exclusive scan of those counts over blocks.
 //   assign        first occurrences get the batch-unique index (rank among
 //                 firsts) and, for new keys, the next shard-local row (rank
 //                 among the shard's new keys): both in CSR order, so the result
-//                 does not depend on thread scheduling.  Two kernels: the ranks
-//                 among firsts always, the new-key numbering only when the
-//                 batch has a new key at all (that kernel also clears the slots'
-//                 scratch words when their range runs out, see Slot::first_occ).
-//   apply_first   one thread per unique key: the key's unique index (and a new
-//                 key's row) at its first occurrence, a new key's row into its
-//                 slot; init_new_rows then fills the new keys' rows from the
-//                 counter-based generator (a lane group per row).
+//                 does not depend on thread scheduling.  A tile forms its own offsets from the two levels of
+//                 counts (no scan pass).  New keys' rows go into their slots and are filled from
+//                 the counter-based generator (a lane group per row).
 //   resolve       every other occurrence takes row and unique index from its
-//                 key's first occurrence.
-//   finish        shard sizes advance, the call's scratch range is retired.
+//                 key's first occurrence; shard sizes advance, the call's scratch range is retired.
 #include "des_internal.cuh"
 
 #define IB 1024  // occurrences per block (tile) in every per-occurrence kernel of this file
@@ -45,18 +41,18 @@ __device__ __forceinline__ Slot load_slot(const Slot* p) {
 // Occurrences per thread and resident blocks per SM: one probe chain per thread at full occupancy
 // measured fastest (more chains per thread cost registers, hence warps in flight; electing one lane
 // per distinct key of a warp costs more in match instructions than the cached slot loads it saves).
-#ifndef PROBE_ILP
 #define PROBE_ILP 1
-#endif
-#ifndef PROBE_MINB
 #define PROBE_MINB 8
-#endif
+#define PROBE_MERGE_WAVES 4
+#define PROBE_MERGE 256   // entries of a block's table of first occurrences (= threads per block)
 
 struct SlotGeom {
   unsigned long long slot_base[DES_MAX_SHARDS + 1];
   uint32_t mod_M, mod_two32;        // constants of the division-free mod S (des_mod_consts)
 };   // kernel parameter: constant-bank reads
 
+// MERGE: the block merges its occurrences before the atomics (see the end of the kernel).
+template <bool MERGE>
 __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
     const unsigned long long* __restrict__ ids, const int32_t* __restrict__ offsets, int nnz, int nbags,
     int S, int F, int partition, int insert, uint32_t world, uint32_t rank, Slot* slots, DevMeta* meta,
@@ -68,6 +64,10 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
   // the bounds of the shards' slot regions, staged once per block: indexing the kernel parameter by a
   // per-lane shard would replay the constant-bank read once per distinct shard of the warp
   __shared__ uint32_t s_base[DES_MAX_SHARDS + 1];
+  __shared__ uint32_t m_slot[PROBE_MERGE], m_occ[PROBE_MERGE];
+  if (MERGE) { m_slot[threadIdx.x] = DES_SLOT_NONE; m_occ[threadIdx.x] = DES_ROW_NONE; }
+  des_pdl_wait(ids, offsets, slots, meta, slot_of, shards, rows);
+  des_pdl_go();
   if (threadIdx.x <= (unsigned)S) s_base[threadIdx.x] = (uint32_t)geom.slot_base[threadIdx.x];
   __syncthreads();
   const uint32_t base = meta->scratch_base - (uint32_t)nnz;   // this call's scratch range (Slot::first_occ)
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
       uint32_t s;
       const unsigned long long h = des_mix64(id[q]);
       if (partition == DES_PART_HASH) s = des_mod_small(h, (uint32_t)S, geom.mod_M, geom.mod_two32);
-      else s = (uint32_t)(des_bag_of(offsets, nbags, j) % F) % (unsigned)S;
+      else s = (uint32_t)(des_bag_near(offsets, nbags, nnz, j) % F) % (unsigned)S;
       shards[j] = (uint8_t)s;
       if (id[q] == DES_KEY_EMPTY) {
         des_raise(meta, DES_ERR_RESERVED_KEY);
@@ -133,17 +133,28 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
       cur[q] = done ? DES_SLOT_NONE : (cur[q] + 1 == hi[q] ? lo[q] : cur[q] + 1);
     }
   }
+  // The slot's scratch word as seen by the probe may be stale (or an earlier call's), but only ever
+  // too LARGE: skipping the atomic when it is already smaller than this occurrence's is safe.  A hot key occurs
+  // dozens of times in a block, and all blocks of a batch that fits the chip at once see the earlier
+  // call's word: 20 k occurrences of one key, 27 us of atomics on one address.  So (MERGE) a block merges its
+  // occurrences first, in a small table (an entry taken by another slot sends the atomic straight on).  In a batch of
+  // many waves the later ones find the word small already, and the barrier costs more than it saves.
 #pragma unroll
   for (int q = 0; q < PROBE_ILP; ++q) {
     const int j = j0 + q * 256;
     if (j >= nnz) continue;
-    // the slot's scratch word as seen by the probe may be stale (or an earlier call's), but only ever
-    // too LARGE: skipping the atomic when it is already smaller than this occurrence's is safe
-    if (found[q] != DES_SLOT_NONE && insert && seen_fo[q] > base + (uint32_t)j)
-      atomicMin(&slots[found[q]].first_occ, base + (uint32_t)j);
+    if (found[q] != DES_SLOT_NONE && insert && seen_fo[q] > base + (uint32_t)j) {
+      const uint32_t e = (found[q] * 0x9E3779B1u) >> 24;
+      const uint32_t old = MERGE ? atomicCAS(&m_slot[e], DES_SLOT_NONE, found[q]) : 0u;
+      if (MERGE && (old == DES_SLOT_NONE || old == found[q])) atomicMin(&m_occ[e], base + (uint32_t)j);
+      else atomicMin(&slots[found[q]].first_occ, base + (uint32_t)j);
+    }
     if (insert) slot_of[j] = found[q];
     else rows[j] = row[q];
   }
+  if (!MERGE || !insert) return;
+  __syncthreads();
+  if (m_slot[threadIdx.x] != DES_SLOT_NONE) atomicMin(&slots[m_slot[threadIdx.x]].first_occ, m_occ[threadIdx.x]);
 }
 
 // flags: bit0 = first occurrence of its key in the batch, bit1 = key is new.  This is the only pass
@@ -153,11 +164,14 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
 __global__ void __launch_bounds__(IB / 4) flag_count_kernel(
     int nnz, int S, const Slot* __restrict__ slots, const DevMeta* __restrict__ meta,
     const uint32_t* __restrict__ slot_of, const uint8_t* __restrict__ shards, uint8_t* __restrict__ flags,
-    uint32_t* __restrict__ rows, uint32_t* __restrict__ first_of, uint32_t* __restrict__ blk_cnt, int nblk_max) {
+    uint32_t* __restrict__ rows, uint32_t* __restrict__ first_of, uint32_t* __restrict__ blk_cnt,
+    uint32_t* __restrict__ sup_cnt, uint32_t* __restrict__ any_new) {
   // IB occurrences per block, IB / 4 threads: a thread's four slot look-ups are in flight together
   __shared__ uint32_t cnt[DES_MAX_SHARDS + 1];
   if (threadIdx.x <= DES_MAX_SHARDS) cnt[threadIdx.x] = 0;
   __syncthreads();
+  des_pdl_wait(slots, meta, slot_of, shards, flags, rows, first_of, blk_cnt, sup_cnt, any_new);
+  des_pdl_go();
   const uint32_t base = meta->scratch_base - (uint32_t)nnz;
   const int j0 = blockIdx.x * IB + threadIdx.x;
   uint32_t so[4];
@@ -189,212 +203,158 @@ __global__ void __launch_bounds__(IB / 4) flag_count_kernel(
     if (fl & 2) atomicAdd(&cnt[1 + shards[j]], 1u);
   }
   __syncthreads();
-  if (threadIdx.x <= S) blk_cnt[(size_t)threadIdx.x * nblk_max + blockIdx.x] = cnt[threadIdx.x];
-}
-
-// One block per sequence (sequence 0 = firsts, 1 + s = new keys of shard s):
-// in-place exclusive scan over the blocks of the batch, total to meta.
-__global__ void __launch_bounds__(1024) scan_blocks_kernel(uint32_t* blk_cnt, int nblk, int nblk_max, DevMeta* meta) {
-  // Warp w owns the contiguous chunk [w * per, (w + 1) * per) of the sequence and walks it 32 entries at a
-  // time (coalesced loads and stores, a warp scan per row, a running carry); the 32 warp totals are scanned
-  // in between, and sequences that are all zero (new keys of a shard in a populated table) are not rewritten.
-  __shared__ uint32_t wsum[32];
-  __shared__ uint32_t s_total;
-  uint32_t* seq = blk_cnt + (size_t)blockIdx.x * nblk_max;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int per = ((nblk + 31) / 32 + 31) / 32 * 32;          // entries per warp, a multiple of 32
-  const int lo = warp * per, hi = min(nblk, lo + per);
-  uint32_t sum = 0;
-  for (int i = lo + lane; i < hi; i += 32) sum += seq[i];
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
-  if (lane == 0) wsum[warp] = sum;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    uint32_t w = wsum[threadIdx.x], wi = w;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      uint32_t v = __shfl_up_sync(0xFFFFFFFFu, wi, d);
-      if (threadIdx.x >= d) wi += v;
+  if (threadIdx.x <= S) {
+    const uint32_t c = cnt[threadIdx.x];
+    blk_cnt[(size_t)blockIdx.x * (S + 1) + threadIdx.x] = c;
+    if (c) {
+      atomicAdd(sup_cnt + (size_t)(blockIdx.x / SUP_TILES) * (S + 1) + threadIdx.x, c);
+      if (threadIdx.x) *any_new = 1u;
     }
-    wsum[threadIdx.x] = wi - w;
-    if (threadIdx.x == 31) {
-      s_total = wi;
-      if (blockIdx.x == 0) meta->n_uniq = wi;
-      else { meta->new_total[blockIdx.x - 1] = wi; if (wi) atomicOr(&meta->any_new, 1u); }
-    }
-  }
-  __syncthreads();
-  if (s_total == 0u) return;                                  // an all-zero sequence is its own exclusive scan
-  uint32_t carry = wsum[warp];
-  for (int base = lo; base < hi; base += 32) {
-    const int i = base + lane;
-    const uint32_t v = (i < hi) ? seq[i] : 0u;
-    uint32_t incl = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (lane >= d) incl += o;
-    }
-    if (i < hi) seq[i] = carry + incl - v;
-    carry += __shfl_sync(0xFFFFFFFFu, incl, 31);
   }
 }
 
-// The common case of assign_kernel below — a batch without a single new key — needs the rank among the
-// first occurrences only: IB occurrences per block, four consecutive ones per thread (their flags are one
-// 32-bit load), one block-wide scan.  Runs always; when the batch does have new keys, assign_kernel
-// rewrites first_j with the new-key marks.
-__global__ void __launch_bounds__(IB / 4) assign_firsts_kernel(int nnz, const uint8_t* __restrict__ flags,
-                                                               const uint32_t* __restrict__ blk_cnt,
-                                                               uint32_t* __restrict__ first_j) {
-  __shared__ uint32_t wsum[IB / 128];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j0 = blockIdx.x * IB + threadIdx.x * 4;
+// Exclusive offset of tile `tile` in sequence c of the two-level counts (0: firsts; 1 + s: new keys of shard s), summed
+// by `n` threads of which this is the i-th (a partial sum).
+__device__ __forceinline__ uint32_t tile_offset_part(const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
+                                                     int S, int tile, int c, int i, int n) {
+  const int sup = tile / (int)SUP_TILES;
+  uint32_t v = 0;
+  for (int x = i; x < sup; x += n) v += __ldg(sup_cnt + (size_t)x * (S + 1) + c);
+#pragma unroll 4
+  for (int x = sup * (int)SUP_TILES + i; x < tile; x += n) v += __ldg(blk_cnt + (size_t)x * (S + 1) + c);
+  return v;
+}
+
+// One tile of IB occurrences per block, four consecutive ones per thread (their flags are one 32-bit load).  First
+// occurrences take the batch-unique index u = rank among firsts: uidx[] at the first occurrence,
+// uniq_rows[u] = table-global row.  New keys (bit 1 of the flag) are listed in CSR order in shared memory and ranked per
+// shard by eight warps, each over a consecutive part of the list; then lane groups fill their rows: weights from
+// the counter-based generator keyed on the id, optimizer state at its start value.
+template <int G>
+__global__ void __launch_bounds__(IB / 4) assign_kernel(
+    int nnz, int ntiles, int S, DevMeta* meta, const unsigned long long* __restrict__ ids, const uint8_t* __restrict__ shards,
+    const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
+    const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx, uint32_t* __restrict__ uniq_rows,
+    uint32_t* __restrict__ n_uniq_out, Slot* slots, unsigned long long total_slots, uint32_t max_nnz, int k, int stride,
+    float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2, unsigned long long seed, float init_scale,
+    float state_init, float lin_state_init) {
+  constexpr int NT = IB / 4, NW = NT / 32;
+  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW], n_base[DES_MAX_SHARDS];
+  __shared__ uint16_t n_warp[NW][DES_MAX_SHARDS];       // new keys per list part and shard, then running ranks
+  __shared__ uint16_t l_off[IB];                        // new keys of the tile: occurrence within the tile, ...
+  __shared__ uint8_t l_shard[IB];
+  __shared__ uint32_t l_grow[IB];                       // ... batch-unique index, then table-global row
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tile = blockIdx.x, j0 = tile * IB + tid * 4;
+  des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2);
+  des_pdl_go();
+  // The slots' scratch range ends with this call (see Slot::first_occ; resolve_kernel then starts a new one): nothing
+  // reads the scratch words after flag_count_kernel, so they are all cleared here, once every few billion occurrences.
+  if (meta->scratch_base - (uint32_t)nnz < max_nnz)
+    for (unsigned long long i = (unsigned long long)blockIdx.x * NT + tid; i < total_slots; i += (unsigned long long)gridDim.x * NT)
+      slots[i].first_occ = DES_ROW_NONE;
   uint32_t w = 0;
-  if (j0 + 3 < nnz) w = *reinterpret_cast<const uint32_t*>(flags + j0);
+  if (j0 + 3 < nnz) w = __ldg(reinterpret_cast<const uint32_t*>(flags + j0));
   else for (int q = 0; q < 4; ++q) if (j0 + q < nnz) w |= (uint32_t)flags[j0 + q] << (8 * q);
-  w &= 0x01010101u;                                           // bit 0 of each flag: first occurrence of its key
-  const uint32_t cnt = __popc(w);
-  uint32_t incl = cnt;
+  uint32_t before = tile_offset_part(blk_cnt, sup_cnt, S, tile, 0, tid, NT);
+  const uint32_t wf = w & 0x01010101u, wn = w & 0x02020202u, cf = __popc(wf), cn = __popc(wn);
+  // what the first occurrences need, in flight while the ranks are formed
+  uint32_t r[4]; uint32_t sh[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const bool f = (wf >> (8 * q)) & 1u;
+    r[q] = f ? rows[j0 + q] : DES_ROW_NONE;
+    sh[q] = f ? __ldg(shards + j0 + q) : 0u;
+  }
+  uint32_t incl = cf | cn << 16;                        // (at most 1024 of each in a tile)
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
     if (lane >= d) incl += v;
   }
-  if (lane == 31) wsum[warp] = incl;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, d);
+  if (lane == 31) { wsum[warp] = incl & 0xFFFFu; wnew[warp] = incl >> 16; }
+  if (lane == 0) wbase[warp] = before;
   __syncthreads();
-  uint32_t before = 0;
-  for (int i = 0; i < warp; ++i) before += wsum[i];
-  uint32_t u = blk_cnt[blockIdx.x] + before + incl - cnt;
+  uint32_t u = (incl & 0xFFFFu) - cf, nrank = (incl >> 16) - cn, tile_firsts = 0, n_new = 0;
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if ((w >> (8 * q)) & 1u) first_j[u++] = (uint32_t)(j0 + q);
-}
-
-// New keys only: first_j[u] gets bit 31 and uniq_rows[u] the key's shard-local row (rank among the
-// shard's new keys on top of the shard's size).  The random slot
-// accesses are left to apply_first_kernel, which runs one thread per unique key.
-__global__ void __launch_bounds__(IB) assign_kernel(
-    int nnz, int nblk, int S, DevMeta* meta, const uint8_t* __restrict__ shards, const uint8_t* __restrict__ flags,
-    const uint32_t* __restrict__ blk_cnt, int nblk_max, uint32_t* __restrict__ first_j,
-    uint32_t* __restrict__ uniq_rows, Slot* slots, unsigned long long total_slots, uint32_t max_nnz) {
-  __shared__ uint32_t wfirst[32];
-  __shared__ uint16_t wnew[32][DES_MAX_SHARDS];
-  // The slots' scratch range ends with this call (see Slot::first_occ; finish_kernel then starts a new one):
-  // nothing reads the scratch words after flag_count_kernel, so this kernel — a few blocks that are idle
-  // in the steady state — clears them all, once every few billion occurrences.
-  if (meta->scratch_base - (uint32_t)nnz < max_nnz)
-    for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < total_slots;
-         i += (unsigned long long)gridDim.x * blockDim.x)
-      slots[i].first_occ = DES_ROW_NONE;
-  // steady state of a populated table: no new key in the whole batch (settled by scan_blocks_kernel, which
-  // ran before this kernel), and assign_firsts_kernel has done all there is to do
-  if (meta->any_new == 0u) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lt = (1u << lane) - 1u;
-  for (int tile = blockIdx.x; tile < nblk; tile += gridDim.x) {   // a few resident blocks walk the tiles
-    const int j = tile * IB + threadIdx.x;
-    const uint8_t fl = (j < nnz) ? flags[j] : 0;
-    const uint32_t s = (j < nnz) ? shards[j] : 0;
-    for (int i = threadIdx.x; i < 32 * DES_MAX_SHARDS; i += IB) (&wnew[0][0])[i] = 0;
-    __syncthreads();
-    // rank among firsts / among the shard's new keys inside the warp (lane order = CSR order)
-    const unsigned fmask = __ballot_sync(0xFFFFFFFFu, fl & 1);
-    const uint32_t frank = __popc(fmask & lt);
-    const unsigned nmask_all = __ballot_sync(0xFFFFFFFFu, fl & 2);
-    uint32_t nrank = 0;
-    if (fl & 2) {
-      unsigned same = __match_any_sync(nmask_all, s);
-      nrank = __popc(same & lt);
-      if ((same >> lane) == 1u) wnew[warp][s] = (uint16_t)__popc(same);   // highest lane of the group
-    }
-    if (lane == 0) wfirst[warp] = __popc(fmask);
-    __syncthreads();
-    // exclusive prefix over warps
-    if (threadIdx.x < 32) {
-      uint32_t v = wfirst[threadIdx.x], in = v;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        uint32_t o = __shfl_up_sync(0xFFFFFFFFu, in, d);
-        if (threadIdx.x >= d) in += o;
-      }
-      wfirst[threadIdx.x] = in - v;
-    } else if (threadIdx.x >= 64 && threadIdx.x < 64 + S) {
-      const int sh = threadIdx.x - 64;
-      uint32_t run = 0;
-      for (int w = 0; w < 32; ++w) { uint16_t v = wnew[w][sh]; wnew[w][sh] = (uint16_t)run; run += v; }
-    }
-    __syncthreads();
-    if (fl & 2) {                                     // (first_j of the other firsts is already in place)
-      const uint32_t u = blk_cnt[tile] + wfirst[warp] + frank;
-      uint32_t local = meta->n_rows[s] + blk_cnt[(size_t)(1 + s) * nblk_max + tile] + wnew[warp][s] + nrank;
-      if (local >= meta->row_cap[s]) { local = DES_ROW_NONE; des_raise(meta, DES_ERR_CAPACITY); }
-      uniq_rows[u] = local;
-      first_j[u] = (uint32_t)j | 0x80000000u;
-    }
-    __syncthreads();                                  // the shared tables are reused by the next tile
+  for (int i = 0; i < NW; ++i) {
+    u += wbase[i] + (i < warp ? wsum[i] : 0u);
+    nrank += i < warp ? wnew[i] : 0u;
+    tile_firsts += wsum[i] + wbase[i];
+    n_new += wnew[i];
   }
-}
-
-// One thread per unique key of the batch: a new key's row number goes into its slot (the only slot
-// access) and into rows[] at its first occurrence; the first occurrence also takes the key's batch-unique
-// index (resolve_kernel hands both on to the key's other occurrences); uniq_rows gets the table-global row.
-__global__ void __launch_bounds__(256) apply_first_kernel(
-    Slot* slots, const DevMeta* __restrict__ meta, const uint32_t* __restrict__ slot_of,
-    const uint8_t* __restrict__ shards, const uint32_t* __restrict__ first_j, uint32_t* __restrict__ rows,
-    uint32_t* __restrict__ uidx, uint32_t* __restrict__ uniq_rows) {
-  const uint32_t U = meta->n_uniq;
-  for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < U; u += gridDim.x * blockDim.x) {
-    const uint32_t fj = first_j[u];
-    const bool is_new = fj >> 31;
-    const uint32_t j = fj & 0x7FFFFFFFu;
-    if (!DES_DBG_OCC_OK(j)) continue;                  // (checking build)
-    const uint32_t s = shards[j];
-    uint32_t local;
-    if (is_new) {
-      local = uniq_rows[u];                            // DES_ROW_NONE: the shard is full
-      if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(slot_of[j])) slots[slot_of[j]].row = local;
-      rows[j] = local;
+  if (tile == ntiles - 1 && tid == 0) { meta->n_uniq = tile_firsts; *n_uniq_out = tile_firsts; }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (!((wf >> (8 * q)) & 1u)) continue;
+    if ((wn >> (8 * q)) & 2u) {
+      l_off[nrank] = (uint16_t)(tid * 4 + q); l_shard[nrank] = (uint8_t)sh[q]; l_grow[nrank] = u;
+      ++nrank;
     } else {
-      local = rows[j];
+      uidx[j0 + q] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : u;
+      uniq_rows[u] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : (uint32_t)(meta->row_base[sh[q]] + r[q]);
     }
-    uidx[j] = (local == DES_ROW_NONE) ? DES_ROW_NONE : u;
-    const unsigned long long g = meta->row_base[s] + local;
-    uniq_rows[u] = (local == DES_ROW_NONE) ? DES_ROW_NONE : (uint32_t)g;
+    ++u;
   }
-}
-
-// Rows of the batch's new keys: weights from the counter-based generator keyed on the id, optimizer state
-// at its start value.  G lanes per unique key (one 16-byte column each); keys that are not new cost one
-// load.  uniq_rows[u] already holds the table-global row (apply_first_kernel).
-template <int G>
-__global__ void __launch_bounds__(256) init_new_rows_kernel(
-    const unsigned long long* __restrict__ ids, int k, int stride, const DevMeta* __restrict__ meta,
-    const uint32_t* __restrict__ first_j, const uint32_t* __restrict__ uniq_rows, float* __restrict__ W,
-    float* __restrict__ A, float* __restrict__ A2, unsigned long long seed, float init_scale, float state_init,
-    float lin_state_init) {
-  if (meta->any_new == 0u) return;                     // steady state of a populated table: nothing to initialise
-  const uint32_t U = meta->n_uniq;
-  const int K4 = k >> 2, c4 = threadIdx.x % G;
-  const long long gstep = (long long)gridDim.x * (256 / G);
-  // every lane of a warp runs the same number of rounds (the squared norm is a warp-level sum)
-  const long long rounds = ((long long)U + gstep - 1) / gstep;
-  long long u = (long long)blockIdx.x * (256 / G) + threadIdx.x / G;
-  for (long long r = 0; r < rounds; ++r, u += gstep) {
-    uint32_t fj = 0, grow = DES_ROW_NONE;
-    if (u < U) { fj = first_j[u]; if (fj >> 31) grow = uniq_rows[u]; }
+  if (n_new == 0) return;                               // (whole block) the steady state of a populated table
+  // ---- new keys: rank among the shard's new keys, on top of the shard's size
+  for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&n_warp[0][0])[i] = 0;
+  if (tid < DES_MAX_SHARDS) n_base[tid] = tid < S ? meta->n_rows[tid] : 0u;
+  __syncthreads();
+  for (int i = tid; i < S * (NT / DES_MAX_SHARDS); i += NT) {
+    const uint32_t v = tile_offset_part(blk_cnt, sup_cnt, S, tile, 1 + i % S, i / S, NT / DES_MAX_SHARDS);
+    if (v) atomicAdd(&n_base[i % S], v);
+  }
+  const int per = (((int)n_new + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min((int)n_new, lo + per);
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i0 = lo; i0 < hi; i0 += 32) {
+      const int i = i0 + lane;
+      const int key = i < hi ? (int)l_shard[i] : -1;
+      const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+      const uint32_t at = i < hi ? n_warp[warp][key] : 0u;
+      __syncwarp();
+      if (i < hi && (same >> lane) == 1u) n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
+      if (pass == 1 && i < hi) {
+        uint32_t local = n_base[key] + at + __popc(same & ((1u << lane) - 1u));
+        if (local >= meta->row_cap[key]) { local = DES_ROW_NONE; des_raise(meta, DES_ERR_CAPACITY); }
+        const int j = tile * IB + l_off[i];
+        const uint32_t uu = l_grow[i];
+        const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : (uint32_t)(meta->row_base[key] + local);
+        if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(slot_of[j])) slots[slot_of[j]].row = local;
+        rows[j] = local;
+        uidx[j] = local == DES_ROW_NONE ? DES_ROW_NONE : uu;
+        uniq_rows[uu] = grow;
+        l_grow[i] = grow;
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    if (pass == 0) {                                     // counts of the list parts -> where each part starts
+      if (tid < S) {
+        uint32_t run = 0;
+        for (int i = 0; i < NW; ++i) { const uint16_t v = n_warp[i][tid]; n_warp[i][tid] = (uint16_t)run; run += v; }
+      }
+      __syncthreads();
+    }
+  }
+  // ---- their rows: G lanes per row, every lane of a warp runs the same rounds (the squared norm is a warp-level sum)
+  const int K4 = k >> 2, c4 = tid % G;
+  const float stamp = des_stamp_bits(meta->clock + 1ull);   // the clock value this call ends with
+  for (int i0 = 0; i0 < (int)n_new; i0 += NT / G) {
+    const int i = i0 + tid / G;
+    const uint32_t grow = i < (int)n_new ? l_grow[i] : DES_ROW_NONE;
     const bool init = grow != DES_ROW_NONE;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (init && c4 < K4) v = des_init4(seed, ids[fj & 0x7FFFFFFFu], (uint32_t)c4, init_scale);
+    if (init && c4 < K4) v = des_init4(seed, __ldg(ids + tile * IB + l_off[i]), (uint32_t)c4, init_scale);
     float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
 #pragma unroll
     for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
     if (!init || DES_DBG_ROW(grow) != grow) continue;
-    float4* w = reinterpret_cast<float4*>(W + (size_t)grow * stride);
-    if (c4 < K4) w[c4] = v;
-    // linear weight, squared norm of the latent vector, age stamp (the clock value this call ends with)
-    if (c4 == 0) w[K4] = make_float4(0.f, n2, des_stamp_bits(meta->clock + 1ull), 0.f);
+    float4* wr = reinterpret_cast<float4*>(W + (size_t)grow * stride);
+    if (c4 < K4) wr[c4] = v;
+    if (c4 == 0) wr[K4] = make_float4(0.f, n2, stamp, 0.f);   // linear weight, squared norm, age stamp
     if (A) {
       float4* a = reinterpret_cast<float4*>(A + (size_t)grow * stride);
       if (c4 < K4) a[c4] = make_float4(state_init, state_init, state_init, state_init);
@@ -411,9 +371,37 @@ __global__ void __launch_bounds__(256) init_new_rows_kernel(
 // Every occurrence that is not its key's first one takes the unique index — and, for a key that was new,
 // the row — from the first one (a look-up in the batch's own arrays, not in the table).  IB occurrences per
 // block, IB / 4 threads: a thread's four look-ups are in flight together.  First occurrences are only read
-// here (apply_first_kernel wrote them), the others only written.
-__global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, const uint32_t* __restrict__ first_of,
-                                                         uint32_t* rows, uint32_t* uidx, DevMeta* meta) {
+// here (assign_kernel wrote them), the others only written.  One more block ends the call: shard sizes advance, the
+// counts are cleared for the next call, the scratch range is retired.
+__global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, int S, uint32_t max_nnz,
+                                                         const uint32_t* __restrict__ first_of, uint32_t* rows, uint32_t* uidx,
+                                                         uint32_t* __restrict__ sup_cnt, DevMeta* meta) {
+  des_pdl_wait(first_of, rows, uidx, sup_cnt, meta);
+  des_pdl_go();
+  if ((int)blockIdx.x == ntiles) {
+    const int nsup = (ntiles + (int)SUP_TILES - 1) / (int)SUP_TILES;
+    for (int c = threadIdx.x; c <= S; c += IB / 4) {
+      uint32_t total = 0;
+      if (c == 0 || meta->any_new) {
+#pragma unroll 8
+        for (int i = 0; i < nsup; ++i) {
+          total += sup_cnt[(size_t)i * (S + 1) + c];
+          sup_cnt[(size_t)i * (S + 1) + c] = 0u;
+        }
+      }
+      if (c) meta->n_rows[c - 1] = min(meta->n_rows[c - 1] + total, meta->row_cap[c - 1]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      meta->any_new = 0u;
+      meta->clock += 1ull;
+      const uint32_t base = meta->scratch_base - (uint32_t)nnz;
+      // the next call may need up to max_nnz below the base; if that is not left, assign_kernel has
+      // cleared every slot's scratch word in this call and the range starts again at the top
+      meta->scratch_base = base < max_nnz ? 0xFFFFFFFFu : base;
+    }
+    return;
+  }
   const int j0 = blockIdx.x * IB + threadIdx.x;
   uint32_t f[4], r[4], u[4];
   bool newrow[4];                                      // the occurrence's row comes from the first occurrence
@@ -445,24 +433,6 @@ __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, const uint32_t
   }
 }
 
-// One block: shard sizes advance, the call's scratch range is retired.
-__global__ void __launch_bounds__(DES_MAX_SHARDS) finish_kernel(int S, int nnz, uint32_t max_nnz, DevMeta* meta,
-                                                                uint32_t* n_uniq_out) {
-  if ((int)threadIdx.x < S) {
-    uint32_t n = meta->n_rows[threadIdx.x] + meta->new_total[threadIdx.x];
-    meta->n_rows[threadIdx.x] = min(n, meta->row_cap[threadIdx.x]);
-  }
-  if (threadIdx.x == 0) {
-    *n_uniq_out = meta->n_uniq;
-    meta->any_new = 0u;
-    meta->clock += 1ull;
-    const uint32_t base = meta->scratch_base - (uint32_t)nnz;
-    // the next call may need up to max_nnz below the base; if that is not left, assign_kernel has
-    // cleared every slot's scratch word in this call and the range starts again at the top
-    meta->scratch_base = base < max_nnz ? 0xFFFFFFFFu : base;
-  }
-}
-
 extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b, int insert, void* stream) {
   des_status_t st = des_check_batch(t, b, insert);
   if (st != DES_OK) return st;
@@ -476,46 +446,37 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
     if (insert) DES_CUDA(cudaMemsetAsync(b->n_uniq, 0, 4, cs));
     return DES_OK;
   }
-  const int nblk = (nnz + IB - 1) / IB;
+  const int ntiles = (nnz + IB - 1) / IB;
   SlotGeom geom;
   for (uint32_t s = 0; s <= t->S; ++s) geom.slot_base[s] = t->h_slot_base[s];
   des_mod_consts(t->S, &geom.mod_M, &geom.mod_two32);
-  probe_claim_kernel<<<(nnz + 256 * PROBE_ILP - 1) / (256 * PROBE_ILP), 256, 0, cs>>>((const unsigned long long*)b->ids, b->offsets, nnz, nbags, t->S, t->F,
-                                          t->cfg.partition, insert, t->cfg.shard_world, t->cfg.shard_rank, t->slots, t->meta, geom,
-                                          t->slot_of, b->shards, b->rows);
+  const bool merge = nnz <= PROBE_MERGE_WAVES * t->sm_count * PROBE_MINB * 256;
+  des_launch(merge ? probe_claim_kernel<true> : probe_claim_kernel<false>, (nnz + 256 * PROBE_ILP - 1) / (256 * PROBE_ILP), 256, 0, cs, (const unsigned long long*)b->ids,
+             b->offsets, nnz, nbags, (int)t->S, (int)t->F, (int)t->cfg.partition, insert, t->cfg.shard_world, t->cfg.shard_rank,
+             t->slots, t->meta, geom, t->slot_of, b->shards, b->rows);
   DES_LAUNCH_CHECK(t, "probe_claim_kernel");
   if (!insert) return DES_OK;
   uint32_t* first_of = t->uslot;
-  flag_count_kernel<<<nblk, IB / 4, 0, cs>>>(nnz, t->S, t->slots, t->meta, t->slot_of, b->shards, t->flags, b->rows,
-                                             first_of, t->blk_cnt, t->nblk_max);
+  des_launch(flag_count_kernel, ntiles, IB / 4, 0, cs, nnz, (int)t->S, t->slots, t->meta, t->slot_of, b->shards, t->flags,
+             b->rows, first_of, t->blk_cnt, t->sup_cnt, &t->meta->any_new);
   DES_LAUNCH_CHECK(t, "flag_count_kernel");
-  scan_blocks_kernel<<<t->S + 1, 1024, 0, cs>>>(t->blk_cnt, nblk, t->nblk_max, t->meta);
-  DES_LAUNCH_CHECK(t, "scan_blocks_kernel");
-  assign_firsts_kernel<<<nblk, IB / 4, 0, cs>>>(nnz, t->flags, t->blk_cnt, t->dest);
-  DES_LAUNCH_CHECK(t, "assign_firsts_kernel");
-  assign_kernel<<<nblk < t->sm_count * 2 ? nblk : t->sm_count * 2, IB, 0, cs>>>(nnz, nblk, t->S, t->meta, b->shards, t->flags,
-                                                                                t->blk_cnt, t->nblk_max, t->dest, b->uniq_rows,
-                                                                                t->slots, t->total_slots, (uint32_t)t->max_nnz);
-  DES_LAUNCH_CHECK(t, "assign_kernel");
-  apply_first_kernel<<<t->sm_count * 8, 256, 0, cs>>>(t->slots, t->meta, t->slot_of, b->shards, t->dest, b->rows,
-                                                      b->uidx, b->uniq_rows);
-  DES_LAUNCH_CHECK(t, "apply_first_kernel");
   {
     const float state_init = t->cfg.optimizer == DES_OPT_ADAGRAD ? t->cfg.init_acc : 0.f;
     const float lin_state_init =
         (t->cfg.lin_optimizer == DES_LIN_FTRL || t->cfg.optimizer != DES_OPT_ADAGRAD) ? 0.f : t->cfg.init_acc;
     int G = 1;
     while (G < (int)t->k / 4) G <<= 1;
-#define INIT(GG) init_new_rows_kernel<GG><<<t->sm_count * 8, 256, 0, cs>>>(                                            \
-        (const unsigned long long*)b->ids, t->k, t->stride, t->meta, t->dest, b->uniq_rows, t->W, t->A, t->A2,         \
-        t->cfg.seed, t->cfg.init_scale, state_init, lin_state_init)
-    switch (G) { case 1: INIT(1); break; case 2: INIT(2); break; case 4: INIT(4); break; case 8: INIT(8); break; default: INIT(16); }
-#undef INIT
-    DES_LAUNCH_CHECK(t, "init_new_rows_kernel");
+#define ASSIGN(GG) des_launch(assign_kernel<GG>, ntiles, IB / 4, 0, cs, nnz, ntiles, (int)t->S, t->meta,                  \
+        (const unsigned long long*)b->ids, b->shards, t->flags, t->blk_cnt, t->sup_cnt, t->slot_of, b->rows, b->uidx,   \
+        b->uniq_rows, b->n_uniq, t->slots, t->total_slots, (uint32_t)t->max_nnz, (int)t->k, (int)t->stride, t->W, t->A, \
+        t->A2, t->cfg.seed, t->cfg.init_scale, state_init, lin_state_init)
+    switch (G) { case 1: ASSIGN(1); break; case 2: ASSIGN(2); break; case 4: ASSIGN(4); break; case 8: ASSIGN(8); break;
+                 default: ASSIGN(16); }
+#undef ASSIGN
+    DES_LAUNCH_CHECK(t, "assign_kernel");
   }
-  resolve_kernel<<<nblk, IB / 4, 0, cs>>>(nnz, first_of, b->rows, b->uidx, t->meta);
+  des_launch(resolve_kernel, ntiles + 1, IB / 4, 0, cs, nnz, ntiles, (int)t->S, (uint32_t)t->max_nnz, first_of, b->rows, b->uidx,
+             t->sup_cnt, t->meta);
   DES_LAUNCH_CHECK(t, "resolve_kernel");
-  finish_kernel<<<1, DES_MAX_SHARDS, 0, cs>>>(t->S, nnz, (uint32_t)t->max_nnz, t->meta, b->n_uniq);
-  DES_LAUNCH_CHECK(t, "finish_kernel");
   return DES_OK;
 }

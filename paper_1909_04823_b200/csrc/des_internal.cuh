@@ -11,6 +11,8 @@
 #define DES_SLOT_NONE 0xFFFFFFFFu
 #define HOT_RCHUNK 16u     // replica rows of a hot key summed by one warp of the backward's replica reduction
 
+#define SUP_TILES 256u     // tiles of find_or_insert per second-level counter
+
 // The few keys that own a large share of a skewed batch ("super" keys) are counted instead of scattered in the
 // backward: a tagged occurrence carries SUPER_TAG | slot where other occurrences carry a gradient row number.
 #define SUPER_T 16u             // slots
@@ -43,7 +45,6 @@ struct DevMeta {
   unsigned long long slot_base[DES_MAX_SHARDS + 1];  // first slot of shard s's region
   uint32_t row_cap[DES_MAX_SHARDS];                  // row capacity of shard s
   uint32_t n_rows[DES_MAX_SHARDS];                   // rows in use
-  uint32_t new_total[DES_MAX_SHARDS];                // new keys of the running insert call
   uint32_t n_uniq;                                   // unique keys of the running insert call
   uint32_t err;                                      // sticky des_status_t raised on device
   uint32_t any_new;                                  // the running insert call has at least one new key
@@ -84,7 +85,8 @@ struct des_table {
   uint32_t* slot_of;                 // [max_nnz]
   uint8_t* flags;                    // [max_nnz]
   uint32_t* uslot;                   // [max_nnz]
-  uint32_t* blk_cnt;                 // [(S+1)][nblk_max]
+  uint32_t* blk_cnt;                 // [nblk_max][S+1] per tile: first occurrences, new keys per shard
+  uint32_t* sup_cnt;                 // [nsup_max][S+1] the same per SUP_TILES tiles; zero between calls
   int32_t* seg_off;                  // [max_batch][S+1] forward routing: (sample, shard) segment bounds
   // backward workspace
   float* Gbuf;                       // [max_uniq + rep_max][stride]: per-unique gradient rows, then
@@ -133,6 +135,35 @@ struct des_table {
 int des_prof_mark(des_table* t, const char* name, int check);
 void des_api_begin(des_table* t, cudaStream_t cs);
 #define DES_LAUNCH_CHECK(t, name) do { if (des_prof_mark((t), (name), 1)) return DES_ERR_CUDA; } while (0)
+
+// Kernels of a step follow one another on a stream and are often only a few microseconds long, so they are
+// launched with programmatic stream serialisation: a kernel's blocks may be set up while the kernel before it drains, and
+// wait in des_pdl_wait for that kernel's completion (memory included) before they touch anything.  EVERY
+// kernel launched through des_launch starts with that wait.  It takes ALL pointers that the kernel reads
+// through: a read-only load (__ldg, const __restrict__) may be moved by the compiler across a mere memory barrier, to
+// before the wait, so the pointers come out of it as new values.  des_pdl_go lets the next kernel be set
+// up; it waits for this one's end all the same.
+template <typename P>
+__device__ __forceinline__ void des_pdl_new(P& p) {
+  static_assert(sizeof(P) == 8, "pointers only");
+  asm volatile("" : "+l"(p)::"memory");
+}
+template <typename... P>
+__device__ __forceinline__ void des_pdl_wait(P&... p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (des_pdl_new(p), ...);
+}
+__device__ __forceinline__ void des_pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+static inline void des_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, (P)args...);        // (errors are picked up by DES_LAUNCH_CHECK)
+}
 
 // ---- device helpers ---------------------------------------------------------
 
@@ -200,6 +231,13 @@ __device__ __forceinline__ int des_bag_of(const int32_t* __restrict__ offsets, i
     if (__ldg(offsets + mid) <= j) lo = mid; else hi = mid;
   }
   return lo;
+}
+
+// The same with a first look at bag j, where one-hot batches (one occurrence per bag) have it: the binary search is a chain
+// of twenty dependent loads at half a million bags, more than the rest of a probe.
+__device__ __forceinline__ int des_bag_near(const int32_t* __restrict__ offsets, int nbags, int nnz, int j) {
+  if (nbags == nnz && __ldg(offsets + j) == j && __ldg(offsets + j + 1) == j + 1) return j;
+  return des_bag_of(offsets, nbags, j);
 }
 
 __device__ __forceinline__ void des_raise(DevMeta* meta, uint32_t code) { atomicCAS(&meta->err, 0u, code); }

@@ -101,7 +101,7 @@ extern "C" des_status_t des_table_destroy(des_table_t* t) {
   if (cudaGetDevice(&caller_dev) != cudaSuccess) { cudaGetLastError(); caller_dev = -1; }
   cudaSetDevice(t->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {t->slots, t->W, t->A, t->A2, t->acc2W1, t->meta, t->slot_of, t->flags, t->uslot, t->blk_cnt, t->seg_off, t->Gbuf, t->hinfo, t->dest, t->hot_base,
+  void* ptrs[] = {t->slots, t->W, t->A, t->A2, t->acc2W1, t->meta, t->slot_of, t->flags, t->uslot, t->blk_cnt, t->sup_cnt, t->seg_off, t->Gbuf, t->hinfo, t->dest, t->hot_base,
                   t->hot_R, t->hot_u, t->hot_ctr, t->hot_work, t->hot_acc, t->super_cnt, t->x_sorted, t->bag_tail,
                   t->W1, t->accW1, t->W1b, t->gW1_part, t->pooled_b, t->gZ_b, t->gemm_ws, t->st_offsets[0], t->st_ids[0], t->st_vals[0], t->st_offsets[1], t->st_ids[1], t->st_vals[1], t->st_rows,
                   t->st_shards, t->st_uidx, t->st_uniq_rows, t->st_n_uniq, t->st_part_small, t->st_out_small};
@@ -198,6 +198,8 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
   A(t->flags, (size_t)t->max_nnz);
   A(t->uslot, (size_t)t->max_nnz * 4);
   A(t->blk_cnt, (size_t)(t->S + 1) * t->nblk_max * 4);
+  const size_t sup_bytes = (size_t)(t->S + 1) * (t->nblk_max / SUP_TILES + 1) * 4;
+  A(t->sup_cnt, sup_bytes);
   A(t->seg_off, (size_t)t->max_batch * (t->S + 1) * 4);
   t->hot_max = 16384;
   t->rep_max = (uint32_t)(t->max_nnz / 256 + t->hot_max + 1024);
@@ -233,6 +235,7 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
   cu &= cudaMemset(t->slots, 0xFF, slots * sizeof(Slot)) == cudaSuccess;
   cu &= cudaMemset(t->W + rows * t->stride, 0, rowbytes) == cudaSuccess;
   cu &= cudaMemset(t->Gbuf, 0, ((size_t)t->max_uniq + t->rep_max) * rowbytes) == cudaSuccess;
+  cu &= cudaMemset(t->sup_cnt, 0, sup_bytes) == cudaSuccess;
   cu &= cudaMemset(t->hinfo, 0, (size_t)t->max_uniq * 4) == cudaSuccess;
   cu &= cudaMemset(t->hot_acc, 0, (size_t)t->hot_max * t->stride * 8) == cudaSuccess;
   cu &= cudaMemcpy(t->meta, &hm, sizeof(hm), cudaMemcpyHostToDevice) == cudaSuccess;
