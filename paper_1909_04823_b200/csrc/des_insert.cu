@@ -24,6 +24,9 @@
 //                 key's first occurrence; shard sizes advance, the call's scratch range is retired.
 #include "des_internal.cuh"
 
+#include <type_traits>
+
+#define ASSIGN_DEEP_TILES 16   // tiles per SM from which a block of assign_kernel takes four of them
 #define IB 1024  // occurrences per block (tile) in every per-occurrence kernel of this file
 
 // A probe may read a slot through L1 although other SMs claim slots meanwhile: a key never changes once
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(IB / 4) flag_count_kernel(
     int nnz, int S, const Slot* __restrict__ slots, const DevMeta* __restrict__ meta,
     const uint32_t* __restrict__ slot_of, const uint8_t* __restrict__ shards, uint8_t* __restrict__ flags,
     uint32_t* __restrict__ rows, uint32_t* __restrict__ first_of, uint32_t* __restrict__ blk_cnt,
-    uint32_t* __restrict__ sup_cnt, uint32_t* __restrict__ any_new) {
+    uint32_t* __restrict__ sup_cnt, int nblk_max, int nsup_max, uint32_t* __restrict__ any_new) {
   // IB occurrences per block, IB / 4 threads: a thread's four slot look-ups are in flight together
   __shared__ uint32_t cnt[DES_MAX_SHARDS + 1];
   if (threadIdx.x <= DES_MAX_SHARDS) cnt[threadIdx.x] = 0;
@@ -205,47 +208,54 @@ __global__ void __launch_bounds__(IB / 4) flag_count_kernel(
   __syncthreads();
   if (threadIdx.x <= S) {
     const uint32_t c = cnt[threadIdx.x];
-    blk_cnt[(size_t)blockIdx.x * (S + 1) + threadIdx.x] = c;
+    const int s = (int)threadIdx.x - 1;                 // -1: firsts
+    uint32_t* bc = s < 0 ? blk_cnt + blockIdx.x : blk_cnt + nblk_max + (size_t)blockIdx.x * S + s;
+    uint32_t* sc = s < 0 ? sup_cnt + blockIdx.x / SUP_TILES : sup_cnt + nsup_max + (size_t)(blockIdx.x / SUP_TILES) * S + s;
+    *bc = c;
     if (c) {
-      atomicAdd(sup_cnt + (size_t)(blockIdx.x / SUP_TILES) * (S + 1) + threadIdx.x, c);
-      if (threadIdx.x) *any_new = 1u;
+      atomicAdd(sc, c);
+      if (s >= 0) *any_new = 1u;
     }
   }
 }
 
-// Exclusive offset of tile `tile` in sequence c of the two-level counts (0: firsts; 1 + s: new keys of shard s), summed
-// by `n` threads of which this is the i-th (a partial sum).
+// Exclusive offset of tile `tile` in one sequence of the two-level counts, summed by `n` threads of which this is the
+// i-th (a partial sum).  The firsts' counts are dense (step 1), those of the new keys [tile][S] (step S).
 __device__ __forceinline__ uint32_t tile_offset_part(const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
-                                                     int S, int tile, int c, int i, int n) {
+                                                     int step, int tile, int i, int n) {
   const int sup = tile / (int)SUP_TILES;
   uint32_t v = 0;
-  for (int x = i; x < sup; x += n) v += __ldg(sup_cnt + (size_t)x * (S + 1) + c);
+  for (int x = i; x < sup; x += n) v += __ldg(sup_cnt + (size_t)x * step);
 #pragma unroll 4
-  for (int x = sup * (int)SUP_TILES + i; x < tile; x += n) v += __ldg(blk_cnt + (size_t)x * (S + 1) + c);
+  for (int x = sup * (int)SUP_TILES + i; x < tile; x += n) v += __ldg(blk_cnt + (size_t)x * step);
   return v;
 }
 
-// One tile of IB occurrences per block, four consecutive ones per thread (their flags are one 32-bit load).  First
+// PER consecutive occurrences per thread: a block covers M = 512 PER / IB counting tiles.  First
 // occurrences take the batch-unique index u = rank among firsts: uidx[] at the first occurrence,
-// uniq_rows[u] = table-global row.  New keys (bit 1 of the flag) are listed in CSR order in shared memory and ranked per
-// shard by eight warps, each over a consecutive part of the list; then lane groups fill their rows: weights from
-// the counter-based generator keyed on the id, optimizer state at its start value.
-template <int G>
-__global__ void __launch_bounds__(IB / 4) assign_kernel(
+// uniq_rows[u] = table-global row.  New keys (bit 1 of the flag) are listed in CSR order in shared memory, up to IB at a time,
+// and ranked per shard by the block's warps, each over a consecutive part of the list; then lane groups fill their
+// rows: weights from the counter-based generator keyed on the id, optimizer state at its start value.
+// PER = 2 gives a small batch enough blocks (and a batch of new keys enough lane groups: 400 k new keys of k = 64
+// take 120 us, 190 us with 256 threads a tile); PER = 8 spreads a block's latency over four times the
+// occurrences once every SM has several blocks (32 M occurrences: 212 -> 70 us).
+template <int G, int PER>
+__global__ void __launch_bounds__(512) assign_kernel(
     int nnz, int ntiles, int S, DevMeta* meta, const unsigned long long* __restrict__ ids, const uint8_t* __restrict__ shards,
     const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
-    const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx, uint32_t* __restrict__ uniq_rows,
-    uint32_t* __restrict__ n_uniq_out, Slot* slots, unsigned long long total_slots, uint32_t max_nnz, int k, int stride,
-    float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2, unsigned long long seed, float init_scale,
-    float state_init, float lin_state_init) {
-  constexpr int NT = IB / 4, NW = NT / 32;
-  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW], n_base[DES_MAX_SHARDS];
+    int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx,
+    uint32_t* __restrict__ uniq_rows, uint32_t* __restrict__ n_uniq_out, Slot* slots, unsigned long long total_slots,
+    uint32_t max_nnz, int k, int stride, float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2,
+    unsigned long long seed, float init_scale, float state_init, float lin_state_init) {
+  constexpr int NT = 512, NW = NT / 32, M = NT * PER / IB;
+  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW], n_base[DES_MAX_SHARDS], s_cap[DES_MAX_SHARDS], s_row[DES_MAX_SHARDS];
   __shared__ uint16_t n_warp[NW][DES_MAX_SHARDS];       // new keys per list part and shard, then running ranks
-  __shared__ uint16_t l_off[IB];                        // new keys of the tile: occurrence within the tile, ...
+  __shared__ uint16_t l_off[IB];                        // listed new keys: occurrence within the block's range, ...
   __shared__ uint8_t l_shard[IB];
+  __shared__ uint32_t l_slot[IB];
   __shared__ uint32_t l_grow[IB];                       // ... batch-unique index, then table-global row
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tile = blockIdx.x, j0 = tile * IB + tid * 4;
+  const int tile0 = blockIdx.x * M, jb = tile0 * IB, j0 = jb + tid * PER;
   des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2);
   des_pdl_go();
   // The slots' scratch range ends with this call (see Slot::first_occ; resolve_kernel then starts a new one): nothing
@@ -253,20 +263,23 @@ __global__ void __launch_bounds__(IB / 4) assign_kernel(
   if (meta->scratch_base - (uint32_t)nnz < max_nnz)
     for (unsigned long long i = (unsigned long long)blockIdx.x * NT + tid; i < total_slots; i += (unsigned long long)gridDim.x * NT)
       slots[i].first_occ = DES_ROW_NONE;
-  uint32_t w = 0;
-  if (j0 + 3 < nnz) w = __ldg(reinterpret_cast<const uint32_t*>(flags + j0));
-  else for (int q = 0; q < 4; ++q) if (j0 + q < nnz) w |= (uint32_t)flags[j0 + q] << (8 * q);
-  uint32_t before = tile_offset_part(blk_cnt, sup_cnt, S, tile, 0, tid, NT);
-  const uint32_t wf = w & 0x01010101u, wn = w & 0x02020202u, cf = __popc(wf), cn = __popc(wn);
+  typedef typename std::conditional<PER == 8, unsigned long long, uint16_t>::type flags_t;
+  unsigned long long w = 0;
+  if (j0 + PER <= nnz) w = __ldg(reinterpret_cast<const flags_t*>(flags + j0));
+  else for (int q = 0; q < PER; ++q) if (j0 + q < nnz) w |= (unsigned long long)flags[j0 + q] << (8 * q);
+  uint32_t before = tile_offset_part(blk_cnt, sup_cnt, 1, tile0, tid, NT);
+  const uint32_t cf = __popcll(w & 0x0101010101010101ull), cn = __popcll(w & 0x0202020202020202ull);
+  auto first = [&](int q) { return (w >> (8 * q)) & 1ull; };
+  auto fresh = [&](int q) { return (w >> (8 * q)) & 2ull; };
   // what the first occurrences need, in flight while the ranks are formed
-  uint32_t r[4]; uint32_t sh[4];
+  uint32_t r[PER], sh[PER];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const bool f = (wf >> (8 * q)) & 1u;
-    r[q] = f ? rows[j0 + q] : DES_ROW_NONE;
-    sh[q] = f ? __ldg(shards + j0 + q) : 0u;
+  for (int q = 0; q < PER; ++q) {
+    r[q] = first(q) ? rows[j0 + q] : DES_ROW_NONE;
+    sh[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
+    if (fresh(q)) r[q] = __ldg(slot_of + j0 + q);       // (a new key has no row yet: its slot instead)
   }
-  uint32_t incl = cf | cn << 16;                        // (at most 1024 of each in a tile)
+  uint32_t incl = cf | cn << 16;                        // (at most 4096 of each in a block)
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
@@ -277,93 +290,126 @@ __global__ void __launch_bounds__(IB / 4) assign_kernel(
   if (lane == 31) { wsum[warp] = incl & 0xFFFFu; wnew[warp] = incl >> 16; }
   if (lane == 0) wbase[warp] = before;
   __syncthreads();
-  uint32_t u = (incl & 0xFFFFu) - cf, nrank = (incl >> 16) - cn, tile_firsts = 0, n_new = 0;
+  uint32_t u = (incl & 0xFFFFu) - cf, nrank = (incl >> 16) - cn, firsts = 0, n_new = 0;
 #pragma unroll
   for (int i = 0; i < NW; ++i) {
     u += wbase[i] + (i < warp ? wsum[i] : 0u);
     nrank += i < warp ? wnew[i] : 0u;
-    tile_firsts += wsum[i] + wbase[i];
+    firsts += wsum[i] + wbase[i];
     n_new += wnew[i];
   }
-  if (tile == ntiles - 1 && tid == 0) { meta->n_uniq = tile_firsts; *n_uniq_out = tile_firsts; }
+  if (blockIdx.x == gridDim.x - 1 && tid == 0) { meta->n_uniq = firsts; *n_uniq_out = firsts; }
+  {
+    uint32_t uu = u;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (!((wf >> (8 * q)) & 1u)) continue;
-    if ((wn >> (8 * q)) & 2u) {
-      l_off[nrank] = (uint16_t)(tid * 4 + q); l_shard[nrank] = (uint8_t)sh[q]; l_grow[nrank] = u;
-      ++nrank;
-    } else {
-      uidx[j0 + q] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : u;
-      uniq_rows[u] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : (uint32_t)(meta->row_base[sh[q]] + r[q]);
+    for (int q = 0; q < PER; ++q) {
+      if (!first(q)) continue;
+      if (!fresh(q)) {
+        uidx[j0 + q] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : uu;
+        uniq_rows[uu] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : (uint32_t)(meta->row_base[sh[q]] + r[q]);
+      }
+      ++uu;
     }
-    ++u;
   }
   if (n_new == 0) return;                               // (whole block) the steady state of a populated table
   // ---- new keys: rank among the shard's new keys, on top of the shard's size
-  for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&n_warp[0][0])[i] = 0;
-  if (tid < DES_MAX_SHARDS) n_base[tid] = tid < S ? meta->n_rows[tid] : 0u;
+  if (tid < S) { n_base[tid] = meta->n_rows[tid]; s_cap[tid] = meta->row_cap[tid]; s_row[tid] = (uint32_t)meta->row_base[tid]; }
   __syncthreads();
   for (int i = tid; i < S * (NT / DES_MAX_SHARDS); i += NT) {
-    const uint32_t v = tile_offset_part(blk_cnt, sup_cnt, S, tile, 1 + i % S, i / S, NT / DES_MAX_SHARDS);
+    const uint32_t v = tile_offset_part(blk_cnt + nblk_max + i % S, sup_cnt + nsup_max + i % S, S, tile0, i / S,
+                                        NT / DES_MAX_SHARDS);
     if (v) atomicAdd(&n_base[i % S], v);
   }
-  const int per = (((int)n_new + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min((int)n_new, lo + per);
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int i0 = lo; i0 < hi; i0 += 32) {
-      const int i = i0 + lane;
-      const int key = i < hi ? (int)l_shard[i] : -1;
-      const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
-      const uint32_t at = i < hi ? n_warp[warp][key] : 0u;
-      __syncwarp();
-      if (i < hi && (same >> lane) == 1u) n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
-      if (pass == 1 && i < hi) {
-        uint32_t local = n_base[key] + at + __popc(same & ((1u << lane) - 1u));
-        if (local >= meta->row_cap[key]) { local = DES_ROW_NONE; des_raise(meta, DES_ERR_CAPACITY); }
-        const int j = tile * IB + l_off[i];
-        const uint32_t uu = l_grow[i];
-        const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : (uint32_t)(meta->row_base[key] + local);
-        if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(slot_of[j])) slots[slot_of[j]].row = local;
-        rows[j] = local;
-        uidx[j] = local == DES_ROW_NONE ? DES_ROW_NONE : uu;
-        uniq_rows[uu] = grow;
-        l_grow[i] = grow;
-      }
-      __syncwarp();
-    }
-    __syncthreads();
-    if (pass == 0) {                                     // counts of the list parts -> where each part starts
-      if (tid < S) {
-        uint32_t run = 0;
-        for (int i = 0; i < NW; ++i) { const uint16_t v = n_warp[i][tid]; n_warp[i][tid] = (uint16_t)run; run += v; }
-      }
-      __syncthreads();
-    }
-  }
-  // ---- their rows: G lanes per row, every lane of a warp runs the same rounds (the squared norm is a warp-level sum)
   const int K4 = k >> 2, c4 = tid % G;
   const float stamp = des_stamp_bits(meta->clock + 1ull);   // the clock value this call ends with
-  for (int i0 = 0; i0 < (int)n_new; i0 += NT / G) {
-    const int i = i0 + tid / G;
-    const uint32_t grow = i < (int)n_new ? l_grow[i] : DES_ROW_NONE;
-    const bool init = grow != DES_ROW_NONE;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (init && c4 < K4) v = des_init4(seed, __ldg(ids + tile * IB + l_off[i]), (uint32_t)c4, init_scale);
-    float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  for (uint32_t win = 0; win < n_new; win += IB) {      // (one round unless PER = 8 and most keys are new)
+    const int n = (int)min(n_new - win, (uint32_t)IB);
+    {
+      uint32_t uu = u, rank = nrank - win;
 #pragma unroll
-    for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
-    if (!init || DES_DBG_ROW(grow) != grow) continue;
-    float4* wr = reinterpret_cast<float4*>(W + (size_t)grow * stride);
-    if (c4 < K4) wr[c4] = v;
-    if (c4 == 0) wr[K4] = make_float4(0.f, n2, stamp, 0.f);   // linear weight, squared norm, age stamp
-    if (A) {
-      float4* a = reinterpret_cast<float4*>(A + (size_t)grow * stride);
-      if (c4 < K4) a[c4] = make_float4(state_init, state_init, state_init, state_init);
-      if (c4 == 0) a[K4] = make_float4(lin_state_init, 0.f, 0.f, 0.f);
+      for (int q = 0; q < PER; ++q) {
+        if (!first(q)) continue;
+        if (fresh(q)) {
+          if (rank < (uint32_t)n) {                     // (unsigned: earlier windows are out of range too)
+            l_off[rank] = (uint16_t)(tid * PER + q); l_slot[rank] = r[q]; l_shard[rank] = (uint8_t)sh[q]; l_grow[rank] = uu;
+          }
+          ++rank;
+        }
+        ++uu;
+      }
     }
-    if (A2) {
-      float4* a2 = reinterpret_cast<float4*>(A2 + (size_t)grow * stride);
-      if (c4 < K4) a2[c4] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c4 == 0) a2[K4] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&n_warp[0][0])[i] = 0;
+    __syncthreads();
+    const int per = ((n + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min(n, lo + per);
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int i0 = lo; i0 < hi; i0 += 32) {
+        const int i = i0 + lane;
+        const int key = i < hi ? (int)l_shard[i] : -1;
+        const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+        const uint32_t at = i < hi ? n_warp[warp][key] : 0u;
+        __syncwarp();
+        if (i < hi && (same >> lane) == 1u) n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
+        if (pass == 1 && i < hi) {
+          uint32_t local = n_base[key] + at + __popc(same & ((1u << lane) - 1u));
+          if (local >= s_cap[key]) { local = DES_ROW_NONE; des_raise(meta, DES_ERR_CAPACITY); }
+          const int j = jb + l_off[i];
+          const uint32_t uu = l_grow[i];
+          const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : s_row[key] + local;
+          if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(l_slot[i])) slots[l_slot[i]].row = local;
+          rows[j] = local;
+          uidx[j] = local == DES_ROW_NONE ? DES_ROW_NONE : uu;
+          uniq_rows[uu] = grow;
+          l_grow[i] = grow;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      if (pass == 0) {                                   // counts of the list parts -> where each part starts
+        if (tid < S) {
+          uint32_t run = 0;
+          for (int i = 0; i < NW; ++i) { const uint16_t v = n_warp[i][tid]; n_warp[i][tid] = (uint16_t)run; run += v; }
+        }
+        __syncthreads();
+      }
+    }
+    // ---- their rows: G lanes per row, every lane of a warp runs the same rounds (the squared norm is a warp-level sum)
+    constexpr int U = 4;                                // rows of a group whose ids are in flight together
+    for (int i0 = 0; i0 < n; i0 += NT / G * U) {
+      uint32_t grow[U];
+      unsigned long long id[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int i = i0 + q * (NT / G) + tid / G;
+        grow[q] = i < n ? l_grow[i] : DES_ROW_NONE;
+        id[q] = i < n ? __ldg(ids + jb + l_off[i]) : 0ull;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c4 < K4) v = des_init4(seed, id[q], (uint32_t)c4, init_scale);
+        float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+        for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
+        if (grow[q] == DES_ROW_NONE || DES_DBG_ROW(grow[q]) != grow[q]) continue;
+        float4* wr = reinterpret_cast<float4*>(W + (size_t)grow[q] * stride);
+        if (c4 < K4) wr[c4] = v;
+        if (c4 == 0) wr[K4] = make_float4(0.f, n2, stamp, 0.f);   // linear weight, squared norm, age stamp
+        if (A) {
+          float4* a = reinterpret_cast<float4*>(A + (size_t)grow[q] * stride);
+          if (c4 < K4) a[c4] = make_float4(state_init, state_init, state_init, state_init);
+          if (c4 == 0) a[K4] = make_float4(lin_state_init, 0.f, 0.f, 0.f);
+        }
+        if (A2) {
+          float4* a2 = reinterpret_cast<float4*>(A2 + (size_t)grow[q] * stride);
+          if (c4 < K4) a2[c4] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (c4 == 0) a2[K4] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+    }
+    if (win + IB < n_new) {                             // another window: the list and the counts are reused
+      __syncthreads();
+      if (tid < S) n_base[tid] += n_warp[NW - 1][tid];
+      __syncthreads();
     }
   }
 }
@@ -375,22 +421,22 @@ __global__ void __launch_bounds__(IB / 4) assign_kernel(
 // counts are cleared for the next call, the scratch range is retired.
 __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, int S, uint32_t max_nnz,
                                                          const uint32_t* __restrict__ first_of, uint32_t* rows, uint32_t* uidx,
-                                                         uint32_t* __restrict__ sup_cnt, DevMeta* meta) {
+                                                         uint32_t* __restrict__ sup_cnt, int nsup_max, DevMeta* meta) {
   des_pdl_wait(first_of, rows, uidx, sup_cnt, meta);
   des_pdl_go();
   if ((int)blockIdx.x == ntiles) {
     const int nsup = (ntiles + (int)SUP_TILES - 1) / (int)SUP_TILES;
-    for (int c = threadIdx.x; c <= S; c += IB / 4) {
-      uint32_t total = 0;
-      if (c == 0 || meta->any_new) {
+    for (int i = threadIdx.x; i < nsup; i += IB / 4) sup_cnt[i] = 0u;
+    if (meta->any_new)
+      for (int c = threadIdx.x; c < S; c += IB / 4) {
+        uint32_t total = 0;
 #pragma unroll 8
         for (int i = 0; i < nsup; ++i) {
-          total += sup_cnt[(size_t)i * (S + 1) + c];
-          sup_cnt[(size_t)i * (S + 1) + c] = 0u;
+          total += sup_cnt[nsup_max + (size_t)i * S + c];
+          sup_cnt[nsup_max + (size_t)i * S + c] = 0u;
         }
+        meta->n_rows[c] = min(meta->n_rows[c] + total, meta->row_cap[c]);
       }
-      if (c) meta->n_rows[c - 1] = min(meta->n_rows[c - 1] + total, meta->row_cap[c - 1]);
-    }
     __syncthreads();
     if (threadIdx.x == 0) {
       meta->any_new = 0u;
@@ -446,7 +492,7 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
     if (insert) DES_CUDA(cudaMemsetAsync(b->n_uniq, 0, 4, cs));
     return DES_OK;
   }
-  const int ntiles = (nnz + IB - 1) / IB;
+  const int ntiles = (nnz + IB - 1) / IB, nsup_max = (int)(t->nblk_max / SUP_TILES) + 1;
   SlotGeom geom;
   for (uint32_t s = 0; s <= t->S; ++s) geom.slot_base[s] = t->h_slot_base[s];
   des_mod_consts(t->S, &geom.mod_M, &geom.mod_two32);
@@ -458,7 +504,7 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
   if (!insert) return DES_OK;
   uint32_t* first_of = t->uslot;
   des_launch(flag_count_kernel, ntiles, IB / 4, 0, cs, nnz, (int)t->S, t->slots, t->meta, t->slot_of, b->shards, t->flags,
-             b->rows, first_of, t->blk_cnt, t->sup_cnt, &t->meta->any_new);
+             b->rows, first_of, t->blk_cnt, t->sup_cnt, (int)t->nblk_max, nsup_max, &t->meta->any_new);
   DES_LAUNCH_CHECK(t, "flag_count_kernel");
   {
     const float state_init = t->cfg.optimizer == DES_OPT_ADAGRAD ? t->cfg.init_acc : 0.f;
@@ -466,17 +512,21 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
         (t->cfg.lin_optimizer == DES_LIN_FTRL || t->cfg.optimizer != DES_OPT_ADAGRAD) ? 0.f : t->cfg.init_acc;
     int G = 1;
     while (G < (int)t->k / 4) G <<= 1;
-#define ASSIGN(GG) des_launch(assign_kernel<GG>, ntiles, IB / 4, 0, cs, nnz, ntiles, (int)t->S, t->meta,                  \
-        (const unsigned long long*)b->ids, b->shards, t->flags, t->blk_cnt, t->sup_cnt, t->slot_of, b->rows, b->uidx,   \
-        b->uniq_rows, b->n_uniq, t->slots, t->total_slots, (uint32_t)t->max_nnz, (int)t->k, (int)t->stride, t->W, t->A, \
-        t->A2, t->cfg.seed, t->cfg.init_scale, state_init, lin_state_init)
+    const bool deep = ntiles >= ASSIGN_DEEP_TILES * t->sm_count;
+#define ASSIGN2(GG, PP) des_launch(assign_kernel<GG, PP>, (ntiles * IB + 512 * PP - 1) / (512 * PP), 512, 0, cs, nnz, ntiles,   \
+        (int)t->S, t->meta, (const unsigned long long*)b->ids, b->shards, t->flags, t->blk_cnt, t->sup_cnt,               \
+        (int)t->nblk_max, nsup_max, t->slot_of, b->rows, b->uidx, b->uniq_rows, b->n_uniq, t->slots, t->total_slots,     \
+        (uint32_t)t->max_nnz, (int)t->k, (int)t->stride, t->W, t->A, t->A2, t->cfg.seed, t->cfg.init_scale, state_init,  \
+        lin_state_init)
+#define ASSIGN(GG) do { if (deep) ASSIGN2(GG, 8); else ASSIGN2(GG, 2); } while (0)
     switch (G) { case 1: ASSIGN(1); break; case 2: ASSIGN(2); break; case 4: ASSIGN(4); break; case 8: ASSIGN(8); break;
                  default: ASSIGN(16); }
+#undef ASSIGN2
 #undef ASSIGN
     DES_LAUNCH_CHECK(t, "assign_kernel");
   }
   des_launch(resolve_kernel, ntiles + 1, IB / 4, 0, cs, nnz, ntiles, (int)t->S, (uint32_t)t->max_nnz, first_of, b->rows, b->uidx,
-             t->sup_cnt, t->meta);
+             t->sup_cnt, nsup_max, t->meta);
   DES_LAUNCH_CHECK(t, "resolve_kernel");
   return DES_OK;
 }

@@ -85,8 +85,8 @@ struct des_table {
   uint32_t* slot_of;                 // [max_nnz]
   uint8_t* flags;                    // [max_nnz]
   uint32_t* uslot;                   // [max_nnz]
-  uint32_t* blk_cnt;                 // [nblk_max][S+1] per tile: first occurrences, new keys per shard
-  uint32_t* sup_cnt;                 // [nsup_max][S+1] the same per SUP_TILES tiles; zero between calls
+  uint32_t* blk_cnt;                 // per tile: first occurrences [nblk_max], then new keys per shard [nblk_max][S]
+  uint32_t* sup_cnt;                 // the same per SUP_TILES tiles; zero between calls
   int32_t* seg_off;                  // [max_batch][S+1] forward routing: (sample, shard) segment bounds
   // backward workspace
   float* Gbuf;                       // [max_uniq + rep_max][stride]: per-unique gradient rows, then

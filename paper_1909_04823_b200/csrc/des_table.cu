@@ -436,17 +436,18 @@ __global__ void __launch_bounds__(256) write_rows_kernel(const uint32_t* __restr
   float n2 = 0.f;
   if (ok)
     for (int c = lane; c < C; c += G) {
-      V v;
-      if (emb) { v = __ldg(reinterpret_cast<const V*>(emb + i * k) + c); reinterpret_cast<V*>(w)[c] = v; }
-      else v = reinterpret_cast<const V*>(w)[c];
+      if (emb) {
+        const V v = __ldg(reinterpret_cast<const V*>(emb + i * k) + c);
+        reinterpret_cast<V*>(w)[c] = v;
+        n2 += rows_sq(v);
+      }
       if (acc_emb && A)
         reinterpret_cast<V*>(A + (size_t)g * stride)[c] = __ldg(reinterpret_cast<const V*>(acc_emb + i * k) + c);
-      n2 += rows_sq(v);
     }
 #pragma unroll
   for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);   // |v|^2, cached in the row's tail
   if (!ok || lane) return;
-  w[k + 1] = n2;
+  if (emb) w[k + 1] = n2;
   if (lin) w[k] = lin[i];
   if (acc_lin && A) A[(size_t)g * stride + k] = acc_lin[i];
 }
