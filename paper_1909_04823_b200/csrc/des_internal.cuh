@@ -146,7 +146,9 @@ void des_api_begin(des_table* t, cudaStream_t cs);
 template <typename P>
 __device__ __forceinline__ void des_pdl_new(P& p) {
   static_assert(sizeof(P) == 8, "pointers only");
-  asm volatile("" : "+l"(p)::"memory");
+  size_t a = __cvta_generic_to_global(p);              // (a plain generic pointer would turn every access into a generic one:
+  asm volatile("" : "+l"(a)::"memory");                // the scatter's atomics took 1124 us instead of 833)
+  p = (P)__cvta_global_to_generic(a);
 }
 template <typename... P>
 __device__ __forceinline__ void des_pdl_wait(P&... p) {
