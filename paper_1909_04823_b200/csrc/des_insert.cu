@@ -46,7 +46,7 @@ __device__ __forceinline__ Slot load_slot(const Slot* p) {
 // per distinct key of a warp costs more in match instructions than the cached slot loads it saves).
 #define PROBE_ILP 1
 #define PROBE_MINB 8
-#define PROBE_MERGE_WAVES 4
+#define PROBE_MERGE_WAVES 24 // waves of resident blocks up to which blocks merge (3.9 M occurrences: 76 against 88 us; 32 M: 350 against 320)
 #define PROBE_MERGE 256   // entries of a block's table of first occurrences (= threads per block)
 
 struct SlotGeom {
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(IB / 4) flag_count_kernel(
     *bc = c;
     if (c) {
       atomicAdd(sc, c);
-      if (s >= 0) *any_new = 1u;
+      if (s >= 0 && !*reinterpret_cast<volatile uint32_t*>(any_new)) *any_new = 1u;   // (not thousands of stores to one word)
     }
   }
 }
@@ -240,7 +240,7 @@ __device__ __forceinline__ uint32_t tile_offset_part(const uint32_t* __restrict_
 // take 120 us, 190 us with 256 threads a tile); PER = 8 spreads a block's latency over four times the
 // occurrences once every SM has several blocks (32 M occurrences: 212 -> 70 us).
 template <int G, int PER>
-__global__ void __launch_bounds__(512) assign_kernel(
+__global__ void __launch_bounds__(512, 3) assign_kernel(
     int nnz, int ntiles, int S, DevMeta* meta, const unsigned long long* __restrict__ ids, const uint8_t* __restrict__ shards,
     const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
     int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx,
@@ -248,6 +248,8 @@ __global__ void __launch_bounds__(512) assign_kernel(
     uint32_t max_nnz, int k, int stride, float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2,
     unsigned long long seed, float init_scale, float state_init, float lin_state_init) {
   constexpr int NT = 512, NW = NT / 32, M = NT * PER / IB;
+  constexpr bool DEEP = PER > 2;
+  __shared__ uint16_t s_first[DEEP ? NT * PER : 1];     // DEEP: the block's first occurrences in order (bit 15: new key)
   __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW], n_base[DES_MAX_SHARDS], s_cap[DES_MAX_SHARDS], s_row[DES_MAX_SHARDS];
   __shared__ uint16_t n_warp[NW][DES_MAX_SHARDS];       // new keys per list part and shard, then running ranks
   __shared__ uint16_t l_off[IB];                        // listed new keys: occurrence within the block's range, ...
@@ -271,14 +273,15 @@ __global__ void __launch_bounds__(512) assign_kernel(
   const uint32_t cf = __popcll(w & 0x0101010101010101ull), cn = __popcll(w & 0x0202020202020202ull);
   auto first = [&](int q) { return (w >> (8 * q)) & 1ull; };
   auto fresh = [&](int q) { return (w >> (8 * q)) & 2ull; };
-  // what the first occurrences need, in flight while the ranks are formed
-  uint32_t r[PER], sh[PER];
+  // PER = 2: what the first occurrences need, in flight while the ranks are formed
+  uint32_t r[DEEP ? 1 : PER], sh[DEEP ? 1 : PER];
+  if (!DEEP)
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    r[q] = first(q) ? rows[j0 + q] : DES_ROW_NONE;
-    sh[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
-    if (fresh(q)) r[q] = __ldg(slot_of + j0 + q);       // (a new key has no row yet: its slot instead)
-  }
+    for (int q = 0; q < PER; ++q) {
+      r[q] = first(q) ? rows[j0 + q] : DES_ROW_NONE;
+      sh[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
+    }
+  if (tid < S) s_row[tid] = (uint32_t)meta->row_base[tid];
   uint32_t incl = cf | cn << 16;                        // (at most 4096 of each in a block)
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -299,21 +302,38 @@ __global__ void __launch_bounds__(512) assign_kernel(
     n_new += wnew[i];
   }
   if (blockIdx.x == gridDim.x - 1 && tid == 0) { meta->n_uniq = firsts; *n_uniq_out = firsts; }
-  {
+  if (DEEP) {
+    // few of a thread's occurrences are first ones: the block lists them and takes one per thread
+    uint32_t nf = 0, rank = (incl & 0xFFFFu) - cf;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) { nf += wsum[i]; rank += i < warp ? wsum[i] : 0u; }
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if (first(q)) s_first[rank++] = (uint16_t)((tid * PER + q) | (fresh(q) ? 0x8000 : 0));
+    __syncthreads();
+    const uint32_t u0 = firsts - nf;
+    for (uint32_t i = tid; i < nf; i += NT) {
+      const uint32_t e = s_first[i];
+      if (e & 0x8000u) continue;
+      const uint32_t row = rows[jb + e], sd = __ldg(shards + jb + e);
+      uidx[jb + e] = row == DES_ROW_NONE ? DES_ROW_NONE : u0 + i;
+      uniq_rows[u0 + i] = row == DES_ROW_NONE ? DES_ROW_NONE : s_row[sd] + row;
+    }
+  } else {
     uint32_t uu = u;
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       if (!first(q)) continue;
       if (!fresh(q)) {
-        uidx[j0 + q] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : uu;
-        uniq_rows[uu] = (r[q] == DES_ROW_NONE) ? DES_ROW_NONE : (uint32_t)(meta->row_base[sh[q]] + r[q]);
+        uidx[j0 + q] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : uu;
+        uniq_rows[uu] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : s_row[sh[q]] + r[q];
       }
       ++uu;
     }
   }
   if (n_new == 0) return;                               // (whole block) the steady state of a populated table
   // ---- new keys: rank among the shard's new keys, on top of the shard's size
-  if (tid < S) { n_base[tid] = meta->n_rows[tid]; s_cap[tid] = meta->row_cap[tid]; s_row[tid] = (uint32_t)meta->row_base[tid]; }
+  if (tid < S) { n_base[tid] = meta->n_rows[tid]; s_cap[tid] = meta->row_cap[tid]; }
   __syncthreads();
   for (int i = tid; i < S * (NT / DES_MAX_SHARDS); i += NT) {
     const uint32_t v = tile_offset_part(blk_cnt + nblk_max + i % S, sup_cnt + nsup_max + i % S, S, tile0, i / S,
@@ -331,7 +351,7 @@ __global__ void __launch_bounds__(512) assign_kernel(
         if (!first(q)) continue;
         if (fresh(q)) {
           if (rank < (uint32_t)n) {                     // (unsigned: earlier windows are out of range too)
-            l_off[rank] = (uint16_t)(tid * PER + q); l_slot[rank] = r[q]; l_shard[rank] = (uint8_t)sh[q]; l_grow[rank] = uu;
+            l_off[rank] = (uint16_t)(tid * PER + q); l_grow[rank] = uu;
           }
           ++rank;
         }
@@ -339,6 +359,8 @@ __global__ void __launch_bounds__(512) assign_kernel(
       }
     }
     for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&n_warp[0][0])[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += NT) { l_shard[i] = __ldg(shards + jb + l_off[i]); l_slot[i] = __ldg(slot_of + jb + l_off[i]); }
     __syncthreads();
     const int per = ((n + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min(n, lo + per);
     for (int pass = 0; pass < 2; ++pass) {
