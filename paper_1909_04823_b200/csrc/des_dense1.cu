@@ -133,18 +133,26 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
 __global__ void w1_update_kernel(const float* __restrict__ part, int slices, size_t n, float* W1, float* acc,
                                  float* acc2, __nv_bfloat16* W1b, const OptParams opt_in,
                                  const DevMeta* __restrict__ meta) {
+  des_pdl_wait(part, W1, acc, acc2, W1b, meta);
+  des_pdl_go();
   const OptParams opt = des_opt_load(opt_in, meta);
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x, st = (size_t)gridDim.x * blockDim.x;
-  for (; i < n; i += st) {
-    float G = 0.f;
-    for (int z = 0; z < slices; ++z) G += __ldg(part + (size_t)z * n + i);
-    float w = W1[i];
-    float s1 = acc[i], s2 = acc2 ? acc2[i] : 0.f;
-    des_opt_step(opt, w, s1, s2, G);
-    acc[i] = s1;
-    if (acc2) acc2[i] = s2;
-    W1[i] = w;
-    W1b[i] = __float2bfloat16_rn(w);
+  const size_t n4 = n / 4, st = (size_t)gridDim.x * blockDim.x;       // (n is a multiple of 4: k and H are)
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += st) {
+    float4 G = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 w = reinterpret_cast<float4*>(W1)[i], s1 = reinterpret_cast<float4*>(acc)[i];
+    float4 s2 = acc2 ? reinterpret_cast<float4*>(acc2)[i] : G;
+#pragma unroll 8
+    for (int z = 0; z < slices; ++z) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(part + (size_t)z * n) + i);
+      G.x += v.x; G.y += v.y; G.z += v.z; G.w += v.w;
+    }
+    des_opt_step(opt, w.x, s1.x, s2.x, G.x); des_opt_step(opt, w.y, s1.y, s2.y, G.y);
+    des_opt_step(opt, w.z, s1.z, s2.z, G.z); des_opt_step(opt, w.w, s1.w, s2.w, G.w);
+    reinterpret_cast<float4*>(acc)[i] = s1;
+    if (acc2) reinterpret_cast<float4*>(acc2)[i] = s2;
+    reinterpret_cast<float4*>(W1)[i] = w;
+    const __nv_bfloat162 a = __floats2bfloat162_rn(w.x, w.y), b = __floats2bfloat162_rn(w.z, w.w);
+    reinterpret_cast<uint2*>(W1b)[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
   }
 }
 
@@ -157,17 +165,26 @@ __global__ void cvt_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __
   }
 }
 
-// two arrays in one launch (the backward's two operands)
-__global__ void cvt_bf16_pair_kernel(const float* __restrict__ s1, __nv_bfloat16* __restrict__ d1, size_t n1,
-                                     const float* __restrict__ s2, __nv_bfloat16* __restrict__ d2, size_t n2) {
-  size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  const size_t st = (size_t)gridDim.x * blockDim.x * 4;
-  for (; i + 3 < n1 + n2; i += st) {                   // n1 and n2 are multiples of 4
-    const float* src = i < n1 ? s1 + i : s2 + (i - n1);
-    __nv_bfloat16* dst = i < n1 ? d1 + i : d2 + (i - n1);
-    const float4 v = *reinterpret_cast<const float4*>(src);
-    __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-    *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
+// two arrays in one launch (the backward's two operands); four 16-byte loads of a thread in flight
+__global__ void __launch_bounds__(256) cvt_bf16_pair_kernel(const float* __restrict__ s1, __nv_bfloat16* __restrict__ d1, size_t n1,
+                                                            const float* __restrict__ s2, __nv_bfloat16* __restrict__ d2, size_t n2) {
+  des_pdl_wait(s1, d1, s2, d2);
+  des_pdl_go();
+  const size_t m1 = n1 / 4, m = m1 + n2 / 4;           // n1 and n2 are multiples of 4
+  const size_t i0 = (size_t)blockIdx.x * 1024 + threadIdx.x;
+  float4 v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const size_t i = i0 + q * 256;
+    if (i < m) v[q] = i < m1 ? __ldg(reinterpret_cast<const float4*>(s1) + i) : __ldg(reinterpret_cast<const float4*>(s2) + (i - m1));
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const size_t i = i0 + q * 256;
+    if (i >= m) continue;
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[q].x, v[q].y), b = __floats2bfloat162_rn(v[q].z, v[q].w);
+    const uint2 o = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    if (i < m1) reinterpret_cast<uint2*>(d1)[i] = o; else reinterpret_cast<uint2*>(d2)[i - m1] = o;
   }
 }
 
@@ -175,6 +192,13 @@ static des_status_t to_bf16(des_table* t, const float* src, __nv_bfloat16* dst, 
   cvt_bf16_kernel<<<t->sm_count * 4, 256, 0, st>>>(src, dst, n);     // n is a multiple of 4 (k and H are)
   DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
   return DES_OK;
+}
+
+// a thread per four weights, as far as the chip holds them at once
+static void launch_w1_update(des_table* t, int slices, cudaStream_t st) {
+  const size_t n = (size_t)t->F * t->k * t->H, blocks = (n / 4 + 255) / 256, most = (size_t)t->sm_count * 8;
+  des_launch(w1_update_kernel, (unsigned)(blocks < most ? blocks : most), 256, 0, st, t->gW1_part, slices, n, t->W1, t->accW1,
+             t->acc2W1, t->W1b, des_opt_params(t), t->meta);
 }
 
 des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float* Z, float* part_dense,
@@ -212,7 +236,8 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
   const int FK = t->F * t->k;
   if (t->use_tc) {
     t->pooled_b_src = nullptr;
-    cvt_bf16_pair_kernel<<<t->sm_count * 4, 256, 0, st>>>(gZ, t->gZ_b, (size_t)B * t->H, pooled, t->pooled_b, (size_t)B * FK);
+    const size_t n1 = (size_t)B * t->H, n2 = (size_t)B * FK;
+    des_launch(cvt_bf16_pair_kernel, (unsigned)(((n1 + n2) / 4 + 1023) / 1024), 256, 0, st, gZ, t->gZ_b, n1, pooled, t->pooled_b, n2);
     DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
     const int rc1 = des_tc_gemm_dgrad(B, FK, t->H, 1, t->gZ_b, t->W1b, gE ? gE : gE_work, gE_work, gE ? 1.f : 0.f,
                                       t->gemm_ws, t->gemm_ws_bytes, st);
@@ -227,8 +252,7 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
                                         t->gemm_ws, t->gemm_ws_bytes, st);
       if (rc2 != 0) return DES_ERR_CUDA;           // same alignment rules as the dgrad: cannot differ
       DES_LAUNCH_CHECK(t, "tc_gemm_wgrad");
-      w1_update_kernel<<<t->sm_count * 2, 256, 0, st>>>(t->gW1_part, L, (size_t)FK * t->H, t->W1, t->accW1, t->acc2W1,
-                                                        t->W1b, des_opt_params(t), t->meta);
+      launch_w1_update(t, L, st);
       DES_LAUNCH_CHECK(t, "w1_update_kernel");
       return DES_OK;
     }
@@ -249,9 +273,7 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
     dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, g.slices);
     gemm_kernel<GEMM_WGRAD><<<grid, 256, 0, st>>>(g);
     DES_LAUNCH_CHECK(t, "gemm_kernel");
-    const size_t n = (size_t)FK * t->H;
-    w1_update_kernel<<<t->sm_count * 2, 256, 0, st>>>(t->gW1_part, g.slices, n, t->W1, t->accW1, t->acc2W1,
-                                                      t->W1b, des_opt_params(t), t->meta);
+    launch_w1_update(t, g.slices, st);
     DES_LAUNCH_CHECK(t, "w1_update_kernel");
   }
   return DES_OK;

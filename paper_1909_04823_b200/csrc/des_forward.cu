@@ -25,16 +25,21 @@
 //                 materialised (with atomics) when the caller asks for it.
 //
 // FIELD partition (field f on shard f mod S): a bag belongs to one shard, so when pooling is among the
-// operators one gather pass (single_gather_kernel: pooled vectors and per-bag sums of the linear weights and
-// squared norms) feeds everything, and field_partials_kernel forms shard s's sub-operators as the sums over
-// the bags of its own fields — no routing pass, no second gather.
+// operators one gather pass (sample_gather_kernel: pooled vectors and per-bag sums of the linear weights and
+// squared norms, kept in shared memory) feeds everything: shard s's sub-operators are the sums over
+// the bags of its own fields — no routing pass, no second gather.  Samples too large for that take two
+// kernels (single_gather_kernel, field_partials_kernel).
 //
 // Accuracy.  A lane never adds more than a few dozen terms into one float32 accumulator (long
 // segments are summed in two levels), and the sum over shards is taken in double and rounded once, so
 // every per-sample sum keeps the stated float32 tolerance even when one key contributes
 // hundreds of equal terms that the other terms cancel.
+#include <type_traits>
+
 #include "des_internal.cuh"
 
+#define SGF_BU 4                  // short bags of a lane group in flight together (sample_gather_kernel)
+#define SGF_SMEM (24u << 10)      // shared memory a block of the FIELD form takes at most, unless one sample needs more
 #ifndef POOL_BLOCKS_PER_SM
 #define POOL_BLOCKS_PER_SM 64   // grid cap of the pooling kernel (it strides over the bags)
 #endif
@@ -50,6 +55,8 @@ __global__ void __launch_bounds__(256) route_kernel(
     int32_t* __restrict__ seg_off) {
   __shared__ uint32_t row_base[DES_MAX_SHARDS];
   __shared__ int cursor[8][DES_MAX_SHARDS];
+  des_pdl_wait(offsets, vals, rows, shards, meta, grow_csr, grow_sorted, x_sorted, seg_off);
+  des_pdl_go();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x < S) row_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x];
   __syncthreads();
@@ -176,6 +183,55 @@ __device__ __forceinline__ void sp_round(const uint32_t* __restrict__ grow_sorte
   }
 }
 
+// A bag walked by LB = G * P lanes together, LB occurrences at a time: every lane looks up the row of one occurrence (and adds
+// its linear weight and squared norm to sums of its own), then the rows are handed round by shuffles, sub-group p taking
+// positions p, p + P, ...  Looked up by all lanes of every occurrence instead, the row number, shard and tail are three of
+// the four loads of an occurrence.
+template <int G, int P, bool HAS_VALS, bool TAIL>
+__device__ __forceinline__ void coop_bag(const uint32_t* __restrict__ rows, const uint8_t* __restrict__ shards,
+                                         const float* __restrict__ vals, const uint32_t* __restrict__ s_base, int lo, int hi,
+                                         int sub, unsigned gmask, const char* __restrict__ Wc, const char* __restrict__ Wt,
+                                         unsigned rowB, uint32_t null_row, float4& acc, float& bl, float& bq) {
+  constexpr int LB = G * P;
+  const int p = sub / G;
+  for (int c0 = lo; c0 < hi; c0 += LB) {
+    const int j = c0 + sub, n = min(LB, hi - c0);
+    uint32_t g = null_row;
+    float x = 0.f;
+    if (j < hi) {
+      const uint32_t r = __ldg(rows + j);
+      if (r != DES_ROW_NONE) g = DES_DBG_ROW(s_base[__ldg(shards + j)] + r);
+      if (HAS_VALS) x = __ldg(vals + j);
+      if (TAIL) {
+        const float2 tl = __ldg(reinterpret_cast<const float2*>(Wt + (size_t)g * rowB));
+        bl += HAS_VALS ? tl.x * x : tl.x;
+        bq += HAS_VALS ? tl.y * x * x : tl.y;
+      }
+    }
+    int t = 0;
+    auto step = [&](auto U) {
+      constexpr int N = decltype(U)::value;
+      float4 v[N]; float xx[N];
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const uint32_t gg = __shfl_sync(gmask, g, t + u * P + p, LB);
+        if (HAS_VALS) xx[u] = __shfl_sync(gmask, x, t + u * P + p, LB);
+        v[u] = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)gg * rowB));
+      }
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        if (HAS_VALS) { v[u].x *= xx[u]; v[u].y *= xx[u]; v[u].z *= xx[u]; v[u].w *= xx[u]; }
+        acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w;
+      }
+      t += N * P;
+    };
+    while (t + 4 * P <= n) step(std::integral_constant<int, 4>());
+    if (t + 2 * P <= n) step(std::integral_constant<int, 2>());
+    if (t + P <= n) step(std::integral_constant<int, 1>());
+    if (t < n) step(std::integral_constant<int, 1>());   // (positions past the end hold the all-zero row)
+  }
+}
+
 // Same for a bag: U rows per lane, optionally also added to the per-shard copy of the pooled sum
 // (MATERIALISE, tests only).
 template <int U, int P, bool HAS_VALS, bool MATERIALISE>
@@ -228,6 +284,8 @@ __global__ void __launch_bounds__(256) shard_partials_kernel(
     int B, int S, int k, uint32_t ops, const float* __restrict__ W, uint32_t null_row, float* __restrict__ part_small,
     float* __restrict__ out_small) {
   constexpr int P = 32 / G;
+  des_pdl_wait(grow_sorted, x_sorted, seg_off, W, part_small, out_small);
+  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -302,6 +360,8 @@ __global__ void __launch_bounds__(256) pool_kernel(
     const uint8_t* __restrict__ shards, long long nbags, int B, int F, int k, const float* __restrict__ W,
     uint32_t null_row, float* __restrict__ pooled, float* __restrict__ part_pooled, __nv_bfloat16* __restrict__ pooled_b) {
   constexpr int LB = G * P;                            // lanes per bag
+  des_pdl_wait(offsets, vals, grow_csr, shards, W, pooled, part_pooled, pooled_b);
+  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
   const bool col = c4 < K4;
@@ -350,6 +410,8 @@ __global__ void __launch_bounds__(256) pool_kernel(
 template <int G>
 __global__ void __launch_bounds__(256) aggregate_small_kernel(const float* __restrict__ part_small, int B, int S, int k,
                                                               uint32_t ops, float* __restrict__ out_small) {
+  des_pdl_wait(part_small, out_small);
+  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = t / G, c4 = t % G;
@@ -416,6 +478,8 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
     __nv_bfloat16* __restrict__ pooled_b) {
   constexpr int LB = G * P;                            // lanes per bag
   __shared__ uint32_t s_base[DES_MAX_SHARDS];
+  des_pdl_wait(offsets, vals, rows, shards, W, meta, pooled, bag_tail, pooled_b);
+  des_pdl_go();
   if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x];
   __syncthreads();
   const int K4 = k >> 2, stride = k + 4;
@@ -459,48 +523,205 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
   }
 }
 
-// A, R_lr, Q and F per sample from the pooled vectors and bag tails of its F bags, added in double in field
-// order.  G lanes per sample, one float4 column each; lane 0 of the group carries the tails.
-template <int G>
-__global__ void __launch_bounds__(256) fused_finish_kernel(const float* __restrict__ pooled, const float2* __restrict__ bag_tail,
-                                                           int B, int F, int k, uint32_t ops, float* __restrict__ out_small) {
+// ---- gather and reduce in one pass ---------------------------------------------------------------------
+// The same sums with a sample's bags kept together: WPS = 8 / T warps take a sample, T samples a block.  Every lane group
+// of a warp walks bags of its own, SGF_BU short ones with their first occurrences in flight together (a one-hot
+// batch is a chain offsets -> row number -> row per bag).
+//  FIELD = false  (the fused form): the groups add their bags in double as they go, and the sample's sums are combined by
+//                 shuffles and, over its warps, in shared memory.  Against single_gather + fused_finish the
+//                 pooled vectors are not read back; and a small batch does not wait for one lane group
+//                 per sample to walk all its fields (48 samples x 39 fields: 12.4 -> 5.2 us; 1500 samples x 100
+//                 bags of 20: 160 -> 141 us).
+//  FIELD = true   (FIELD partition, per-shard partials wanted): the pooled vectors of the block's samples stay in
+//                 shared memory, where each shard's own fields are added in field order; with out_small the shards'
+//                 partials are added in double in shard order and passed through F, as aggregate_small_kernel does.
+//                 (16384 x 39 fields, k = 32: 92 -> 79 us against single_gather + field_partials.)
+// The sums over fields are taken in double in a fixed order that depends on WPS, i.e. on the batch size.
+template <int G, int P, bool HAS_VALS, bool FIELD>
+__global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
+    const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ rows,
+    const uint8_t* __restrict__ shards, int B, int F, int S, int k, int T, uint32_t ops, const float* __restrict__ W,
+    const DevMeta* __restrict__ meta, uint32_t null_row, float* __restrict__ pooled, __nv_bfloat16* __restrict__ pooled_b,
+    float* __restrict__ part_small, float* __restrict__ out_small) {
+  constexpr int LB = G * P, GW = 32 / LB;              // lanes per bag, bags per warp
+  constexpr bool COOP = P > 1;
+  constexpr int BU = COOP ? 1 : SGF_BU;                // bags of a group in flight together (long bags: their own rows are)
+  extern __shared__ __align__(16) unsigned char sg_smem[];
+  __shared__ uint32_t s_base[DES_MAX_SHARDS];
+  __shared__ double s_red[FIELD ? 1 : 8][FIELD ? 1 : G][4], s_tail[FIELD ? 1 : 8][2];
+  des_pdl_wait(offsets, vals, rows, shards, W, meta, pooled, pooled_b, part_small, out_small);
+  des_pdl_go();
+  if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x];
+  __syncthreads();
   const int K4 = k >> 2, stride = k + 4;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int b = t / G, c4 = t % G;
-  const bool live = b < B;
-  const bool lr = ops & DES_OP_LR, fm = ops & DES_OP_FM;
-  double ax = 0.0, ay = 0.0, az = 0.0, aw = 0.0, tr = 0.0, tq = 0.0;
-  if (live) {
-    const float4* pb = reinterpret_cast<const float4*>(pooled + (size_t)b * F * k) + c4;
-    const float2* tb = bag_tail + (size_t)b * F;
-    int f = 0;
-    for (; f + 4 <= F; f += 4) {                       // four bags in flight
-      float4 v[4]; float2 tl[4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sub = lane % LB, c4 = sub % G, p = sub / G;
+  const bool col = c4 < K4, fm = ops & DES_OP_FM, lr = ops & DES_OP_LR;
+  const unsigned rowB = (unsigned)stride * 4u;
+  const char* Wc = reinterpret_cast<const char*>(W) + (col ? c4 : 0) * 16;
+  const char* Wt = reinterpret_cast<const char*>(W + k);
+  const int wps = 8 / T, st = warp / wps, ws = warp % wps;             // sample within the block, warp within the sample
+  const int b = blockIdx.x * T + st;
+  const int gs = ws * GW + lane / LB, ng = wps * GW;                   // this group among the sample's
+  // FIELD: pooled vectors of sample st [F][K4] and bag tails [F]
+  float4* s_pool = reinterpret_cast<float4*>(sg_smem) + (size_t)st * F * K4;
+  float2* s_bt = reinterpret_cast<float2*>(sg_smem + (size_t)T * F * k * 4) + (size_t)st * F;
+  const int32_t* off = offsets + (size_t)b * F;
+  double Ax = 0.0, Ay = 0.0, Az = 0.0, Aw = 0.0, R = 0.0, Q = 0.0;
+  const int rounds = b < B ? (F + ng * BU - 1) / (ng * BU) : 0;   // (same for every lane of a warp)
+  int lo_n[BU], hi_n[BU];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        v[q] = (c4 < K4 && fm) ? __ldg(pb + (size_t)(f + q) * K4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        tl[q] = (c4 == 0) ? __ldg(tb + f + q) : make_float2(0.f, 0.f);
+  for (int q = 0; q < BU; ++q) {
+    const int f = gs + q * ng;
+    lo_n[q] = 0; hi_n[q] = 0;
+    if (b < B && f < F) { lo_n[q] = __ldg(off + f); hi_n[q] = __ldg(off + f + 1); }
+  }
+  for (int r = 0; r < rounds; ++r) {
+    int lo[BU], hi[BU];
+    float4 acc[BU]; float bl[BU], bq[BU];
+#pragma unroll
+    for (int q = 0; q < BU; ++q) {
+      lo[q] = lo_n[q]; hi[q] = hi_n[q];
+      const int f = gs + ((r + 1) * BU + q) * ng;      // the next round's bounds are fetched ahead
+      lo_n[q] = 0; hi_n[q] = 0;
+      if (f < F) { lo_n[q] = __ldg(off + f); hi_n[q] = __ldg(off + f + 1); }
+      acc[q] = make_float4(0.f, 0.f, 0.f, 0.f); bl[q] = 0.f; bq[q] = 0.f;
+    }
+    if (BU > 1) {                                      // the bags' first occurrences
+      uint32_t g[BU]; float x[BU];
+#pragma unroll
+      for (int q = 0; q < BU; ++q) {
+        const int j = lo[q] + p;
+        g[q] = null_row; x[q] = 1.f;
+        if (j < hi[q]) {
+          const uint32_t rr = __ldg(rows + j);
+          if (rr != DES_ROW_NONE) g[q] = s_base[__ldg(shards + j)] + rr;
+          if (HAS_VALS) x[q] = __ldg(vals + j);
+        }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        ax += (double)v[q].x; ay += (double)v[q].y; az += (double)v[q].z; aw += (double)v[q].w;
-        tr += (double)tl[q].x; tq += (double)tl[q].y;
+      for (int q = 0; q < BU; ++q) {
+        const size_t o = (size_t)DES_DBG_ROW(g[q]) * rowB;
+        acc[q] = __ldg(reinterpret_cast<const float4*>(Wc + o));
+        const float2 tl = __ldg(reinterpret_cast<const float2*>(Wt + o));
+        bl[q] = tl.x; bq[q] = tl.y;
+        if (HAS_VALS) {
+          acc[q].x *= x[q]; acc[q].y *= x[q]; acc[q].z *= x[q]; acc[q].w *= x[q];
+          bl[q] *= x[q]; bq[q] *= x[q] * x[q];
+        }
       }
     }
-    for (; f < F; ++f) {
-      if (c4 < K4 && fm) { const float4 v = __ldg(pb + (size_t)f * K4); ax += (double)v.x; ay += (double)v.y; az += (double)v.z; aw += (double)v.w; }
-      if (c4 == 0) { const float2 tl = __ldg(tb + f); tr += (double)tl.x; tq += (double)tl.y; }
+    if (COOP) {
+      coop_bag<G, P, HAS_VALS, true>(rows, shards, vals, s_base, lo[0], hi[0], sub, 0xFFFFFFFFu, Wc, Wt, rowB, null_row, acc[0], bl[0], bq[0]);
+    } else
+#pragma unroll
+    for (int q = 0; q < BU; ++q) {                 // the rest of each bag
+      int i0 = lo[q] + P;
+      const int h = hi[q];
+#define SG_STEP(U) sg_step<U, P, HAS_VALS>(rows, shards, vals, s_base, i0 + p, Wc, Wt, rowB, null_row, acc[q], bl[q], bq[q])
+      for (; i0 + 4 * P <= h; i0 += 4 * P) SG_STEP(4);
+      if (i0 + 2 * P <= h) { SG_STEP(2); i0 += 2 * P; }
+      if (i0 + P <= h) { SG_STEP(1); i0 += P; }
+      if (i0 + p < h) SG_STEP(1);
+#undef SG_STEP
+    }
+#pragma unroll
+    for (int q = 0; q < BU; ++q) {
+      const int f = gs + (r * BU + q) * ng;
+#pragma unroll
+      for (int d = G; d < LB; d <<= 1) {               // combine the bag's sub-groups
+        acc[q].x += __shfl_xor_sync(0xFFFFFFFFu, acc[q].x, d); acc[q].y += __shfl_xor_sync(0xFFFFFFFFu, acc[q].y, d);
+        acc[q].z += __shfl_xor_sync(0xFFFFFFFFu, acc[q].z, d); acc[q].w += __shfl_xor_sync(0xFFFFFFFFu, acc[q].w, d);
+        if (!COOP) { bl[q] += __shfl_xor_sync(0xFFFFFFFFu, bl[q], d); bq[q] += __shfl_xor_sync(0xFFFFFFFFu, bq[q], d); }
+      }
+      if (COOP && FIELD)
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) { bl[q] += __shfl_xor_sync(0xFFFFFFFFu, bl[q], d); bq[q] += __shfl_xor_sync(0xFFFFFFFFu, bq[q], d); }
+      if (COOP && !FIELD) { R += (double)bl[q]; Q += (double)bq[q]; }   // (every lane its own occurrences)
+      if (f < F && p == 0) {
+        if (col) {
+          const size_t o = ((size_t)b * F + f) * K4 + c4;
+          reinterpret_cast<float4*>(pooled)[o] = acc[q];
+          if (pooled_b) store_bf16x4(pooled_b + o * 4, acc[q]);
+        }
+        if (FIELD) {
+          if (col) s_pool[f * K4 + c4] = acc[q];
+          if (c4 == 0) s_bt[f] = make_float2(bl[q], bq[q]);
+        } else {
+          Ax += (double)acc[q].x; Ay += (double)acc[q].y; Az += (double)acc[q].z; Aw += (double)acc[q].w;
+          if (!COOP) { R += (double)bl[q]; Q += (double)bq[q]; }
+        }
+      }
     }
   }
-  if (!lr) tr = 0.0;
-  if (!fm) tq = 0.0;
-  double aa = ax * ax + ay * ay + az * az + aw * aw;
+  if (!FIELD) {
+    // groups of the warp (p > 0 lanes hold zeros), then warps of the sample
 #pragma unroll
-  for (int d = 1; d < G; d <<= 1) aa += __shfl_xor_sync(0xFFFFFFFFu, aa, d);
-  if (!live) return;
-  float4* o = reinterpret_cast<float4*>(out_small + (size_t)b * stride);
-  if (c4 < K4) o[c4] = make_float4((float)ax, (float)ay, (float)az, (float)aw);
-  if (c4 == 0) o[K4] = make_float4((float)tr, fm ? (float)(0.5 * aa - 0.5 * tq) : 0.f, (float)tq, 0.f);
+    for (int d = G; d < 32; d <<= 1) {
+      Ax += __shfl_xor_sync(0xFFFFFFFFu, Ax, d); Ay += __shfl_xor_sync(0xFFFFFFFFu, Ay, d);
+      Az += __shfl_xor_sync(0xFFFFFFFFu, Az, d); Aw += __shfl_xor_sync(0xFFFFFFFFu, Aw, d);
+    }
+#pragma unroll
+    for (int d = COOP ? 1 : G; d < 32; d <<= 1) { R += __shfl_xor_sync(0xFFFFFFFFu, R, d); Q += __shfl_xor_sync(0xFFFFFFFFu, Q, d); }
+    if (wps > 1) {
+      if (lane < G) {
+        s_red[warp][lane][0] = Ax; s_red[warp][lane][1] = Ay; s_red[warp][lane][2] = Az; s_red[warp][lane][3] = Aw;
+        if (lane == 0) { s_tail[warp][0] = R; s_tail[warp][1] = Q; }
+      }
+      __syncthreads();
+      if (ws != 0) return;                             // whole warp
+      Ax = Ay = Az = Aw = R = Q = 0.0;
+      for (int i = 0; i < wps; ++i) {
+        Ax += s_red[warp + i][lane % G][0]; Ay += s_red[warp + i][lane % G][1];
+        Az += s_red[warp + i][lane % G][2]; Aw += s_red[warp + i][lane % G][3];
+        R += s_tail[warp + i][0]; Q += s_tail[warp + i][1];
+      }
+    }
+    if (b >= B) return;                                // whole warp
+    if (!lr) R = 0.0;
+    if (!fm) { Ax = Ay = Az = Aw = 0.0; Q = 0.0; }
+    double aa = (lane < G && col) ? Ax * Ax + Ay * Ay + Az * Az + Aw * Aw : 0.0;
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) aa += __shfl_xor_sync(0xFFFFFFFFu, aa, d);
+    float4* o = reinterpret_cast<float4*>(out_small + (size_t)b * stride);
+    if (lane < G && col) o[c4] = make_float4((float)Ax, (float)Ay, (float)Az, (float)Aw);
+    if (lane == 0) o[K4] = make_float4((float)R, fm ? (float)(0.5 * aa - 0.5 * Q) : 0.f, (float)Q, 0.f);
+    return;
+  }
+  __syncthreads();
+  // one shard's partial of one sample, column c (K4 = the tail): its own fields in field order
+  auto shard_sum = [&](int t, int s, int c) {
+    const float4* sp = reinterpret_cast<const float4*>(sg_smem) + (size_t)t * F * K4;
+    const float2* sb = reinterpret_cast<const float2*>(sg_smem + (size_t)T * F * k * 4) + (size_t)t * F;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c < K4) {
+      if (fm) for (int f = s; f < F; f += S) { const float4 v = sp[f * K4 + c]; a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w; }
+    } else {
+      for (int f = s; f < F; f += S) { const float2 v = sb[f]; a.x += v.x; a.y += v.y; }
+      if (!lr) a.x = 0.f;
+      if (!fm) a.y = 0.f;
+    }
+    return a;
+  };
+  if (part_small)
+    for (int i = threadIdx.x; i < T * S * (K4 + 1); i += 256) {
+      const int c = i % (K4 + 1), x = i / (K4 + 1), t = x % T, s = x / T, bb = blockIdx.x * T + t;
+      if (bb < B) reinterpret_cast<float4*>(part_small + ((size_t)s * B + bb) * stride)[c] = shard_sum(t, s, c);
+    }
+  if (out_small && ws == 0 && b < B) {                 // the sample's first warp; lanes 0 .. G-1 a column each
+    double ax = 0.0, ay = 0.0, az = 0.0, aw = 0.0, tr = 0.0, tq = 0.0;
+    if (lane < G)
+      for (int s = 0; s < S; ++s) {
+        if (col) { const float4 v = shard_sum(st, s, c4); ax += (double)v.x; ay += (double)v.y; az += (double)v.z; aw += (double)v.w; }
+        if (lane == 0) { const float4 v = shard_sum(st, s, K4); tr += (double)v.x; tq += (double)v.y; }
+      }
+    double aa = ax * ax + ay * ay + az * az + aw * aw;
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) aa += __shfl_xor_sync(0xFFFFFFFFu, aa, d);
+    float4* o = reinterpret_cast<float4*>(out_small + (size_t)b * stride);
+    if (lane < G && col) o[c4] = make_float4((float)ax, (float)ay, (float)az, (float)aw);
+    if (lane == 0) o[K4] = make_float4((float)tr, fm ? (float)(0.5 * aa - 0.5 * tq) : 0.f, (float)tq, 0.f);
+  }
 }
 
 // FIELD partition: a bag belongs to one shard (field f lives on shard f mod S), so the sub-operators of shard s
@@ -512,6 +733,8 @@ template <int G, bool FUSED>
 __global__ void __launch_bounds__(256) field_partials_kernel(const float* __restrict__ pooled, const float2* __restrict__ bag_tail,
                                                              int B, int F, int S, int k, uint32_t ops,
                                                              float* __restrict__ part_small, float* __restrict__ out_small) {
+  des_pdl_wait(pooled, bag_tail, part_small, out_small);
+  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = t / G, c4 = t % G;
@@ -554,6 +777,8 @@ __global__ void __launch_bounds__(256) field_partials_kernel(const float* __rest
 
 // sum over shards of a dense [S][B][n] tensor (materialised pooled / dense partials)
 __global__ void reduce_shards_kernel(const float* __restrict__ part, size_t per_shard, int S, float* __restrict__ out) {
+  des_pdl_wait(part, out);
+  des_pdl_go();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x, st = (size_t)gridDim.x * blockDim.x;
   for (; i < per_shard; i += st) {
     float a = 0.f;
@@ -565,6 +790,9 @@ __global__ void reduce_shards_kernel(const float* __restrict__ part, size_t per_
 static int group_for(int k) { int K4 = k / 4, G = 1; while (G < K4) G <<= 1; return G; }
 
 static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, float* pooled, cudaStream_t cs);
+static bool sample_gather_fits(const des_table* t) { return (size_t)t->F * (t->k + 2) * 4 <= (48u << 10); }   // FIELD form, one sample
+static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, bool field, float* pooled,
+                                         float* part_small, float* out_small, cudaStream_t cs);
 
 // shared by des_forward_partials (fused_out == NULL) and des_forward_fused
 static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t* b, const des_partials_t* part,
@@ -588,10 +816,12 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
   const int G = group_for(t->k);
   if (t->cfg.partition == DES_PART_FIELD && pl && !pp && (ps || fused_out)) {
     // FIELD partition with pooling among the operators: one gather pass (pooled vectors + bag tails), then the
-    // per-shard sub-operators as sums over each shard's own fields — no routing pass, no second gather
+    // per-shard sub-operators as sums over each shard's own fields — no routing pass, no second gather.  In one kernel
+    // unless a sample's pooled vectors do not fit its shared memory.
+    if (sample_gather_fits(t)) return launch_sample_gather(t, ops, b, true, pl, ps, fused_out, cs);
     if ((st = launch_single_gather(t, ops, b, pl, cs)) != DES_OK) return st;
     const int grid = (int)(((long long)B * G + 255) / 256);
-#define FP2(GG, FU) field_partials_kernel<GG, FU><<<grid, 256, 0, cs>>>(pl, t->bag_tail, B, (int)t->F, (int)t->S, t->k, ops, ps, fused_out)
+#define FP2(GG, FU) des_launch(field_partials_kernel<GG, FU>, grid, 256, 0, cs, (const float*)pl, t->bag_tail, B, (int)t->F, (int)t->S, (int)t->k, ops, ps, fused_out)
 #define FP(GG) do { if (fused_out) FP2(GG, true); else FP2(GG, false); } while (0)
     switch (G) { case 1: FP(1); break; case 2: FP(2); break; case 4: FP(4); break; case 8: FP(8); break; default: FP(16); }
 #undef FP
@@ -601,17 +831,16 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
   }
   // routing: rows of every occurrence in shard-major order per sample (workspace shared with find_or_insert,
   // which has finished with it by the time a forward can run on the same stream)
-  uint32_t* grow_csr = t->uslot;
   uint32_t* grow_sorted = t->slot_of;
   float* x_sorted = t->x_sorted;
-  route_kernel<<<(B + 7) / 8 < t->sm_count * 8 ? (B + 7) / 8 : t->sm_count * 8, 256, 0, cs>>>(
-      b->offsets, b->vals, b->rows, b->shards, B, t->F, t->S, t->meta, (uint32_t)t->total_rows, grow_csr, grow_sorted,
-      x_sorted, t->seg_off);
+  uint32_t* grow_csr = t->uslot;
+  des_launch(route_kernel, (B + 7) / 8 < t->sm_count * 8 ? (B + 7) / 8 : t->sm_count * 8, 256, 0, cs, b->offsets, b->vals, b->rows,
+             b->shards, B, (int)t->F, (int)t->S, t->meta, (uint32_t)t->total_rows, grow_csr, grow_sorted, x_sorted, t->seg_off);
   DES_LAUNCH_CHECK(t, "route_kernel");
   if (ps || fused_out) {
     const unsigned grid = (unsigned)((B + 7) / 8);      // one warp per sample
-#define SP3(GG, HV, FU) shard_partials_kernel<GG, HV, FU><<<grid, 256, 0, cs>>>(grow_sorted, x_sorted, t->seg_off, B, t->S, \
-                                                                              t->k, ops, t->W, (uint32_t)t->total_rows, ps, fused_out)
+#define SP3(GG, HV, FU) des_launch(shard_partials_kernel<GG, HV, FU>, grid, 256, 0, cs, grow_sorted, x_sorted, t->seg_off, B,   \
+                                   (int)t->S, (int)t->k, ops, t->W, (uint32_t)t->total_rows, ps, fused_out)
 #define SP(GG) do { if (fused_out) { if (b->vals) SP3(GG, true, true); else SP3(GG, false, true); } \
                     else { if (b->vals) SP3(GG, true, false); else SP3(GG, false, false); } } while (0)
     switch (G) { case 1: SP(1); break; case 2: SP(2); break; case 4: SP(4); break; case 8: SP(8); break; default: SP(16); }
@@ -630,8 +859,8 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
     // with the first layer among the operators the pooled vectors are also left as bfloat16, the operand
     // format of the tensor-core product that follows (one conversion pass less)
     __nv_bfloat16* pb = ((ops & DES_OP_DENSE1) && t->use_tc && !pp) ? t->pooled_b : nullptr;
-#define PK5(GG, PP, HV, MT, BO) pool_kernel<GG, PP, HV, MT, BO><<<grid, 256, 0, cs>>>(                                 \
-        b->offsets, b->vals, grow_csr, b->shards, nbags, B, t->F, t->k, t->W, (uint32_t)t->total_rows, pl, pp, pb)
+#define PK5(GG, PP, HV, MT, BO) des_launch(pool_kernel<GG, PP, HV, MT, BO>, grid, 256, 0, cs, b->offsets, b->vals, grow_csr,    \
+        b->shards, nbags, B, (int)t->F, (int)t->k, t->W, (uint32_t)t->total_rows, pl, pp, pb)
 #define PK3(GG, HV, MT, BO) do { if (wide) PK5(GG, 32 / GG, HV, MT, BO); else PK5(GG, 1, HV, MT, BO); } while (0)
 #define PK2(GG, HV) do { if (pp) PK3(GG, HV, true, false); else if (pb) PK3(GG, HV, false, true); else PK3(GG, HV, false, false); } while (0)
 #define PK(GG) do { if (b->vals) PK2(GG, true); else PK2(GG, false); } while (0)
@@ -661,9 +890,8 @@ static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des
   if (blocks > (long long)t->sm_count * POOL_BLOCKS_PER_SM) blocks = (long long)t->sm_count * POOL_BLOCKS_PER_SM;
   const unsigned grid = (unsigned)blocks;
   __nv_bfloat16* pb = ((ops & DES_OP_DENSE1) && t->use_tc) ? t->pooled_b : nullptr;
-#define SG3(GG, PP, HV) single_gather_kernel<GG, PP, HV><<<grid, 256, 0, cs>>>(b->offsets, b->vals, b->rows, b->shards, nbags,   \
-                                                                              (int)t->S, t->k, t->W, t->meta,                 \
-                                                                              (uint32_t)t->total_rows, pooled, t->bag_tail, pb)
+#define SG3(GG, PP, HV) des_launch(single_gather_kernel<GG, PP, HV>, grid, 256, 0, cs, b->offsets, b->vals, b->rows, b->shards, nbags, \
+                                   (int)t->S, (int)t->k, t->W, t->meta, (uint32_t)t->total_rows, pooled, t->bag_tail, pb)
 #define SG2(GG, HV) do { if (wide) SG3(GG, 32 / GG, HV); else SG3(GG, 1, HV); } while (0)
 #define SG(GG) do { if (b->vals) SG2(GG, true); else SG2(GG, false); } while (0)
   switch (G) { case 1: SG(1); break; case 2: SG(2); break; case 4: SG(4); break; case 8: SG(8); break; default: SG(16); }
@@ -675,17 +903,32 @@ static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des
   return DES_OK;
 }
 
-// des_forward_fused with pooling among the operators: one gather pass for everything.
-static des_status_t forward_single_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, float* pooled,
-                                          float* out_small, cudaStream_t cs) {
-  des_status_t st = launch_single_gather(t, ops, b, pooled, cs);
-  if (st != DES_OK) return st;
-  const int B = b->batch, G = group_for(t->k);
-  const int grid = (int)(((long long)B * G + 255) / 256);
-#define FF(GG) fused_finish_kernel<GG><<<grid, 256, 0, cs>>>(pooled, t->bag_tail, B, (int)t->F, t->k, ops, out_small)
-  switch (G) { case 1: FF(1); break; case 2: FF(2); break; case 4: FF(4); break; case 8: FF(8); break; default: FF(16); }
-#undef FF
-  DES_LAUNCH_CHECK(t, "fused_finish_kernel");
+// Samples per block: one warp per sample once there are samples for the chip, more warps per sample below that (as long as
+// they have bags to take), and always for samples of many long bags, whose lengths differ too much for one warp each.
+static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, bool field, float* pooled,
+                                         float* part_small, float* out_small, cudaStream_t cs) {
+  const int B = b->batch, F = (int)t->F, G = group_for(t->k);
+  const bool wide = b->nnz >= 8ll * B * F;
+  const int per_warp = wide ? 1 : 32 / G * SGF_BU;      // bags a warp has in flight
+  int T = 8;
+  while (T > 1 && (B < t->sm_count * 4 * T || (wide && b->nnz >= 256ll * B)) && F > per_warp * (8 / T)) T >>= 1;
+  const size_t per_sample = field ? (size_t)F * (t->k + 2) * 4 : 0;
+  while (T > 1 && T * per_sample > SGF_SMEM) T >>= 1;
+  const unsigned grid = (unsigned)((B + T - 1) / T);
+  __nv_bfloat16* pb = ((ops & DES_OP_DENSE1) && t->use_tc) ? t->pooled_b : nullptr;
+#define SF4(GG, PP, HV, FD) des_launch(sample_gather_kernel<GG, PP, HV, FD>, grid, 256, T * per_sample, cs, b->offsets, b->vals,     \
+                                       b->rows, b->shards, B, F, (int)t->S, (int)t->k, T, ops, t->W, t->meta,                     \
+                                       (uint32_t)t->total_rows, pooled, pb, part_small, out_small)
+#define SF3(GG, PP, HV) do { if (field) SF4(GG, PP, HV, true); else SF4(GG, PP, HV, false); } while (0)
+#define SF2(GG, HV) do { if (wide) SF3(GG, 32 / GG, HV); else SF3(GG, 1, HV); } while (0)
+#define SF(GG) do { if (b->vals) SF2(GG, true); else SF2(GG, false); } while (0)
+  switch (G) { case 1: SF(1); break; case 2: SF(2); break; case 4: SF(4); break; case 8: SF(8); break; default: SF(16); }
+#undef SF
+#undef SF2
+#undef SF3
+#undef SF4
+  DES_LAUNCH_CHECK(t, "sample_gather_kernel");
+  t->pooled_b_src = pb ? pooled : nullptr;
   return DES_OK;
 }
 
@@ -705,7 +948,7 @@ extern "C" des_status_t des_forward_fused(des_table_t* t, uint32_t ops, const de
     if (!part->pooled || ((ops & DES_OP_DENSE1) && !t->H)) return DES_ERR_INVALID_ARG;
     des_api_begin(t, (cudaStream_t)stream);
     DES_DBG_ARM(t, (cudaStream_t)stream);
-    st = forward_single_gather(t, ops, b, part->pooled, out->out_small, (cudaStream_t)stream);
+    st = launch_sample_gather(t, ops, b, false, part->pooled, nullptr, out->out_small, (cudaStream_t)stream);
   } else {
     st = forward_impl(t, ops, b, part, out->out_small, stream);
   }
@@ -726,13 +969,15 @@ extern "C" des_status_t des_aggregate(des_table_t* t, uint32_t ops, const des_ba
     const int G = group_for(t->k);
     const long long threads = (long long)B * G;
     const int grid = (int)((threads + 255) / 256);
+#define AGG(GG) des_launch(aggregate_small_kernel<GG>, grid, 256, 0, cs, part->part_small, B, (int)t->S, (int)t->k, ops, out->out_small)
     switch (G) {
-      case 1: aggregate_small_kernel<1><<<grid, 256, 0, cs>>>(part->part_small, B, t->S, t->k, ops, out->out_small); break;
-      case 2: aggregate_small_kernel<2><<<grid, 256, 0, cs>>>(part->part_small, B, t->S, t->k, ops, out->out_small); break;
-      case 4: aggregate_small_kernel<4><<<grid, 256, 0, cs>>>(part->part_small, B, t->S, t->k, ops, out->out_small); break;
-      case 8: aggregate_small_kernel<8><<<grid, 256, 0, cs>>>(part->part_small, B, t->S, t->k, ops, out->out_small); break;
-      default: aggregate_small_kernel<16><<<grid, 256, 0, cs>>>(part->part_small, B, t->S, t->k, ops, out->out_small); break;
+      case 1: AGG(1); break;
+      case 2: AGG(2); break;
+      case 4: AGG(4); break;
+      case 8: AGG(8); break;
+      default: AGG(16); break;
     }
+#undef AGG
     DES_LAUNCH_CHECK(t, "aggregate_small_kernel");
   }
   if (ops & (DES_OP_POOL | DES_OP_DENSE1)) {
@@ -740,7 +985,7 @@ extern "C" des_status_t des_aggregate(des_table_t* t, uint32_t ops, const des_ba
     const size_t n = (size_t)B * t->F * t->k;
     if (part->part_pooled) {
       // materialised per-shard pooled partials: aggregate them in shard order
-      reduce_shards_kernel<<<t->sm_count * 4, 256, 0, cs>>>(part->part_pooled, n, t->S, out->pooled);
+      des_launch(reduce_shards_kernel, t->sm_count * 4, 256, 0, cs, part->part_pooled, n, (int)t->S, out->pooled);
       DES_LAUNCH_CHECK(t, "reduce_shards_kernel");
       t->pooled_b_src = nullptr;
     } else if (out->pooled != part->pooled) {
@@ -752,7 +997,7 @@ extern "C" des_status_t des_aggregate(des_table_t* t, uint32_t ops, const des_ba
     des_status_t st = des_dense1_forward(t, out->pooled, B, out->Z, part->part_dense, part->part_pooled, cs);
     if (st != DES_OK) return st;
     if (part->part_dense) {
-      reduce_shards_kernel<<<t->sm_count * 4, 256, 0, cs>>>(part->part_dense, (size_t)B * t->H, t->S, out->Z);
+      des_launch(reduce_shards_kernel, t->sm_count * 4, 256, 0, cs, part->part_dense, (size_t)B * t->H, (int)t->S, out->Z);
       DES_LAUNCH_CHECK(t, "reduce_shards_kernel");
     }
   }
@@ -765,7 +1010,7 @@ extern "C" des_status_t des_rank_partial(des_table_t* t, int32_t batch, const fl
   if (!t || !d_part_small || !d_rank_part || batch <= 0 || batch > t->max_batch) return DES_ERR_INVALID_ARG;
   cudaStream_t cs = (cudaStream_t)stream;
   des_api_begin(t, cs);
-  reduce_shards_kernel<<<t->sm_count * 4, 256, 0, cs>>>(d_part_small, (size_t)batch * t->stride, t->S, d_rank_part);
+  des_launch(reduce_shards_kernel, t->sm_count * 4, 256, 0, cs, d_part_small, (size_t)batch * t->stride, (int)t->S, d_rank_part);
   DES_LAUNCH_CHECK(t, "reduce_shards_kernel");
   return DES_OK;
 }
@@ -779,13 +1024,15 @@ extern "C" des_status_t des_aggregate_ranks(des_table_t* t, uint32_t ops, int32_
   des_api_begin(t, cs);
   const int G = group_for(t->k);
   const int grid = (int)(((long long)batch * G + 255) / 256);
+#define AGG(GG) des_launch(aggregate_small_kernel<GG>, grid, 256, 0, cs, d_rank_parts, batch, world, (int)t->k, ops, d_out_small)
   switch (G) {   // the processes' messages are added like shards' partials: fixed (rank) order, then F
-    case 1: aggregate_small_kernel<1><<<grid, 256, 0, cs>>>(d_rank_parts, batch, world, t->k, ops, d_out_small); break;
-    case 2: aggregate_small_kernel<2><<<grid, 256, 0, cs>>>(d_rank_parts, batch, world, t->k, ops, d_out_small); break;
-    case 4: aggregate_small_kernel<4><<<grid, 256, 0, cs>>>(d_rank_parts, batch, world, t->k, ops, d_out_small); break;
-    case 8: aggregate_small_kernel<8><<<grid, 256, 0, cs>>>(d_rank_parts, batch, world, t->k, ops, d_out_small); break;
-    default: aggregate_small_kernel<16><<<grid, 256, 0, cs>>>(d_rank_parts, batch, world, t->k, ops, d_out_small); break;
+    case 1: AGG(1); break;
+    case 2: AGG(2); break;
+    case 4: AGG(4); break;
+    case 8: AGG(8); break;
+    default: AGG(16); break;
   }
+#undef AGG
   DES_LAUNCH_CHECK(t, "aggregate_small_kernel");
   return DES_OK;
 }

@@ -15,6 +15,8 @@ __global__ void __launch_bounds__(256) head_kernel(
     const float* __restrict__ out_small, const float* __restrict__ Z, const float* __restrict__ pooled,
     const float* __restrict__ xdense, const float* __restrict__ y, float* __restrict__ logit, float* __restrict__ loss,
     float* __restrict__ gL, float* __restrict__ gF, float* __restrict__ gZ, float* __restrict__ gE) {
+  des_pdl_wait(u, b1, q, d, out_small, Z, pooled, xdense, y, logit, loss, gL, gF, gZ, gE);
+  des_pdl_go();
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;                                  // whole warp
@@ -82,10 +84,9 @@ extern "C" des_status_t des_head(des_table_t* t, uint32_t ops, int32_t batch, co
   if (head->n_dense < 0 || (head->n_dense > 0 && head->d && !d_xdense)) return DES_ERR_INVALID_ARG;
   cudaStream_t cs = (cudaStream_t)stream;
   des_api_begin(t, cs);
-  head_kernel<<<(batch + 7) / 8, 256, 0, cs>>>(batch, (int)t->k, (int)t->H, (int)(t->F * t->k), head->n_dense, ops, head->b0,
-                                               head->c_lr, head->c_fm, head->u, head->b1, head->q,
-                                               head->n_dense > 0 ? head->d : nullptr, out->out_small, out->Z, out->pooled,
-                                               d_xdense, d_y, d_logit, d_loss, g->gL, g->gF, g->gZ, g->gE);
+  des_launch(head_kernel, (batch + 7) / 8, 256, 0, cs, batch, (int)t->k, (int)t->H, (int)(t->F * t->k), head->n_dense, ops, head->b0,
+             head->c_lr, head->c_fm, head->u, head->b1, head->q, head->n_dense > 0 ? head->d : nullptr, out->out_small, out->Z,
+             out->pooled, d_xdense, d_y, d_logit, d_loss, g->gL, g->gF, g->gZ, g->gE);
   DES_LAUNCH_CHECK(t, "head_kernel");
   return DES_OK;
 }

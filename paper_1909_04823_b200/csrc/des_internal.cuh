@@ -163,7 +163,9 @@ static inline void des_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at; cfg.numAttrs = 1;
+  // (a launch of many waves gains nothing, and its waiting blocks take room in the last wave of the kernel before: a step
+  // of 32 M occurrences 4.56 ms with this rule, 4.59 without)
+  cfg.attrs = &at; cfg.numAttrs = grid.x <= 8192u ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, (P)args...);        // (errors are picked up by DES_LAUNCH_CHECK)
 }
 

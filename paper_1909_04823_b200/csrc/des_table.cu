@@ -359,6 +359,8 @@ __global__ void __launch_bounds__(256) read_rows_kernel(const uint32_t* __restri
                                                         float* __restrict__ lin, float* __restrict__ acc_emb,
                                                         float* __restrict__ acc_lin) {
   constexpr int VW = sizeof(V) / 4;
+  des_pdl_wait(grows, W, A, emb, lin, acc_emb, acc_lin);
+  des_pdl_go();
   const int C = k / VW, lane = threadIdx.x % G;
   // a warp's groups take neighbouring rows, its ROWS_U rounds too
   const long long i0 = ((long long)blockIdx.x * 256 + (threadIdx.x & ~31)) / G * ROWS_U + (threadIdx.x & 31) / G;
@@ -411,8 +413,8 @@ extern "C" des_status_t des_table_read_rows(des_table_t* t, const uint32_t* d_gl
   if (!d_global_rows) return DES_ERR_INVALID_ARG;
   des_api_begin(t, (cudaStream_t)stream);
   const int G = rows_group((int)t->k);
-#define RR(GG, VV) read_rows_kernel<GG, VV><<<rows_grid(n, GG), 256, 0, (cudaStream_t)stream>>>(                       \
-      d_global_rows, n, t->k, t->stride, t->total_rows, t->W, t->A, d_emb, d_lin, d_acc_emb, d_acc_lin)
+#define RR(GG, VV) des_launch(read_rows_kernel<GG, VV>, rows_grid(n, GG), 256, 0, (cudaStream_t)stream, d_global_rows, (long long)n,  \
+      (int)t->k, (int)t->stride, (unsigned long long)t->total_rows, t->W, t->A, d_emb, d_lin, d_acc_emb, d_acc_lin)
   if (!rows_vec(d_emb, d_acc_emb)) RR(16, float);
   else switch (G) { case 1: RR(1, float4); break; case 2: RR(2, float4); break; case 4: RR(4, float4); break;
                     case 8: RR(8, float4); break; default: RR(16, float4); }
