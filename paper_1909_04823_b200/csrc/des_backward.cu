@@ -17,225 +17,93 @@
 // Hot keys.  CTR ids are Zipf distributed: a handful of keys own most of a
 // batch's occurrences.  Millions of float atomics on one gradient row would
 // serialise in L2 and, summed one after the other in fp32, lose the 1e-5
-// accuracy the step must keep.  So before the scatter, occurrences are counted
+// accuracy the step must keep.  So find_or_insert counts the occurrences
 // per unique key on a sample of the batch; a key whose estimated count reaches
-// HOT_MIN gets R = count / CHAIN private replica rows, every occurrence is sent
-// to replica hash(j) mod R, and after the scatter the replicas of a key are
-// summed in double into its gradient row.  No accumulator ever takes more than
+// HOT_MIN gets R = count / HOT_CHAIN private replica rows, every occurrence is sent
+// to replica hash(j) mod R, and the update sums the replicas of a key
+// in double.  No accumulator ever takes more than
 // a few hundred float additions, and no address is shared by more than that
 // many atomics.
+//
+// Two kernels, then (a small batch's scatter looks an occurrence's gradient row up itself: batch-unique index -> the
+// key's word of hinfo -> replica; a large batch has it done in a pass before): the update's first blocks take the hot keys.  Six kernels and two memsets around the same
+// two took 40 us of a 100 us step at 10 k occurrences, and 180 us of passes over index arrays at 32 M.
+#include <type_traits>
+
 #include "des_internal.cuh"
 
-#define HOT_MIN 512u      // estimated occurrences from which a key is treated as hot
-#define HOT_CHAIN 256u    // target number of additions per replica row
-#define SUPER_R 64u       // replica rows of a super key (they only take one partial sum per lane group)
 #ifndef SC_BLOCKS_PER_SM
 #define SC_BLOCKS_PER_SM 64     // grid cap of the scatter (it strides over the bags)
 #endif
 
-__device__ __forceinline__ uint32_t hash_u32(uint32_t x) {
-  x ^= x >> 16; x *= 0x7FEB352Du; x ^= x >> 15; x *= 0x846CA68Bu; x ^= x >> 16;
-  return x;
-}
-
-// hinfo[u] += 1 for a 1 / 2^shift sample of the occurrences.  A hot key would draw tens of
-// thousands of atomics on one word, which L2 serialises; so counts are first merged per warp
-// (lanes holding the same key), then per block in a small shared-memory table keyed by a hash of
-// the key (a slot taken by another key sends the count straight to memory), and each block adds
-// its table to hinfo once.
-#define SC_THREADS 1024
-#define SC_SLOTS 1024
-#ifndef SC_PER
-#define SC_PER 4
-#endif
-__global__ void __launch_bounds__(SC_THREADS) sample_count_kernel(const uint32_t* __restrict__ uidx, int nnz, int shift,
-                                                                  long long max_uniq, uint32_t* hinfo) {
-  __shared__ uint32_t s_key[SC_SLOTS], s_cnt[SC_SLOTS];
-  for (int i = threadIdx.x; i < SC_SLOTS; i += SC_THREADS) { s_key[i] = DES_ROW_NONE; s_cnt[i] = 0u; }
-  __syncthreads();
-  // SC_PER samples per thread, their loads in flight together
-  uint32_t u[SC_PER];
+// The gradient row of occurrence j: its key's own row, one of the key's replicas, or the tag of a key that is counted
+// instead (batch-unique index -> the key's word of hinfo -> replica).
+struct DestMap {
+  const uint32_t* uidx;
+  const uint32_t* hinfo;
+  const uint2* hot_rep;
+  uint32_t max_uniq;
+  uint32_t* dest;
+};
+template <int U>
+__device__ __forceinline__ void dest_rows(const DestMap& m, int i, int step, uint32_t (&d)[U]) {
+  uint32_t h[U];
 #pragma unroll
-  for (int q = 0; q < SC_PER; ++q) {
-    const long long i = ((long long)blockIdx.x * SC_PER + q) * SC_THREADS + threadIdx.x;
-    const long long j = (i << shift) + (shift ? (hash_u32((uint32_t)i) & ((1u << shift) - 1u)) : 0u);
-    u[q] = DES_ROW_NONE;
-    if (j < nnz) u[q] = __ldg(uidx + j);
+  for (int u = 0; u < U; ++u) d[u] = __ldg(m.uidx + i + u * step);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (d[u] >= m.max_uniq) d[u] = DES_ROW_NONE;        // no row, or more keys than the gradient buffer holds
+    h[u] = d[u] != DES_ROW_NONE ? __ldg(m.hinfo + d[u]) : 0u;
   }
 #pragma unroll
-  for (int q = 0; q < SC_PER; ++q) {
-    const bool ok = u[q] != DES_ROW_NONE && (long long)u[q] < max_uniq;
-    const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
-    if (ok) {
-      const unsigned same = __match_any_sync(act, u[q]);
-      if ((threadIdx.x & 31) == __ffs(same) - 1) {
-        const uint32_t c = (uint32_t)__popc(same), slot = hash_u32(u[q]) & (SC_SLOTS - 1);
-        const uint32_t old = atomicCAS(&s_key[slot], DES_ROW_NONE, u[q]);
-        if (old == DES_ROW_NONE || old == u[q]) atomicAdd(&s_cnt[slot], c);
-        else atomicAdd(hinfo + u[q], c);
+  for (int u = 0; u < U; ++u)
+    if (h[u] & HOT_FLAG) {
+      const uint32_t sup = (h[u] >> 24) & 0x7Fu;
+      if (sup) {
+        d[u] = SUPER_TAG | (sup - 1u);
+      } else {   // replica floor(hash * R / 2^32): uniform over the R replicas without a division
+        const uint2 rp = __ldg(m.hot_rep + (h[u] & 0xFFFFFFu));
+        d[u] = m.max_uniq + rp.x + __umulhi(des_hash32((uint32_t)(i + u * step)), rp.y);
       }
     }
-  }
-  __syncthreads();
-  for (int s = threadIdx.x; s < SC_SLOTS; s += SC_THREADS)
-    if (s_cnt[s]) atomicAdd(hinfo + s_key[s], s_cnt[s]);
 }
 
-// Turns the sampled counts into the hot list: hinfo[u] becomes the key's hot
-// index, or DES_ROW_NONE for a cold key.  ctr[0] = hot keys, ctr[1] = replica rows.
-__global__ void __launch_bounds__(256) hot_select_kernel(uint32_t* hinfo, const uint32_t* __restrict__ n_uniq,
-                                                         long long max_uniq, int shift, uint32_t* hot_base,
-                                                         uint32_t* hot_R, uint32_t* hot_u, uint32_t* ctr,
-                                                         uint32_t h_max, uint32_t rep_max, DevMeta* meta,
-                                                         uint32_t* hot_work, uint32_t work_max, uint32_t super_min) {
-  long long U = *n_uniq;
-  if (U > max_uniq) U = max_uniq;   // more unique keys than the gradient buffer holds: the backward reports it
-  for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < U; u += (long long)gridDim.x * blockDim.x) {
-    const uint32_t est = hinfo[u] << shift;
-    uint32_t h = DES_ROW_NONE;
-    if (est >= HOT_MIN) {
-      // the few keys that own a large share of the batch (super_min = 0: feature off) take one of
-      // SUPER_T slots: ctr[3] = slots claimed, ctr[4 + slot] = hot index; hinfo carries slot + 1 in bits 24..
-      bool sup = false;
-      uint32_t ts = 0;
-      if (super_min && est >= super_min) { ts = atomicAdd(&ctr[3], 1u); sup = ts < SUPER_T; }
-      // (capped so that a key's chunk number fits the 18 bits of a work item; longer chains only cost accuracy)
-      const uint32_t R = sup ? SUPER_R : min((est + HOT_CHAIN - 1) / HOT_CHAIN, 0x3FFFFu * HOT_RCHUNK);
-      const uint32_t hh = atomicAdd(&ctr[0], 1u);
-      if (hh < h_max) {
-        const uint32_t base = atomicAdd(&ctr[1], R);
-        const uint32_t nchunk = (R + HOT_RCHUNK - 1) / HOT_RCHUNK;
-        bool ok = base + R <= rep_max;
-        uint32_t wbase = 0;
-        if (ok) { wbase = atomicAdd(&ctr[2], nchunk); ok = wbase + nchunk <= work_max; }
-        if (ok) {
-          hot_base[hh] = base; hot_R[hh] = R; hot_u[hh] = (uint32_t)u;
-          h = hh | (sup ? (ts + 1u) << 24 : 0u);
-          for (uint32_t i = 0; i < nchunk; ++i) hot_work[wbase + i] = (hh << 18) | i;
-        } else {
-          hot_R[hh] = 0;
-        }
-      }
-      if (sup) ctr[HOT_CTR_SLOT + ts] = (h == DES_ROW_NONE) ? DES_ROW_NONE : (h & 0xFFFFFFu);
-    }
-    hinfo[u] = h;
-  }
-}
-
-// dest[j] = gradient row of occurrence j: the key's own row, one of its replicas, or the tag of a
-// register-summed key.  Four occurrences per thread: their look-up chains are in flight together.
-__global__ void __launch_bounds__(256) make_dest_kernel(const uint32_t* __restrict__ uidx, int nnz,
-                                                        const uint32_t* __restrict__ hinfo,
-                                                        const uint32_t* __restrict__ hot_base,
-                                                        const uint32_t* __restrict__ hot_R, long long max_uniq,
-                                                        uint32_t* __restrict__ dest) {
+// dest[j] for a batch of many occurrences.  In the scatter every lane of a group would do the look-up (830 + 74 us with
+// this pass against 1466 us without at 32 M occurrences of k = 64; handing rows round by shuffles instead: 1127 us); below
+// DEST_INLINE occurrences the scatter waits on latency anyway and does it itself, a launch less.
+#define DEST_INLINE (1 << 19)
+__global__ void __launch_bounds__(256) make_dest_kernel(DestMap dm, int nnz) {
+  des_pdl_wait(dm.uidx, dm.hinfo, dm.hot_rep, dm.dest);
+  des_pdl_go();
   const int j0 = blockIdx.x * 1024 + threadIdx.x;
-  uint32_t u[4], hv[4], d[4];
+  if (j0 + 3 * 256 < nnz) {                             // four look-up chains in flight per thread
+    uint32_t d[4];
+    dest_rows<4>(dm, j0, 256, d);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int j = j0 + q * 256;
-    u[q] = (j < nnz) ? __ldg(uidx + j) : DES_ROW_NONE;
-    if (u[q] != DES_ROW_NONE && (long long)u[q] >= max_uniq) u[q] = DES_ROW_NONE;
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) hv[q] = (u[q] != DES_ROW_NONE) ? __ldg(hinfo + u[q]) : DES_ROW_NONE;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int j = j0 + q * 256;
-    d[q] = u[q];                                          // cold key (or no row)
-    if (u[q] != DES_ROW_NONE && hv[q] != DES_ROW_NONE) {
-      if (hv[q] >> 24) d[q] = SUPER_TAG | ((hv[q] >> 24) - 1u);
-      else   // replica floor(hash * R / 2^32): uniform over the R replicas without a division
-        d[q] = (uint32_t)max_uniq + __ldg(hot_base + hv[q]) + __umulhi(hash_u32((uint32_t)j), __ldg(hot_R + hv[q]));
+    for (int q = 0; q < 4; ++q) dm.dest[j0 + q * 256] = d[q];
+  } else {
+    for (int j = j0; j < nnz; j += 256) {
+      uint32_t d[1];
+      dest_rows<1>(dm, j, 0, d);
+      dm.dest[j] = d[0];
     }
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int j = j0 + q * 256;
-    if (j < nnz) dest[j] = d[q];
-  }
-}
-
-// Replica reduction, stage 1: one warp per work item = HOT_RCHUNK replica rows
-// of one hot key.  Columns are spread over the lanes, sums are taken in double
-// and added (double atomics, a few hundred per key at most) to the key's row of
-// hot_acc; the replica rows are cleared for the next step.
-__global__ void __launch_bounds__(256) hot_reduce_kernel(const uint32_t* __restrict__ ctr, uint32_t work_max,
-                                                         const uint32_t* __restrict__ hot_work,
-                                                         const uint32_t* __restrict__ hot_base,
-                                                         const uint32_t* __restrict__ hot_R, long long max_uniq,
-                                                         int k, float* __restrict__ Gbuf, double* __restrict__ hot_acc) {
-  const int stride = k + 4, lane = threadIdx.x & 31;
-  uint32_t nw = ctr[2];
-  if (nw > work_max) nw = work_max;
-  const uint32_t wstep = gridDim.x * (blockDim.x >> 5);
-  for (uint32_t wi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); wi < nw; wi += wstep) {
-    const uint32_t item = hot_work[wi], h = item >> 18, chunk = item & 0x3FFFFu;
-    const uint32_t R = hot_R[h];
-    const uint32_t r_lo = chunk * HOT_RCHUNK, r_hi = min(R, r_lo + HOT_RCHUNK);
-    float* rep = Gbuf + ((size_t)max_uniq + hot_base[h]) * stride;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    const bool c0 = lane < stride, c1 = lane + 32 < stride, c2 = lane + 64 < stride;
-    uint32_t r = r_lo;
-    for (; r + 4 <= r_hi; r += 4) {                    // four rows in flight
-      float v0[4], v1[4], v2[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float* row = rep + (size_t)(r + q) * stride;
-        v0[q] = c0 ? row[lane] : 0.f; v1[q] = c1 ? row[lane + 32] : 0.f; v2[q] = c2 ? row[lane + 64] : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float* row = rep + (size_t)(r + q) * stride;
-        a0 += (double)v0[q]; a1 += (double)v1[q]; a2 += (double)v2[q];
-        if (c0) row[lane] = 0.f;
-        if (c1) row[lane + 32] = 0.f;
-        if (c2) row[lane + 64] = 0.f;
-      }
-    }
-    for (; r < r_hi; ++r) {
-      float* row = rep + (size_t)r * stride;
-      if (c0) { a0 += (double)row[lane]; row[lane] = 0.f; }
-      if (c1) { a1 += (double)row[lane + 32]; row[lane + 32] = 0.f; }
-      if (c2) { a2 += (double)row[lane + 64]; row[lane + 64] = 0.f; }
-    }
-    double* dst = hot_acc + (size_t)h * stride;
-    if (lane < stride) atomicAdd(dst + lane, a0);
-    if (lane + 32 < stride) atomicAdd(dst + lane + 32, a1);
-    if (lane + 64 < stride) atomicAdd(dst + lane + 64, a2);
-  }
-}
-
-// Stage 2: the double sums go into the hot keys' gradient rows; hot_acc is cleared.
-__global__ void __launch_bounds__(256) hot_finish_kernel(const uint32_t* __restrict__ ctr, uint32_t h_max,
-                                                         const uint32_t* __restrict__ hot_R,
-                                                         const uint32_t* __restrict__ hot_u, int k,
-                                                         float* __restrict__ Gbuf, double* __restrict__ hot_acc) {
-  const int stride = k + 4;
-  uint32_t nh = ctr[0];
-  if (nh > h_max) nh = h_max;
-  const long long n = (long long)nh * stride;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const uint32_t h = (uint32_t)(i / stride), c = (uint32_t)(i % stride);
-    if (hot_R[h] == 0) continue;
-    Gbuf[(size_t)hot_u[h] * stride + c] += (float)hot_acc[i];
-    hot_acc[i] = 0.0;
   }
 }
 
 // U occurrences i, i + P, ... of a bag: one vector atomic per lane into the occurrence's gradient
-// row (lane 0 of the sub-group also adds the linear-weight tail).  SUPER: occurrences marked
-// dest = SUPER_TAG | slot send nothing; lane t counts those of slot t.
-template <int U, int P, bool HAS_VALS, bool SUPER>
-__device__ __forceinline__ void scatter_step(const uint32_t* __restrict__ dest, const float* __restrict__ vals, int i,
+// row (lane 0 of the sub-group also adds the linear-weight tail).  SUPER: occurrences of the keys tagged
+// SUPER_TAG | slot send nothing; lane t counts those of slot t.
+template <int U, int P, bool HAS_VALS, bool SUPER, bool INLINE>
+__device__ __forceinline__ void scatter_step(const DestMap& dm, const float* __restrict__ vals, int i,
                                              char* gcol, char* gtail, unsigned rowB, bool col, bool lead,
                                              const float4& c, float gl, float gf, uint32_t mine, uint32_t& cnt) {
   uint32_t d[U]; float x[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    d[u] = __ldg(dest + i + u * P);
+    if (!INLINE) d[u] = __ldg(dm.dest + i + u * P);
     if (HAS_VALS) x[u] = __ldg(vals + i + u * P);
   }
+  if (INLINE) dest_rows<U>(dm, i, P, d);
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     if (SUPER) cnt += (d[u] == mine);
@@ -260,12 +128,17 @@ __device__ __forceinline__ void scatter_step(const uint32_t* __restrict__ dest, 
 // and the atomics.  SUPER (G = 16 only): occurrences of the few keys that own a large share of a
 // skewed batch send no atomics; lane t counts the bag's occurrences of slot t and the counts go
 // to super_cnt[bag][16]; super_dense_kernel turns them into the keys' gradient sums.
-template <int G, int P, bool HAS_VALS, bool SUPER>
-__global__ void __launch_bounds__(256) grad_scatter_kernel(
-    const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ dest,
+// (Resident warps: eight blocks per SM are worth 15 % without SUPER — 16384 x 39 fields 57 -> 45 us —, and cost 7 % with
+// it, where the 32 registers spill and the gradient buffer's address is best kept in registers.)
+template <int G, int P, bool HAS_VALS, bool SUPER, bool INLINE>
+__global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatter_kernel(
+    const int32_t* __restrict__ offsets, const float* __restrict__ vals, DestMap dm,
     long long nbags, int F, int k, uint32_t ops, const float* __restrict__ out_small,
     const float* __restrict__ gL, const float* __restrict__ gF, const float* __restrict__ gE, float* Gbuf,
     float* __restrict__ super_cnt) {
+  const int zero = des_pdl_wait0();
+  if (SUPER) des_pdl_new(Gbuf);
+  des_pdl_go();
   constexpr int LB = G * P;
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
@@ -278,7 +151,7 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(
   // fetched while the current bag is scattered, so only the destination loads wait on them
   const long long slots = (long long)gridDim.x * (256 / LB);
   const long long rounds = (nbags + slots - 1) / slots;
-  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB;
+  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB + zero;
   int lo_n = 0, hi_n = 0;
   if (bag < nbags) { lo_n = __ldg(offsets + bag); hi_n = __ldg(offsets + bag + 1); }
   for (long long r = 0; r < rounds; ++r, bag += slots) {
@@ -305,7 +178,7 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(
     }
     uint32_t cnt = 0;
     int i0 = lo;
-#define SC_STEP(U) scatter_step<U, P, HAS_VALS, SUPER>(dest, vals, i0 + p, gcol, gtail, rowB, col, lead, c, gl, gf, mine, cnt)
+#define SC_STEP(U) scatter_step<U, P, HAS_VALS, SUPER, INLINE>(dm, vals, i0 + p, gcol, gtail, rowB, col, lead, c, gl, gf, mine, cnt)
     for (; i0 + 4 * P <= hi; i0 += 4 * P) SC_STEP(4);
     if (i0 + 2 * P <= hi) { SC_STEP(2); i0 += 2 * P; }
     if (i0 + P <= hi) { SC_STEP(1); i0 += P; }
@@ -324,7 +197,7 @@ __global__ void __launch_bounds__(256) grad_scatter_kernel(
 // with c_bag rebuilt from gE and the aggregated forward exactly as in the scatter.  A CTA
 // stages SD_TILE bags (c_bag rows, counts, gL / gF) in shared memory; thread (t, c4) owns the
 // accumulator of key t, 16-byte column c4.  Each CTA adds its sums to one replica row per key
-// (summed in double by hot_reduce).  All feature values are 1 on this path.
+// (summed in double by the update).  All feature values are 1 on this path.
 #define SD_TILE 32
 #define SD_STAGES 4
 #define SD_THREADS 288   // 256 column threads + one warp for the linear-weight tails
@@ -350,7 +223,7 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
     const float* __restrict__ super_cnt, int nbags, int F, int k, uint32_t ops,
     const float* __restrict__ out_small, const float* __restrict__ gL, const float* __restrict__ gF,
     const float* __restrict__ gE, float* Gbuf, const uint32_t* __restrict__ ctr,
-    const uint32_t* __restrict__ hot_base, const uint32_t* __restrict__ hot_R, long long max_uniq) {
+    const uint2* __restrict__ hot_rep, long long max_uniq) {
   uint32_t ns = __ldg(ctr + 3);
   if (ns == 0) return;
   if (ns > SUPER_T) ns = SUPER_T;
@@ -436,14 +309,14 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
   }
   sd_cp_wait<0>();
   // each (CTA, bag subset) hands its sums to one replica row per key
-  const uint32_t salt = hash_u32(blockIdx.x * 8u + (uint32_t)(tailw ? th : sub));
+  const uint32_t salt = des_hash32(blockIdx.x * 8u + (uint32_t)(tailw ? th : sub));
   if (tailw) {
     if ((uint32_t)tt >= ns) return;
     const uint32_t hh = __ldg(ctr + HOT_CTR_SLOT + tt);
     if (hh == DES_ROW_NONE) return;
-    const uint32_t R = __ldg(hot_R + hh);
-    if (R == 0) return;
-    float* row = Gbuf + ((size_t)max_uniq + __ldg(hot_base + hh) + salt % R) * stride;
+    const uint2 rp = __ldg(hot_rep + hh);
+    if (rp.y == 0) return;
+    float* row = Gbuf + ((size_t)max_uniq + rp.x + salt % rp.y) * stride;
     atomicAdd(reinterpret_cast<float4*>(row) + K4, make_float4(tw, tq, 0.f, 0.f));
     return;
   }
@@ -453,9 +326,9 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
     if (key >= ns || !col) continue;
     const uint32_t hh = __ldg(ctr + HOT_CTR_SLOT + key);
     if (hh == DES_ROW_NONE) continue;
-    const uint32_t R = __ldg(hot_R + hh);
-    if (R == 0) continue;
-    float* row = Gbuf + ((size_t)max_uniq + __ldg(hot_base + hh) + salt % R) * stride;
+    const uint2 rp = __ldg(hot_rep + hh);
+    if (rp.y == 0) continue;
+    float* row = Gbuf + ((size_t)max_uniq + rp.x + salt % rp.y) * stride;
     atomicAdd(reinterpret_cast<float4*>(row) + c4, acc[q]);
   }
 }
@@ -466,6 +339,7 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
 #ifndef UP_UNROLL
 #define UP_UNROLL 4
 #endif
+#define UP_GRID 8
 
 // Advances Adam's step count and recomputes the bias corrections 1 - beta^t in double.
 __global__ void adam_tick_kernel(DevMeta* meta, float beta1, float beta2) {
@@ -475,104 +349,311 @@ __global__ void adam_tick_kernel(DevMeta* meta, float beta1, float beta2) {
   meta->adam_c2 = (float)(1.0 - pow((double)beta2, (double)t));
 }
 
-// One optimizer application per unique key.  A group of G lanes owns a key (one
-// 16-byte column each, lane 0 also the linear weight); it works on UP_UNROLL
-// keys at a time so that their gradient rows, row numbers, weights and state
-// are all in flight together: the kernel is a pure stream of 272-byte rows.
+// What a group of G lanes holds of one key (a 16-byte column each, lane 0 also the linear weight).
+template <bool ADAM>
+struct KeyState {
+  float4 v, s, s2;
+  float2 st;                    // linear weight's two state words
+  float lw;
+};
+
+struct UpdateArgs {
+  int k, stride;
+  bool upd_v, upd_w;
+  float stamp;                  // "updated in the step of the current batch" (eviction by age)
+  float *W, *A, *A2;
+  OptParams opt;
+};
+
+template <bool ADAM>
+__device__ __forceinline__ void key_load(const UpdateArgs& a, uint32_t row, int c4, bool col, bool lead, KeyState<ADAM>& x) {
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  x.v = zero; x.s = zero; x.lw = 0.f; x.st = make_float2(0.f, 0.f);
+  if (ADAM) x.s2 = zero;
+  if (row == DES_ROW_NONE) return;
+  const float4* w = reinterpret_cast<const float4*>(a.W + (size_t)row * a.stride);
+  const float4* ac = a.A ? reinterpret_cast<const float4*>(a.A + (size_t)row * a.stride) : nullptr;
+  if (col) {
+    x.v = w[c4];
+    if (ac && a.upd_v) x.s = ac[c4];
+    if (ADAM && a.upd_v) x.s2 = reinterpret_cast<const float4*>(a.A2 + (size_t)row * a.stride)[c4];
+  }
+  if (lead) {
+    x.lw = *reinterpret_cast<const float*>(w + (a.k >> 2));
+    if (ac && a.upd_w) x.st = *reinterpret_cast<const float2*>(ac + (a.k >> 2));
+  }
+}
+
+// One optimizer application: g = the key's summed gradient column, tail = (G_w, sum x^2 gF).  All lanes of the warp.
 template <int G, bool ADAM>
+__device__ __forceinline__ void key_apply(const UpdateArgs& a, uint32_t row, int c4, bool col, bool lead, const float4& g,
+                                          const float2& tail, KeyState<ADAM>& x) {
+  const bool mapped = row != DES_ROW_NONE;
+  if (mapped && col && a.upd_v) {
+    const float t1 = tail.y;
+    des_opt_step(a.opt, x.v.x, x.s.x, x.s2.x, g.x - x.v.x * t1);
+    des_opt_step(a.opt, x.v.y, x.s.y, x.s2.y, g.y - x.v.y * t1);
+    des_opt_step(a.opt, x.v.z, x.s.z, x.s2.z, g.z - x.v.z * t1);
+    des_opt_step(a.opt, x.v.w, x.s.w, x.s2.w, g.w - x.v.w * t1);
+  }
+  // squared norm of the (new) latent vector, kept in the row's tail for the forward's M_2
+  float n2 = x.v.x * x.v.x + x.v.y * x.v.y + x.v.z * x.v.z + x.v.w * x.v.w;
+#pragma unroll
+  for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
+  if (!mapped) return;
+  const int K4 = a.k >> 2;
+  float4* w = reinterpret_cast<float4*>(a.W + (size_t)row * a.stride);
+  float4* ac = a.A ? reinterpret_cast<float4*>(a.A + (size_t)row * a.stride) : nullptr;
+  if (col && a.upd_v) {
+    w[c4] = x.v;
+    if (ac) ac[c4] = x.s;
+    if (ADAM) reinterpret_cast<float4*>(a.A2 + (size_t)row * a.stride)[c4] = x.s2;
+  }
+  if (lead) {
+    if (a.upd_w) {     // linear weight: its two state words sit side by side in the state row's tail
+      if (a.opt.lin_optimizer == DES_LIN_FTRL) des_ftrl_step(a.opt, x.lw, x.st.x, x.st.y, tail.x);
+      else des_opt_step(a.opt, x.lw, x.st.x, x.st.y, tail.x);
+    }
+    w[K4] = make_float4(x.lw, n2, a.stamp, 0.f);
+    if (ac && a.upd_w) ac[K4] = make_float4(x.st.x, x.st.y, 0.f, 0.f);
+  }
+}
+
+#define HOT_GROUP_R 16u
+#define HOT_LIST 256      // keys of a hot block that can be beyond that, looked through at a time
+// Rows first, first + step, ... below R of a replica block: their sum, then zeros.
+__device__ __forceinline__ void replica_sum(float* rep, uint32_t first, uint32_t step, uint32_t R, int stride, int K4, int c4,
+                                            bool col, bool lead, double (&a)[4], double (&t)[2]) {
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) a[q] = 0.0;
+  t[0] = t[1] = 0.0;
+  for (uint32_t r0 = first; r0 < R; r0 += 4 * step) {   // four rows in flight
+    float4 v[4]; float2 tl[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[q] = zero; tl[q] = make_float2(0.f, 0.f);
+      if (r0 + q * step < R) {
+        const float4* row = reinterpret_cast<const float4*>(rep + (size_t)(r0 + q * step) * stride);
+        if (col) v[q] = row[c4];
+        if (lead) tl[q] = *reinterpret_cast<const float2*>(row + K4);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (r0 + q * step < R) {
+        float4* row = reinterpret_cast<float4*>(rep + (size_t)(r0 + q * step) * stride);
+        if (col) row[c4] = zero;
+        if (lead) row[K4] = zero;
+      }
+      a[0] += (double)v[q].x; a[1] += (double)v[q].y; a[2] += (double)v[q].z; a[3] += (double)v[q].w;
+      t[0] += (double)tl[q].x; t[1] += (double)tl[q].y;
+    }
+  }
+}
+
+// Hot keys of one block's share: a hot key's replica rows are added in double and cleared, and done(h, R, lanes with the
+// sum, column sums, tail sums) takes the result.  A group of G lanes takes a key of up to HOT_GROUP_R
+// replicas by itself (most hot keys have a handful), the whole block one of more.  (R is at most
+// a few thousand rows: the keys that would have more are counted instead of scattered and have SUPER_R.)
+template <int G>
+struct HotShared {
+  double sum[256 / G][G][4], tail[256 / G][2];
+  uint32_t list[HOT_LIST];
+  int n;
+};
+template <int G, typename F>
+__device__ __forceinline__ void hot_keys(HotShared<G>& sh, int blk, int nblk, uint32_t nh, const uint2* __restrict__ hot_rep,
+                                         float* rep0, int stride, int K4, int c4, bool col, bool lead, F&& done) {
+  constexpr int NG = 256 / G;
+  const int grp = (int)(threadIdx.x / G);
+  // keys for one group; whole warps stay together
+  for (uint32_t h0 = (uint32_t)blk * NG; h0 < nh; h0 += (uint32_t)nblk * NG) {
+    const uint32_t h = h0 + grp;
+    const uint2 rp = h < nh ? __ldg(hot_rep + h) : make_uint2(0u, 0u);
+    const bool mine = rp.y > 0u && rp.y <= HOT_GROUP_R;   // (R = 0: no replica rows were left, a cold key)
+    double a[4], tl[2];
+    replica_sum(rep0 + (size_t)rp.x * stride, 0u, 1u, mine ? rp.y : 0u, stride, K4, c4, col, lead, a, tl);
+    done(h, mine, a, tl);
+  }
+  // keys for the whole block: looked for by its threads, HOT_LIST at a time
+  for (uint32_t h0 = (uint32_t)blk; h0 < nh; h0 += (uint32_t)nblk * HOT_LIST) {
+    if (threadIdx.x == 0) sh.n = 0;
+    __syncthreads();
+    const uint32_t hc = h0 + threadIdx.x * (uint32_t)nblk;
+    if (hc < nh && __ldg(hot_rep + hc).y > HOT_GROUP_R) sh.list[atomicAdd(&sh.n, 1)] = hc;
+    __syncthreads();
+    for (int e = 0; e < sh.n; ++e) {
+      const uint32_t h = sh.list[e];
+      const uint2 rp = __ldg(hot_rep + h);
+      double a[4], tl[2];
+      replica_sum(rep0 + (size_t)rp.x * stride, (uint32_t)grp, (uint32_t)NG, rp.y, stride, K4, c4, col, lead, a, tl);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sh.sum[grp][c4][q] = a[q];
+      if (lead) { sh.tail[grp][0] = tl[0]; sh.tail[grp][1] = tl[1]; }
+      __syncthreads();
+      if (threadIdx.x < 32) {                           // one warp; its first group has the key
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = 0.0;
+        tl[0] = tl[1] = 0.0;
+        if (grp == 0) {
+          const int n = rp.y < (uint32_t)NG ? (int)rp.y : NG;
+          for (int i = 0; i < n; ++i) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a[q] += sh.sum[i][c4][q];
+            if (lead) { tl[0] += sh.tail[i][0]; tl[1] += sh.tail[i][1]; }
+          }
+        }
+        done(h, grp == 0, a, tl);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// The hot keys' sums into their own gradient rows (all zero until then), for a batch of many keys: the update is then a pure
+// stream.  One warp per work item = HOT_RCHUNK replica rows of a hot key, columns over the lanes, sums in double; the warp
+// that finishes a key's last item writes the row.  (A key's rows left to one block: 58 us instead of 12 at 3.9 M
+// occurrences, all of it the hottest key's 1800 rows.)
+__global__ void __launch_bounds__(256) hot_sum_kernel(int k, long long max_uniq, float* __restrict__ Gbuf,
+                                                      const uint32_t* __restrict__ hot_u, const uint2* __restrict__ hot_rep,
+                                                      const uint32_t* __restrict__ hot_ctr, uint32_t work_max,
+                                                      const uint32_t* __restrict__ hot_work, double* hot_acc, uint32_t* hot_done) {
+  des_pdl_wait(Gbuf, hot_u, hot_rep, hot_ctr, hot_work, hot_acc, hot_done);
+  des_pdl_go();
+  const int stride = k + 4, lane = threadIdx.x & 31;
+  const bool c0 = lane < stride, c1 = lane + 32 < stride, c2 = lane + 64 < stride;
+  const uint32_t nw = min(__ldg(hot_ctr + HOT_CTR_WORK), work_max);
+  for (uint32_t wi = blockIdx.x * 8 + (threadIdx.x >> 5); wi < nw; wi += gridDim.x * 8) {
+    const uint32_t item = __ldg(hot_work + wi), h = item >> HOT_WORK_BITS, chunk = item & ((1u << HOT_WORK_BITS) - 1u);
+    if (item == DES_ROW_NONE) continue;
+    const uint2 rp = __ldg(hot_rep + h);
+    const uint32_t r_lo = chunk * HOT_RCHUNK, r_hi = min(rp.y, r_lo + HOT_RCHUNK);
+    float* rep = Gbuf + ((size_t)max_uniq + rp.x) * stride;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    for (uint32_t r = r_lo; r < r_hi; r += 8) {        // eight rows in flight
+      float v0[8], v1[8], v2[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float* row = rep + (size_t)(r + q) * stride;
+        const bool in = r + q < r_hi;
+        v0[q] = in && c0 ? row[lane] : 0.f; v1[q] = in && c1 ? row[lane + 32] : 0.f; v2[q] = in && c2 ? row[lane + 64] : 0.f;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        float* row = rep + (size_t)(r + q) * stride;
+        a0 += (double)v0[q]; a1 += (double)v1[q]; a2 += (double)v2[q];
+        if (r + q >= r_hi) continue;
+        if (c0) row[lane] = 0.f;
+        if (c1) row[lane + 32] = 0.f;
+        if (c2) row[lane + 64] = 0.f;
+      }
+    }
+    if (rp.y > HOT_RCHUNK) {
+      double* acc = hot_acc + (size_t)h * stride;
+      if (c0) atomicAdd(acc + lane, a0);
+      if (c1) atomicAdd(acc + lane + 32, a1);
+      if (c2) atomicAdd(acc + lane + 64, a2);
+      __threadfence();
+      __syncwarp();
+      uint32_t before = 0;
+      if (lane == 0) before = atomicAdd(hot_done + h, 1u);
+      if (__shfl_sync(0xFFFFFFFFu, before, 0) != (rp.y + HOT_RCHUNK - 1) / HOT_RCHUNK - 1) continue;
+      __threadfence();
+      if (c0) { a0 = __ldcg(acc + lane); acc[lane] = 0.0; }
+      if (c1) { a1 = __ldcg(acc + lane + 32); acc[lane + 32] = 0.0; }
+      if (c2) { a2 = __ldcg(acc + lane + 64); acc[lane + 64] = 0.0; }
+      if (lane == 0) hot_done[h] = 0u;
+    }
+    float* row = Gbuf + (size_t)__ldg(hot_u + h) * stride;
+    if (c0) row[lane] = (float)a0;
+    if (c1) row[lane + 32] = (float)a1;
+    if (c2) row[lane + 64] = (float)a2;
+  }
+}
+
+// One optimizer application per unique key: a group of G lanes owns a key and works on UP_UNROLL keys at a time so that
+// their gradient rows, row numbers, weights and state are all in flight together: a pure stream of 272-byte rows, bound
+// by memory (1.5 M keys of k = 64 with Adagrad state: 2.5 GB in 615 us).
+// HOT, for a batch of few keys: the first hot_blocks of the grid take the hot keys, replicas and all, a launch less than
+// hot_sum_kernel before it; the others skip them.
+template <int G, bool ADAM, bool HOT>
 __global__ void __launch_bounds__(256, UP_MINB) update_rows_kernel(
-    const uint32_t* __restrict__ uniq_rows, const uint32_t* __restrict__ n_uniq, long long max_uniq, int k,
-    uint32_t ops, const OptParams opt_in, DevMeta* __restrict__ meta, float* __restrict__ Gbuf,
-    float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2) {
+    int hot_blocks, const uint32_t* __restrict__ uniq_rows, const uint32_t* __restrict__ n_uniq, long long max_uniq, int k,
+    uint32_t ops, const OptParams opt_in, DevMeta* __restrict__ meta, float* __restrict__ Gbuf, float* __restrict__ W,
+    float* __restrict__ A, float* __restrict__ A2, const uint32_t* __restrict__ hinfo, const uint32_t* __restrict__ hot_u,
+    const uint2* __restrict__ hot_rep, const uint32_t* __restrict__ hot_ctr, uint32_t hot_max) {
+  constexpr int NG = 256 / G;
+  __shared__ typename std::conditional<HOT, HotShared<G>, int>::type sh;
+  const int z0 = des_pdl_wait0();
+  meta += z0; n_uniq += z0; hot_ctr += z0;
+  des_pdl_go();
+  UpdateArgs ua;
+  ua.k = k; ua.stride = k + 4; ua.W = W; ua.A = A; ua.A2 = A2;
+  ua.opt = des_opt_load(opt_in, meta);
+  ua.stamp = des_stamp_bits(meta->clock);
+  ua.upd_v = ops & (DES_OP_FM | DES_OP_POOL | DES_OP_DENSE1); ua.upd_w = ops & DES_OP_LR;
   const int K4 = k >> 2, stride = k + 4;
-  const OptParams opt = des_opt_load(opt_in, meta);
-  const float stamp = des_stamp_bits(meta->clock);     // "updated in the step of the current batch" (eviction by age)
+  const int c4 = (int)(threadIdx.x % G), grp = (int)(threadIdx.x / G);
+  const bool col = c4 < K4, lead = c4 == 0;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  if constexpr (HOT) {
+    if ((int)blockIdx.x < hot_blocks) {
+      hot_keys<G>(sh, (int)blockIdx.x + z0, hot_blocks, min(__ldg(hot_ctr), hot_max), hot_rep, Gbuf + (size_t)max_uniq * stride, stride,
+                  K4, c4, col, lead, [&](uint32_t h, bool mine, const double (&a)[4], const double (&tl)[2]) {
+                    uint32_t row = mine ? __ldg(uniq_rows + __ldg(hot_u + h)) : DES_ROW_NONE;
+                    if (row != DES_ROW_NONE && DES_DBG_ROW(row) != row) row = DES_ROW_NONE;      // (checking build)
+                    KeyState<ADAM> x;
+                    key_load<ADAM>(ua, row, c4, col, lead, x);
+                    // (the tail's sums are lane 0's; every lane of the group needs the second)
+                    const float2 tail = make_float2((float)tl[0], __shfl_sync(0xFFFFFFFFu, (float)tl[1], (threadIdx.x & 31) / G * G));
+                    key_apply<G, ADAM>(ua, row, c4, col, lead, make_float4((float)a[0], (float)a[1], (float)a[2], (float)a[3]), tail, x);
+                  });
+      return;
+    }
+  }
+  const long long blk = (long long)blockIdx.x - hot_blocks, nblk = (long long)gridDim.x - hot_blocks;
   long long U = *n_uniq;
   if (U > max_uniq) {           // the gradient buffer cannot hold this batch: report, update what fits
-    if (blockIdx.x == 0 && threadIdx.x == 0) des_raise(meta, DES_ERR_CAPACITY);
+    if (blk == 0 && threadIdx.x == 0) des_raise(meta, DES_ERR_CAPACITY);
     U = max_uniq;
   }
-  const int c4 = (int)(threadIdx.x % G);
-  const bool col = c4 < K4, lead = c4 == 0;
-  const bool upd_v = ops & (DES_OP_FM | DES_OP_POOL | DES_OP_DENSE1), upd_w = ops & DES_OP_LR;
-  const long long gstep = (long long)gridDim.x * (blockDim.x / G);
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const long long gstep = nblk * NG;
   // every lane of a warp runs the same number of iterations (keys past U are masked off)
   const long long iters = (U + gstep * UP_UNROLL - 1) / (gstep * UP_UNROLL);
-  long long u0 = (long long)blockIdx.x * (blockDim.x / G) + threadIdx.x / G;
+  long long u0 = blk * NG + grp + z0;
   for (long long it = 0; it < iters; ++it, u0 += gstep * UP_UNROLL) {
     uint32_t r[UP_UNROLL];
-    float4 g[UP_UNROLL], v[UP_UNROLL], s[UP_UNROLL], s2[ADAM ? UP_UNROLL : 1];
-    float2 tail[UP_UNROLL], st[UP_UNROLL];   // gradient tail (G_w, sum x^2 gF); linear weight's two state words
-    float lw[UP_UNROLL];                      // linear weight (lead lane)
+    float4 g[UP_UNROLL];
+    float2 tail[UP_UNROLL];
+    bool cold[UP_UNROLL];
+    KeyState<ADAM> x[UP_UNROLL];
 #pragma unroll
     for (int q = 0; q < UP_UNROLL; ++q) {
       const long long u = u0 + q * gstep;
-      r[q] = (u < U) ? __ldg(uniq_rows + u) : DES_ROW_NONE;
+      r[q] = u < U ? __ldg(uniq_rows + u) : DES_ROW_NONE;
+      cold[q] = u < U && !(HOT && (__ldg(hinfo + u) & HOT_FLAG));
+      if (HOT && !cold[q]) r[q] = DES_ROW_NONE;
       if (r[q] != DES_ROW_NONE && DES_DBG_ROW(r[q]) != r[q]) r[q] = DES_ROW_NONE;   // (checking build)
       g[q] = zero; tail[q] = make_float2(0.f, 0.f);
-      if (u < U) {
+      if (u < U) {                                      // (a hot key's own row is all zero: nothing to clear)
         const float4* grow = reinterpret_cast<const float4*>(Gbuf + (size_t)u * stride);
         if (col) g[q] = grow[c4];
         tail[q] = *reinterpret_cast<const float2*>(grow + K4);
       }
     }
 #pragma unroll
-    for (int q = 0; q < UP_UNROLL; ++q) {
-      v[q] = zero; s[q] = zero; lw[q] = 0.f; st[q] = make_float2(0.f, 0.f);
-      if (ADAM) s2[ADAM ? q : 0] = zero;
-      if (r[q] != DES_ROW_NONE) {
-        const float4* w = reinterpret_cast<const float4*>(W + (size_t)r[q] * stride);
-        const float4* a = A ? reinterpret_cast<const float4*>(A + (size_t)r[q] * stride) : nullptr;
-        if (col) {
-          v[q] = w[c4];
-          if (a && upd_v) s[q] = a[c4];
-          if (ADAM && upd_v) s2[ADAM ? q : 0] = reinterpret_cast<const float4*>(A2 + (size_t)r[q] * stride)[c4];
-        }
-        if (lead) {
-          lw[q] = *reinterpret_cast<const float*>(w + K4);
-          if (a && upd_w) st[q] = *reinterpret_cast<const float2*>(a + K4);
-        }
-      }
-    }
+    for (int q = 0; q < UP_UNROLL; ++q) key_load<ADAM>(ua, r[q], c4, col, lead, x[q]);
     __syncwarp();   // all lanes of a group have read the gradient row before its lead lane clears it
 #pragma unroll
     for (int q = 0; q < UP_UNROLL; ++q) {
       const long long u = u0 + q * gstep;
-      const bool live = u < U, mapped = r[q] != DES_ROW_NONE;
-      if (live) {
+      if (cold[q]) {
         float4* grow = reinterpret_cast<float4*>(Gbuf + (size_t)u * stride);
         if (col) grow[c4] = zero;
         if (lead) grow[K4] = zero;
       }
-      float4& m2 = s2[ADAM ? q : 0];            // Adam's second moment (unused otherwise)
-      if (mapped && col && upd_v) {
-        const float t1 = tail[q].y;
-        des_opt_step(opt, v[q].x, s[q].x, m2.x, g[q].x - v[q].x * t1);
-        des_opt_step(opt, v[q].y, s[q].y, m2.y, g[q].y - v[q].y * t1);
-        des_opt_step(opt, v[q].z, s[q].z, m2.z, g[q].z - v[q].z * t1);
-        des_opt_step(opt, v[q].w, s[q].w, m2.w, g[q].w - v[q].w * t1);
-      }
-      // squared norm of the (new) latent vector, kept in the row's tail for the forward's M_2
-      float n2 = v[q].x * v[q].x + v[q].y * v[q].y + v[q].z * v[q].z + v[q].w * v[q].w;
-#pragma unroll
-      for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
-      if (!mapped) continue;
-      float4* w = reinterpret_cast<float4*>(W + (size_t)r[q] * stride);
-      float4* a = A ? reinterpret_cast<float4*>(A + (size_t)r[q] * stride) : nullptr;
-      if (col && upd_v) {
-        w[c4] = v[q];
-        if (a) a[c4] = s[q];
-        if (ADAM) reinterpret_cast<float4*>(A2 + (size_t)r[q] * stride)[c4] = m2;
-      }
-      if (lead) {
-        if (upd_w) {     // linear weight: its two state words sit side by side in the state row's tail
-          if (opt.lin_optimizer == DES_LIN_FTRL) des_ftrl_step(opt, lw[q], st[q].x, st[q].y, tail[q].x);
-          else des_opt_step(opt, lw[q], st[q].x, st[q].y, tail[q].x);
-        }
-        w[K4] = make_float4(lw[q], n2, stamp, 0.f);
-        if (a && upd_w) a[K4] = make_float4(st[q].x, st[q].y, 0.f, 0.f);
-      }
+      key_apply<G, ADAM>(ua, r[q], c4, col, lead, g[q], tail[q], x[q]);
     }
   }
 }
@@ -582,34 +663,9 @@ static int group_for(int k) { int K4 = k / 4, G = 1; while (G < K4) G <<= 1; ret
 // Skewed-batch path: 16-lane groups, unit feature values, batches large enough to fill a persistent grid.
 // The dense product of the backward costs time per BAG, the atomics it replaces per OCCURRENCE: it pays from
 // about ten ids per bag on (measured: 20 ids per bag 1.50 -> 0.85 + 0.25 ms; 4 ids per bag 0.43 -> 0.39 + 0.29 ms).
-static bool super_path(const des_table* t, const des_batch_t* b) {
+bool des_super_path(const des_table* t, const des_batch_t* b) {
   const long long nbags = (long long)b->batch * t->F;
   return group_for(t->k) == 16 && !b->vals && b->nnz >= (1 << 20) && t->super_cnt && b->nnz >= 8 * nbags;
-}
-
-des_status_t des_tags_ensure(des_table* t, const des_batch_t* b, cudaStream_t cs) {
-  if (t->tag_valid && t->tag_uidx == (const void*)b->uidx && t->tag_nnz == (long long)b->nnz) return DES_OK;
-  t->tag_valid = 0;
-  if (b->nnz == 0) return DES_OK;
-  const int nnz = (int)b->nnz;
-  int shift = 0;
-  while (shift < 6 && ((long long)nnz >> shift) > (1ll << 20)) ++shift;
-  DES_CUDA(cudaMemsetAsync(t->hot_ctr, 0, HOT_CTR_WORDS * 4, cs));
-  DES_CUDA(cudaMemsetAsync(t->hinfo, 0, (size_t)t->max_uniq * 4, cs));
-  const bool use_super = super_path(t, b);
-  const uint32_t super_min = use_super ? (uint32_t)(nnz >> 7) : 0u;
-  const int n = (nnz >> shift) + 1;
-  sample_count_kernel<<<(n + SC_THREADS * SC_PER - 1) / (SC_THREADS * SC_PER), SC_THREADS, 0, cs>>>(b->uidx, nnz, shift, t->max_uniq, t->hinfo);
-  DES_LAUNCH_CHECK(t, "sample_count_kernel");
-  hot_select_kernel<<<t->sm_count * 4, 256, 0, cs>>>(t->hinfo, b->n_uniq, t->max_uniq, shift, t->hot_base, t->hot_R,
-                                                     t->hot_u, t->hot_ctr, t->hot_max, t->rep_max, t->meta,
-                                                     t->hot_work, t->work_max, super_min);
-  DES_LAUNCH_CHECK(t, "hot_select_kernel");
-  make_dest_kernel<<<(nnz + 1023) / 1024, 256, 0, cs>>>(b->uidx, nnz, t->hinfo, t->hot_base, t->hot_R, t->max_uniq,
-                                                      t->dest);
-  DES_LAUNCH_CHECK(t, "make_dest_kernel");
-  t->tag_uidx = b->uidx; t->tag_nnz = (long long)b->nnz; t->tag_super = use_super ? 1 : 0; t->tag_valid = 1;
-  return DES_OK;
 }
 
 extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const des_batch_t* b,
@@ -640,10 +696,16 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
   const int G = group_for(t->k);
   const int nnz = (int)b->nnz;
   const long long nbags = (long long)B * t->F;
-  // hot-key detection on a sample, replica assignment, per-occurrence destination row (kept if this very batch
-  // has been through it since its find_or_insert)
-  if ((st = des_tags_ensure(t, b, cs)) != DES_OK) return st;
+  // counts and hot keys of this batch: find_or_insert has left them unless it has seen another batch since
+  if ((st = des_count_batch(t, b, cs)) != DES_OK) return st;
   const bool use_super = t->tag_super;
+  DestMap dm;
+  dm.uidx = b->uidx; dm.hinfo = t->hinfo; dm.hot_rep = t->hot_rep; dm.max_uniq = (uint32_t)t->max_uniq; dm.dest = t->dest;
+  const bool inl = nnz < DEST_INLINE;
+  if (!inl) {
+    des_launch(make_dest_kernel, (nnz + 1023) / 1024, 256, 0, cs, dm, nnz);
+    DES_LAUNCH_CHECK(t, "make_dest_kernel");
+  }
   {
     // long bags: a whole warp per bag (its sub-groups take alternate occurrences); short bags: G lanes per bag
     const bool wide = (long long)nnz >= 8 * nbags;   // (at 4 ids per bag the narrow form measured faster)
@@ -651,18 +713,20 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
     long long blocks = (threads + 255) / 256;
     if (blocks > (long long)t->sm_count * SC_BLOCKS_PER_SM) blocks = (long long)t->sm_count * SC_BLOCKS_PER_SM;
     const unsigned grid = (unsigned)blocks;
-#define SC4(GG, PP, HV, SU) grad_scatter_kernel<GG, PP, HV, SU><<<grid, 256, 0, cs>>>(                                  \
-        b->offsets, b->vals, t->dest, nbags, t->F, t->k, ops, out->out_small, gr->gL, gr->gF, gE, t->Gbuf, t->super_cnt)
-#define SC3(GG, HV) do { if (wide) SC4(GG, 32 / GG, HV, false); else SC4(GG, 1, HV, false); } while (0)
+#define SC5(GG, PP, HV, SU, IL) des_launch(grad_scatter_kernel<GG, PP, HV, SU, IL>, grid, 256, 0, cs, b->offsets, b->vals, dm,    \
+        nbags, (int)t->F, (int)t->k, ops, (const float*)out->out_small, gr->gL, gr->gF, gE, t->Gbuf, t->super_cnt)
+#define SC4(GG, PP, HV) do { if (inl) SC5(GG, PP, HV, false, true); else SC5(GG, PP, HV, false, false); } while (0)
+#define SC3(GG, HV) do { if (wide) SC4(GG, 32 / GG, HV); else SC4(GG, 1, HV); } while (0)
 #define SC(GG) do { if (b->vals) SC3(GG, true); else SC3(GG, false); } while (0)
-    if (use_super) {
-      if (wide) SC4(16, 2, false, true); else SC4(16, 1, false, true);
+    if (use_super) {                                    // (at least 2^20 occurrences, 8 per bag)
+      SC5(16, 2, false, true, false);
     } else {
       switch (G) { case 1: SC(1); break; case 2: SC(2); break; case 4: SC(4); break; case 8: SC(8); break; default: SC(16); }
     }
 #undef SC
 #undef SC3
 #undef SC4
+#undef SC5
     DES_LAUNCH_CHECK(t, "grad_scatter_kernel");
   }
   if (use_super) {
@@ -670,28 +734,36 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
     // (an attribute of the function on the current device, not a stream operation: legal under capture)
     if (cudaFuncSetAttribute(super_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sd_smem) != cudaSuccess)
       return DES_ERR_CUDA;
-    super_dense_kernel<<<t->sm_count * 3, SD_THREADS, sd_smem, cs>>>(t->super_cnt, (int)nbags, t->F, t->k, ops, out->out_small,
-                                                               gr->gL, gr->gF, gE, t->Gbuf, t->hot_ctr, t->hot_base,
-                                                               t->hot_R, t->max_uniq);
+    // (not chained: its shared memory would be taken from the L1 of the scatter that it waits for)
+    des_launch_if(false, super_dense_kernel, t->sm_count * 3, SD_THREADS, sd_smem, cs, t->super_cnt, (int)nbags, (int)t->F, (int)t->k, ops,
+               (const float*)out->out_small, gr->gL, gr->gF, gE, t->Gbuf, t->hot_ctr, t->hot_rep, (long long)t->max_uniq);
     DES_LAUNCH_CHECK(t, "super_dense_kernel");
   }
-  hot_reduce_kernel<<<t->sm_count * 8, 256, 0, cs>>>(t->hot_ctr, t->work_max, t->hot_work, t->hot_base, t->hot_R,
-                                                     t->max_uniq, t->k, t->Gbuf, t->hot_acc);
-  DES_LAUNCH_CHECK(t, "hot_reduce_kernel");
-  hot_finish_kernel<<<t->sm_count * 2, 256, 0, cs>>>(t->hot_ctr, t->hot_max, t->hot_R, t->hot_u, t->k, t->Gbuf,
-                                                     t->hot_acc);
-  DES_LAUNCH_CHECK(t, "hot_finish_kernel");
   {
-#ifndef UP_GRID
-#define UP_GRID 8
-#endif
-    const unsigned grid = (unsigned)(t->sm_count * UP_GRID);
-#define UP2(GG, AD) update_rows_kernel<GG, AD><<<grid, 256, 0, cs>>>(b->uniq_rows, b->n_uniq, t->max_uniq, t->k, ops, \
-                                                                   opt, t->meta, t->Gbuf, t->W, t->A, t->A2)
+    // stream blocks: enough for every key the batch can have, at most UP_GRID per SM; hot blocks in front: one per key
+    // that can be hot, at most two per SM
+    const long long keys = nnz < t->max_uniq ? nnz : t->max_uniq, per = 256 / G * UP_UNROLL;
+    long long blocks = (keys + per - 1) / per;
+    if (blocks > (long long)t->sm_count * UP_GRID) blocks = (long long)t->sm_count * UP_GRID;
+    int hot = nnz / (int)HOT_MIN(0) + 1;
+    if (hot > t->sm_count * 2) hot = t->sm_count * 2;
+    // (up to DEST_INLINE occurrences the two kernels in one are a launch less; beyond, the flag look-up per key costs more)
+    if (!inl) {
+      des_launch(hot_sum_kernel, t->sm_count * 8, 256, 0, cs, (int)t->k, (long long)t->max_uniq, t->Gbuf, t->hot_u, t->hot_rep,
+                 t->hot_ctr, t->work_max, t->hot_work, t->hot_acc, t->hot_done);
+      DES_LAUNCH_CHECK(t, "hot_sum_kernel");
+      hot = 0;
+    }
+    const unsigned grid = (unsigned)(blocks + hot);
+#define UP3(GG, AD, HT) des_launch(update_rows_kernel<GG, AD, HT>, grid, 256, 0, cs, hot, b->uniq_rows, b->n_uniq,                  \
+                                   (long long)t->max_uniq, (int)t->k, ops, opt, t->meta, t->Gbuf, t->W, t->A, t->A2, t->hinfo,       \
+                                   t->hot_u, t->hot_rep, t->hot_ctr, t->hot_max)
+#define UP2(GG, AD) do { if (inl) UP3(GG, AD, true); else UP3(GG, AD, false); } while (0)
 #define UP(GG) do { if (t->A2) UP2(GG, true); else UP2(GG, false); } while (0)
     switch (G) { case 1: UP(1); break; case 2: UP(2); break; case 4: UP(4); break; case 8: UP(8); break; default: UP(16); }
 #undef UP
 #undef UP2
+#undef UP3
     DES_LAUNCH_CHECK(t, "update_rows_kernel");
   }
   return DES_OK;

@@ -284,11 +284,11 @@ __global__ void __launch_bounds__(256) shard_partials_kernel(
     int B, int S, int k, uint32_t ops, const float* __restrict__ W, uint32_t null_row, float* __restrict__ part_small,
     float* __restrict__ out_small) {
   constexpr int P = 32 / G;
-  des_pdl_wait(grow_sorted, x_sorted, seg_off, W, part_small, out_small);
+  const int zero = des_pdl_wait0();
   des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int b = blockIdx.x * 8 + (threadIdx.x >> 5) + zero;
   if (b >= B) return;                                  // whole warp
   const int c4 = lane % G, p = lane / G;
   const bool col = c4 < K4;
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(256) pool_kernel(
     const uint8_t* __restrict__ shards, long long nbags, int B, int F, int k, const float* __restrict__ W,
     uint32_t null_row, float* __restrict__ pooled, float* __restrict__ part_pooled, __nv_bfloat16* __restrict__ pooled_b) {
   constexpr int LB = G * P;                            // lanes per bag
-  des_pdl_wait(offsets, vals, grow_csr, shards, W, pooled, part_pooled, pooled_b);
+  const int zero = des_pdl_wait0();
   des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(256) pool_kernel(
   // fetched while the current bag is summed
   const long long slots = (long long)gridDim.x * (256 / LB);
   const long long rounds = (nbags + slots - 1) / slots;
-  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB;
+  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB + zero;
   int lo_n = 0, hi_n = 0;
   if (bag < nbags) { lo_n = __ldg(offsets + bag); hi_n = __ldg(offsets + bag + 1); }
   for (long long r = 0; r < rounds; ++r, bag += slots) {
@@ -478,9 +478,9 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
     __nv_bfloat16* __restrict__ pooled_b) {
   constexpr int LB = G * P;                            // lanes per bag
   __shared__ uint32_t s_base[DES_MAX_SHARDS];
-  des_pdl_wait(offsets, vals, rows, shards, W, meta, pooled, bag_tail, pooled_b);
+  const int zero = des_pdl_wait0();
   des_pdl_go();
-  if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x];
+  if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x + zero];
   __syncthreads();
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
   const char* Wt = reinterpret_cast<const char*>(W + k);
   const long long slots = (long long)gridDim.x * (256 / LB);
   const long long rounds = (nbags + slots - 1) / slots;
-  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB;
+  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB + zero;
   int lo_n = 0, hi_n = 0;
   if (bag < nbags) { lo_n = __ldg(offsets + bag); hi_n = __ldg(offsets + bag + 1); }
   for (long long r = 0; r < rounds; ++r, bag += slots) {
@@ -549,9 +549,9 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
   extern __shared__ __align__(16) unsigned char sg_smem[];
   __shared__ uint32_t s_base[DES_MAX_SHARDS];
   __shared__ double s_red[FIELD ? 1 : 8][FIELD ? 1 : G][4], s_tail[FIELD ? 1 : 8][2];
-  des_pdl_wait(offsets, vals, rows, shards, W, meta, pooled, pooled_b, part_small, out_small);
+  const int zero = des_pdl_wait0();
   des_pdl_go();
-  if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x];
+  if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x + zero];
   __syncthreads();
   const int K4 = k >> 2, stride = k + 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
   const char* Wc = reinterpret_cast<const char*>(W) + (col ? c4 : 0) * 16;
   const char* Wt = reinterpret_cast<const char*>(W + k);
   const int wps = 8 / T, st = warp / wps, ws = warp % wps;             // sample within the block, warp within the sample
-  const int b = blockIdx.x * T + st;
+  const int b = blockIdx.x * T + st + zero;
   const int gs = ws * GW + lane / LB, ng = wps * GW;                   // this group among the sample's
   // FIELD: pooled vectors of sample st [F][K4] and bag tails [F]
   float4* s_pool = reinterpret_cast<float4*>(sg_smem) + (size_t)st * F * K4;

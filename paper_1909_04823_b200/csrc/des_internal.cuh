@@ -9,8 +9,6 @@
 
 #define DES_MAX_SHARDS 64
 #define DES_SLOT_NONE 0xFFFFFFFFu
-#define HOT_RCHUNK 16u     // replica rows of a hot key summed by one warp of the backward's replica reduction
-
 #define SUP_TILES 256u     // tiles of find_or_insert per second-level counter
 
 // The few keys that own a large share of a skewed batch ("super" keys) are counted instead of scattered in the
@@ -18,10 +16,21 @@
 #define SUPER_T 16u             // slots
 #define SUPER_TAG 0xFFFFFF00u   // tag | slot; DES_ROW_NONE (low byte 0xFF) is not a tag
 // Layout of the hot-key counter block (des_table::hot_ctr, 64 words):
-//   [0] hot keys  [1] replica rows  [2] work items  [3] super slots claimed
-//   [4 + t]   hot index of super slot t (DES_ROW_NONE: slot unused)
+//   [0] keys listed  [1] replica rows  [2] ticket of the counting kernel's blocks  [3] super slots claimed
+//   [4 + t]   hot index of super slot t (DES_ROW_NONE: slot unused)  [HOT_CTR_WORK] work items of the replica sums
 #define HOT_CTR_WORDS 64
 #define HOT_CTR_SLOT 4
+#define HOT_CTR_WORK 32
+#define HOT_RCHUNK 16u     // replica rows of a work item (hot index << HOT_WORK_BITS | chunk)
+#define HOT_WORK_BITS 17
+// A key is hot from HOT_MIN occurrences on (estimated from a 1 / 2^shift sample: at least 8 of them) and gets one replica row per
+// HOT_CHAIN.
+#define HOT_MIN(shift) ((shift) < 4 ? 128u : (shift) < 6 ? 256u : 512u)
+#define HOT_CHAIN(shift) ((shift) < 4 ? 128u : 256u)
+#define SUPER_R 64u        // replica rows of a super key (they only take one partial sum per lane group)
+// A batch-unique key's word (des_table::hinfo) once the batch is counted: below HOT_FLAG a sampled count (cold key);
+// else HOT_FLAG | (super slot + 1) << 24 | hot index.
+#define HOT_FLAG 0x80000000u
 
 // One open-addressing slot: 16 bytes, read with a single vector load.
 //   key        DES_KEY_EMPTY until claimed by a 64-bit CAS; never changes after.
@@ -91,16 +100,17 @@ struct des_table {
   // backward workspace
   float* Gbuf;                       // [max_uniq + rep_max][stride]: per-unique gradient rows, then
                                      // hot-key replica rows; all zero between calls
-  uint32_t* hinfo;                   // [max_uniq] sampled count, then hot index; zero between calls
-  uint32_t* dest;                    // [max_nnz] gradient row of each occurrence (or SUPER_TAG | slot), made by the
-                                     // hot-key pass that opens the backward; scratch of find_or_insert before that
+  uint32_t* hinfo;                   // [max_uniq] sampled count, or hot index (HOT_FLAG)
+  uint32_t* dest;                    // [max_nnz] gradient row of each occurrence (or SUPER_TAG | slot), large batches
   float* x_sorted;                   // [max_nnz] forward routing: feature values in shard-major order
   float2* bag_tail;                  // [max_batch * F] single-gather forward: per-bag sums of (w x, |v|^2 x^2)
-  // which batch the tags in dest[] / the hot lists belong to (they are rebuilt when another batch comes)
+  // which batch hinfo and the hot list belong to (the backward counts again when another batch comes)
   const void* tag_uidx; long long tag_nnz; int tag_valid; int tag_super;
-  uint32_t *hot_base, *hot_R, *hot_u, *hot_ctr;   // hot list [hot_max] and its two counters
-  uint32_t* hot_work;                // [work_max] (hot index << 18 | chunk) items of the replica reduction
+  uint32_t *hot_u, *hot_ctr;         // hot keys [hot_max] and their counters
+  uint2* hot_rep;                    // [hot_max] (first replica row, replica rows) of a hot key
+  uint32_t* hot_work;                // [work_max] work items of the replica sums
   double* hot_acc;                   // [hot_max][stride] double sums of the replicas; zero between calls
+  uint32_t* hot_done;                // [hot_max] finished items of a key; zero between calls
   float* super_cnt;                  // [max_batch * F][16] per-bag counts of the register-summed keys (k > 28 only)
   uint32_t hot_max, rep_max, work_max;
   // first dense layer
@@ -155,9 +165,16 @@ __device__ __forceinline__ void des_pdl_wait(P&... p) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   (des_pdl_new(p), ...);
 }
+// The same for a kernel whose every load is indexed from one number (a bag, a sample, a row): the number takes 0 from the wait
+// and the pointers stay kernel parameters, which cost no registers (a scatter of 11 pointers: 36 -> 30 registers).
+__device__ __forceinline__ int des_pdl_wait0() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
+  return zero;
+}
 __device__ __forceinline__ void des_pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
-static inline void des_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+static inline void des_launch_if(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute at;
@@ -165,8 +182,13 @@ static inline void des_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_
   at.val.programmaticStreamSerializationAllowed = 1;
   // (a launch of many waves gains nothing, and its waiting blocks take room in the last wave of the kernel before: a step
   // of 32 M occurrences 4.56 ms with this rule, 4.59 without)
-  cfg.attrs = &at; cfg.numAttrs = grid.x <= 8192u ? 1 : 0;
+  cfg.attrs = &at; cfg.numAttrs = chain && grid.x <= 8192u ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, (P)args...);        // (errors are picked up by DES_LAUNCH_CHECK)
+}
+
+template <typename... P, typename... A>
+static inline void des_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  des_launch_if(true, kernel, grid, block, smem, st, args...);
 }
 
 // ---- device helpers ---------------------------------------------------------
@@ -224,6 +246,11 @@ __device__ __forceinline__ float4 des_init4(unsigned long long seed, unsigned lo
   uint4 r = des_philox(make_uint4(q, 0u, (uint32_t)seed, (uint32_t)(seed >> 32)),
                        make_uint2((uint32_t)id, (uint32_t)(id >> 32)));
   return make_float4(des_u24(r.x, scale), des_u24(r.y, scale), des_u24(r.z, scale), des_u24(r.w, scale));
+}
+
+__device__ __forceinline__ uint32_t des_hash32(uint32_t x) {
+  x ^= x >> 16; x *= 0x7FEB352Du; x ^= x >> 15; x *= 0x846CA68Bu; x ^= x >> 16;
+  return x;
 }
 
 // Index of the bag that holds occurrence j: largest i with offsets[i] <= j
@@ -334,6 +361,8 @@ des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float*
                                 const float* part_pooled, cudaStream_t st);
 des_status_t des_dense1_backward(des_table* t, const float* pooled, const float* gE, const float* gZ,
                                  float* gE_work, int B, cudaStream_t st);
-// Hot-key pass over a batch's unique indices (sampled counts, hot list, replica assignment, dest[] with
-// the super-key tags); a no-op when dest[] already belongs to this batch (a second backward over it).
-des_status_t des_tags_ensure(des_table* t, const des_batch_t* b, cudaStream_t st);
+// Whether the keys that own a large share of the batch are counted instead of scattered in the backward.
+bool des_super_path(const des_table* t, const des_batch_t* b);
+// Counts a batch's occurrences per unique key (a sample) and makes the hot list, for a backward whose batch is not the
+// one that find_or_insert counted last.
+des_status_t des_count_batch(des_table* t, const des_batch_t* b, cudaStream_t cs);

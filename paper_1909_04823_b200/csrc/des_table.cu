@@ -101,8 +101,8 @@ extern "C" des_status_t des_table_destroy(des_table_t* t) {
   if (cudaGetDevice(&caller_dev) != cudaSuccess) { cudaGetLastError(); caller_dev = -1; }
   cudaSetDevice(t->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {t->slots, t->W, t->A, t->A2, t->acc2W1, t->meta, t->slot_of, t->flags, t->uslot, t->blk_cnt, t->sup_cnt, t->seg_off, t->Gbuf, t->hinfo, t->dest, t->hot_base,
-                  t->hot_R, t->hot_u, t->hot_ctr, t->hot_work, t->hot_acc, t->super_cnt, t->x_sorted, t->bag_tail,
+  void* ptrs[] = {t->slots, t->W, t->A, t->A2, t->acc2W1, t->meta, t->slot_of, t->flags, t->uslot, t->blk_cnt, t->sup_cnt, t->seg_off, t->Gbuf, t->hinfo, t->dest,
+                  t->hot_rep, t->hot_u, t->hot_ctr, t->hot_work, t->hot_acc, t->hot_done, t->super_cnt, t->x_sorted, t->bag_tail,
                   t->W1, t->accW1, t->W1b, t->gW1_part, t->pooled_b, t->gZ_b, t->gemm_ws, t->st_offsets[0], t->st_ids[0], t->st_vals[0], t->st_offsets[1], t->st_ids[1], t->st_vals[1], t->st_rows,
                   t->st_shards, t->st_uidx, t->st_uniq_rows, t->st_n_uniq, t->st_part_small, t->st_out_small};
   for (void* p : ptrs) dfree(t->cfg, p);
@@ -205,16 +205,16 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
   t->rep_max = (uint32_t)(t->max_nnz / 256 + t->hot_max + 1024);
   A(t->Gbuf, ((size_t)t->max_uniq + t->rep_max) * rowbytes);
   A(t->hinfo, (size_t)t->max_uniq * 4);
-  A(t->dest, (size_t)t->max_nnz * 4);
+  if (t->max_nnz >= (1 << 18)) A(t->dest, (size_t)t->max_nnz * 4);    // (used from DEST_INLINE occurrences on)
   A(t->x_sorted, (size_t)t->max_nnz * 4);
   A(t->bag_tail, (size_t)t->max_batch * t->F * sizeof(float2));
-  A(t->hot_base, (size_t)t->hot_max * 4);
-  A(t->hot_R, (size_t)t->hot_max * 4);
-  A(t->hot_u, (size_t)t->hot_max * 4);
-  A(t->hot_ctr, HOT_CTR_WORDS * 4);
+  A(t->hot_rep, (size_t)t->hot_max * sizeof(uint2));
   t->work_max = t->rep_max / HOT_RCHUNK + t->hot_max;
   A(t->hot_work, (size_t)t->work_max * 4);
   A(t->hot_acc, (size_t)t->hot_max * t->stride * 8);
+  A(t->hot_done, (size_t)t->hot_max * 4);
+  A(t->hot_u, (size_t)t->hot_max * 4);
+  A(t->hot_ctr, HOT_CTR_WORDS * 4);
   if (t->k > 28 && t->max_nnz >= (1 << 20)) A(t->super_cnt, (size_t)t->max_batch * t->F * 16 * sizeof(float));
   if (t->H) {
     A(t->W1, FKH * 4); A(t->accW1, FKH * 4); A(t->W1b, FKH * 2);
@@ -237,7 +237,9 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
   cu &= cudaMemset(t->Gbuf, 0, ((size_t)t->max_uniq + t->rep_max) * rowbytes) == cudaSuccess;
   cu &= cudaMemset(t->sup_cnt, 0, sup_bytes) == cudaSuccess;
   cu &= cudaMemset(t->hinfo, 0, (size_t)t->max_uniq * 4) == cudaSuccess;
+  cu &= cudaMemset(t->hot_ctr, 0, HOT_CTR_WORDS * 4) == cudaSuccess;
   cu &= cudaMemset(t->hot_acc, 0, (size_t)t->hot_max * t->stride * 8) == cudaSuccess;
+  cu &= cudaMemset(t->hot_done, 0, (size_t)t->hot_max * 4) == cudaSuccess;
   cu &= cudaMemcpy(t->meta, &hm, sizeof(hm), cudaMemcpyHostToDevice) == cudaSuccess;
   if (t->H) {
     cu &= cudaMemset(t->W1, 0, FKH * 4) == cudaSuccess;
