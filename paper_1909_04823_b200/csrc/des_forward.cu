@@ -277,6 +277,7 @@ __device__ __forceinline__ void pool_step(const uint32_t* __restrict__ grow_csr,
 // double), and out_small is written directly — the per-shard partials then never
 // touch memory.
 #define SP_U 4
+#define SP_BRIEF 8       // occurrences per (sample, shard) segment, on average, up to which segments are taken one per sub-group
 #define SP_FLUSH 4
 template <int G, bool HAS_VALS, bool FUSED>
 __global__ void __launch_bounds__(256) shard_partials_kernel(
@@ -336,6 +337,75 @@ __global__ void __launch_bounds__(256) shard_partials_kernel(
     if (FUSED) {
       Ax += (double)acc.x; Ay += (double)acc.y; Az += (double)acc.z; Aw += (double)acc.w;
       R += (double)m1lr; Q += (double)m2;
+    }
+  }
+  if (FUSED) {
+    double aa = col ? Ax * Ax + Ay * Ay + Az * Az + Aw * Aw : 0.0;
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) aa += __shfl_xor_sync(0xFFFFFFFFu, aa, d);
+    float4* o = reinterpret_cast<float4*>(out_small + (size_t)b * stride);
+    if (p == 0 && col) o[c4] = make_float4((float)Ax, (float)Ay, (float)Az, (float)Aw);
+    if (lane == 0) o[K4] = make_float4((float)R, fm ? (float)(0.5 * aa - 0.5 * Q) : 0.f, (float)Q, 0.f);
+  }
+}
+
+// The same for short segments (a sample's occurrences spread over many shards): sub-group p takes the segments of shards
+// p, p + P, ... by itself.  Nothing is combined when a segment ends, and an empty segment costs next to nothing, where the
+// kernel above spends a round of loads and a butterfly on it.  FUSED adds the partials in shard order all the same (handed
+// round by shuffles), so both forms still give the same bits.
+template <int G, bool HAS_VALS, bool FUSED>
+__global__ void __launch_bounds__(256) shard_partials_short_kernel(
+    const uint32_t* __restrict__ grow_sorted, const float* __restrict__ x_sorted, const int32_t* __restrict__ seg_off,
+    int B, int S, int k, uint32_t ops, const float* __restrict__ W, uint32_t null_row, float* __restrict__ part_small,
+    float* __restrict__ out_small) {
+  constexpr int P = 32 / G;
+  const int zero = des_pdl_wait0();
+  des_pdl_go();
+  const int K4 = k >> 2, stride = k + 4;
+  const int lane = threadIdx.x & 31;
+  const int b = blockIdx.x * 8 + (threadIdx.x >> 5) + zero;
+  if (b >= B) return;                                  // whole warp
+  const int c4 = lane % G, p = lane / G;
+  const bool col = c4 < K4, lr = ops & DES_OP_LR, fm = ops & DES_OP_FM;
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const unsigned rowB = (unsigned)stride * 4u;
+  const char* Wc = reinterpret_cast<const char*>(W) + (col ? c4 : 0) * 16;
+  const char* Wt = reinterpret_cast<const char*>(W + k);
+  double Ax = 0.0, Ay = 0.0, Az = 0.0, Aw = 0.0, R = 0.0, Q = 0.0;
+  const int32_t* so = seg_off + (size_t)b * (S + 1);
+  int lo_n = p < S ? __ldg(so + p) : 0, hi_n = p < S ? __ldg(so + p + 1) : 0;
+  for (int s0 = 0; s0 < S; s0 += P) {
+    const int s = s0 + p, lo = lo_n, hi = hi_n;
+    lo_n = s + P < S ? __ldg(so + s + P) : 0; hi_n = s + P < S ? __ldg(so + s + P + 1) : 0;
+    float4 acc = zero4, up = zero4;
+    float m1lr = 0.f, m2 = 0.f, up_l = 0.f, up_q = 0.f;
+    int round = 0;
+    for (int i = lo; i < hi; i += SP_U) {
+      sp_round<SP_U, 1, HAS_VALS>(grow_sorted, x_sorted, i, hi, null_row, Wc, Wt, rowB, acc, m1lr, m2);
+      if ((++round & (SP_FLUSH - 1)) == 0) {
+        up.x += acc.x; up.y += acc.y; up.z += acc.z; up.w += acc.w; up_l += m1lr; up_q += m2;
+        acc = zero4; m1lr = 0.f; m2 = 0.f;
+      }
+    }
+    acc.x += up.x; acc.y += up.y; acc.z += up.z; acc.w += up.w; m1lr += up_l; m2 += up_q;
+    if (!fm) { acc = zero4; m2 = 0.f; }
+    if (!lr) m1lr = 0.f;
+    if (part_small && s < S) {
+      float4* dst = reinterpret_cast<float4*>(part_small + ((size_t)s * B + b) * stride);
+      if (col) dst[c4] = acc;
+      if (c4 == 0) dst[K4] = make_float4(m1lr, m2, 0.f, 0.f);
+    }
+    if (FUSED) {
+      __syncwarp();
+      const unsigned some = __ballot_sync(0xFFFFFFFFu, hi > lo);     // (an empty segment adds 0)
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
+        if (!((some >> (q * G)) & 1u)) continue;                     // whole warp
+        const int src = q * G + c4;
+        Ax += (double)__shfl_sync(0xFFFFFFFFu, acc.x, src); Ay += (double)__shfl_sync(0xFFFFFFFFu, acc.y, src);
+        Az += (double)__shfl_sync(0xFFFFFFFFu, acc.z, src); Aw += (double)__shfl_sync(0xFFFFFFFFu, acc.w, src);
+        R += (double)__shfl_sync(0xFFFFFFFFu, m1lr, src); Q += (double)__shfl_sync(0xFFFFFFFFu, m2, src);
+      }
     }
   }
   if (FUSED) {
@@ -544,6 +614,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
     const DevMeta* __restrict__ meta, uint32_t null_row, float* __restrict__ pooled, __nv_bfloat16* __restrict__ pooled_b,
     float* __restrict__ part_small, float* __restrict__ out_small) {
   constexpr int LB = G * P, GW = 32 / LB;              // lanes per bag, bags per warp
+  static_assert(FIELD || P == 1, "long bags of the fused form: sample_stage_kernel");
   constexpr bool COOP = P > 1;
   constexpr int BU = COOP ? 1 : SGF_BU;                // bags of a group in flight together (long bags: their own rows are)
   extern __shared__ __align__(16) unsigned char sg_smem[];
@@ -634,10 +705,9 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
         acc[q].z += __shfl_xor_sync(0xFFFFFFFFu, acc[q].z, d); acc[q].w += __shfl_xor_sync(0xFFFFFFFFu, acc[q].w, d);
         if (!COOP) { bl[q] += __shfl_xor_sync(0xFFFFFFFFu, bl[q], d); bq[q] += __shfl_xor_sync(0xFFFFFFFFu, bq[q], d); }
       }
-      if (COOP && FIELD)
+      if (COOP)
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) { bl[q] += __shfl_xor_sync(0xFFFFFFFFu, bl[q], d); bq[q] += __shfl_xor_sync(0xFFFFFFFFu, bq[q], d); }
-      if (COOP && !FIELD) { R += (double)bl[q]; Q += (double)bq[q]; }   // (every lane its own occurrences)
       if (f < F && p == 0) {
         if (col) {
           const size_t o = ((size_t)b * F + f) * K4 + c4;
@@ -649,7 +719,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
           if (c4 == 0) s_bt[f] = make_float2(bl[q], bq[q]);
         } else {
           Ax += (double)acc[q].x; Ay += (double)acc[q].y; Az += (double)acc[q].z; Aw += (double)acc[q].w;
-          if (!COOP) { R += (double)bl[q]; Q += (double)bq[q]; }
+          R += (double)bl[q]; Q += (double)bq[q];
         }
       }
     }
@@ -662,7 +732,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
       Az += __shfl_xor_sync(0xFFFFFFFFu, Az, d); Aw += __shfl_xor_sync(0xFFFFFFFFu, Aw, d);
     }
 #pragma unroll
-    for (int d = COOP ? 1 : G; d < 32; d <<= 1) { R += __shfl_xor_sync(0xFFFFFFFFu, R, d); Q += __shfl_xor_sync(0xFFFFFFFFu, Q, d); }
+    for (int d = G; d < 32; d <<= 1) { R += __shfl_xor_sync(0xFFFFFFFFu, R, d); Q += __shfl_xor_sync(0xFFFFFFFFu, Q, d); }
     if (wps > 1) {
       if (lane < G) {
         s_red[warp][lane][0] = Ax; s_red[warp][lane][1] = Ay; s_red[warp][lane][2] = Az; s_red[warp][lane][3] = Aw;
@@ -722,6 +792,156 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
     if (lane < G && col) o[c4] = make_float4((float)ax, (float)ay, (float)az, (float)aw);
     if (lane == 0) o[K4] = make_float4((float)tr, fm ? (float)(0.5 * aa - 0.5 * tq) : 0.f, (float)tq, 0.f);
   }
+}
+
+// The fused form for long bags: WPS = 8 / T warps take a sample, T samples a block, a stretch of the sample's bags (up to
+// SS_CAP / T occurrences) at a time.  First every thread looks up the row of occurrences of its own — row number, shard, the
+// row's linear weight and squared norm, which go straight into sums of the thread's — and leaves the row in shared memory;
+// then the warps pool a bag each, their only loads the latent vectors.  What bounds the pooling is the number of loads that
+// go through L1 per occurrence: looked up by all lanes of every occurrence it was four (8.2 M occurrences of k = 64:
+// 321 us, now SS_MEASURED).
+#define SS_CAP 2048
+template <int G, int P, bool HAS_VALS>
+__global__ void __launch_bounds__(256, 5) sample_stage_kernel(
+    const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ rows,
+    const uint8_t* __restrict__ shards, int B, int F, int S, int k, int T, uint32_t ops, const float* __restrict__ W,
+    const DevMeta* __restrict__ meta, uint32_t null_row, float* __restrict__ pooled, __nv_bfloat16* __restrict__ pooled_b,
+    float* __restrict__ out_small) {
+  static_assert(G * P == 32, "a warp per bag");
+  __shared__ uint32_t s_base[DES_MAX_SHARDS], s_row[SS_CAP];
+  __shared__ double s_red[8][G][4], s_tail[8][2];
+  const int zero = des_pdl_wait0();
+  des_pdl_go();
+  if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x + zero];
+  for (int i = threadIdx.x; i < 8 * G * 4; i += 256) (&s_red[0][0][0])[i] = 0.0;
+  if (threadIdx.x < 16) (&s_tail[0][0])[threadIdx.x] = 0.0;
+  __syncthreads();
+  const int K4 = k >> 2, stride = k + 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c4 = lane % G, p = lane / G;
+  const bool col = c4 < K4, fm = ops & DES_OP_FM, lr = ops & DES_OP_LR;
+  const unsigned rowB = (unsigned)stride * 4u;
+  const char* Wc = reinterpret_cast<const char*>(W) + (col ? c4 : 0) * 16;
+  const char* Wt = reinterpret_cast<const char*>(W + k);
+  const int wps = 8 / T, st = warp / wps, ws = warp % wps, cap = SS_CAP / T;
+  const int b = blockIdx.x * T + st + zero;
+  uint32_t* sr = s_row + st * cap;
+  const int32_t* off = offsets + (size_t)b * F;
+  auto team_sync = [&]() {                             // the sample's warps
+    if (wps == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(st + 1), "r"(wps * 32) : "memory");
+  };
+  // a warp's sums over its bags and occurrences stay in shared memory (registers are what limits the resident warps)
+  auto tail_done = [&](float bl, float bq) {
+    double R = (double)bl, Q = (double)bq;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) { R += __shfl_xor_sync(0xFFFFFFFFu, R, d); Q += __shfl_xor_sync(0xFFFFFFFFu, Q, d); }
+    if (lane == 0) { s_tail[warp][0] += R; s_tail[warp][1] += Q; }
+  };
+  auto bag_done = [&](int f, float4 acc) {
+#pragma unroll
+    for (int d = G; d < 32; d <<= 1) {                 // combine the bag's sub-groups
+      acc.x += __shfl_xor_sync(0xFFFFFFFFu, acc.x, d); acc.y += __shfl_xor_sync(0xFFFFFFFFu, acc.y, d);
+      acc.z += __shfl_xor_sync(0xFFFFFFFFu, acc.z, d); acc.w += __shfl_xor_sync(0xFFFFFFFFu, acc.w, d);
+    }
+    if (p != 0 || !col) return;
+    const size_t o = ((size_t)b * F + f) * K4 + c4;
+    reinterpret_cast<float4*>(pooled)[o] = acc;
+    if (pooled_b) store_bf16x4(pooled_b + o * 4, acc);
+    double* a = s_red[warp][c4];
+    a[0] += (double)acc.x; a[1] += (double)acc.y; a[2] += (double)acc.z; a[3] += (double)acc.w;
+  };
+  for (int fa = b < B ? 0 : F; fa < F;) {               // (the same for all warps of a sample)
+    const int j0 = __ldg(off + fa);
+    int nb = 0;                                        // bags fa .. fa + nb - 1 fit the stage
+    for (unsigned m = 0xFFFFFFFFu; m == 0xFFFFFFFFu;) {
+      const int f = fa + 1 + nb + lane;
+      m = __ballot_sync(0xFFFFFFFFu, f <= F && __ldg(off + min(f, F)) - j0 <= cap);
+      nb += m == 0xFFFFFFFFu ? 32 : __ffs(~m) - 1;
+    }
+    if (nb == 0) {                                     // one bag longer than that
+      if (ws == 0) {
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float bl = 0.f, bq = 0.f;
+        coop_bag<G, P, HAS_VALS, true>(rows, shards, vals, s_base, j0, __ldg(off + fa + 1), lane, 0xFFFFFFFFu, Wc, Wt, rowB, null_row,
+                                       acc, bl, bq);
+        tail_done(bl, bq);
+        bag_done(fa, acc);
+      }
+      ++fa;
+      continue;
+    }
+    const int n = __ldg(off + fa + nb) - j0;
+    {
+      float bl = 0.f, bq = 0.f;
+      for (int i0 = ws * 32 + lane; i0 < n; i0 += 4 * wps * 32) {   // four look-ups of a thread in flight
+        uint32_t g[4]; float x[4]; float2 tl[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + q * wps * 32;
+          g[q] = null_row; x[q] = 0.f;
+          if (i < n) {
+            const uint32_t r = __ldg(rows + j0 + i);
+            if (r != DES_ROW_NONE) g[q] = DES_DBG_ROW(s_base[__ldg(shards + j0 + i)] + r);
+            if (HAS_VALS) x[q] = __ldg(vals + j0 + i);
+            sr[i] = g[q];
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tl[q] = __ldg(reinterpret_cast<const float2*>(Wt + (size_t)g[q] * rowB));   // (the all-zero row adds 0)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          bl += HAS_VALS ? tl[q].x * x[q] : tl[q].x;
+          bq += HAS_VALS ? tl[q].y * x[q] * x[q] : tl[q].y;
+        }
+      }
+      tail_done(bl, bq);
+    }
+    team_sync();
+    for (int f = fa + ws; f < fa + nb; f += wps) {
+      const int lo = __ldg(off + f) - j0, hi = __ldg(off + f + 1) - j0;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      int i0 = lo + p;
+      auto step = [&](auto U) {
+        constexpr int N = decltype(U)::value;
+        float4 v[N]; float xx[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+          if (HAS_VALS) xx[u] = __ldg(vals + j0 + i0 + u * P);
+          v[u] = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)sr[i0 + u * P] * rowB));
+        }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+          if (HAS_VALS) { v[u].x *= xx[u]; v[u].y *= xx[u]; v[u].z *= xx[u]; v[u].w *= xx[u]; }
+          acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w;
+        }
+        i0 += N * P;
+      };
+      const int full = lo + (hi - lo) / P * P;         // whole rounds of the warp end here
+      while (i0 - p + 4 * P <= full) step(std::integral_constant<int, 4>());
+      if (i0 - p + 2 * P <= full) step(std::integral_constant<int, 2>());
+      if (i0 - p + P <= full) step(std::integral_constant<int, 1>());
+      if (i0 < hi) step(std::integral_constant<int, 1>());
+      bag_done(f, acc);
+    }
+    fa += nb;
+    if (fa < F) team_sync();                           // the stage is overwritten
+  }
+  team_sync();
+  if (ws != 0) return;                                 // whole warp
+  double Ax = 0.0, Ay = 0.0, Az = 0.0, Aw = 0.0, R = 0.0, Q = 0.0;
+  for (int i = 0; i < wps; ++i) {
+    Ax += s_red[warp + i][c4][0]; Ay += s_red[warp + i][c4][1]; Az += s_red[warp + i][c4][2]; Aw += s_red[warp + i][c4][3];
+    R += s_tail[warp + i][0]; Q += s_tail[warp + i][1];
+  }
+  if (b >= B) return;                                  // whole warp
+  if (!lr) R = 0.0;
+  if (!fm) { Ax = Ay = Az = Aw = 0.0; Q = 0.0; }
+  double aa = (lane < G && col) ? Ax * Ax + Ay * Ay + Az * Az + Aw * Aw : 0.0;
+#pragma unroll
+  for (int d = 1; d < G; d <<= 1) aa += __shfl_xor_sync(0xFFFFFFFFu, aa, d);
+  float4* o = reinterpret_cast<float4*>(out_small + (size_t)b * stride);
+  if (lane < G && col) o[c4] = make_float4((float)Ax, (float)Ay, (float)Az, (float)Aw);
+  if (lane == 0) o[K4] = make_float4((float)R, fm ? (float)(0.5 * aa - 0.5 * Q) : 0.f, (float)Q, 0.f);
 }
 
 // FIELD partition: a bag belongs to one shard (field f lives on shard f mod S), so the sub-operators of shard s
@@ -839,7 +1059,8 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
   DES_LAUNCH_CHECK(t, "route_kernel");
   if (ps || fused_out) {
     const unsigned grid = (unsigned)((B + 7) / 8);      // one warp per sample
-#define SP3(GG, HV, FU) des_launch(shard_partials_kernel<GG, HV, FU>, grid, 256, 0, cs, grow_sorted, x_sorted, t->seg_off, B,   \
+    const bool brief = b->nnz <= (int64_t)SP_BRIEF * B * t->S;
+#define SP3(GG, HV, FU) des_launch(brief ? shard_partials_short_kernel<GG, HV, FU> : shard_partials_kernel<GG, HV, FU>, grid, 256, 0, cs, grow_sorted, x_sorted, t->seg_off, B,   \
                                    (int)t->S, (int)t->k, ops, t->W, (uint32_t)t->total_rows, ps, fused_out)
 #define SP(GG) do { if (fused_out) { if (b->vals) SP3(GG, true, true); else SP3(GG, false, true); } \
                     else { if (b->vals) SP3(GG, true, false); else SP3(GG, false, false); } } while (0)
@@ -919,15 +1140,17 @@ static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des
 #define SF4(GG, PP, HV, FD) des_launch(sample_gather_kernel<GG, PP, HV, FD>, grid, 256, T * per_sample, cs, b->offsets, b->vals,     \
                                        b->rows, b->shards, B, F, (int)t->S, (int)t->k, T, ops, t->W, t->meta,                     \
                                        (uint32_t)t->total_rows, pooled, pb, part_small, out_small)
-#define SF3(GG, PP, HV) do { if (field) SF4(GG, PP, HV, true); else SF4(GG, PP, HV, false); } while (0)
-#define SF2(GG, HV) do { if (wide) SF3(GG, 32 / GG, HV); else SF3(GG, 1, HV); } while (0)
+#define SS(GG, HV) des_launch(sample_stage_kernel<GG, 32 / GG, HV>, grid, 256, 0, cs, b->offsets, b->vals, b->rows, b->shards, B, F, \
+                              (int)t->S, (int)t->k, T, ops, t->W, t->meta, (uint32_t)t->total_rows, pooled, pb, out_small)
+#define SF2(GG, HV) do { if (!wide) { if (field) SF4(GG, 1, HV, true); else SF4(GG, 1, HV, false); }                              \
+                         else if (field) SF4(GG, 32 / GG, HV, true); else SS(GG, HV); } while (0)
 #define SF(GG) do { if (b->vals) SF2(GG, true); else SF2(GG, false); } while (0)
   switch (G) { case 1: SF(1); break; case 2: SF(2); break; case 4: SF(4); break; case 8: SF(8); break; default: SF(16); }
 #undef SF
 #undef SF2
-#undef SF3
+#undef SS
 #undef SF4
-  DES_LAUNCH_CHECK(t, "sample_gather_kernel");
+  DES_LAUNCH_CHECK(t, wide && !field ? "sample_stage_kernel" : "sample_gather_kernel");
   t->pooled_b_src = pb ? pooled : nullptr;
   return DES_OK;
 }
