@@ -403,8 +403,9 @@ des_status_t des_step_host(des_table_t* t, uint32_t ops, int32_t batch, int64_t 
  * building and the optimizer phase follow each other every iteration).
  * des_step_host_submit returns as soon as the step is enqueued: the host
  * buffers are copied on a stream of the table's own into one of two staging
- * slots, the kernels and the read-back of out_small run on `stream` once the
- * copy has landed, so the copy of step i+1 overlaps the kernels of step i.
+ * slots, the kernels run on `stream` once the copy has landed, so the copy of
+ * step i+1 overlaps the kernels of step i.  The read-back of out_small overlaps the
+ * step's own backward; `stream` passes the step when it is done.
  * *ticket names the slot; des_step_host_wait(ticket) blocks until that step is
  * over (h_out_small written).  At most two steps are in flight: a third submit
  * first waits for the step that used its slot.  Host buffers (inputs and

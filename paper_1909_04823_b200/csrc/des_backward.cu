@@ -74,7 +74,6 @@ __device__ __forceinline__ void dest_rows(const DestMap& m, int i, int step, uin
 #define DEST_INLINE (1 << 19)
 __global__ void __launch_bounds__(256) make_dest_kernel(DestMap dm, int nnz) {
   des_pdl_wait(dm.uidx, dm.hinfo, dm.hot_rep, dm.dest);
-  des_pdl_go();
   const int j0 = blockIdx.x * 1024 + threadIdx.x;
   if (j0 + 3 * 256 < nnz) {                             // four look-up chains in flight per thread
     uint32_t d[4];
@@ -138,7 +137,6 @@ __global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatte
     float* __restrict__ super_cnt) {
   const int zero = des_pdl_wait0();
   if (SUPER) des_pdl_new(Gbuf);
-  des_pdl_go();
   constexpr int LB = G * P;
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
@@ -520,7 +518,6 @@ __global__ void __launch_bounds__(256) hot_sum_kernel(int k, long long max_uniq,
                                                       const uint32_t* __restrict__ hot_ctr, uint32_t work_max,
                                                       const uint32_t* __restrict__ hot_work, double* hot_acc, uint32_t* hot_done) {
   des_pdl_wait(Gbuf, hot_u, hot_rep, hot_ctr, hot_work, hot_acc, hot_done);
-  des_pdl_go();
   const int stride = k + 4, lane = threadIdx.x & 31;
   const bool c0 = lane < stride, c1 = lane + 32 < stride, c2 = lane + 64 < stride;
   const uint32_t nw = min(__ldg(hot_ctr + HOT_CTR_WORK), work_max);
@@ -587,7 +584,6 @@ __global__ void __launch_bounds__(256, UP_MINB) update_rows_kernel(
   __shared__ typename std::conditional<HOT, HotShared<G>, int>::type sh;
   const int z0 = des_pdl_wait0();
   meta += z0; n_uniq += z0; hot_ctr += z0;
-  des_pdl_go();
   UpdateArgs ua;
   ua.k = k; ua.stride = k + 4; ua.W = W; ua.A = A; ua.A2 = A2;
   ua.opt = des_opt_load(opt_in, meta);
@@ -770,41 +766,26 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
 }
 
 // ---- whole step from host buffers ---------------------------------------------
-static void* st_alloc(des_table* t, size_t bytes) {
-  if (t->cfg.alloc) return t->cfg.alloc(bytes ? bytes : 256, t->cfg.alloc_ctx);
-  void* p = nullptr;
-  if (cudaMalloc(&p, bytes ? bytes : 256) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-  return p;
-}
-
 // Device staging of the host-buffer step, sized for the largest batch (first call: allocates, synchronises).
-// The batch inputs (offsets, ids, values) have two slots so that the copy of one step can overlap the
-// kernels of the step before; everything the kernels produce is single (kernels of consecutive steps run
+// The batch inputs (offsets, ids, values) and the results have two slots so that the copies of one step can overlap
+// kernels; everything else the kernels produce is single (kernels of consecutive steps run
 // in order on the caller's stream).
 static des_status_t st_prepare(des_table* t) {
   if (t->st_ready) return DES_OK;
-  if (t->st_ids[0]) return DES_ERR_CUDA;               // an earlier attempt ran out of memory half-way
-  const size_t nb = (size_t)t->max_batch * t->F + 1;
-  for (int s = 0; s < 2; ++s) {
-    t->st_offsets[s] = (int32_t*)st_alloc(t, nb * 4);
-    t->st_ids[s] = (unsigned long long*)st_alloc(t, (size_t)t->max_nnz * 8);
-    t->st_vals[s] = (float*)st_alloc(t, (size_t)t->max_nnz * 4);
-    if (!t->st_offsets[s] || !t->st_ids[s] || !t->st_vals[s]) return DES_ERR_CUDA;
-  }
-  t->st_rows = (uint32_t*)st_alloc(t, (size_t)t->max_nnz * 4);
-  t->st_shards = (uint8_t*)st_alloc(t, (size_t)t->max_nnz);
-  t->st_uidx = (uint32_t*)st_alloc(t, (size_t)t->max_nnz * 4);
-  t->st_uniq_rows = (uint32_t*)st_alloc(t, (size_t)t->max_nnz * 4);
-  t->st_n_uniq = (uint32_t*)st_alloc(t, 256);
-  t->st_part_small = (float*)st_alloc(t, (size_t)t->S * t->max_batch * t->stride * 4);
-  t->st_out_small = (float*)st_alloc(t, (size_t)t->max_batch * t->stride * 4);
-  if (!t->st_rows || !t->st_shards || !t->st_uidx || !t->st_uniq_rows || !t->st_n_uniq || !t->st_part_small ||
-      !t->st_out_small)
-    return DES_ERR_CUDA;
+  if (t->st_slab) return DES_ERR_CUDA;                 // an earlier attempt failed half-way
+  const size_t nb = (size_t)t->max_batch * t->F + 1, n = (size_t)t->max_nnz, out = (size_t)t->max_batch * t->stride * 4;
+  const DesSlabItem items[] = {
+      {(void**)&t->st_offsets[0], nb * 4}, {(void**)&t->st_ids[0], n * 8}, {(void**)&t->st_vals[0], n * 4},
+      {(void**)&t->st_offsets[1], nb * 4}, {(void**)&t->st_ids[1], n * 8}, {(void**)&t->st_vals[1], n * 4},
+      {(void**)&t->st_rows, n * 4}, {(void**)&t->st_shards, n}, {(void**)&t->st_uidx, n * 4}, {(void**)&t->st_uniq_rows, n * 4},
+      {(void**)&t->st_n_uniq, 256}, {(void**)&t->st_out_small[0], out}, {(void**)&t->st_out_small[1], out}};
+  t->st_slab = des_slab_alloc(t->cfg, items, (int)(sizeof(items) / sizeof(items[0])));
+  if (!t->st_slab) return DES_ERR_CUDA;
   if (cudaStreamCreateWithFlags(&t->st_copy_stream, cudaStreamNonBlocking) != cudaSuccess) return DES_ERR_CUDA;
+  if (cudaStreamCreateWithFlags(&t->st_out_stream, cudaStreamNonBlocking) != cudaSuccess) return DES_ERR_CUDA;
   for (int s = 0; s < 2; ++s) {
-    if (cudaEventCreateWithFlags(&t->st_copied[s], cudaEventDisableTiming) != cudaSuccess) return DES_ERR_CUDA;
-    if (cudaEventCreateWithFlags(&t->st_done[s], cudaEventDisableTiming) != cudaSuccess) return DES_ERR_CUDA;
+    for (cudaEvent_t* e : {&t->st_copied[s], &t->st_done[s], &t->st_fwd[s], &t->st_out[s]})
+      if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return DES_ERR_CUDA;
     t->st_busy[s] = 0;
   }
   t->st_ready = 1;
@@ -812,7 +793,11 @@ static des_status_t st_prepare(des_table* t) {
 }
 
 // Enqueues one whole step from host buffers: inputs go to staging slot `slot` on `copy` (the caller's
-// stream itself, or the table's copy stream), the kernels and the read-back of out_small on `cs`.
+// stream itself, or the table's copy stream), the kernels on `cs`.  The per-shard partials are not among the results, so the
+// forward is the fused one in shard order: the same bits without writing them out (two steps of 2 M occurrences
+// 1680 -> 1452 us with the read-back below).  The read-back of out_small starts as soon as the forward has it and, from ST_ASIDE
+// bytes on, runs beside the backward (a copy of 4.4 MB held the kernels up for 80 us); `cs` waits for it at the end.
+#define ST_ASIDE (256u << 10)
 static des_status_t st_enqueue(des_table* t, int slot, cudaStream_t copy, uint32_t ops, int32_t batch, int64_t nnz,
                                const int32_t* h_offsets, const uint64_t* h_ids, const float* h_vals,
                                const des_grads_t* d_grads, float* d_pooled, float* d_Z, float* h_out_small,
@@ -829,14 +814,23 @@ static des_status_t st_enqueue(des_table* t, int slot, cudaStream_t copy, uint32
   b.batch = batch; b.nnz = nnz; b.offsets = t->st_offsets[slot]; b.ids = (const uint64_t*)t->st_ids[slot];
   b.vals = h_vals ? t->st_vals[slot] : nullptr; b.rows = t->st_rows; b.shards = t->st_shards; b.uidx = t->st_uidx;
   b.uniq_rows = t->st_uniq_rows; b.n_uniq = t->st_n_uniq;
-  des_partials_t p; p.part_small = t->st_part_small; p.pooled = d_pooled; p.part_pooled = nullptr; p.part_dense = nullptr;
-  des_outputs_t o; o.out_small = t->st_out_small; o.pooled = d_pooled; o.Z = d_Z;
+  des_partials_t p; p.part_small = nullptr; p.pooled = d_pooled; p.part_pooled = nullptr; p.part_dense = nullptr;
+  des_outputs_t o; o.out_small = t->st_out_small[slot]; o.pooled = d_pooled; o.Z = d_Z;
+  const size_t out_bytes = (size_t)batch * t->stride * 4;
+  const bool aside = out_bytes >= ST_ASIDE;
+  if (ops & ~15u) return DES_ERR_INVALID_ARG;
   des_status_t st;
   if ((st = des_find_or_insert(t, &b, 1, cs)) != DES_OK) return st;
-  if ((st = des_forward_partials(t, ops, &b, &p, cs)) != DES_OK) return st;
-  if ((st = des_aggregate(t, ops, &b, &p, &o, cs)) != DES_OK) return st;
+  if ((st = des_forward_fused(t, ops | DES_FUSED_SHARD_ORDER, &b, &p, &o, cs)) != DES_OK) return st;
+  if (aside) {
+    DES_CUDA(cudaEventRecord(t->st_fwd[slot], cs));
+    DES_CUDA(cudaStreamWaitEvent(t->st_out_stream, t->st_fwd[slot], 0));
+    DES_CUDA(cudaMemcpyAsync(h_out_small, t->st_out_small[slot], out_bytes, cudaMemcpyDeviceToHost, t->st_out_stream));
+    DES_CUDA(cudaEventRecord(t->st_out[slot], t->st_out_stream));
+  }
   if ((st = des_backward_update(t, ops, &b, &o, d_grads, cs)) != DES_OK) return st;
-  DES_CUDA(cudaMemcpyAsync(h_out_small, t->st_out_small, (size_t)batch * t->stride * 4, cudaMemcpyDeviceToHost, cs));
+  if (aside) DES_CUDA(cudaStreamWaitEvent(cs, t->st_out[slot], 0));
+  else DES_CUDA(cudaMemcpyAsync(h_out_small, t->st_out_small[slot], out_bytes, cudaMemcpyDeviceToHost, cs));
   return DES_OK;
 }
 

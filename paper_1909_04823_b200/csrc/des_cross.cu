@@ -137,7 +137,6 @@ __global__ void __launch_bounds__(512) cross_forward_rows_kernel(int B, CrossGeo
                                                                  float4* __restrict__ y) {
   __shared__ float s_part[2][CX_R][16];
   des_pdl_wait(x0, x, w, bias, P, y);
-  des_pdl_go();
   const int grp = threadIdx.x / cg.tpr, c = threadIdx.x % cg.tpr, nw = cg.tpr / 32;
   const bool act = c < cg.d4;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -180,7 +179,6 @@ __global__ void __launch_bounds__(512) cross_backward_vec_kernel(int B, CrossGeo
   __shared__ float s_part[2][CX_R][16];
   __shared__ float4 s_sum[2][512];
   des_pdl_wait(x0, x, w, P, gY, gx0, gx, pw, pb);
-  des_pdl_go();
   const int grp = threadIdx.x / cg.tpr, c = threadIdx.x % cg.tpr, nw = cg.tpr / 32;
   const bool act = c < cg.d4;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -232,7 +230,6 @@ __global__ void __launch_bounds__(256) cross_backward_sums_kernel(int d, int blo
                                                                   const float* __restrict__ pb, float* __restrict__ gw,
                                                                   float* __restrict__ gb) {
   des_pdl_wait(pw, pb, gw, gb);
-  des_pdl_go();
   const int c = threadIdx.x & 7, part = threadIdx.x >> 3, i = blockIdx.x * 8 + c;
   __shared__ float s_w[32][8], s_b[32][8];
   float aw = 0.f, ab = 0.f;

@@ -134,7 +134,6 @@ __global__ void w1_update_kernel(const float* __restrict__ part, int slices, siz
                                  float* acc2, __nv_bfloat16* W1b, const OptParams opt_in,
                                  const DevMeta* __restrict__ meta) {
   des_pdl_wait(part, W1, acc, acc2, W1b, meta);
-  des_pdl_go();
   const OptParams opt = des_opt_load(opt_in, meta);
   const size_t n4 = n / 4, st = (size_t)gridDim.x * blockDim.x;       // (n is a multiple of 4: k and H are)
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += st) {
@@ -169,7 +168,6 @@ __global__ void cvt_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __
 __global__ void __launch_bounds__(256) cvt_bf16_pair_kernel(const float* __restrict__ s1, __nv_bfloat16* __restrict__ d1, size_t n1,
                                                             const float* __restrict__ s2, __nv_bfloat16* __restrict__ d2, size_t n2) {
   des_pdl_wait(s1, d1, s2, d2);
-  des_pdl_go();
   const size_t m1 = n1 / 4, m = m1 + n2 / 4;           // n1 and n2 are multiples of 4
   const size_t i0 = (size_t)blockIdx.x * 1024 + threadIdx.x;
   float4 v[4];

@@ -56,7 +56,6 @@ __global__ void __launch_bounds__(256) route_kernel(
   __shared__ uint32_t row_base[DES_MAX_SHARDS];
   __shared__ int cursor[8][DES_MAX_SHARDS];
   des_pdl_wait(offsets, vals, rows, shards, meta, grow_csr, grow_sorted, x_sorted, seg_off);
-  des_pdl_go();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x < S) row_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x];
   __syncthreads();
@@ -286,7 +285,6 @@ __global__ void __launch_bounds__(256) shard_partials_kernel(
     float* __restrict__ out_small) {
   constexpr int P = 32 / G;
   const int zero = des_pdl_wait0();
-  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5) + zero;
@@ -360,7 +358,6 @@ __global__ void __launch_bounds__(256) shard_partials_short_kernel(
     float* __restrict__ out_small) {
   constexpr int P = 32 / G;
   const int zero = des_pdl_wait0();
-  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5) + zero;
@@ -431,7 +428,6 @@ __global__ void __launch_bounds__(256) pool_kernel(
     uint32_t null_row, float* __restrict__ pooled, float* __restrict__ part_pooled, __nv_bfloat16* __restrict__ pooled_b) {
   constexpr int LB = G * P;                            // lanes per bag
   const int zero = des_pdl_wait0();
-  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
   const bool col = c4 < K4;
@@ -481,7 +477,6 @@ template <int G>
 __global__ void __launch_bounds__(256) aggregate_small_kernel(const float* __restrict__ part_small, int B, int S, int k,
                                                               uint32_t ops, float* __restrict__ out_small) {
   des_pdl_wait(part_small, out_small);
-  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = t / G, c4 = t % G;
@@ -549,7 +544,6 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
   constexpr int LB = G * P;                            // lanes per bag
   __shared__ uint32_t s_base[DES_MAX_SHARDS];
   const int zero = des_pdl_wait0();
-  des_pdl_go();
   if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x + zero];
   __syncthreads();
   const int K4 = k >> 2, stride = k + 4;
@@ -621,7 +615,6 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
   __shared__ uint32_t s_base[DES_MAX_SHARDS];
   __shared__ double s_red[FIELD ? 1 : 8][FIELD ? 1 : G][4], s_tail[FIELD ? 1 : 8][2];
   const int zero = des_pdl_wait0();
-  des_pdl_go();
   if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x + zero];
   __syncthreads();
   const int K4 = k >> 2, stride = k + 4;
@@ -799,7 +792,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
 // row's linear weight and squared norm, which go straight into sums of the thread's — and leaves the row in shared memory;
 // then the warps pool a bag each, their only loads the latent vectors.  What bounds the pooling is the number of loads that
 // go through L1 per occurrence: looked up by all lanes of every occurrence it was four (8.2 M occurrences of k = 64:
-// 321 us, now SS_MEASURED).
+// 321 us, now 302; the rest is latency at the 40 warps that fit an SM).
 #define SS_CAP 2048
 template <int G, int P, bool HAS_VALS>
 __global__ void __launch_bounds__(256, 5) sample_stage_kernel(
@@ -811,7 +804,6 @@ __global__ void __launch_bounds__(256, 5) sample_stage_kernel(
   __shared__ uint32_t s_base[DES_MAX_SHARDS], s_row[SS_CAP];
   __shared__ double s_red[8][G][4], s_tail[8][2];
   const int zero = des_pdl_wait0();
-  des_pdl_go();
   if (threadIdx.x < S) s_base[threadIdx.x] = (uint32_t)meta->row_base[threadIdx.x + zero];
   for (int i = threadIdx.x; i < 8 * G * 4; i += 256) (&s_red[0][0][0])[i] = 0.0;
   if (threadIdx.x < 16) (&s_tail[0][0])[threadIdx.x] = 0.0;
@@ -954,7 +946,6 @@ __global__ void __launch_bounds__(256) field_partials_kernel(const float* __rest
                                                              int B, int F, int S, int k, uint32_t ops,
                                                              float* __restrict__ part_small, float* __restrict__ out_small) {
   des_pdl_wait(pooled, bag_tail, part_small, out_small);
-  des_pdl_go();
   const int K4 = k >> 2, stride = k + 4;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int b = t / G, c4 = t % G;
@@ -998,7 +989,6 @@ __global__ void __launch_bounds__(256) field_partials_kernel(const float* __rest
 // sum over shards of a dense [S][B][n] tensor (materialised pooled / dense partials)
 __global__ void reduce_shards_kernel(const float* __restrict__ part, size_t per_shard, int S, float* __restrict__ out) {
   des_pdl_wait(part, out);
-  des_pdl_go();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x, st = (size_t)gridDim.x * blockDim.x;
   for (; i < per_shard; i += st) {
     float a = 0.f;

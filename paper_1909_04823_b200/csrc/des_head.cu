@@ -16,7 +16,6 @@ __global__ void __launch_bounds__(256) head_kernel(
     const float* __restrict__ xdense, const float* __restrict__ y, float* __restrict__ logit, float* __restrict__ loss,
     float* __restrict__ gL, float* __restrict__ gF, float* __restrict__ gZ, float* __restrict__ gE) {
   des_pdl_wait(u, b1, q, d, out_small, Z, pooled, xdense, y, logit, loss, gL, gF, gZ, gE);
-  des_pdl_go();
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;                                  // whole warp

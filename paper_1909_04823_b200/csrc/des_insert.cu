@@ -72,7 +72,6 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
   __shared__ uint32_t m_slot[PROBE_MERGE], m_occ[PROBE_MERGE];
   if (MERGE) { m_slot[threadIdx.x] = DES_SLOT_NONE; m_occ[threadIdx.x] = DES_ROW_NONE; }
   des_pdl_wait(ids, offsets, slots, meta, slot_of, shards, rows);
-  des_pdl_go();
   if (threadIdx.x <= (unsigned)S) s_base[threadIdx.x] = (uint32_t)geom.slot_base[threadIdx.x];
   __syncthreads();
   const uint32_t base = meta->scratch_base - (uint32_t)nnz;   // this call's scratch range (Slot::first_occ)
@@ -176,7 +175,6 @@ __global__ void __launch_bounds__(IB / 4) flag_count_kernel(
   if (threadIdx.x <= DES_MAX_SHARDS) cnt[threadIdx.x] = 0;
   __syncthreads();
   des_pdl_wait(slots, meta, slot_of, shards, flags, rows, first_of, blk_cnt, sup_cnt, any_new);
-  des_pdl_go();
   const uint32_t base = meta->scratch_base - (uint32_t)nnz;
   const int j0 = blockIdx.x * IB + threadIdx.x;
   uint32_t so[4];
@@ -262,7 +260,6 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile0 = blockIdx.x * M, jb = tile0 * IB, j0 = jb + tid * PER;
   des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2, hinfo, hot_ctr);
-  des_pdl_go();
   // The slots' scratch range ends with this call (see Slot::first_occ; resolve_kernel then starts a new one): nothing
   // reads the scratch words after flag_count_kernel, so they are all cleared here, once every few billion occurrences.
   if (meta->scratch_base - (uint32_t)nnz < max_nnz)
@@ -528,7 +525,6 @@ __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, in
   __shared__ uint32_t s_key[COUNT ? CT_SLOTS : 1], s_cnt[COUNT ? CT_SLOTS : 1];
   if (COUNT) count_begin(s_key, s_cnt);
   des_pdl_wait(first_of, rows, uidx, sup_cnt, meta, ca.hinfo, ca.hot_u, ca.hot_ctr, ca.hot_rep);
-  des_pdl_go();
   if (blockIdx.x == gridDim.x - 1) {
     const int nsup = (ntiles + (int)SUP_TILES - 1) / (int)SUP_TILES;
     for (int i = threadIdx.x; i < nsup; i += IB / 4) sup_cnt[i] = 0u;
@@ -601,7 +597,6 @@ __global__ void __launch_bounds__(CK_THREADS) count_kernel(const uint32_t* __res
   __shared__ uint32_t s_key[CT_SLOTS], s_cnt[CT_SLOTS];
   count_begin(s_key, s_cnt);
   des_pdl_wait(uidx, ca.hinfo, ca.hot_u, ca.hot_ctr, ca.hot_rep);
-  des_pdl_go();
   __syncthreads();
   uint32_t u[CK_PER];
 #pragma unroll

@@ -126,10 +126,12 @@ struct des_table {
   // host-step staging
   int32_t* st_offsets[2]; unsigned long long* st_ids[2]; float* st_vals[2];   // two input slots (pipelined submit)
   cudaStream_t st_copy_stream; cudaEvent_t st_copied[2], st_done[2]; int st_busy[2]; uint64_t st_next;
+  cudaStream_t st_out_stream; cudaEvent_t st_fwd[2], st_out[2];   // read-back of large results beside the backward
   void* evict_ws; size_t evict_ws_bytes;   // temporaries of the eviction calls, kept while small
   int st_ready;                      // staging, copy stream and events all exist
   uint32_t* st_rows; uint8_t* st_shards; uint32_t* st_uidx; uint32_t* st_uniq_rows; uint32_t* st_n_uniq;
-  float* st_part_small; float* st_out_small;
+  float* st_out_small[2];
+  void *slab, *st_slab;              // the allocations behind the workspace and the staging (des_slab_alloc)
   uint64_t launches;
   int sm_count;
   // optional per-launch timing (des_profile_*): one event after every launch, and one at API entry
@@ -139,6 +141,11 @@ struct des_table {
   const char** prof_name;            // [DES_PROF_MAX], NULL = API-entry marker
 };
 #define DES_PROF_MAX 16384
+
+// Many arrays, one allocation: every array starts on a 256-byte boundary.  (A table made 25 allocations of its own, and each
+// can take milliseconds when the driver has to find memory.)  Returns NULL when there is no memory.
+struct DesSlabItem { void** p; size_t bytes; };
+void* des_slab_alloc(const des_config_t& c, const DesSlabItem* items, int n);
 
 #define DES_CUDA(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return DES_ERR_CUDA; } while (0)
 // after every kernel launch: count it, check the launch, and (when profiling) drop an event behind it
@@ -151,8 +158,9 @@ void des_api_begin(des_table* t, cudaStream_t cs);
 // wait in des_pdl_wait for that kernel's completion (memory included) before they touch anything.  EVERY
 // kernel launched through des_launch starts with that wait.  It takes ALL pointers that the kernel reads
 // through: a read-only load (__ldg, const __restrict__) may be moved by the compiler across a mere memory barrier, to
-// before the wait, so the pointers come out of it as new values.  des_pdl_go lets the next kernel be set
-// up; it waits for this one's end all the same.
+// before the wait, so the pointers come out of it as new values.  No kernel lets the next one in before its
+// blocks end: blocks that wait on an SM take room and end up unevenly spread (512 x 8 LR + FM step 47 -> 42 us
+// without, a 2379-sample prediction 204 -> 184).
 template <typename P>
 __device__ __forceinline__ void des_pdl_new(P& p) {
   static_assert(sizeof(P) == 8, "pointers only");
@@ -172,7 +180,6 @@ __device__ __forceinline__ int des_pdl_wait0() {
   asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
   return zero;
 }
-__device__ __forceinline__ void des_pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
 static inline void des_launch_if(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};

@@ -2,6 +2,7 @@
 // workspace, status, size, export, row read-back (Section 5, "Dynamic Hash
 // Table": the storage behind lookup / insert / update).
 #include <new>
+#include <vector>
 #include <math.h>
 #include <string.h>
 
@@ -18,6 +19,16 @@ static void* dalloc(const des_config_t& c, size_t bytes) {
 static void dfree(const des_config_t& c, void* p) {
   if (!p) return;
   if (c.dealloc) c.dealloc(p, c.alloc_ctx); else cudaFree(p);
+}
+
+void* des_slab_alloc(const des_config_t& c, const DesSlabItem* items, int n) {
+  size_t total = 0;
+  for (int i = 0; i < n; ++i) total += (items[i].bytes + 255) / 256 * 256 + 256;   // (an empty array keeps an address of its own)
+  unsigned char* base = (unsigned char*)dalloc(c, total);
+  if (!base) return nullptr;
+  size_t at = 0;
+  for (int i = 0; i < n; ++i) { *items[i].p = base + at; at += (items[i].bytes + 255) / 256 * 256 + 256; }
+  return base;
 }
 
 __global__ void fill_f32_kernel(float* p, size_t n, float v) {
@@ -101,15 +112,14 @@ extern "C" des_status_t des_table_destroy(des_table_t* t) {
   if (cudaGetDevice(&caller_dev) != cudaSuccess) { cudaGetLastError(); caller_dev = -1; }
   cudaSetDevice(t->device);
   cudaDeviceSynchronize();
-  void* ptrs[] = {t->slots, t->W, t->A, t->A2, t->acc2W1, t->meta, t->slot_of, t->flags, t->uslot, t->blk_cnt, t->sup_cnt, t->seg_off, t->Gbuf, t->hinfo, t->dest,
-                  t->hot_rep, t->hot_u, t->hot_ctr, t->hot_work, t->hot_acc, t->hot_done, t->super_cnt, t->x_sorted, t->bag_tail,
-                  t->W1, t->accW1, t->W1b, t->gW1_part, t->pooled_b, t->gZ_b, t->gemm_ws, t->st_offsets[0], t->st_ids[0], t->st_vals[0], t->st_offsets[1], t->st_ids[1], t->st_vals[1], t->st_rows,
-                  t->st_shards, t->st_uidx, t->st_uniq_rows, t->st_n_uniq, t->st_part_small, t->st_out_small};
+  void* ptrs[] = {t->slots, t->W, t->A, t->A2, t->slab, t->st_slab};
   for (void* p : ptrs) dfree(t->cfg, p);
   cudaFree(t->evict_ws);
   if (t->st_copy_stream) {
     cudaStreamDestroy(t->st_copy_stream);
-    for (int s = 0; s < 2; ++s) { if (t->st_copied[s]) cudaEventDestroy(t->st_copied[s]); if (t->st_done[s]) cudaEventDestroy(t->st_done[s]); }
+    if (t->st_out_stream) cudaStreamDestroy(t->st_out_stream);
+    for (int s = 0; s < 2; ++s)
+      for (cudaEvent_t e : {t->st_copied[s], t->st_done[s], t->st_fwd[s], t->st_out[s]}) if (e) cudaEventDestroy(e);
   }
   if (t->prof_ev) { for (int i = 0; i < DES_PROF_MAX; ++i) cudaEventDestroy(t->prof_ev[i]); delete[] t->prof_ev; }
   delete[] t->prof_name;
@@ -185,14 +195,16 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
   const size_t rowbytes = (size_t)t->stride * 4;
   const size_t FKH = (size_t)t->F * t->k * t->H;
   bool ok = true;
-  auto A = [&](auto*& p, size_t bytes) {
+  auto big = [&](auto*& p, size_t bytes) {
     p = (typename std::remove_reference<decltype(p)>::type)dalloc(c, bytes);
     if (!p) ok = false;
   };
-  A(t->slots, slots * sizeof(Slot));
-  A(t->W, (rows + 1) * rowbytes);          // one all-zero row behind the table stands for "no row" in gathers
-  if (c.optimizer != DES_OPT_SGD || c.lin_optimizer == DES_LIN_FTRL) A(t->A, rows * rowbytes);
-  if (c.optimizer == DES_OPT_ADAM) A(t->A2, rows * rowbytes);
+  std::vector<DesSlabItem> items;                      // the workspace: one allocation
+  auto A = [&](auto*& p, size_t bytes) { items.push_back({(void**)&p, bytes}); };
+  big(t->slots, slots * sizeof(Slot));
+  big(t->W, (rows + 1) * rowbytes);          // one all-zero row behind the table stands for "no row" in gathers
+  if (c.optimizer != DES_OPT_SGD || c.lin_optimizer == DES_LIN_FTRL) big(t->A, rows * rowbytes);
+  if (c.optimizer == DES_OPT_ADAM) big(t->A2, rows * rowbytes);
   A(t->meta, sizeof(DevMeta));
   A(t->slot_of, (size_t)t->max_nnz * 4);
   A(t->flags, (size_t)t->max_nnz);
@@ -227,6 +239,10 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
     A(t->gZ_b, (size_t)t->max_batch * t->H * 2);
     t->gemm_ws_bytes = 8u << 20;
     A(t->gemm_ws, t->gemm_ws_bytes);
+  }
+  if (ok) {
+    t->slab = des_slab_alloc(c, items.data(), (int)items.size());
+    ok = t->slab != nullptr;
   }
   if (!ok) { des_table_destroy(t); return DES_ERR_CUDA; }
   t->dbg.rows = rows + 1; t->dbg.slots = slots; t->dbg.grad_rows = (unsigned long long)t->max_uniq + t->rep_max;
@@ -362,7 +378,6 @@ __global__ void __launch_bounds__(256) read_rows_kernel(const uint32_t* __restri
                                                         float* __restrict__ acc_lin) {
   constexpr int VW = sizeof(V) / 4;
   des_pdl_wait(grows, W, A, emb, lin, acc_emb, acc_lin);
-  des_pdl_go();
   const int C = k / VW, lane = threadIdx.x % G;
   // a warp's groups take neighbouring rows, its ROWS_U rounds too
   const long long i0 = ((long long)blockIdx.x * 256 + (threadIdx.x & ~31)) / G * ROWS_U + (threadIdx.x & 31) / G;
