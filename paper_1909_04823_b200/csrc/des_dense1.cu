@@ -164,17 +164,21 @@ __global__ void cvt_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __
   }
 }
 
-// two arrays in one launch (the backward's two operands); four 16-byte loads of a thread in flight
+// two arrays in one launch (the backward's two operands), zeros from n to the padded length; four 16-byte loads of a thread
+// in flight
 __global__ void __launch_bounds__(256) cvt_bf16_pair_kernel(const float* __restrict__ s1, __nv_bfloat16* __restrict__ d1, size_t n1,
-                                                            const float* __restrict__ s2, __nv_bfloat16* __restrict__ d2, size_t n2) {
+                                                            size_t pad1, const float* __restrict__ s2,
+                                                            __nv_bfloat16* __restrict__ d2, size_t n2, size_t pad2) {
   des_pdl_wait(s1, d1, s2, d2);
-  const size_t m1 = n1 / 4, m = m1 + n2 / 4;           // n1 and n2 are multiples of 4
+  const size_t m1 = pad1 / 4, m = m1 + pad2 / 4;       // every length is a multiple of 4
   const size_t i0 = (size_t)blockIdx.x * 1024 + threadIdx.x;
   float4 v[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const size_t i = i0 + q * 256;
-    if (i < m) v[q] = i < m1 ? __ldg(reinterpret_cast<const float4*>(s1) + i) : __ldg(reinterpret_cast<const float4*>(s2) + (i - m1));
+    v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < m1) { if (i < n1 / 4) v[q] = __ldg(reinterpret_cast<const float4*>(s1) + i); }
+    else if (i - m1 < n2 / 4) v[q] = __ldg(reinterpret_cast<const float4*>(s2) + (i - m1));
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -234,19 +238,25 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
   const int FK = t->F * t->k;
   if (t->use_tc) {
     t->pooled_b_src = nullptr;
-    const size_t n1 = (size_t)B * t->H, n2 = (size_t)B * FK;
-    des_launch(cvt_bf16_pair_kernel, (unsigned)(((n1 + n2) / 4 + 1023) / 1024), 256, 0, st, gZ, t->gZ_b, n1, pooled, t->pooled_b, n2);
+    // The weight gradient has few output tiles (F*k x H) and a long contraction (the batch): the batch is cut into L pieces so
+    // that every SM gets a tile (L partial products, added in piece order by w1_update_kernel).  The pieces are of
+    // equal length, a multiple of 64 samples; zero rows fill the last one up.
+    const int tiles = ((FK + 127) / 128) * ((t->H + 63) / 64);
+    int L = t->sm_count / tiles;
+    if (L > B / 256) L = B / 256;
+    if (L > t->gw1_splits) L = t->gw1_splits;
+    if (L < 1) L = 1;
+    const int piece = L == 1 ? B : ((B + L - 1) / L + 63) / 64 * 64;
+    L = (B + piece - 1) / piece;
+    const size_t n1 = (size_t)B * t->H, n2 = (size_t)B * FK, p1 = (size_t)piece * L * t->H, p2 = (size_t)piece * L * FK;
+    des_launch(cvt_bf16_pair_kernel, (unsigned)(((p1 + p2) / 4 + 1023) / 1024), 256, 0, st, gZ, t->gZ_b, n1, p1, pooled, t->pooled_b,
+               n2, p2);
     DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
     const int rc1 = des_tc_gemm_dgrad(B, FK, t->H, 1, t->gZ_b, t->W1b, gE ? gE : gE_work, gE_work, gE ? 1.f : 0.f,
                                       t->gemm_ws, t->gemm_ws_bytes, st);
     if (rc1 == 0) {
       DES_LAUNCH_CHECK(t, "tc_gemm_dgrad");
-      // The product has few output tiles (F*k x H) and a long contraction (the batch): cut the batch into L
-      // pieces so that every SM gets tiles (L partial products, added in piece order by w1_update_kernel).
-      const int tiles = ((FK + 127) / 128) * ((t->H + 127) / 128);
-      int L = 1;
-      while (L < t->gw1_splits && tiles * L < 2 * t->sm_count && B % (2 * L * 64) == 0) L *= 2;
-      const int rc2 = des_tc_gemm_wgrad(FK, t->H, B / L, L, t->pooled_b, t->gZ_b, t->gW1_part, t->gW1_part, 0.f,
+      const int rc2 = des_tc_gemm_wgrad(FK, t->H, piece, L, t->pooled_b, t->gZ_b, t->gW1_part, t->gW1_part, 0.f,
                                         t->gemm_ws, t->gemm_ws_bytes, st);
       if (rc2 != 0) return DES_ERR_CUDA;           // same alignment rules as the dgrad: cannot differ
       DES_LAUNCH_CHECK(t, "tc_gemm_wgrad");

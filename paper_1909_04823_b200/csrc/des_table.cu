@@ -235,8 +235,9 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
     A(t->gW1_part, (size_t)t->gw1_splits * FKH * 4);
     // TMA needs 16-byte rows: every contiguous extent of a bf16 operand a multiple of 8
     t->use_tc = ((t->F * t->k) % 8 == 0) && (t->H % 8 == 0);
-    A(t->pooled_b, (size_t)t->max_batch * t->F * t->k * 2);
-    A(t->gZ_b, (size_t)t->max_batch * t->H * 2);
+    // (room for the zero rows behind the batch: 64 per piece of the weight gradient's contraction)
+    A(t->pooled_b, ((size_t)t->max_batch + 64 * t->gw1_splits) * t->F * t->k * 2);
+    A(t->gZ_b, ((size_t)t->max_batch + 64 * t->gw1_splits) * t->H * 2);
     t->gemm_ws_bytes = 8u << 20;
     A(t->gemm_ws, t->gemm_ws_bytes);
   }

@@ -1,0 +1,43 @@
+"""The first layer's products at sizes where the tile or the number of batch pieces changes: few samples, odd batches (the
+last piece of the weight gradient is filled up with zero rows), the narrow and the wide tile, and a smaller batch after
+a larger one (stale rows behind it must not count).  Against float64 products of the bfloat16 operands."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("F,k,H", [(39, 32, 400), (5, 16, 136), (20, 8, 24), (1, 8, 8)])
+@pytest.mark.parametrize("batches", [(300, 7), (1025, 512), (4099, 777), (12000, 8192)])
+def test_first_layer_products(F, k, H, batches):
+    from paper_1909_04823_b200 import binding as D
+    B0 = max(batches)
+    t = D.Table(2, F, k, hidden=H, partition=D.PART_FIELD, optimizer=D.OPT_SGD, lr=1.0, max_rows=4000, max_nnz=B0 * F, max_batch=B0)
+    assert t.uses_tensor_cores()
+    try:
+        g = torch.Generator(device="cuda").manual_seed(F + H)
+        rn = lambda *s: torch.randn(*s, generator=g, device="cuda")
+        for B in batches:
+            ids = torch.arange(F, device="cuda").repeat(B) + 5          # one key per field
+            db = D.DeviceBatch(torch.arange(B * F + 1, device="cuda"), ids, None, B)
+            t.find_or_insert(db)
+            W1, gZ, gE, pooled = rn(F * k, H) / 8, rn(B, H), rn(B, F * k), rn(B, F * k)
+            t.dense1_set(W1)
+            Z, work = torch.empty(B, H, device="cuda"), torch.empty(B, F * k, device="cuda")
+            ops = D.OP_POOL | D.OP_DENSE1
+            t.aggregate(ops, db, pooled=pooled, Z=Z)
+            t.backward_update(ops, db, None, pooled, Z, None, None, gE, gZ, work)
+            Vb, Wb, gb = pooled.bfloat16().double(), W1.bfloat16().double(), gZ.bfloat16().double()
+            gW = (W1 - t.dense1_get()).double()                         # lr = 1: the gradient, rounded at W1's size
+
+            def close(got, ref, absum, what, extra=0.0):   # float32 accumulation over the contraction
+                err = (got.double() - ref).abs()
+                assert bool((err <= 2e-6 * absum + extra + 1e-6).all()), (what, B, float(err.max()))
+
+            close(Z, Vb @ Wb, Vb.abs() @ Wb.abs(), "Z")
+            close(work, gE.double() + gb @ Wb.T, gE.double().abs() + gb.abs() @ Wb.abs().T, "gE")
+            ref = Vb.T @ gb
+            close(gW, ref, Vb.abs().T @ gb.abs(), "gW1", extra=1.2e-7 * (ref.abs() + W1.abs().double()))
+        assert t.status() == 0
+    finally:
+        t.close()
