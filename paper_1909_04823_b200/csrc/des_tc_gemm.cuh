@@ -20,6 +20,7 @@
 #if defined(DES_TC_GEMM_DECL_ONLY)
 /* prototypes only */
 #elif !defined(DES_NO_CUTLASS)
+#define CUTLASS_ENABLE_GDC_FOR_SM100 1    // the kernels wait for the one before them themselves (chained launches)
 #include "cutlass/cutlass.h"
 #include "cute/tensor.hpp"
 #include "cutlass/gemm/device/gemm_universal_adapter.h"
@@ -75,7 +76,7 @@
       if (gemm.can_implement(args) != cutlass::Status::kSuccess) return 1;                                            \
       if (Gemm::get_workspace_size(args) > ws_bytes) return 2;                                                        \
       if (gemm.initialize(args, workspace, stream) != cutlass::Status::kSuccess) return 3;                            \
-      if (gemm.run(stream) != cutlass::Status::kSuccess) return 4;                                                    \
+      if (gemm.run(stream, nullptr, true) != cutlass::Status::kSuccess) return 4;                                                    \
       return 0;                                                                                                       \
     }                                                                                                                 \
   };
