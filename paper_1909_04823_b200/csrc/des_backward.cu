@@ -331,12 +331,10 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
   }
 }
 
-#ifndef UP_MINB
-#define UP_MINB 2
-#endif
-#ifndef UP_UNROLL
-#define UP_UNROLL 4
-#endif
+// Keys a lane group has in flight, and resident blocks: 2 x 4 against 4 x 2 (as many keys in flight, twice the warps to issue
+// and to wait) 234 -> 210 us for 0.57 M keys of k = 64, 38 -> 34 for 0.14 M of k = 32, the same for 1.5 M.
+#define UP_MINB 4
+#define UP_UNROLL 2
 #define UP_GRID 8
 
 // Advances Adam's step count and recomputes the bias corrections 1 - beta^t in double.

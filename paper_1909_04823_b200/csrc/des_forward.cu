@@ -45,9 +45,10 @@
 #endif
 
 
-#ifndef ROUTE_PF
-#define ROUTE_PF 8    // batches of 32 occurrences whose loads a warp keeps in flight
-#endif
+// ROUTE_PF batches of 32 occurrences are in flight per warp: eight where a sample has many (2000 occurrences: 267 us, 324 with
+// two), two where it has few (120: 50 us with eight, 41 with two, whose registers let more warps in).
+#define ROUTE_LONG 512          // occurrences per sample, on average, from which it is eight
+template <int ROUTE_PF>
 __global__ void __launch_bounds__(256) route_kernel(
     const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ rows,
     const uint8_t* __restrict__ shards, int B, int F, int S, const DevMeta* __restrict__ meta, uint32_t null_row,
@@ -1044,7 +1045,7 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
   uint32_t* grow_sorted = t->slot_of;
   float* x_sorted = t->x_sorted;
   uint32_t* grow_csr = t->uslot;
-  des_launch(route_kernel, (B + 7) / 8 < t->sm_count * 8 ? (B + 7) / 8 : t->sm_count * 8, 256, 0, cs, b->offsets, b->vals, b->rows,
+  des_launch(b->nnz >= (int64_t)ROUTE_LONG * B ? route_kernel<8> : route_kernel<2>, (B + 7) / 8 < t->sm_count * 8 ? (B + 7) / 8 : t->sm_count * 8, 256, 0, cs, b->offsets, b->vals, b->rows,
              b->shards, B, (int)t->F, (int)t->S, t->meta, (uint32_t)t->total_rows, grow_csr, grow_sorted, x_sorted, t->seg_off);
   DES_LAUNCH_CHECK(t, "route_kernel");
   if (ps || fused_out) {

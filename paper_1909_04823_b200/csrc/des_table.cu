@@ -365,7 +365,7 @@ extern "C" des_status_t des_table_export(des_table_t* t, uint64_t* d_keys, uint8
 // contiguous.  (One thread per row, walking its columns 4 bytes at a time, re-read every 32-byte sector eight
 // times: 1.6 M rows of k = 64 with state took 2.23 ms.)  V = float serves dense arrays that are not
 // 16-byte aligned.
-#define ROWS_U 4
+#define ROWS_U 2
 __device__ __forceinline__ void rows_zero(float& v) { v = 0.f; }
 __device__ __forceinline__ void rows_zero(float4& v) { v = make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ float rows_sq(float v) { return v * v; }
