@@ -127,16 +127,16 @@ __device__ __forceinline__ void scatter_step(const DestMap& dm, const float* __r
 // and the atomics.  SUPER (G = 16 only): occurrences of the few keys that own a large share of a
 // skewed batch send no atomics; lane t counts the bag's occurrences of slot t and the counts go
 // to super_cnt[bag][16]; super_dense_kernel turns them into the keys' gradient sums.
-// (Resident warps: eight blocks per SM are worth 15 % without SUPER — 16384 x 39 fields 57 -> 45 us —, and cost 7 % with
-// it, where the 32 registers spill and the gradient buffer's address is best kept in registers.)
+// (What it waits for are the look-ups, so resident warps count: eight blocks per SM at 32 registers against six or seven, 16384
+// x 39 fields 57 -> 45 us.  With SUPER the wait of a chained launch costs the registers that makes them spill, 831 -> 890 us at
+// 32 M occurrences, and saves nothing there: that form is launched the plain way.)
 template <int G, int P, bool HAS_VALS, bool SUPER, bool INLINE>
-__global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatter_kernel(
+__global__ void __launch_bounds__(256, HAS_VALS ? 6 : 8) grad_scatter_kernel(
     const int32_t* __restrict__ offsets, const float* __restrict__ vals, DestMap dm,
-    long long nbags, int F, int k, uint32_t ops, const float* __restrict__ out_small,
+    uint32_t nbags, int F, int k, uint32_t ops, const float* __restrict__ out_small,
     const float* __restrict__ gL, const float* __restrict__ gF, const float* __restrict__ gE, float* Gbuf,
     float* __restrict__ super_cnt) {
-  const int zero = des_pdl_wait0();
-  if (SUPER) des_pdl_new(Gbuf);
+  const int zero = SUPER ? 0 : des_pdl_wait0();         // (SUPER is not a chained launch)
   constexpr int LB = G * P;
   const int K4 = k >> 2, stride = k + 4;
   const int sub = threadIdx.x % LB, c4 = sub % G, p = sub / G;
@@ -147,12 +147,12 @@ __global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatte
   const uint32_t mine = SUPER_TAG | (uint32_t)c4;
   // grid-stride over bags (every lane of a warp runs the same number of rounds); the next bag's bounds are
   // fetched while the current bag is scattered, so only the destination loads wait on them
-  const long long slots = (long long)gridDim.x * (256 / LB);
-  const long long rounds = (nbags + slots - 1) / slots;
-  long long bag = (long long)blockIdx.x * (256 / LB) + threadIdx.x / LB + zero;
+  const uint32_t slots = gridDim.x * (256 / LB);        // (bags < 2^31: 32 bits hold every sum)
+  const uint32_t rounds = (nbags + slots - 1) / slots;
+  uint32_t bag = blockIdx.x * (256 / LB) + threadIdx.x / LB + zero;
   int lo_n = 0, hi_n = 0;
   if (bag < nbags) { lo_n = __ldg(offsets + bag); hi_n = __ldg(offsets + bag + 1); }
-  for (long long r = 0; r < rounds; ++r, bag += slots) {
+  for (uint32_t r = 0; r < rounds; ++r, bag += slots) {
     const bool live = bag < nbags;
     const int lo = lo_n, hi = hi_n;
     lo_n = 0; hi_n = 0;
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatte
     float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
     float gf = 0.f, gl = 0.f;
     if (lo < hi) {
-      const long long b = (long long)((unsigned)bag / (unsigned)F);   // bags < 2^31: no 64-bit division
+      const long long b = (long long)(bag / (uint32_t)F);
       if (ops & DES_OP_FM) gf = __ldg(gF + b);
       if (ops & DES_OP_LR) gl = __ldg(gL + b);
       if (col) {
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatte
           c = make_float4(gf * a.x, gf * a.y, gf * a.z, gf * a.w);
         }
         if (gE) {
-          const float4 e = __ldg(reinterpret_cast<const float4*>(gE + bag * k) + c4);
+          const float4 e = __ldg(reinterpret_cast<const float4*>(gE + (size_t)bag * k) + c4);
           c.x += e.x; c.y += e.y; c.z += e.z; c.w += e.w;
         }
       }
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(256, SUPER ? 1 : HAS_VALS ? 6 : 8) grad_scatte
     if (SUPER) {
 #pragma unroll
       for (int d = G; d < LB; d <<= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, d);
-      if (live && p == 0) super_cnt[bag * 16 + c4] = (float)cnt;
+      if (live && p == 0) super_cnt[(size_t)bag * 16 + c4] = (float)cnt;
     }
   }
 }
@@ -707,8 +707,8 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
     long long blocks = (threads + 255) / 256;
     if (blocks > (long long)t->sm_count * SC_BLOCKS_PER_SM) blocks = (long long)t->sm_count * SC_BLOCKS_PER_SM;
     const unsigned grid = (unsigned)blocks;
-#define SC5(GG, PP, HV, SU, IL) des_launch(grad_scatter_kernel<GG, PP, HV, SU, IL>, grid, 256, 0, cs, b->offsets, b->vals, dm,    \
-        nbags, (int)t->F, (int)t->k, ops, (const float*)out->out_small, gr->gL, gr->gF, gE, t->Gbuf, t->super_cnt)
+#define SC5(GG, PP, HV, SU, IL) des_launch_if(!SU, grad_scatter_kernel<GG, PP, HV, SU, IL>, grid, 256, 0, cs, b->offsets, b->vals, dm, \
+        (uint32_t)nbags, (int)t->F, (int)t->k, ops, (const float*)out->out_small, gr->gL, gr->gF, gE, t->Gbuf, t->super_cnt)
 #define SC4(GG, PP, HV) do { if (inl) SC5(GG, PP, HV, false, true); else SC5(GG, PP, HV, false, false); } while (0)
 #define SC3(GG, HV) do { if (wide) SC4(GG, 32 / GG, HV); else SC4(GG, 1, HV); } while (0)
 #define SC(GG) do { if (b->vals) SC3(GG, true); else SC3(GG, false); } while (0)
