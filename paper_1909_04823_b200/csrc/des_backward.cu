@@ -21,13 +21,13 @@
 // per unique key on a sample of the batch; a key whose estimated count reaches
 // HOT_MIN gets R = count / HOT_CHAIN private replica rows, every occurrence is sent
 // to replica hash(j) mod R, and the update sums the replicas of a key
-// in double.  No accumulator ever takes more than
-// a few hundred float additions, and no address is shared by more than that
-// many atomics.
+// in double.  No accumulator ever takes more than a few hundred float additions, and no address is shared by
+// more than that many atomics.
 //
 // Two kernels, then (a small batch's scatter looks an occurrence's gradient row up itself: batch-unique index -> the
-// key's word of hinfo -> replica; a large batch has it done in a pass before): the update's first blocks take the hot keys.  Six kernels and two memsets around the same
-// two took 40 us of a 100 us step at 10 k occurrences, and 180 us of passes over index arrays at 32 M.
+// key's word of hinfo -> replica; a large batch has it done in a pass before): the update's first blocks take the hot
+// keys.  Six kernels and two memsets around the same two took 40 us of a 100 us step at 10 k occurrences, and 180 us of
+// passes over index arrays at 32 M.
 #include <type_traits>
 
 #include "des_internal.cuh"

@@ -28,7 +28,8 @@
 // operators one gather pass (sample_gather_kernel: pooled vectors and per-bag sums of the linear weights and
 // squared norms, kept in shared memory) feeds everything: shard s's sub-operators are the sums over
 // the bags of its own fields — no routing pass, no second gather.  Samples too large for that take two
-// kernels (single_gather_kernel, field_partials_kernel).
+// kernels (single_gather_kernel, field_partials_kernel).  des_forward_fused with pooling among the operators takes one
+// gather pass under HASH too: sample_gather_kernel for short bags, sample_stage_kernel for long ones.
 //
 // Accuracy.  A lane never adds more than a few dozen terms into one float32 accumulator (long
 // segments are summed in two levels), and the sum over shards is taken in double and rounded once, so
@@ -279,8 +280,9 @@ __device__ __forceinline__ void pool_step(const uint32_t* __restrict__ grow_csr,
 #define SP_U 4
 #define SP_BRIEF 8       // occurrences per (sample, shard) segment, on average, up to which segments are taken one per sub-group
 #define SP_FLUSH 4
+// (36 registers, seven blocks per SM: 776 -> 763 us at 32 M occurrences of k = 64; FUSED 64, four: 127 -> 118 at 2.5 M of k = 40)
 template <int G, bool HAS_VALS, bool FUSED>
-__global__ void __launch_bounds__(256) shard_partials_kernel(
+__global__ void __launch_bounds__(256, FUSED || HAS_VALS ? 4 : 7) shard_partials_kernel(
     const uint32_t* __restrict__ grow_sorted, const float* __restrict__ x_sorted, const int32_t* __restrict__ seg_off,
     int B, int S, int k, uint32_t ops, const float* __restrict__ W, uint32_t null_row, float* __restrict__ part_small,
     float* __restrict__ out_small) {
@@ -353,7 +355,7 @@ __global__ void __launch_bounds__(256) shard_partials_kernel(
 // kernel above spends a round of loads and a butterfly on it.  FUSED adds the partials in shard order all the same (handed
 // round by shuffles), so both forms still give the same bits.
 template <int G, bool HAS_VALS, bool FUSED>
-__global__ void __launch_bounds__(256) shard_partials_short_kernel(
+__global__ void __launch_bounds__(256, FUSED || HAS_VALS ? 4 : 6) shard_partials_short_kernel(
     const uint32_t* __restrict__ grow_sorted, const float* __restrict__ x_sorted, const int32_t* __restrict__ seg_off,
     int B, int S, int k, uint32_t ops, const float* __restrict__ W, uint32_t null_row, float* __restrict__ part_small,
     float* __restrict__ out_small) {
@@ -793,10 +795,10 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
 // row's linear weight and squared norm, which go straight into sums of the thread's — and leaves the row in shared memory;
 // then the warps pool a bag each, their only loads the latent vectors.  What bounds the pooling is the number of loads that
 // go through L1 per occurrence: looked up by all lanes of every occurrence it was four (8.2 M occurrences of k = 64:
-// 321 us, now 302; the rest is latency at the 40 warps that fit an SM).
+// 321 us, staged 302, eight rows of a lane in flight at 32 warps per SM instead of four at 40 282; the rest is that latency).
 #define SS_CAP 2048
 template <int G, int P, bool HAS_VALS>
-__global__ void __launch_bounds__(256, 5) sample_stage_kernel(
+__global__ void __launch_bounds__(256, 4) sample_stage_kernel(
     const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ rows,
     const uint8_t* __restrict__ shards, int B, int F, int S, int k, int T, uint32_t ops, const float* __restrict__ W,
     const DevMeta* __restrict__ meta, uint32_t null_row, float* __restrict__ pooled, __nv_bfloat16* __restrict__ pooled_b,
@@ -910,7 +912,8 @@ __global__ void __launch_bounds__(256, 5) sample_stage_kernel(
         i0 += N * P;
       };
       const int full = lo + (hi - lo) / P * P;         // whole rounds of the warp end here
-      while (i0 - p + 4 * P <= full) step(std::integral_constant<int, 4>());
+      while (i0 - p + 8 * P <= full) step(std::integral_constant<int, 8>());
+      if (i0 - p + 4 * P <= full) step(std::integral_constant<int, 4>());
       if (i0 - p + 2 * P <= full) step(std::integral_constant<int, 2>());
       if (i0 - p + P <= full) step(std::integral_constant<int, 1>());
       if (i0 < hi) step(std::integral_constant<int, 1>());
