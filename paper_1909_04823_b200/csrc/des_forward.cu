@@ -280,9 +280,10 @@ __device__ __forceinline__ void pool_step(const uint32_t* __restrict__ grow_csr,
 #define SP_U 4
 #define SP_BRIEF 8       // occurrences per (sample, shard) segment, on average, up to which segments are taken one per sub-group
 #define SP_FLUSH 4
-// (36 registers, seven blocks per SM: 776 -> 763 us at 32 M occurrences of k = 64; FUSED 64, four: 127 -> 118 at 2.5 M of k = 40)
+// (40 registers, six blocks per SM: 776 -> 752 us at 32 M occurrences of k = 64, 32 and eight: 770; FUSED 64, four: 127 -> 118 at
+// 2.5 M of k = 40)
 template <int G, bool HAS_VALS, bool FUSED>
-__global__ void __launch_bounds__(256, FUSED || HAS_VALS ? 4 : 7) shard_partials_kernel(
+__global__ void __launch_bounds__(256, FUSED || HAS_VALS ? 4 : 6) shard_partials_kernel(
     const uint32_t* __restrict__ grow_sorted, const float* __restrict__ x_sorted, const int32_t* __restrict__ seg_off,
     int B, int S, int k, uint32_t ops, const float* __restrict__ W, uint32_t null_row, float* __restrict__ part_small,
     float* __restrict__ out_small) {
