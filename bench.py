@@ -210,18 +210,17 @@ class ClockSampler:
 # own batch on a 4e6-key table (the 2e8-key table cannot be captured under multi-pass replay).  The scatter's traffic does not depend on
 # the table; kernels that touch table rows move fewer DRAM bytes there (U = 1.06 M instead of 1.81 M).
 NCU_DRAM_TRAFFIC = {
-    ("cfg5", "grad_scatter_kernel"): 1807e6,
+    ("cfg5", "grad_scatter_kernel"): 1811e6,
     ("cfg5", "super_dense_kernel"): 533e6,
-    ("cfg5", "shard_partials_kernel"): 962e6,
-    ("cfg5", "pool_kernel"): 1213e6,
-    ("cfg5", "update_rows_kernel"): 1933e6,
+    ("cfg5", "shard_partials_kernel"): 979e6,
+    ("cfg5", "pool_kernel"): 1212e6,
+    ("cfg5", "update_rows_kernel"): 1945e6,
     ("cfg5", "probe_claim_kernel"): 596e6,
-    ("cfg5", "flag_count_kernel"): 566e6,
+    ("cfg5", "flag_count_kernel"): 565e6,
     ("cfg5", "resolve_kernel"): 421e6,
     ("cfg5", "make_dest_kernel"): 225e6,
-    ("cfg5", "route_kernel"): 456e6,
-    ("cfg5", "single_gather_kernel"): 1290e6,
-    ("cfg5", "fused_finish_kernel"): 440e6,
+    ("cfg5", "route_kernel"): 453e6,
+    ("cfg5", "sample_stage_kernel"): 1270e6,
 }
 
 
@@ -247,12 +246,12 @@ def kernel_bytes(name, st):
         return 4 * B * (S + 1) + 4 * nnz + row * U + 4 * S * B * (k + 4)
     if name == "pool_kernel":
         return 4 * (B * F + 1) + 4 * nnz + 4 * k * U + 4 * B * F * k
+    if name in ("sample_gather_kernel", "sample_stage_kernel"):   # rows + shards in, every unique row once, pooled + aggregates out
+        return 4 * (B * F + 1) + 5 * nnz + row * U + (4 * B * F * k if pool else 0) + 4 * B * (k + 4)
     if name == "single_gather_kernel":   # rows + shards in, every unique row once, pooled + bag tails out
         return 4 * (B * F + 1) + 5 * nnz + row * U + 4 * B * F * k + 8 * B * F
     if name == "field_partials_kernel":   # pooled vectors and bag tails in, per-shard partials out
         return 4 * B * F * k + 8 * B * F + 4 * S * B * (k + 4)
-    if name == "fused_finish_kernel":
-        return 4 * B * F * k + 8 * B * F + 4 * B * (k + 4)
     if name == "aggregate_small_kernel":
         return 4 * S * B * (k + 4) + 4 * B * (k + 4)
     if name == "make_dest_kernel":
@@ -264,9 +263,9 @@ def kernel_bytes(name, st):
         return 4 * (B * F + 1) + 4 * nnz + (4 * B * F * k if pool else 0) + 4 * B * (k + 4) + 8 * B + row * (U + R)
     if name == "super_dense_kernel":
         return 64 * B * F + (4 * B * F * k if pool else 0) + 4 * B * (k + 4) + 8 * B
-    if name == "sample_count_kernel":
+    if name == "count_kernel":
         return 4 * (nnz >> st["shift"]) + 4 * U
-    if name == "hot_reduce_kernel":
+    if name == "hot_sum_kernel":
         return 2 * row * R
     if name == "update_rows_kernel":
         return U * (2 * row + 2 * row * (1 + state) + 8)
@@ -281,7 +280,7 @@ def occurrence_bytes(name, st):
     nnz, k = st["nnz"], st["k"]
     if name == "pool_kernel":
         return 4 * k * nnz
-    if name in ("shard_partials_kernel", "single_gather_kernel"):
+    if name in ("shard_partials_kernel", "single_gather_kernel", "sample_gather_kernel", "sample_stage_kernel"):
         return (4 * k + 32) * nnz          # the vector and the 32-byte sector that holds the row's tail
     return None
 
@@ -306,10 +305,10 @@ def kernel_flops(name, st):
 # while only the unique rows come from HBM.
 BOUND_NOTES = {
     "grad_scatter_kernel": "busiest unit per ncu: L1TEX 87 % / L2 67 % (one 16-byte vector atomic per lane and occurrence); DRAM 26 %",
-    "shard_partials_kernel": "busiest unit per ncu: L1TEX 73 % (a 272-byte row per occurrence through L1); DRAM 15 %",
+    "shard_partials_kernel": "busiest unit per ncu: L1TEX 80 % (a 272-byte row per occurrence through L1); DRAM 15 %",
     "pool_kernel": "busiest unit per ncu: L1TEX 77 % (a 256-byte vector per occurrence through L1); DRAM 27 %",
-    "single_gather_kernel": "busiest unit per ncu: L1TEX 65 % (a 272-byte row per occurrence through L1); DRAM 16 %",
-    "update_rows_kernel": "random 272-byte rows of weights and state: DRAM-bound (56 % on a small table under ncu)",
+    "sample_stage_kernel": "latency of the row gathers at 32 warps per SM; L1TEX 68 % per ncu (a 272-byte row per occurrence); DRAM 15 %",
+    "update_rows_kernel": "random 272-byte rows of weights and state: DRAM-bound (57 % on a small table under ncu)",
 }
 TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on the benchmark's own batch with a "
                   "4e6-key table (the 2e8-key table cannot be captured under multi-pass replay); constant, not measured "
@@ -574,7 +573,8 @@ def run_workload(args, cfg_index, w, ctx, *, steps, warmup, repeats, modes, want
                 ms_mode[name] = max_over_ranks(e0.elapsed_time(e1) / n_e2e, world, dev)
             ms_e = ms_mode["pipelined"]
             e2e = {"value": job_throughput(B, world, ms_e), "unit": UNIT, "ms_per_step": ms_e,
-                   "mode": "des_step_host_submit / des_step_host_wait from pinned host buffers, two steps in flight; "
+                   "mode": "des_step_host_submit / des_step_host_wait from pinned host buffers, two steps in flight, "
+                           "forward fused (per-shard partials summed on chip in shard order); "
                            "copied every step: offsets + ids host to device, out_small [B][k+4] back; resident on the "
                            "device: the upstream gradients gL / gF / gE (they come from the rest of the model) and the "
                            "pooled output (its consumer)",

@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
 // of a warp walks bags of its own, SGF_BU short ones with their first occurrences in flight together (a one-hot
 // batch is a chain offsets -> row number -> row per bag).
 //  FIELD = false  (the fused form): the groups add their bags in double as they go, and the sample's sums are combined by
-//                 shuffles and, over its warps, in shared memory.  Against single_gather + fused_finish the
+//                 shuffles and, over its warps, in shared memory.  Against a gather and a second pass over its output the
 //                 pooled vectors are not read back; and a small batch does not wait for one lane group
 //                 per sample to walk all its fields (48 samples x 39 fields: 12.4 -> 5.2 us; 1500 samples x 100
 //                 bags of 20: 160 -> 141 us).
