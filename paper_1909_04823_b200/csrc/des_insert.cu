@@ -494,17 +494,30 @@ __device__ __forceinline__ void count_end(const CountArgs& a, const uint32_t* s_
   if (!s_last) return;
   __threadfence();
   const uint32_t nh = min(__ldcg(a.hot_ctr), a.hot_max);
-  for (uint32_t h = threadIdx.x; h < nh; h += blockDim.x) {
-    const uint32_t u = __ldcg(a.hot_u + h), est = __ldcg(a.hinfo + u) << a.shift;
+  const int lane = threadIdx.x & 31;
+  for (uint32_t h0 = 0; h0 < nh; h0 += blockDim.x) {   // whole warps; a warp takes its keys' space with one addition
+    const uint32_t h = h0 + threadIdx.x;
+    const bool in = h < nh;
+    const uint32_t u = in ? __ldcg(a.hot_u + h) : 0u, est = in ? __ldcg(a.hinfo + u) << a.shift : 0u;
     // the few keys that own a large share of the batch take one of SUPER_T slots
     uint32_t ts = SUPER_T;
-    if (a.super_min && est >= a.super_min) ts = atomicAdd(a.hot_ctr + 3, 1u);
+    if (in && a.super_min && est >= a.super_min) ts = atomicAdd(a.hot_ctr + 3, 1u);
     const bool sup = ts < SUPER_T;
-    uint32_t R = sup ? SUPER_R : (est + HOT_CHAIN(a.shift) - 1) / HOT_CHAIN(a.shift);
+    uint32_t R = !in ? 0u : sup ? SUPER_R : (est + HOT_CHAIN(a.shift) - 1) / HOT_CHAIN(a.shift);
     // (a key's chunk number has to fit a work item; longer chains only cost accuracy)
     R = min(R, (1u << HOT_WORK_BITS) * HOT_RCHUNK);
     const uint32_t nchunk = (R + HOT_RCHUNK - 1) / HOT_RCHUNK;
-    const uint32_t base = atomicAdd(a.hot_ctr + 1, R), wbase = atomicAdd(a.hot_ctr + HOT_CTR_WORK, nchunk);
+    uint32_t base = R, wbase = nchunk;                 // inclusive sums over the warp, then where the key's space starts
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, base, d), y = __shfl_up_sync(0xFFFFFFFFu, wbase, d);
+      if (lane >= d) { base += x; wbase += y; }
+    }
+    uint32_t b0 = 0, w0 = 0;
+    if (lane == 31) { b0 = atomicAdd(a.hot_ctr + 1, base); w0 = atomicAdd(a.hot_ctr + HOT_CTR_WORK, wbase); }
+    base += __shfl_sync(0xFFFFFFFFu, b0, 31) - R;
+    wbase += __shfl_sync(0xFFFFFFFFu, w0, 31) - nchunk;
+    if (!in) continue;
     const bool ok = base + R <= a.rep_max && wbase + nchunk <= a.work_max;   // nothing left: the key is treated as a cold one
     for (uint32_t i = 0; i < nchunk && wbase + i < a.work_max; ++i) a.hot_work[wbase + i] = ok ? h << HOT_WORK_BITS | i : DES_ROW_NONE;
     a.hot_rep[h] = make_uint2(base, ok ? R : 0u);
