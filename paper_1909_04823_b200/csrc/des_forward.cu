@@ -41,6 +41,7 @@
 
 #define SGF_BU 4                  // short bags of a lane group in flight together (sample_gather_kernel)
 #define SGF_SMEM (24u << 10)      // shared memory a block of the FIELD form takes at most, unless one sample needs more
+#define SGF_ONE (47u << 10)       // and at most for one sample: a launch has 48 KiB, the kernel's own arrays (s_base and the like) included
 #ifndef POOL_BLOCKS_PER_SM
 #define POOL_BLOCKS_PER_SM 64   // grid cap of the pooling kernel (it strides over the bags)
 #endif
@@ -1005,7 +1006,7 @@ __global__ void reduce_shards_kernel(const float* __restrict__ part, size_t per_
 static int group_for(int k) { int K4 = k / 4, G = 1; while (G < K4) G <<= 1; return G; }
 
 static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, float* pooled, cudaStream_t cs);
-static bool sample_gather_fits(const des_table* t) { return (size_t)t->F * (t->k + 2) * 4 <= (48u << 10); }   // FIELD form, one sample
+static bool sample_gather_fits(const des_table* t) { return (size_t)t->F * (t->k + 2) * 4 <= SGF_ONE; }   // FIELD form, one sample
 static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, bool field, float* pooled,
                                          float* part_small, float* out_small, cudaStream_t cs);
 

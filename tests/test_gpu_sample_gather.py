@@ -41,7 +41,10 @@ def _setup(D, B, F, k, S, partition, mean, vals, seed):
 @pytest.mark.parametrize("B,F,k,S,partition,mean,vals", [
     (1, 1, 4, 1, 1, 1, False), (48, 39, 32, 16, 1, 1, False), (700, 8, 8, 4, 0, 2, True), (1300, 39, 16, 5, 1, 1, True),
     (2500, 40, 20, 7, 1, 1, False), (5000, 26, 16, 8, 1, 1, False), (33, 100, 64, 64, 0, 20, False), (5000, 3, 64, 3, 0, 12, True),
-    (20, 400, 64, 9, 1, 1, False)])
+    (20, 400, 64, 9, 1, 1, False),
+    # about the largest sample whose pooled vectors a block holds, and the sizes behind it
+    *[(20, F, 64, 9, 1, 1, False) for F in (182, 183, 185, 186, 187)], (20, 360, 32, 7, 1, 1, True), (20, 361, 32, 7, 1, 1, False),
+    (20, 682, 16, 5, 1, 1, False)])
 def test_sums_of_a_sample(B, F, k, S, partition, mean, vals):
     from paper_1909_04823_b200 import binding as D
     t, db, bag, v, w, nnz = _setup(D, B, F, k, S, partition, mean, vals, B + F)
