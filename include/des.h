@@ -258,7 +258,9 @@ des_status_t des_forward_fused(des_table_t* t, uint32_t ops, const des_batch_t* 
  * summed per unique key, then one SGD / Adagrad application per key with the
  * state kept in the shard.  With DENSE1: gE_work = gE + gZ W1^T (each shard's
  * own column block), gW1 = pooled^T gZ, and the same optimizer on W1.
- * `out` supplies A (out_small) and pooled. */
+ * `out` supplies A (out_small) and pooled.  Of the batch the call uses what its arrays hold when its kernels run: the table
+ * may have seen other batches since, the arrays may have been copied, and a captured call may be replayed for
+ * whatever find_or_insert (or a copy of its results) has put into the same buffers. */
 des_status_t des_backward_update(des_table_t* t, uint32_t ops, const des_batch_t* batch,
                                  const des_outputs_t* out, const des_grads_t* grads, void* stream);
 

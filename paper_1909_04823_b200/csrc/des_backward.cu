@@ -17,14 +17,14 @@
 // Hot keys.  CTR ids are Zipf distributed: a handful of keys own most of a
 // batch's occurrences.  Millions of float atomics on one gradient row would
 // serialise in L2 and, summed one after the other in fp32, lose the 1e-5
-// accuracy the step must keep.  So find_or_insert counts the occurrences
-// per unique key on a sample of the batch; a key whose estimated count reaches
+// accuracy the step must keep.  So the backward first counts the occurrences
+// per unique key (on a sample of a large batch); a key whose estimated count reaches
 // HOT_MIN gets R = count / HOT_CHAIN private replica rows, every occurrence is sent
 // to replica hash(j) mod R, and the update sums the replicas of a key
 // in double.  No accumulator ever takes more than a few hundred float additions, and no address is shared by
 // more than that many atomics.
 //
-// Two kernels, then (a small batch's scatter looks an occurrence's gradient row up itself: batch-unique index -> the
+// Three kernels, then (a small batch's scatter looks an occurrence's gradient row up itself: batch-unique index -> the
 // key's word of hinfo -> replica; a large batch has it done in a pass before): the update's first blocks take the hot
 // keys.  Six kernels and two memsets around the same two took 40 us of a 100 us step at 10 k occurrences, and 180 us of
 // passes over index arrays at 32 M.
@@ -222,9 +222,8 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
     const float* __restrict__ out_small, const float* __restrict__ gL, const float* __restrict__ gF,
     const float* __restrict__ gE, float* Gbuf, const uint32_t* __restrict__ ctr,
     const uint2* __restrict__ hot_rep, long long max_uniq) {
-  uint32_t ns = __ldg(ctr + 3);
+  const uint32_t ns = __ldg(ctr + HOT_N_SUPER);
   if (ns == 0) return;
-  if (ns > SUPER_T) ns = SUPER_T;
   extern __shared__ __align__(16) unsigned char sd_smem[];
   typedef float4 (*tile_t)[SD_TILE][16];
   tile_t s_c = reinterpret_cast<tile_t>(sd_smem);                                      // gE rows
@@ -310,7 +309,7 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
   const uint32_t salt = des_hash32(blockIdx.x * 8u + (uint32_t)(tailw ? th : sub));
   if (tailw) {
     if ((uint32_t)tt >= ns) return;
-    const uint32_t hh = __ldg(ctr + HOT_CTR_SLOT + tt);
+    const uint32_t hh = __ldg(ctr + HOT_N_SLOT + tt);
     if (hh == DES_ROW_NONE) return;
     const uint2 rp = __ldg(hot_rep + hh);
     if (rp.y == 0) return;
@@ -322,7 +321,7 @@ __global__ void __launch_bounds__(SD_THREADS) super_dense_kernel(
   for (int q = 0; q < 8; ++q) {
     const uint32_t key = (uint32_t)(kg * 8 + q);
     if (key >= ns || !col) continue;
-    const uint32_t hh = __ldg(ctr + HOT_CTR_SLOT + key);
+    const uint32_t hh = __ldg(ctr + HOT_N_SLOT + key);
     if (hh == DES_ROW_NONE) continue;
     const uint2 rp = __ldg(hot_rep + hh);
     if (rp.y == 0) continue;
@@ -513,12 +512,12 @@ __device__ __forceinline__ void hot_keys(HotShared<G>& sh, int blk, int nblk, ui
 // occurrences, all of it the hottest key's 1800 rows.)
 __global__ void __launch_bounds__(256) hot_sum_kernel(int k, long long max_uniq, float* __restrict__ Gbuf,
                                                       const uint32_t* __restrict__ hot_u, const uint2* __restrict__ hot_rep,
-                                                      const uint32_t* __restrict__ hot_ctr, uint32_t work_max,
+                                                      const uint32_t* __restrict__ hot_ctr,
                                                       const uint32_t* __restrict__ hot_work, double* hot_acc, uint32_t* hot_done) {
   des_pdl_wait(Gbuf, hot_u, hot_rep, hot_ctr, hot_work, hot_acc, hot_done);
   const int stride = k + 4, lane = threadIdx.x & 31;
   const bool c0 = lane < stride, c1 = lane + 32 < stride, c2 = lane + 64 < stride;
-  const uint32_t nw = min(__ldg(hot_ctr + HOT_CTR_WORK), work_max);
+  const uint32_t nw = __ldg(hot_ctr + HOT_N_WORK);
   for (uint32_t wi = blockIdx.x * 8 + (threadIdx.x >> 5); wi < nw; wi += gridDim.x * 8) {
     const uint32_t item = __ldg(hot_work + wi), h = item >> HOT_WORK_BITS, chunk = item & ((1u << HOT_WORK_BITS) - 1u);
     if (item == DES_ROW_NONE) continue;
@@ -576,8 +575,8 @@ template <int G, bool ADAM, bool HOT>
 __global__ void __launch_bounds__(256, UP_MINB) update_rows_kernel(
     int hot_blocks, const uint32_t* __restrict__ uniq_rows, const uint32_t* __restrict__ n_uniq, long long max_uniq, int k,
     uint32_t ops, const OptParams opt_in, DevMeta* __restrict__ meta, float* __restrict__ Gbuf, float* __restrict__ W,
-    float* __restrict__ A, float* __restrict__ A2, const uint32_t* __restrict__ hinfo, const uint32_t* __restrict__ hot_u,
-    const uint2* __restrict__ hot_rep, const uint32_t* __restrict__ hot_ctr, uint32_t hot_max) {
+    float* __restrict__ A, float* __restrict__ A2, uint32_t* hinfo, const uint32_t* __restrict__ hot_u,
+    const uint2* __restrict__ hot_rep, const uint32_t* __restrict__ hot_ctr) {
   constexpr int NG = 256 / G;
   __shared__ typename std::conditional<HOT, HotShared<G>, int>::type sh;
   const int z0 = des_pdl_wait0();
@@ -593,7 +592,7 @@ __global__ void __launch_bounds__(256, UP_MINB) update_rows_kernel(
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (HOT) {
     if ((int)blockIdx.x < hot_blocks) {
-      hot_keys<G>(sh, (int)blockIdx.x + z0, hot_blocks, min(__ldg(hot_ctr), hot_max), hot_rep, Gbuf + (size_t)max_uniq * stride, stride,
+      hot_keys<G>(sh, (int)blockIdx.x + z0, hot_blocks, __ldg(hot_ctr + HOT_N_KEYS), hot_rep, Gbuf + (size_t)max_uniq * stride, stride,
                   K4, c4, col, lead, [&](uint32_t h, bool mine, const double (&a)[4], const double (&tl)[2]) {
                     uint32_t row = mine ? __ldg(uniq_rows + __ldg(hot_u + h)) : DES_ROW_NONE;
                     if (row != DES_ROW_NONE && DES_DBG_ROW(row) != row) row = DES_ROW_NONE;      // (checking build)
@@ -626,7 +625,7 @@ __global__ void __launch_bounds__(256, UP_MINB) update_rows_kernel(
     for (int q = 0; q < UP_UNROLL; ++q) {
       const long long u = u0 + q * gstep;
       r[q] = u < U ? __ldg(uniq_rows + u) : DES_ROW_NONE;
-      cold[q] = u < U && !(HOT && (__ldg(hinfo + u) & HOT_FLAG));
+      cold[q] = u < U && !(HOT && (hinfo[u] & HOT_FLAG));
       if (HOT && !cold[q]) r[q] = DES_ROW_NONE;
       if (r[q] != DES_ROW_NONE && DES_DBG_ROW(r[q]) != r[q]) r[q] = DES_ROW_NONE;   // (checking build)
       g[q] = zero; tail[q] = make_float2(0.f, 0.f);
@@ -638,10 +637,11 @@ __global__ void __launch_bounds__(256, UP_MINB) update_rows_kernel(
     }
 #pragma unroll
     for (int q = 0; q < UP_UNROLL; ++q) key_load<ADAM>(ua, r[q], c4, col, lead, x[q]);
-    __syncwarp();   // all lanes of a group have read the gradient row before its lead lane clears it
+    __syncwarp();   // all lanes of a group have read the gradient row and hinfo before its lead lane clears them
 #pragma unroll
     for (int q = 0; q < UP_UNROLL; ++q) {
       const long long u = u0 + q * gstep;
+      if (lead && u < U) hinfo[u] = 0u;
       if (cold[q]) {
         float4* grow = reinterpret_cast<float4*>(Gbuf + (size_t)u * stride);
         if (col) grow[c4] = zero;
@@ -690,9 +690,8 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
   const int G = group_for(t->k);
   const int nnz = (int)b->nnz;
   const long long nbags = (long long)B * t->F;
-  // counts and hot keys of this batch: find_or_insert has left them unless it has seen another batch since
   if ((st = des_count_batch(t, b, cs)) != DES_OK) return st;
-  const bool use_super = t->tag_super;
+  const bool use_super = des_super_path(t, b);
   DestMap dm;
   dm.uidx = b->uidx; dm.hinfo = t->hinfo; dm.hot_rep = t->hot_rep; dm.max_uniq = (uint32_t)t->max_uniq; dm.dest = t->dest;
   const bool inl = nnz < DEST_INLINE;
@@ -744,14 +743,14 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
     // (up to DEST_INLINE occurrences the two kernels in one are a launch less; beyond, the flag look-up per key costs more)
     if (!inl) {
       des_launch(hot_sum_kernel, t->sm_count * 8, 256, 0, cs, (int)t->k, (long long)t->max_uniq, t->Gbuf, t->hot_u, t->hot_rep,
-                 t->hot_ctr, t->work_max, t->hot_work, t->hot_acc, t->hot_done);
+                 t->hot_ctr, t->hot_work, t->hot_acc, t->hot_done);
       DES_LAUNCH_CHECK(t, "hot_sum_kernel");
       hot = 0;
     }
     const unsigned grid = (unsigned)(blocks + hot);
 #define UP3(GG, AD, HT) des_launch(update_rows_kernel<GG, AD, HT>, grid, 256, 0, cs, hot, b->uniq_rows, b->n_uniq,                  \
                                    (long long)t->max_uniq, (int)t->k, ops, opt, t->meta, t->Gbuf, t->W, t->A, t->A2, t->hinfo,       \
-                                   t->hot_u, t->hot_rep, t->hot_ctr, t->hot_max)
+                                   t->hot_u, t->hot_rep, t->hot_ctr)
 #define UP2(GG, AD) do { if (inl) UP3(GG, AD, true); else UP3(GG, AD, false); } while (0)
 #define UP(GG) do { if (t->A2) UP2(GG, true); else UP2(GG, false); } while (0)
     switch (G) { case 1: UP(1); break; case 2: UP(2); break; case 4: UP(4); break; case 8: UP(8); break; default: UP(16); }

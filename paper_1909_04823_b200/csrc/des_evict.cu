@@ -353,7 +353,6 @@ static des_status_t evict_run(des_table_t* t, const uint64_t* d_keys, int64_t n,
   DES_CUDA(cudaGetDevice(&dev));
   if (dev != t->device) return DES_ERR_INVALID_ARG;
   DES_CUDA(cudaDeviceSynchronize());
-  t->tag_valid = 0;                                    // rows move: whatever was derived from a batch is stale
   des_api_begin(t, 0);
   if (!by_age && n == 0) return DES_OK;
   const int S = (int)t->S;

@@ -21,9 +21,8 @@
 //                 counts (no scan pass).  New keys' rows go into their slots and are filled from
 //                 the counter-based generator (a lane group per row).
 //   resolve       every other occurrence takes row and unique index from its
-//                 key's first occurrence; shard sizes advance, the call's scratch range is retired.  The
-//                 occurrences are counted per unique key on the way (a sample of a large batch) and the hot keys
-//                 listed: what the backward needs to know of the batch before it can scatter.
+//                 key's first occurrence; shard sizes advance, the call's scratch range is retired.
+// A fifth kernel (count_kernel) is the backward's: it counts the occurrences per unique key and lists the hot keys.
 #include "des_internal.cuh"
 
 #include <type_traits>
@@ -246,8 +245,7 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
     int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx,
     uint32_t* __restrict__ uniq_rows, uint32_t* __restrict__ n_uniq_out, Slot* slots, unsigned long long total_slots,
     uint32_t max_nnz, int k, int stride, float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2,
-    unsigned long long seed, float init_scale, float state_init, float lin_state_init, uint32_t* __restrict__ hinfo,
-    long long max_uniq, uint32_t* __restrict__ hot_ctr) {
+    unsigned long long seed, float init_scale, float state_init, float lin_state_init) {
   constexpr int NT = 512, NW = NT / 32, M = NT * PER / IB;
   constexpr bool DEEP = PER > 2;
   __shared__ uint16_t s_first[DEEP ? NT * PER : 1];     // DEEP: the block's first occurrences in order (bit 15: new key)
@@ -259,13 +257,12 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
   __shared__ uint32_t l_grow[IB];                       // ... batch-unique index, then table-global row
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile0 = blockIdx.x * M, jb = tile0 * IB, j0 = jb + tid * PER;
-  des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2, hinfo, hot_ctr);
+  des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2);
   // The slots' scratch range ends with this call (see Slot::first_occ; resolve_kernel then starts a new one): nothing
   // reads the scratch words after flag_count_kernel, so they are all cleared here, once every few billion occurrences.
   if (meta->scratch_base - (uint32_t)nnz < max_nnz)
     for (unsigned long long i = (unsigned long long)blockIdx.x * NT + tid; i < total_slots; i += (unsigned long long)gridDim.x * NT)
       slots[i].first_occ = DES_ROW_NONE;
-  if (blockIdx.x == 0 && tid < HOT_CTR_SLOT + 1) hot_ctr[tid < HOT_CTR_SLOT ? tid : HOT_CTR_WORK] = 0u;        // (counted by resolve_kernel)
   typedef typename std::conditional<PER == 8, unsigned long long, uint16_t>::type flags_t;
   unsigned long long w = 0;
   if (j0 + PER <= nnz) w = __ldg(reinterpret_cast<const flags_t*>(flags + j0));
@@ -315,7 +312,6 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
     const uint32_t u0 = firsts - nf;
     for (uint32_t i = tid; i < nf; i += NT) {
       const uint32_t e = s_first[i];
-      if ((long long)(u0 + i) < max_uniq) hinfo[u0 + i] = 0u;
       if (e & 0x8000u) continue;
       const uint32_t row = rows[jb + e], sd = __ldg(shards + jb + e);
       uidx[jb + e] = row == DES_ROW_NONE ? DES_ROW_NONE : u0 + i;
@@ -326,7 +322,6 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       if (!first(q)) continue;
-      if ((long long)uu < max_uniq) hinfo[uu] = 0u;
       if (!fresh(q)) {
         uidx[j0 + q] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : uu;
         uniq_rows[uu] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : s_row[sh[q]] + r[q];
@@ -439,105 +434,15 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
   }
 }
 
-// ---- counting ------------------------------------------------------------------------------------------------------
-// hinfo[u] += occurrences of key u among a 1 / 2^shift sample.  A hot key would draw tens of thousands of atomics on one
-// word, which L2 serialises, so counts are merged per warp (lanes holding the same key), then per block in a small
-// shared-memory table keyed by a hash of the key (an entry taken by another key sends the count straight to memory), and
-// each block adds its table once.  The addition that takes a key over the threshold lists it; the block that
-// finishes last turns the list into replica rows.
-#define CT_SLOTS 1024
-// resolve_kernel counts on the way up to CT_INLINE occurrences, whole up to CT_WHOLE and one of a thread's four beyond
-// (16384 x 39 fields: 18 us for the sample, 38 whole); larger batches are counted by count_kernel, from 1 / 16 to 1 / 64.
-#define CT_WHOLE (1 << 17)
-#define CT_INLINE (1 << 20)
-struct CountArgs {
-  uint32_t *hinfo, *hot_u, *hot_ctr;
-  uint2* hot_rep;
-  long long max_uniq;
-  int shift;
-  uint32_t* hot_work;
-  uint32_t work_max, hot_max, rep_max, super_min;                // super_min = 0: no key is counted instead of scattered
-};
-
-__device__ __forceinline__ void count_flush(const CountArgs& a, uint32_t u, uint32_t c) {
-  const uint32_t thr = HOT_MIN(a.shift) >> a.shift, old = atomicAdd(a.hinfo + u, c);
-  if (old < thr && old + c >= thr) {
-    const uint32_t h = atomicAdd(a.hot_ctr, 1u);
-    if (h < a.hot_max) a.hot_u[h] = u;
-  }
-}
-// whole warp; u = DES_ROW_NONE: nothing to count
-__device__ __forceinline__ void count_one(const CountArgs& a, uint32_t* s_key, uint32_t* s_cnt, uint32_t u) {
-  const bool ok = (long long)u < a.max_uniq;
-  const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
-  if (!ok) return;
-  const unsigned same = __match_any_sync(act, u);
-  if ((threadIdx.x & 31) != __ffs(same) - 1) return;
-  const uint32_t e = des_hash32(u) & (CT_SLOTS - 1), c = (uint32_t)__popc(same);
-  const uint32_t old = atomicCAS(&s_key[e], DES_ROW_NONE, u);
-  if (old == DES_ROW_NONE || old == u) atomicAdd(&s_cnt[e], c);
-  else count_flush(a, u, c);
-}
-__device__ __forceinline__ void count_begin(uint32_t* s_key, uint32_t* s_cnt) {
-  for (int i = threadIdx.x; i < CT_SLOTS; i += blockDim.x) { s_key[i] = DES_ROW_NONE; s_cnt[i] = 0u; }
-}
-// whole block; `blocks` blocks take part
-__device__ __forceinline__ void count_end(const CountArgs& a, const uint32_t* s_key, const uint32_t* s_cnt, uint32_t blocks) {
-  __shared__ bool s_last;
-  __syncthreads();
-  for (int i = threadIdx.x; i < CT_SLOTS; i += blockDim.x)
-    if (s_cnt[i]) count_flush(a, s_key[i], s_cnt[i]);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(a.hot_ctr + 2, 1u) == blocks - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const uint32_t nh = min(__ldcg(a.hot_ctr), a.hot_max);
-  const int lane = threadIdx.x & 31;
-  for (uint32_t h0 = 0; h0 < nh; h0 += blockDim.x) {   // whole warps; a warp takes its keys' space with one addition
-    const uint32_t h = h0 + threadIdx.x;
-    const bool in = h < nh;
-    const uint32_t u = in ? __ldcg(a.hot_u + h) : 0u, est = in ? __ldcg(a.hinfo + u) << a.shift : 0u;
-    // the few keys that own a large share of the batch take one of SUPER_T slots
-    uint32_t ts = SUPER_T;
-    if (in && a.super_min && est >= a.super_min) ts = atomicAdd(a.hot_ctr + 3, 1u);
-    const bool sup = ts < SUPER_T;
-    uint32_t R = !in ? 0u : sup ? SUPER_R : (est + HOT_CHAIN(a.shift) - 1) / HOT_CHAIN(a.shift);
-    // (a key's chunk number has to fit a work item; longer chains only cost accuracy)
-    R = min(R, (1u << HOT_WORK_BITS) * HOT_RCHUNK);
-    const uint32_t nchunk = (R + HOT_RCHUNK - 1) / HOT_RCHUNK;
-    uint32_t base = R, wbase = nchunk;                 // inclusive sums over the warp, then where the key's space starts
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, base, d), y = __shfl_up_sync(0xFFFFFFFFu, wbase, d);
-      if (lane >= d) { base += x; wbase += y; }
-    }
-    uint32_t b0 = 0, w0 = 0;
-    if (lane == 31) { b0 = atomicAdd(a.hot_ctr + 1, base); w0 = atomicAdd(a.hot_ctr + HOT_CTR_WORK, wbase); }
-    base += __shfl_sync(0xFFFFFFFFu, b0, 31) - R;
-    wbase += __shfl_sync(0xFFFFFFFFu, w0, 31) - nchunk;
-    if (!in) continue;
-    const bool ok = base + R <= a.rep_max && wbase + nchunk <= a.work_max;   // nothing left: the key is treated as a cold one
-    for (uint32_t i = 0; i < nchunk && wbase + i < a.work_max; ++i) a.hot_work[wbase + i] = ok ? h << HOT_WORK_BITS | i : DES_ROW_NONE;
-    a.hot_rep[h] = make_uint2(base, ok ? R : 0u);
-    a.hinfo[u] = ok ? HOT_FLAG | (sup ? (ts + 1u) << 24 : 0u) | h : 0u;
-    if (sup) a.hot_ctr[HOT_CTR_SLOT + ts] = ok ? h : DES_ROW_NONE;
-  }
-}
-
 // Every occurrence that is not its key's first one takes the unique index — and, for a key that was new,
 // the row — from the first one (a look-up in the batch's own arrays, not in the table).  IB occurrences at a time per
 // block of IB / 4 threads: a thread's four look-ups are in flight together.  First occurrences are only read
 // here (assign_kernel wrote them), the others only written.  One more block ends the call: shard sizes advance, the
 // two-level counts are cleared for the next call, the scratch range is retired.
-template <bool COUNT>
 __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, int S, uint32_t max_nnz,
                                                          const uint32_t* __restrict__ first_of, uint32_t* rows, uint32_t* uidx,
-                                                         uint32_t* __restrict__ sup_cnt, int nsup_max, DevMeta* meta, CountArgs ca) {
-  __shared__ uint32_t s_key[COUNT ? CT_SLOTS : 1], s_cnt[COUNT ? CT_SLOTS : 1];
-  if (COUNT) count_begin(s_key, s_cnt);
-  des_pdl_wait(first_of, rows, uidx, sup_cnt, meta, ca.hinfo, ca.hot_u, ca.hot_ctr, ca.hot_rep);
+                                                         uint32_t* __restrict__ sup_cnt, int nsup_max, DevMeta* meta) {
+  des_pdl_wait(first_of, rows, uidx, sup_cnt, meta);
   if (blockIdx.x == gridDim.x - 1) {
     const int nsup = (ntiles + (int)SUP_TILES - 1) / (int)SUP_TILES;
     for (int i = threadIdx.x; i < nsup; i += IB / 4) sup_cnt[i] = 0u;
@@ -562,7 +467,6 @@ __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, in
     }
     return;
   }
-  __syncthreads();
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x - 1) {
     const int j0 = tile * IB + threadIdx.x;
     uint32_t f[4], r[4], u[4];
@@ -581,77 +485,165 @@ __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, in
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + q * (IB / 4);
       u[q] = DES_ROW_NONE;
-      if (f[q] != DES_ROW_NONE) {
-        if (COUNT || f[q] != (uint32_t)j) u[q] = uidx[f[q]];
-        if (f[q] != (uint32_t)j && r[q] == DES_ROW_NONE) { r[q] = rows[f[q]]; newrow[q] = true; }
+      if (f[q] != DES_ROW_NONE && f[q] != (uint32_t)j) {
+        u[q] = uidx[f[q]];
+        if (r[q] == DES_ROW_NONE) { r[q] = rows[f[q]]; newrow[q] = true; }
       }
-    }
-    if (COUNT && ca.shift) {                           // (positions past the end hold "no row")
-      const uint32_t pick = des_hash32((uint32_t)j0) & 3u;
-      count_one(ca, s_key, s_cnt, pick == 0 ? u[0] : pick == 1 ? u[1] : pick == 2 ? u[2] : u[3]);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + q * (IB / 4);
-      if (COUNT && ca.shift == 0) count_one(ca, s_key, s_cnt, u[q]);
-      if (j >= nnz) continue;
-      if (f[q] == (uint32_t)j) continue;
+      if (j >= nnz || f[q] == (uint32_t)j) continue;
       if (newrow[q]) rows[j] = r[q];                   // (every other row is in place since flag_count_kernel)
       uidx[j] = u[q];
     }
   }
-  if (COUNT) count_end(ca, s_key, s_cnt, gridDim.x - 1);
 }
 
-// The counts alone: of a large batch, or of one that find_or_insert did not see last.
-#define CK_THREADS 1024
-#define CK_PER 4
-__global__ void __launch_bounds__(CK_THREADS) count_kernel(const uint32_t* __restrict__ uidx, int nnz, CountArgs ca) {
-  __shared__ uint32_t s_key[CT_SLOTS], s_cnt[CT_SLOTS];
-  count_begin(s_key, s_cnt);
-  des_pdl_wait(uidx, ca.hinfo, ca.hot_u, ca.hot_ctr, ca.hot_rep);
-  __syncthreads();
-  uint32_t u[CK_PER];
+// ---- counting ------------------------------------------------------------------------------------------------------
+// hinfo[u] += occurrences of key u among a 1 / 2^shift sample.  A hot key would draw tens of thousands of atomics on one
+// word, which L2 serialises, so counts are merged per warp (lanes holding the same key), then per block in a small
+// shared-memory table keyed by a hash of the key (an entry taken by another key sends the count straight to memory), and
+// each block adds its table once.  The addition that takes a key over the threshold lists it; the block that
+// finishes last turns the list into replica rows, publishes its sizes and leaves the counters at zero.
+// Every backward counts its own batch, from the index array it is given: counts kept from find_or_insert would have to
+// be recognised by that array's address, which says nothing about what a captured graph or a copy has put there since.
+// (Against counts taken on the way by resolve_kernel a launch more: a 10 k-occurrence step 42.7 -> 40.3 us all the same, with the
+// shorter chains below, 0.21 M 135.9 -> 137.9, 32 M 4528 -> 4496, where two memsets went.)
+// What a small batch waits for here is a chain of dependent accesses, so as few of them as possible follow one another: a
+// block's table takes a key at one of CT_PROBES entries before a count goes straight to memory, all the entries that a
+// thread adds are in flight together, and the last block hands out replica rows by sums of its own.
+#define CT_SLOTS 1024
+#define CT_PROBES 4
+// counted whole up to CT_WHOLE occurrences, one in four up to CT_QUARTER, beyond that one in 16 to 64
+#define CT_WHOLE (1 << 17)
+#define CT_QUARTER (1 << 20)
+struct CountArgs {
+  uint32_t *hinfo, *hot_u, *hot_ctr;
+  uint2* hot_rep;
+  long long max_uniq;
+  int shift;
+  uint32_t* hot_work;
+  uint32_t work_max, hot_max, rep_max, super_min;                // super_min = 0: no key is counted instead of scattered
+};
+
+__device__ __forceinline__ void count_added(const CountArgs& a, uint32_t u, uint32_t old, uint32_t c) {
+  const uint32_t thr = HOT_MIN(a.shift) >> a.shift;
+  if (old < thr && old + c >= thr) {
+    const uint32_t h = atomicAdd(a.hot_ctr + HOT_CTR_LIST, 1u);
+    if (h < a.hot_max) a.hot_u[h] = u;
+  }
+}
+// whole warp; u = DES_ROW_NONE: nothing to count
+__device__ __forceinline__ void count_one(const CountArgs& a, uint32_t* s_key, uint32_t* s_cnt, uint32_t u) {
+  const bool ok = (long long)u < a.max_uniq;
+  const unsigned act = __ballot_sync(0xFFFFFFFFu, ok);
+  if (!ok) return;
+  const unsigned same = __match_any_sync(act, u);
+  if ((threadIdx.x & 31) != __ffs(same) - 1) return;
+  const uint32_t e = des_hash32(u), c = (uint32_t)__popc(same);
+  for (uint32_t p = 0; p < CT_PROBES; ++p) {
+    const uint32_t i = (e + p) & (CT_SLOTS - 1), old = atomicCAS(&s_key[i], DES_ROW_NONE, u);
+    if (old == DES_ROW_NONE || old == u) { atomicAdd(&s_cnt[i], c); return; }
+  }
+  count_added(a, u, atomicAdd(a.hinfo + u, c), c);
+}
+
+template <int T, int PER>
+__global__ void __launch_bounds__(T) count_kernel(const uint32_t* __restrict__ uidx, int nnz, CountArgs ca) {
+  __shared__ uint32_t s_key[CT_SLOTS], s_cnt[CT_SLOTS], s_rows, s_work, s_super;
+  __shared__ bool s_last;
+  constexpr int E = CT_SLOTS / T;
 #pragma unroll
-  for (int q = 0; q < CK_PER; ++q) {
-    const long long i = ((long long)blockIdx.x * CK_PER + q) * CK_THREADS + threadIdx.x;
+  for (int i = 0; i < E; ++i) { s_key[threadIdx.x + i * T] = DES_ROW_NONE; s_cnt[threadIdx.x + i * T] = 0u; }
+  if (threadIdx.x == 0) { s_rows = 0u; s_work = 0u; s_super = 0u; }
+  des_pdl_wait(uidx, ca.hinfo, ca.hot_u, ca.hot_ctr, ca.hot_rep, ca.hot_work);
+  uint32_t u[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const long long i = ((long long)blockIdx.x * PER + q) * T + threadIdx.x;
     const long long j = (i << ca.shift) + (des_hash32((uint32_t)i) & ((1u << ca.shift) - 1u));   // (shift 0: all)
     u[q] = j < nnz ? __ldg(uidx + j) : DES_ROW_NONE;
   }
+  __syncthreads();
 #pragma unroll
-  for (int q = 0; q < CK_PER; ++q) count_one(ca, s_key, s_cnt, u[q]);
-  count_end(ca, s_key, s_cnt, gridDim.x);
+  for (int q = 0; q < PER; ++q) count_one(ca, s_key, s_cnt, u[q]);
+  __syncthreads();
+  {
+    uint32_t old[E];
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      const uint32_t c = s_cnt[threadIdx.x + i * T];
+      old[i] = c ? atomicAdd(ca.hinfo + s_key[threadIdx.x + i * T], c) : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < E; ++i)
+      if (const uint32_t c = s_cnt[threadIdx.x + i * T]) count_added(ca, s_key[threadIdx.x + i * T], old[i], c);
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(ca.hot_ctr + HOT_CTR_TICKET, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // ---- the last block: replica rows for the listed keys
+  const uint32_t nh = min(__ldcg(ca.hot_ctr + HOT_CTR_LIST), ca.hot_max);
+  const int lane = threadIdx.x & 31;
+  for (uint32_t h0 = 0; h0 < nh; h0 += T) {            // whole warps; a warp takes its keys' space with one addition
+    const uint32_t h = h0 + threadIdx.x;
+    const bool in = h < nh;
+    const uint32_t u = in ? __ldcg(ca.hot_u + h) : 0u, est = in ? __ldcg(ca.hinfo + u) << ca.shift : 0u;
+    // the few keys that own a large share of the batch take one of SUPER_T slots
+    uint32_t ts = SUPER_T;
+    if (in && ca.super_min && est >= ca.super_min) ts = atomicAdd(&s_super, 1u);
+    const bool sup = ts < SUPER_T;
+    uint32_t R = !in ? 0u : sup ? SUPER_R : (est + HOT_CHAIN(ca.shift) - 1) / HOT_CHAIN(ca.shift);
+    // (a key's chunk number has to fit a work item; longer chains only cost accuracy)
+    R = min(R, (1u << HOT_WORK_BITS) * HOT_RCHUNK);
+    const uint32_t nchunk = (R + HOT_RCHUNK - 1) / HOT_RCHUNK;
+    uint32_t base = R, wbase = nchunk;                 // inclusive sums over the warp, then where the key's space starts
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, base, d), y = __shfl_up_sync(0xFFFFFFFFu, wbase, d);
+      if (lane >= d) { base += x; wbase += y; }
+    }
+    uint32_t b0 = 0, w0 = 0;
+    if (lane == 31) { b0 = atomicAdd(&s_rows, base); w0 = atomicAdd(&s_work, wbase); }
+    base += __shfl_sync(0xFFFFFFFFu, b0, 31) - R;
+    wbase += __shfl_sync(0xFFFFFFFFu, w0, 31) - nchunk;
+    if (!in) continue;
+    const bool ok = base + R <= ca.rep_max && wbase + nchunk <= ca.work_max;   // nothing left: the key is treated as a cold one
+    for (uint32_t i = 0; i < nchunk && wbase + i < ca.work_max; ++i) ca.hot_work[wbase + i] = ok ? h << HOT_WORK_BITS | i : DES_ROW_NONE;
+    ca.hot_rep[h] = make_uint2(base, ok ? R : 0u);
+    ca.hinfo[u] = ok ? HOT_FLAG | (sup ? (ts + 1u) << 24 : 0u) | h : 0u;
+    if (sup) ca.hot_ctr[HOT_N_SLOT + ts] = ok ? h : DES_ROW_NONE;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ca.hot_ctr[HOT_N_KEYS] = nh;
+    ca.hot_ctr[HOT_N_SUPER] = min(s_super, SUPER_T);
+    ca.hot_ctr[HOT_N_WORK] = min(s_work, ca.work_max);
+    ca.hot_ctr[HOT_CTR_LIST] = 0u;
+    ca.hot_ctr[HOT_CTR_TICKET] = 0u;
+  }
 }
 
-static CountArgs count_args(const des_table* t, const des_batch_t* b) {
+des_status_t des_count_batch(des_table* t, const des_batch_t* b, cudaStream_t cs) {
   CountArgs a;
   a.hinfo = t->hinfo; a.hot_u = t->hot_u; a.hot_ctr = t->hot_ctr; a.hot_rep = t->hot_rep;
   a.max_uniq = t->max_uniq; a.hot_max = t->hot_max; a.rep_max = t->rep_max;
   a.hot_work = t->hot_work; a.work_max = t->work_max;
   a.shift = 0;
   if (b->nnz > CT_WHOLE) a.shift = 2;
-  if (b->nnz > CT_INLINE) a.shift = 4;
+  if (b->nnz > CT_QUARTER) a.shift = 4;
   while (a.shift >= 4 && a.shift < 6 && (b->nnz >> a.shift) > (1 << 20)) ++a.shift;
   a.super_min = des_super_path(t, b) ? (uint32_t)(b->nnz >> 7) : 0u;
-  return a;
-}
-static void counted(des_table* t, const des_batch_t* b, const CountArgs& a) {
-  t->tag_uidx = b->uidx; t->tag_nnz = (long long)b->nnz; t->tag_super = a.super_min ? 1 : 0; t->tag_valid = 1;
-}
-
-des_status_t des_count_batch(des_table* t, const des_batch_t* b, cudaStream_t cs) {
-  if (b->nnz == 0) return DES_OK;
-  if (t->tag_valid && t->tag_uidx == (const void*)b->uidx && t->tag_nnz == (long long)b->nnz &&
-      t->tag_super == (des_super_path(t, b) ? 1 : 0))
-    return DES_OK;
-  const CountArgs a = count_args(t, b);
-  DES_CUDA(cudaMemsetAsync(t->hot_ctr, 0, HOT_CTR_WORDS * 4, cs));
-  DES_CUDA(cudaMemsetAsync(t->hinfo, 0, (size_t)t->max_uniq * 4, cs));
+  // small blocks as long as the chip holds them all at once; larger ones merge more before their atomics
   const int64_t n = (b->nnz >> a.shift) + 1;
-  des_launch(count_kernel, (unsigned)((n + CK_THREADS * CK_PER - 1) / (CK_THREADS * CK_PER)), CK_THREADS, 0, cs,
-             (const uint32_t*)b->uidx, (int)b->nnz, a);
+#define CK(T, PER) des_launch(count_kernel<T, PER>, (unsigned)((n + T * PER - 1) / (T * PER)), T, 0, cs, (const uint32_t*)b->uidx, (int)b->nnz, a)
+  if (n <= (int64_t)t->sm_count * 8 * 256 * 2) CK(256, 2); else CK(1024, 4);
+#undef CK
   DES_LAUNCH_CHECK(t, "count_kernel");
-  counted(t, b, a);
   return DES_OK;
 }
 
@@ -677,11 +669,7 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
              t->slots, t->meta, geom, t->slot_of, b->shards, b->rows);
   DES_LAUNCH_CHECK(t, "probe_claim_kernel");
   if (!insert) return DES_OK;
-  t->tag_valid = 0;
   uint32_t* first_of = t->uslot;
-  // a batch of up to CT_INLINE occurrences is counted on the way (a launch and two memsets less for the backward), a
-  // larger one when its backward asks for it
-  const CountArgs ca = count_args(t, b);
   des_launch(flag_count_kernel, ntiles, IB / 4, 0, cs, nnz, (int)t->S, t->slots, t->meta, t->slot_of, b->shards, t->flags,
              b->rows, first_of, t->blk_cnt, t->sup_cnt, (int)t->nblk_max, nsup_max, &t->meta->any_new);
   DES_LAUNCH_CHECK(t, "flag_count_kernel");
@@ -696,7 +684,7 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
         (int)t->S, t->meta, (const unsigned long long*)b->ids, b->shards, t->flags, t->blk_cnt, t->sup_cnt,               \
         (int)t->nblk_max, nsup_max, t->slot_of, b->rows, b->uidx, b->uniq_rows, b->n_uniq, t->slots, t->total_slots,     \
         (uint32_t)t->max_nnz, (int)t->k, (int)t->stride, t->W, t->A, t->A2, t->cfg.seed, t->cfg.init_scale, state_init,  \
-        lin_state_init, t->hinfo, (long long)(nnz <= CT_INLINE ? t->max_uniq : 0), t->hot_ctr)
+        lin_state_init)
 #define ASSIGN(GG) do { if (deep) ASSIGN2(GG, 8); else ASSIGN2(GG, 2); } while (0)
     switch (G) { case 1: ASSIGN(1); break; case 2: ASSIGN(2); break; case 4: ASSIGN(4); break; case 8: ASSIGN(8); break;
                  default: ASSIGN(16); }
@@ -704,11 +692,8 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
 #undef ASSIGN
     DES_LAUNCH_CHECK(t, "assign_kernel");
   }
-  const bool count = nnz <= CT_INLINE;
-  const int most = t->sm_count * 8, rblocks = count && ntiles > most ? most : ntiles;
-  des_launch(count ? resolve_kernel<true> : resolve_kernel<false>, rblocks + 1, IB / 4, 0, cs, nnz, ntiles, (int)t->S,
-             (uint32_t)t->max_nnz, first_of, b->rows, b->uidx, t->sup_cnt, nsup_max, t->meta, ca);
+  des_launch(resolve_kernel, ntiles + 1, IB / 4, 0, cs, nnz, ntiles, (int)t->S, (uint32_t)t->max_nnz, first_of, b->rows, b->uidx,
+             t->sup_cnt, nsup_max, t->meta);
   DES_LAUNCH_CHECK(t, "resolve_kernel");
-  if (count) counted(t, b, ca);
   return DES_OK;
 }

@@ -15,12 +15,15 @@
 // backward: a tagged occurrence carries SUPER_TAG | slot where other occurrences carry a gradient row number.
 #define SUPER_T 16u             // slots
 #define SUPER_TAG 0xFFFFFF00u   // tag | slot; DES_ROW_NONE (low byte 0xFF) is not a tag
-// Layout of the hot-key counter block (des_table::hot_ctr, 64 words):
-//   [0] keys listed  [1] replica rows  [2] ticket of the counting kernel's blocks  [3] super slots claimed
-//   [4 + t]   hot index of super slot t (DES_ROW_NONE: slot unused)  [HOT_CTR_WORK] work items of the replica sums
+// Layout of the hot-key counter block (des_table::hot_ctr): the counting kernel's own counters, zero between calls, ...
+#define HOT_CTR_LIST 0     // keys listed
+#define HOT_CTR_TICKET 1   // blocks that are through
+// ... and what it leaves for the rest of the backward
+#define HOT_N_KEYS 8       // hot keys
+#define HOT_N_SUPER 9      // super slots taken
+#define HOT_N_WORK 10      // work items of the replica sums
+#define HOT_N_SLOT 16      // + t: hot index of super slot t (DES_ROW_NONE: slot unused)
 #define HOT_CTR_WORDS 64
-#define HOT_CTR_SLOT 4
-#define HOT_CTR_WORK 32
 #define HOT_RCHUNK 16u     // replica rows of a work item (hot index << HOT_WORK_BITS | chunk)
 #define HOT_WORK_BITS 17
 // A key is hot from HOT_MIN occurrences on (estimated from a 1 / 2^shift sample: at least 8 of them) and gets one replica row per
@@ -28,8 +31,8 @@
 #define HOT_MIN(shift) ((shift) < 4 ? 128u : (shift) < 6 ? 256u : 512u)
 #define HOT_CHAIN(shift) ((shift) < 4 ? 128u : 256u)
 #define SUPER_R 64u        // replica rows of a super key (they only take one partial sum per lane group)
-// A batch-unique key's word (des_table::hinfo) once the batch is counted: below HOT_FLAG a sampled count (cold key);
-// else HOT_FLAG | (super slot + 1) << 24 | hot index.
+// A batch-unique key's word (des_table::hinfo) once the backward has counted the batch: below HOT_FLAG a sampled count
+// (cold key); else HOT_FLAG | (super slot + 1) << 24 | hot index.  The update clears it: zero between calls.
 #define HOT_FLAG 0x80000000u
 
 // One open-addressing slot: 16 bytes, read with a single vector load.
@@ -100,12 +103,10 @@ struct des_table {
   // backward workspace
   float* Gbuf;                       // [max_uniq + rep_max][stride]: per-unique gradient rows, then
                                      // hot-key replica rows; all zero between calls
-  uint32_t* hinfo;                   // [max_uniq] sampled count, or hot index (HOT_FLAG)
+  uint32_t* hinfo;                   // [max_uniq] sampled count, or hot index (HOT_FLAG); zero between calls
   uint32_t* dest;                    // [max_nnz] gradient row of each occurrence (or SUPER_TAG | slot), large batches
   float* x_sorted;                   // [max_nnz] forward routing: feature values in shard-major order
   float2* bag_tail;                  // [max_batch * F] single-gather forward: per-bag sums of (w x, |v|^2 x^2)
-  // which batch hinfo and the hot list belong to (the backward counts again when another batch comes)
-  const void* tag_uidx; long long tag_nnz; int tag_valid; int tag_super;
   uint32_t *hot_u, *hot_ctr;         // hot keys [hot_max] and their counters
   uint2* hot_rep;                    // [hot_max] (first replica row, replica rows) of a hot key
   uint32_t* hot_work;                // [work_max] work items of the replica sums
@@ -370,6 +371,5 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
                                  float* gE_work, int B, cudaStream_t st);
 // Whether the keys that own a large share of the batch are counted instead of scattered in the backward.
 bool des_super_path(const des_table* t, const des_batch_t* b);
-// Counts a batch's occurrences per unique key (a sample) and makes the hot list, for a backward whose batch is not the
-// one that find_or_insert counted last.
+// Counts a batch's occurrences per unique key (a sample of a large batch) and makes the hot list: opens a backward.
 des_status_t des_count_batch(des_table* t, const des_batch_t* b, cudaStream_t cs);
