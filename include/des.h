@@ -395,7 +395,9 @@ des_status_t des_table_write_state2(des_table_t* t, const uint32_t* d_global_row
  * call returns after synchronising.  Upstream gradients stay device resident
  * (they come from the rest of the model, which lives on the GPU).  d_pooled
  * [B][F*k] is device scratch/output for POOL.  Requires max_nnz/max_batch
- * workspace like the other calls. */
+ * workspace like the other calls.  A call that some part of the step would refuse
+ * (DES_ERR_INVALID_ARG) enqueues nothing, and no copy from or to the host buffers is in
+ * flight behind any error. */
 des_status_t des_step_host(des_table_t* t, uint32_t ops, int32_t batch, int64_t nnz,
                            const int32_t* h_offsets, const uint64_t* h_ids, const float* h_vals,
                            const des_grads_t* d_grads, float* d_pooled, float* d_Z,

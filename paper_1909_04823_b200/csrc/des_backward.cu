@@ -662,15 +662,20 @@ bool des_super_path(const des_table* t, const des_batch_t* b) {
   return group_for(t->k) == 16 && !b->vals && b->nnz >= (1 << 20) && t->super_cnt && b->nnz >= 8 * nbags;
 }
 
-extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const des_batch_t* b,
-                                            const des_outputs_t* out, const des_grads_t* gr, void* stream) {
-  des_status_t st = des_check_batch(t, b, 1);
-  if (st != DES_OK) return st;
+static des_status_t backward_args(const des_table* t, uint32_t ops, const des_outputs_t* out, const des_grads_t* gr) {
   if (!out || !gr || (ops & ~15u) || ops == 0) return DES_ERR_INVALID_ARG;
   if ((ops & DES_OP_LR) && !gr->gL) return DES_ERR_INVALID_ARG;
   if ((ops & DES_OP_FM) && (!gr->gF || !out->out_small)) return DES_ERR_INVALID_ARG;
   if ((ops & DES_OP_POOL) && !(ops & DES_OP_DENSE1) && !gr->gE) return DES_ERR_INVALID_ARG;
   if ((ops & DES_OP_DENSE1) && (!t->H || !gr->gZ || !gr->gE_work || !out->pooled)) return DES_ERR_INVALID_ARG;
+  return DES_OK;
+}
+
+extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const des_batch_t* b,
+                                            const des_outputs_t* out, const des_grads_t* gr, void* stream) {
+  des_status_t st = des_check_batch(t, b, 1);
+  if (st != DES_OK) return st;
+  if ((st = backward_args(t, ops, out, gr)) != DES_OK) return st;
   cudaStream_t cs = (cudaStream_t)stream;
   des_api_begin(t, cs);
   DES_DBG_ARM(t, cs);
@@ -763,6 +768,8 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
 }
 
 // ---- whole step from host buffers ---------------------------------------------
+#define ST_ASIDE (256u << 10)      // bytes of out_small from which its read-back runs beside the backward
+
 // Device staging of the host-buffer step, sized for the largest batch (first call: allocates, synchronises).
 // The batch inputs (offsets, ids, values) and the results have two slots so that the copies of one step can overlap
 // kernels; everything else the kernels produce is single (kernels of consecutive steps run
@@ -794,41 +801,57 @@ static des_status_t st_prepare(des_table* t) {
 // forward is the fused one in shard order: the same bits without writing them out (two steps of 2 M occurrences
 // 1680 -> 1452 us with the read-back below).  The read-back of out_small starts as soon as the forward has it and, from ST_ASIDE
 // bytes on, runs beside the backward (a copy of 4.4 MB held the kernels up for 80 us); `cs` waits for it at the end.
-#define ST_ASIDE (256u << 10)
-static des_status_t st_enqueue(des_table* t, int slot, cudaStream_t copy, uint32_t ops, int32_t batch, int64_t nnz,
-                               const int32_t* h_offsets, const uint64_t* h_ids, const float* h_vals,
-                               const des_grads_t* d_grads, float* d_pooled, float* d_Z, float* h_out_small,
-                               cudaStream_t cs) {
-  const size_t nb = (size_t)batch * t->F + 1;
+static des_status_t st_issue(des_table* t, int slot, cudaStream_t copy, uint32_t ops, const des_batch_t* b,
+                             const int32_t* h_offsets, const uint64_t* h_ids, const float* h_vals, const des_grads_t* d_grads,
+                             const des_outputs_t* o, float* h_out_small, cudaStream_t cs) {
+  const size_t nb = (size_t)b->batch * t->F + 1, nnz = (size_t)b->nnz;
   DES_CUDA(cudaMemcpyAsync(t->st_offsets[slot], h_offsets, nb * 4, cudaMemcpyHostToDevice, copy));
-  if (nnz) DES_CUDA(cudaMemcpyAsync(t->st_ids[slot], h_ids, (size_t)nnz * 8, cudaMemcpyHostToDevice, copy));
-  if (h_vals && nnz) DES_CUDA(cudaMemcpyAsync(t->st_vals[slot], h_vals, (size_t)nnz * 4, cudaMemcpyHostToDevice, copy));
+  if (nnz) DES_CUDA(cudaMemcpyAsync(t->st_ids[slot], h_ids, nnz * 8, cudaMemcpyHostToDevice, copy));
+  if (h_vals && nnz) DES_CUDA(cudaMemcpyAsync(t->st_vals[slot], h_vals, nnz * 4, cudaMemcpyHostToDevice, copy));
   if (copy != cs) {
     DES_CUDA(cudaEventRecord(t->st_copied[slot], copy));
     DES_CUDA(cudaStreamWaitEvent(cs, t->st_copied[slot], 0));
   }
-  des_batch_t b;
-  b.batch = batch; b.nnz = nnz; b.offsets = t->st_offsets[slot]; b.ids = (const uint64_t*)t->st_ids[slot];
-  b.vals = h_vals ? t->st_vals[slot] : nullptr; b.rows = t->st_rows; b.shards = t->st_shards; b.uidx = t->st_uidx;
-  b.uniq_rows = t->st_uniq_rows; b.n_uniq = t->st_n_uniq;
-  des_partials_t p; p.part_small = nullptr; p.pooled = d_pooled; p.part_pooled = nullptr; p.part_dense = nullptr;
-  des_outputs_t o; o.out_small = t->st_out_small[slot]; o.pooled = d_pooled; o.Z = d_Z;
-  const size_t out_bytes = (size_t)batch * t->stride * 4;
+  des_partials_t p; p.part_small = nullptr; p.pooled = o->pooled; p.part_pooled = nullptr; p.part_dense = nullptr;
+  const size_t out_bytes = (size_t)b->batch * t->stride * 4;
   const bool aside = out_bytes >= ST_ASIDE;
-  if (ops & ~15u) return DES_ERR_INVALID_ARG;
   des_status_t st;
-  if ((st = des_find_or_insert(t, &b, 1, cs)) != DES_OK) return st;
-  if ((st = des_forward_fused(t, ops | DES_FUSED_SHARD_ORDER, &b, &p, &o, cs)) != DES_OK) return st;
+  if ((st = des_find_or_insert(t, b, 1, cs)) != DES_OK) return st;
+  if ((st = des_forward_fused(t, ops | DES_FUSED_SHARD_ORDER, b, &p, o, cs)) != DES_OK) return st;
   if (aside) {
     DES_CUDA(cudaEventRecord(t->st_fwd[slot], cs));
     DES_CUDA(cudaStreamWaitEvent(t->st_out_stream, t->st_fwd[slot], 0));
     DES_CUDA(cudaMemcpyAsync(h_out_small, t->st_out_small[slot], out_bytes, cudaMemcpyDeviceToHost, t->st_out_stream));
     DES_CUDA(cudaEventRecord(t->st_out[slot], t->st_out_stream));
   }
-  if ((st = des_backward_update(t, ops, &b, &o, d_grads, cs)) != DES_OK) return st;
+  if ((st = des_backward_update(t, ops, b, o, d_grads, cs)) != DES_OK) return st;
   if (aside) DES_CUDA(cudaStreamWaitEvent(cs, t->st_out[slot], 0));
   else DES_CUDA(cudaMemcpyAsync(h_out_small, t->st_out_small[slot], out_bytes, cudaMemcpyDeviceToHost, cs));
   return DES_OK;
+}
+
+// Nothing is enqueued for a step whose arguments some call of it refuses; a step that fails on the way is waited for.  Either
+// way no copy to or from the caller's buffers is left in flight behind an error.
+static des_status_t st_enqueue(des_table* t, int slot, cudaStream_t copy, uint32_t ops, int32_t batch, int64_t nnz,
+                               const int32_t* h_offsets, const uint64_t* h_ids, const float* h_vals,
+                               const des_grads_t* d_grads, float* d_pooled, float* d_Z, float* h_out_small,
+                               cudaStream_t cs) {
+  des_batch_t b;
+  b.batch = batch; b.nnz = nnz; b.offsets = t->st_offsets[slot]; b.ids = (const uint64_t*)t->st_ids[slot];
+  b.vals = h_vals ? t->st_vals[slot] : nullptr; b.rows = t->st_rows; b.shards = t->st_shards; b.uidx = t->st_uidx;
+  b.uniq_rows = t->st_uniq_rows; b.n_uniq = t->st_n_uniq;
+  des_outputs_t o; o.out_small = t->st_out_small[slot]; o.pooled = d_pooled; o.Z = d_Z;
+  des_status_t st = backward_args(t, ops, &o, d_grads);
+  if (st != DES_OK) return st;
+  if ((ops & (DES_OP_POOL | DES_OP_DENSE1)) && !d_pooled) return DES_ERR_INVALID_ARG;
+  if ((ops & DES_OP_DENSE1) && !d_Z) return DES_ERR_INVALID_ARG;
+  if ((st = st_issue(t, slot, copy, ops, &b, h_offsets, h_ids, h_vals, d_grads, &o, h_out_small, cs)) != DES_OK) {
+    cudaStreamSynchronize(copy);
+    cudaStreamSynchronize(cs);
+    if (t->st_out_stream) cudaStreamSynchronize(t->st_out_stream);
+    cudaGetLastError();
+  }
+  return st;
 }
 
 static des_status_t st_check_args(des_table* t, int32_t batch, int64_t nnz, const int32_t* h_offsets,
