@@ -12,9 +12,9 @@
 //   starts + repair   linear probing must never meet a deleted slot, and there are no tombstones: the run of
 //             occupied slots around a removed key is put back in order by one thread.  Runs are disjoint
 //             and short (a handful of slots at load 0.5), so this costs per removed key, not per key of the table
-//             (emptying and refilling the shards' regions, which remains for a region without a single empty
-//             slot, took 107 us for 0.25 M of 1.25 M keys; this takes 25 us and its cost does not
-//             grow with the table).
+//             (emptying and refilling the shards' regions took 107 us for 0.25 M of 1.25 M keys; this takes 25 us and
+//             its cost does not grow with the table).  The regions are rebuilt where one has no empty slot, or holds
+//             keys without a row (their insert met a full shard), which an eviction drops.
 //   relabel   survivors that changed rows get their new row number (one pass over the slots, only when any did)
 // The host learns the outcome with one copy at the end; nothing in between waits for it, and the temporaries
 // stay with the table unless they are large (allocating and freeing them took 1.8 ms a call).
@@ -28,7 +28,8 @@ struct EvictCtl {                                      // zero at the start of a
   uint32_t gone[DES_MAX_SHARDS];                       // rows to go
   uint32_t pairs[DES_MAX_SHARDS];                      // rows that move
   uint32_t n_list;                                     // slots of keys to go
-  uint32_t owned[DES_MAX_SHARDS];                      // a run of the shard has found its start (see ev_full)
+  uint32_t owned[DES_MAX_SHARDS];                      // a run of the shard has found its start
+  uint32_t rebuild[DES_MAX_SHARDS];                    // there are keys without a row
   uint32_t any_pairs;
   uint32_t n_live;                                     // (rebuild only)
 };
@@ -58,11 +59,14 @@ __device__ __forceinline__ uint32_t ev_append(uint32_t* counter, bool want) {   
 }
 
 // A shard that loses keys has a run that starts behind an empty slot — unless its region has no empty slot at all.
+__host__ __device__ __forceinline__ bool ev_rebuilt(const EvictCtl* ctl, int s) {
+  return ctl->gone[s] && (!ctl->owned[s] || ctl->rebuild[s]);
+}
 // Whole block.
-__device__ __forceinline__ bool ev_full(const EvictCtl* ctl, int S) {
-  bool full = false;
-  for (int s = threadIdx.x; s < S; s += blockDim.x) full |= ctl->gone[s] && !ctl->owned[s];
-  return __syncthreads_or(full);
+__device__ __forceinline__ bool ev_any_rebuilt(const EvictCtl* ctl, int S) {
+  bool any = false;
+  for (int s = threadIdx.x; s < S; s += blockDim.x) any |= ev_rebuilt(ctl, s);
+  return __syncthreads_or(any);
 }
 
 // by list: one thread per key (HASH: the key's own shard; FIELD: thread (key, shard) looks in every shard)
@@ -224,7 +228,9 @@ __global__ void __launch_bounds__(256) evict_starts_kernel(const Slot* __restric
     const int s = shard_of_pos(meta->slot_base, S, cur);
     const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cap = hi - lo;
     uint32_t start = EV_NONE;
-    for (uint32_t step = 1; step < cap; ++step) {
+    const bool rebuild = meta->rowless[s];
+    if (rebuild && !ctl->rebuild[s]) ctl->rebuild[s] = 1u;
+    for (uint32_t step = 1; !rebuild && step < cap; ++step) {
       const uint32_t prev = cur == lo ? hi - 1 : cur - 1;
       const Slot sl = slots[prev];
       if (sl.key == DES_KEY_EMPTY) { start = cur; break; }
@@ -238,12 +244,11 @@ __global__ void __launch_bounds__(256) evict_starts_kernel(const Slot* __restric
 
 // Slots of a run are taken out one after the other and, unless removed, put back from their home slot: everything
 // between the home and the slot just emptied has been through this, so a key never lands behind where it was,
-// and the result is what inserting the survivors in that order gives.  Keys without a row (their insert
-// met a full shard) are dropped on the way.
+// and the result is what inserting the survivors in that order gives.
 __global__ void __launch_bounds__(128) evict_repair_kernel(Slot* slots, int S, const DevMeta* __restrict__ meta,
                                                           const uint32_t* __restrict__ bits, const uint32_t* __restrict__ starts,
                                                           const EvictCtl* ctl) {
-  if (ev_full(ctl, S)) return;
+  if (ev_any_rebuilt(ctl, S)) return;
   const uint32_t n = ctl->n_list;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     uint32_t cur = starts[i];
@@ -254,7 +259,7 @@ __global__ void __launch_bounds__(128) evict_repair_kernel(Slot* slots, int S, c
     for (uint32_t step = 0; step < cap; ++step) {
       const Slot sl = slots[cur];
       if (sl.key == DES_KEY_EMPTY) break;               // the run's end
-      if (sl.row == DES_ROW_NONE || ev_gone(bits, meta, s, sl.row)) {
+      if (ev_gone(bits, meta, s, sl.row)) {
         slots[cur] = empty;
       } else {
         uint32_t at = des_slot_home(des_mix64(sl.key), lo, cap);
@@ -270,7 +275,7 @@ __global__ void __launch_bounds__(128) evict_repair_kernel(Slot* slots, int S, c
 __global__ void __launch_bounds__(256) evict_relabel_kernel(Slot* slots, unsigned long long total_slots, int S,
                                                            const DevMeta* __restrict__ meta, const EvictCtl* ctl,
                                                            const uint32_t* __restrict__ holes, const uint32_t* __restrict__ movers) {
-  if (!ctl->any_pairs || ev_full(ctl, S)) return;
+  if (!ctl->any_pairs || ev_any_rebuilt(ctl, S)) return;
   __shared__ unsigned long long off[DES_MAX_SHARDS];
   for (int s = threadIdx.x; s < S; s += blockDim.x) off[s] = ev_list_off(meta, ctl, s);
   __syncthreads();
@@ -289,11 +294,14 @@ __global__ void __launch_bounds__(256) evict_relabel_kernel(Slot* slots, unsigne
 }
 
 __global__ void evict_finish_kernel(DevMeta* meta, const EvictCtl* ctl, int S) {
-  if ((int)threadIdx.x < S) meta->n_rows[threadIdx.x] -= ctl->gone[threadIdx.x];
+  const int s = threadIdx.x;
+  if (s >= S) return;
+  meta->n_rows[s] -= ctl->gone[s];
+  if (ctl->rebuild[s]) meta->rowless[s] = 0u;
 }
 
-// A region without a single empty slot (only keys whose insert failed can fill it up): the survivors of the shards
-// that lose a key are collected, the regions emptied, the survivors put back.  Runs before evict_finish_kernel.
+// Rebuild: the survivors of the shards that lose a key are collected, the regions emptied, the survivors put back.  Runs
+// before evict_finish_kernel.
 __global__ void __launch_bounds__(256) evict_collect_kernel(const Slot* __restrict__ slots, unsigned long long total_slots,
                                                             int S, const DevMeta* __restrict__ meta, EvictCtl* ctl,
                                                             const uint32_t* __restrict__ bits, const uint32_t* __restrict__ holes,
@@ -412,7 +420,7 @@ static des_status_t evict_run(des_table_t* t, const uint64_t* d_keys, int64_t n,
   EvictCtl h;
   EV_CUDA(cudaMemcpy(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost));
   bool full = false;
-  for (int s = 0; s < S; ++s) full |= h.gone[s] && !h.owned[s];
+  for (int s = 0; s < S; ++s) full |= ev_rebuilt(&h, s);
   if (full) {
     EV_CUDA(cudaMalloc(&live, (t->total_rows + 1) * sizeof(LiveKey)));
     evict_collect_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl, bits, holes, movers, live);

@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
         if (i < hi && (same >> lane) == 1u) n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
         if (pass == 1 && i < hi) {
           uint32_t local = n_base[key] + at + __popc(same & ((1u << lane) - 1u));
-          if (local >= s_cap[key]) { local = DES_ROW_NONE; des_raise(meta, DES_ERR_CAPACITY); }
+          if (local >= s_cap[key]) { local = DES_ROW_NONE; meta->rowless[key] = 1u; des_raise(meta, DES_ERR_CAPACITY); }
           const int j = jb + l_off[i];
           const uint32_t uu = l_grow[i];
           const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : s_row[key] + local;

@@ -59,6 +59,7 @@ struct DevMeta {
   uint32_t n_rows[DES_MAX_SHARDS];                   // rows in use
   uint32_t n_uniq;                                   // unique keys of the running insert call
   uint32_t err;                                      // sticky des_status_t raised on device
+  uint32_t rowless[DES_MAX_SHARDS];                  // the shard has been full: slots may hold keys without a row
   uint32_t any_new;                                  // the running insert call has at least one new key
   uint32_t scratch_base;                             // see Slot::first_occ: the last insert call's base
   uint32_t field_order[1024];                        // fields sorted by (owning shard, field)
