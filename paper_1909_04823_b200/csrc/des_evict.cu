@@ -13,8 +13,10 @@
 //             occupied slots around a removed key is put back in order by one thread.  Runs are disjoint
 //             and short (a handful of slots at load 0.5), so this costs per removed key, not per key of the table
 //             (emptying and refilling the shards' regions took 107 us for 0.25 M of 1.25 M keys; this takes 25 us and
-//             its cost does not grow with the table).  The regions are rebuilt where one has no empty slot, or holds
-//             keys without a row (their insert met a full shard), which an eviction drops.
+//             its cost does not grow with the table).  The regions are rebuilt (all threads take part) where one has
+//             a run of more than EV_RUN slots around a removed key, which one thread would walk and probe for
+//             milliseconds, where one has no empty slot, and where one holds keys without a row (their insert met a
+//             full shard), which an eviction drops.
 //   relabel   survivors that changed rows get their new row number (one pass over the slots, only when any did)
 // The host learns the outcome with one copy at the end; nothing in between waits for it, and the temporaries
 // stay with the table unless they are large (allocating and freeing them took 1.8 ms a call).
@@ -23,13 +25,18 @@
 
 #define EV_NONE 0xFFFFFFFFu
 #define EV_KEEP_BYTES (64ull << 20)                    // temporaries up to this size stay allocated with the table
+#ifdef DES_DEBUG
+#define EV_RUN 64u                                     // (checking build: small tables get there)
+#else
+#define EV_RUN 2048u                                   // slots of the longest run that one thread repairs
+#endif
 
 struct EvictCtl {                                      // zero at the start of a call
   uint32_t gone[DES_MAX_SHARDS];                       // rows to go
   uint32_t pairs[DES_MAX_SHARDS];                      // rows that move
   uint32_t n_list;                                     // slots of keys to go
   uint32_t owned[DES_MAX_SHARDS];                      // a run of the shard has found its start
-  uint32_t rebuild[DES_MAX_SHARDS];                    // there are keys without a row
+  uint32_t rebuild[DES_MAX_SHARDS];                    // a run is too long, or there are keys without a row
   uint32_t any_pairs;
   uint32_t n_live;                                     // (rebuild only)
 };
@@ -227,17 +234,24 @@ __global__ void __launch_bounds__(256) evict_starts_kernel(const Slot* __restric
     uint32_t cur = list[i];
     const int s = shard_of_pos(meta->slot_base, S, cur);
     const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cap = hi - lo;
-    uint32_t start = EV_NONE;
-    const bool rebuild = meta->rowless[s];
-    if (rebuild && !ctl->rebuild[s]) ctl->rebuild[s] = 1u;
-    for (uint32_t step = 1; !rebuild && step < cap; ++step) {
+    uint32_t start = EV_NONE, len = 1;
+    bool rebuild = meta->rowless[s];
+    while (!rebuild && len < cap) {                     // back to the run's start
       const uint32_t prev = cur == lo ? hi - 1 : cur - 1;
       const Slot sl = slots[prev];
       if (sl.key == DES_KEY_EMPTY) { start = cur; break; }
       if (sl.row != DES_ROW_NONE && ev_gone(bits, meta, s, sl.row)) break;
       cur = prev;
+      rebuild = ++len > EV_RUN;
     }
-    starts[i] = start;
+    cur = list[i];
+    while (!rebuild && start != EV_NONE) {              // on to its end: an empty slot, at the latest the one before the start
+      cur = cur + 1 == hi ? lo : cur + 1;
+      if (slots[cur].key == DES_KEY_EMPTY) break;
+      rebuild = ++len > EV_RUN;
+    }
+    starts[i] = rebuild ? EV_NONE : start;
+    if (rebuild && !ctl->rebuild[s]) ctl->rebuild[s] = 1u;
     if (start != EV_NONE && !ctl->owned[s]) ctl->owned[s] = 1u;
   }
 }

@@ -1,4 +1,5 @@
-"""Evictions whose shards are rebuilt instead of repaired run by run: keys without a row (their insert met a full shard)."""
+"""Evictions whose shards are rebuilt instead of repaired run by run: runs of occupied slots too long for one thread, and keys
+without a row (their insert met a full shard)."""
 import pytest
 import torch
 
@@ -26,6 +27,35 @@ def _check(D, t, ids, gone, found0, emb0):
     for s, m in enumerate(t.size()):
         mine = rows[found][(rows[found] >= base[s]) & (rows[found] < base[s + 1])] - base[s]
         assert torch.equal(torch.sort(mine).values, torch.arange(m, device="cuda", dtype=mine.dtype))
+
+
+# full at load 0.9 a region of 200 k slots has runs of a thousand and more, one of 2 k some of hundreds.  In the checking build a
+# run of 64 slots is a long one: all shards of the first cases are rebuilt, some of the last one
+@pytest.mark.parametrize("shards,rows,load", [(1, 200_000, 0.9), (3, 60_000, 0.9), (8, 1800, 0.9), (40, 1500, 0.6)])
+@pytest.mark.parametrize("share", [0.0005, 0.2])
+@pytest.mark.parametrize("checking", [False, True])
+def test_long_runs(shards, rows, load, share, checking):
+    from paper_1909_04823_b200 import binding as D
+    n = shards * rows
+    prev = D.use_debug_library(checking)
+    try:
+        t = _table(D, shards, rows, load, n)
+    finally:
+        D.use_debug_library(prev)
+    try:
+        ids = _some_ids(n, n - 3 * shards * int(rows ** 0.5) if shards > 1 else n)
+        t.find_or_insert(_batch(D, ids))
+        assert t.status() == 0
+        found0, emb0, _ = _contents(D, t, ids)
+        assert bool(found0.all())
+        gone = torch.zeros(ids.numel(), dtype=torch.bool, device="cuda")
+        gone[torch.randperm(ids.numel(), device="cuda")[:max(1, int(ids.numel() * share))]] = True
+        assert t.evict_keys(ids[gone]) == int(gone.sum())
+        _check(D, t, ids, gone, found0, emb0)
+        t.find_or_insert(_batch(D, ids))                   # back in, as new keys
+        assert t.status() == 0 and bool(_contents(D, t, ids)[0].all())
+    finally:
+        t.close()
 
 
 @pytest.mark.parametrize("seed", range(6))
