@@ -370,8 +370,10 @@ des_status_t des_table_write_rows(des_table_t* t, const uint32_t* d_global_rows,
  * *h_n_evicted (optional) = number of rows removed.  Maintenance calls: they synchronise the
  * device and take temporaries with cudaMalloc (16 bytes per key to remove — evict_keys under
  * DES_PART_FIELD: per key and shard; evict_stale: per table row — and a bit per table row).  Up to
- * 64 MiB of them stay with the table for its next eviction, more are freed before returning.  Not for use inside a
- * stream capture.  Errors: DES_ERR_INVALID_ARG, DES_ERR_CUDA (also: out of memory). */
+ * 64 MiB of them stay with the table for its next eviction, more are freed before returning.  A shard that loses keys is
+ * rebuilt, with 16 more bytes per row of its capacity, when its slots hold keys that found no row, when none of them is empty or
+ * when a run of more than 2048 occupied ones has to be repaired.  Out of memory the table is unchanged.  Not for use inside
+ * a stream capture.  Errors: DES_ERR_INVALID_ARG, DES_ERR_CUDA (also: out of memory). */
 des_status_t des_table_evict_keys(des_table_t* t, const uint64_t* d_keys, int64_t n, uint64_t* h_n_evicted);
 des_status_t des_table_evict_stale(des_table_t* t, uint64_t min_clock, uint64_t* h_n_evicted);
 des_status_t des_table_clock(des_table_t* t, uint64_t* h_clock);

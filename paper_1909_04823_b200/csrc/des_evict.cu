@@ -6,21 +6,25 @@
 // A maintenance operation, not part of the training step: it synchronises on entry and once at the end.
 //   mark      a bit per row to go (by probing the listed keys, or by comparing age stamps), the counts per
 //             shard, and the list of the slots concerned
+//   starts    for every removed key, the start of the run of occupied slots it lies in; shards that need a rebuild
 //   pair      the freed rows below a shard's new size m (ascending) are paired with the surviving rows at or
 //             beyond m (ascending): one block per shard walks the shard's bits in order
 //   move      the surviving row's weights and state are copied into the freed row
-//   starts + repair   linear probing must never meet a deleted slot, and there are no tombstones: the run of
+//   repair    linear probing must never meet a deleted slot, and there are no tombstones: the run of
 //             occupied slots around a removed key is put back in order by one thread.  Runs are disjoint
 //             and short (a handful of slots at load 0.5), so this costs per removed key, not per key of the table
 //             (emptying and refilling the shards' regions took 107 us for 0.25 M of 1.25 M keys; this takes 25 us and
-//             its cost does not grow with the table).  The regions are rebuilt (all threads take part) where one has
-//             a run of more than EV_RUN slots around a removed key, which one thread would walk and probe for
-//             milliseconds, where one has no empty slot, and where one holds keys without a row (their insert met a
-//             full shard), which an eviction drops.
+//             its cost does not grow with the table).
 //   relabel   survivors that changed rows get their new row number (one pass over the slots, only when any did)
+// A shard whose region is rebuilt instead (all threads take part: collected, emptied, put back): one with a run of more than
+// EV_RUN slots around a removed key, which one thread would walk and probe for milliseconds; one without an empty slot;
+// and one that holds keys without a row (their insert met a full shard), which an eviction drops.
 // The host learns the outcome with one copy at the end; nothing in between waits for it, and the temporaries
-// stay with the table unless they are large (allocating and freeing them took 1.8 ms a call).
+// stay with the table unless they are large (allocating and freeing them took 1.8 ms a call).  Only where a shard is rebuilt
+// nothing is changed before that copy, so that the memory for it is there before the first row moves.
 // Every loop is bounded (probes by the region size); a full region raises the sticky status word.
+#include <cstdlib>
+
 #include "des_internal.cuh"
 
 #define EV_NONE 0xFFFFFFFFu
@@ -69,10 +73,11 @@ __device__ __forceinline__ uint32_t ev_append(uint32_t* counter, bool want) {   
 __host__ __device__ __forceinline__ bool ev_rebuilt(const EvictCtl* ctl, int s) {
   return ctl->gone[s] && (!ctl->owned[s] || ctl->rebuild[s]);
 }
-// Whole block.
-__device__ __forceinline__ bool ev_any_rebuilt(const EvictCtl* ctl, int S) {
+// The kernels that change the table are launched once, and again (`planned`) when the host has seen that a shard is to
+// be rebuilt: the first time they then do nothing.  Whole block.
+__device__ __forceinline__ bool ev_wait(const EvictCtl* ctl, int S, int planned) {
   bool any = false;
-  for (int s = threadIdx.x; s < S; s += blockDim.x) any |= ev_rebuilt(ctl, s);
+  if (!planned) for (int s = threadIdx.x; s < S; s += blockDim.x) any |= ev_rebuilt(ctl, s);
   return __syncthreads_or(any);
 }
 
@@ -209,7 +214,8 @@ __global__ void __launch_bounds__(1024) evict_pair_kernel(const uint32_t* __rest
 // one warp per pair: the surviving row's weights and state move into the freed row
 __global__ void __launch_bounds__(256) evict_move_kernel(const DevMeta* __restrict__ meta, const EvictCtl* ctl,
                                                          const uint32_t* __restrict__ holes, const uint32_t* __restrict__ movers,
-                                                         int stride, float* W, float* A, float* A2) {
+                                                         int S, int planned, int stride, float* W, float* A, float* A2) {
+  if (ev_wait(ctl, S, planned)) return;
   const int s = blockIdx.y, lane = threadIdx.x & 31;
   const uint32_t np = ctl->pairs[s];
   if (np == 0) return;
@@ -261,13 +267,14 @@ __global__ void __launch_bounds__(256) evict_starts_kernel(const Slot* __restric
 // and the result is what inserting the survivors in that order gives.
 __global__ void __launch_bounds__(128) evict_repair_kernel(Slot* slots, int S, const DevMeta* __restrict__ meta,
                                                           const uint32_t* __restrict__ bits, const uint32_t* __restrict__ starts,
-                                                          const EvictCtl* ctl) {
-  if (ev_any_rebuilt(ctl, S)) return;
+                                                          const EvictCtl* ctl, int planned) {
+  if (ev_wait(ctl, S, planned)) return;
   const uint32_t n = ctl->n_list;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     uint32_t cur = starts[i];
     if (cur == EV_NONE) continue;
     const int s = shard_of_pos(meta->slot_base, S, cur);
+    if (ev_rebuilt(ctl, s)) continue;
     const uint32_t lo = (uint32_t)meta->slot_base[s], hi = (uint32_t)meta->slot_base[s + 1], cap = hi - lo;
     Slot empty; empty.key = DES_KEY_EMPTY; empty.row = DES_ROW_NONE; empty.first_occ = DES_ROW_NONE;
     for (uint32_t step = 0; step < cap; ++step) {
@@ -288,8 +295,9 @@ __global__ void __launch_bounds__(128) evict_repair_kernel(Slot* slots, int S, c
 // survivors that changed rows
 __global__ void __launch_bounds__(256) evict_relabel_kernel(Slot* slots, unsigned long long total_slots, int S,
                                                            const DevMeta* __restrict__ meta, const EvictCtl* ctl,
-                                                           const uint32_t* __restrict__ holes, const uint32_t* __restrict__ movers) {
-  if (!ctl->any_pairs || ev_any_rebuilt(ctl, S)) return;
+                                                           const uint32_t* __restrict__ holes, const uint32_t* __restrict__ movers,
+                                                           int planned) {
+  if (!ctl->any_pairs || ev_wait(ctl, S, planned)) return;
   __shared__ unsigned long long off[DES_MAX_SHARDS];
   for (int s = threadIdx.x; s < S; s += blockDim.x) off[s] = ev_list_off(meta, ctl, s);
   __syncthreads();
@@ -299,7 +307,7 @@ __global__ void __launch_bounds__(256) evict_relabel_kernel(Slot* slots, unsigne
     const Slot sl = slots[i];
     if (sl.key == DES_KEY_EMPTY || sl.row == DES_ROW_NONE) continue;
     const int s = shard_of_pos(meta->slot_base, S, i);
-    if (sl.row < meta->n_rows[s] - ctl->gone[s] || !ctl->pairs[s]) continue;
+    if (sl.row < meta->n_rows[s] - ctl->gone[s] || !ctl->pairs[s] || ev_rebuilt(ctl, s)) continue;
     const uint32_t* mv = movers + off[s];
     uint32_t a = 0, b = ctl->pairs[s];                  // mv[a] <= row < mv[b]: the row is in the list
     while (b - a > 1) { const uint32_t mid = (a + b) >> 1; if (mv[mid] <= sl.row) a = mid; else b = mid; }
@@ -311,11 +319,10 @@ __global__ void evict_finish_kernel(DevMeta* meta, const EvictCtl* ctl, int S) {
   const int s = threadIdx.x;
   if (s >= S) return;
   meta->n_rows[s] -= ctl->gone[s];
-  if (ctl->rebuild[s]) meta->rowless[s] = 0u;
+  if (ev_rebuilt(ctl, s)) meta->rowless[s] = 0u;
 }
 
-// Rebuild: the survivors of the shards that lose a key are collected, the regions emptied, the survivors put back.  Runs
-// before evict_finish_kernel.
+// Rebuilt shards: the survivors are collected, the regions emptied, the survivors put back.  Runs before evict_finish_kernel.
 __global__ void __launch_bounds__(256) evict_collect_kernel(const Slot* __restrict__ slots, unsigned long long total_slots,
                                                             int S, const DevMeta* __restrict__ meta, EvictCtl* ctl,
                                                             const uint32_t* __restrict__ bits, const uint32_t* __restrict__ holes,
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(256) evict_collect_kernel(const Slot* __restri
   const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
   for (; i < total_slots; i += st) {
     const int s = shard_of_pos(meta->slot_base, S, i);
-    if (ctl->gone[s] == 0) continue;
+    if (!ev_rebuilt(ctl, s)) continue;
     const Slot sl = slots[i];
     if (sl.key == DES_KEY_EMPTY || sl.row == DES_ROW_NONE || ev_gone(bits, meta, s, sl.row)) continue;
     LiveKey lk; lk.key = sl.key; lk.row = sl.row; lk.shard = (uint32_t)s;
@@ -343,7 +350,7 @@ __global__ void __launch_bounds__(256) evict_clear_kernel(Slot* slots, unsigned 
   unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned long long st = (unsigned long long)gridDim.x * blockDim.x;
   for (; i < total_slots; i += st) {
-    if (ctl->gone[shard_of_pos(meta->slot_base, S, i)] == 0) continue;
+    if (!ev_rebuilt(ctl, shard_of_pos(meta->slot_base, S, i))) continue;
     Slot e; e.key = DES_KEY_EMPTY; e.row = DES_ROW_NONE; e.first_occ = DES_ROW_NONE;
     slots[i] = e;
   }
@@ -366,6 +373,14 @@ __global__ void __launch_bounds__(256) evict_reinsert_kernel(Slot* slots, DevMet
     }
     if (!placed) des_raise(meta, DES_ERR_CAPACITY);      // cannot happen: the region held these keys before
   }
+}
+
+static bool ev_no_memory() {
+#ifdef DES_DEBUG
+  return getenv("DES_DEBUG_EVICT_NO_MEMORY") != nullptr;   // checking build only: the memory for a rebuild is not to be had
+#else
+  return false;
+#endif
 }
 
 static des_status_t evict_run(des_table_t* t, const uint64_t* d_keys, int64_t n, uint64_t min_clock, int by_age,
@@ -420,23 +435,29 @@ static des_status_t evict_run(des_table_t* t, const uint64_t* d_keys, int64_t n,
                                                                       (int)t->cfg.partition, M, two32, t->slots, t->meta, bits, list, ctl);
     EV_LAUNCH("evict_mark_keys_kernel");
   }
-  evict_pair_kernel<<<S, 1024>>>(bits, t->meta, ctl, holes, movers);
-  EV_LAUNCH("evict_pair_kernel");
-  evict_move_kernel<<<dim3((unsigned)((t->sm_count * 8 + S - 1) / S), (unsigned)S), 256>>>(t->meta, ctl, holes, movers,
-                                                                                         (int)t->stride, t->W, t->A, t->A2);
-  EV_LAUNCH("evict_move_kernel");
   evict_starts_kernel<<<wide, 256>>>(t->slots, S, t->meta, bits, list, starts, ctl);
   EV_LAUNCH("evict_starts_kernel");
-  evict_repair_kernel<<<wide * 2, 128>>>(t->slots, S, t->meta, bits, starts, ctl);
-  EV_LAUNCH("evict_repair_kernel");
-  evict_relabel_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl, holes, movers);
-  EV_LAUNCH("evict_relabel_kernel");
+  evict_pair_kernel<<<S, 1024>>>(bits, t->meta, ctl, holes, movers);
+  EV_LAUNCH("evict_pair_kernel");
+  auto change = [&](int planned) {
+    evict_move_kernel<<<dim3((unsigned)((t->sm_count * 8 + S - 1) / S), (unsigned)S), 256>>>(t->meta, ctl, holes, movers, S, planned,
+                                                                                           (int)t->stride, t->W, t->A, t->A2);
+    if (des_prof_mark(t, "evict_move_kernel", 1)) return false;
+    evict_repair_kernel<<<wide * 2, 128>>>(t->slots, S, t->meta, bits, starts, ctl, planned);
+    if (des_prof_mark(t, "evict_repair_kernel", 1)) return false;
+    evict_relabel_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl, holes, movers, planned);
+    return !des_prof_mark(t, "evict_relabel_kernel", 1);
+  };
+  if (!change(0)) return bail(DES_ERR_CUDA);
   EvictCtl h;
   EV_CUDA(cudaMemcpy(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost));
-  bool full = false;
-  for (int s = 0; s < S; ++s) full |= ev_rebuilt(&h, s);
-  if (full) {
-    EV_CUDA(cudaMalloc(&live, (t->total_rows + 1) * sizeof(LiveKey)));
+  uint64_t n_live = 0;                                 // rows of the shards to rebuild
+  bool rebuild = false;
+  for (int s = 0; s < S; ++s)
+    if (ev_rebuilt(&h, s)) { rebuild = true; n_live += t->h_row_base[s + 1] - t->h_row_base[s]; }
+  if (rebuild) {
+    if (ev_no_memory() || cudaMalloc(&live, n_live * sizeof(LiveKey)) != cudaSuccess) { live = nullptr; return bail(DES_ERR_CUDA); }
+    if (!change(1)) return bail(DES_ERR_CUDA);
     evict_collect_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl, bits, holes, movers, live);
     EV_LAUNCH("evict_collect_kernel");
     evict_clear_kernel<<<wide, 256>>>(t->slots, t->total_slots, S, t->meta, ctl);

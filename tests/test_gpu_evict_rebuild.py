@@ -1,5 +1,5 @@
-"""Evictions whose shards are rebuilt instead of repaired run by run: runs of occupied slots too long for one thread, and keys
-without a row (their insert met a full shard)."""
+"""Evictions whose shards are rebuilt instead of repaired run by run: runs of occupied slots too long for one thread, keys without
+a row (their insert met a full shard), and a rebuild whose memory is not to be had."""
 import pytest
 import torch
 
@@ -78,3 +78,29 @@ def test_keys_without_a_row_are_dropped(seed):
         assert bool(found[0]) and int(found.sum()) == 1 and int(rows[0]) == 199
     finally:
         t.close()
+
+
+def test_no_memory_for_a_rebuild_changes_nothing(monkeypatch):
+    from paper_1909_04823_b200 import binding as D
+    prev = D.use_debug_library(True)
+    try:
+        t = _table(D, 2, 300, 0.5, 2048)
+        try:
+            ids = _some_ids(1, 900)
+            t.find_or_insert(_batch(D, ids))               # about 450 keys a shard for 300 rows
+            assert t.status() == 3 and t.size() == [300, 300]
+            found0, emb0, rows0 = _contents(D, t, ids)
+            gone = torch.zeros(900, dtype=torch.bool, device="cuda")
+            gone[torch.nonzero(found0)[::3, 0]] = True
+            monkeypatch.setenv("DES_DEBUG_EVICT_NO_MEMORY", "1")
+            with pytest.raises(D.DesError):
+                t.evict_keys(ids[gone])
+            found, emb, rows = _contents(D, t, ids)
+            assert torch.equal(found, found0) and torch.equal(emb, emb0) and torch.equal(rows, rows0) and t.size() == [300, 300]
+            monkeypatch.delenv("DES_DEBUG_EVICT_NO_MEMORY")
+            assert t.evict_keys(ids[gone]) == int(gone.sum())
+            _check(D, t, ids, gone, found0, emb0)
+        finally:
+            t.close()
+    finally:
+        D.use_debug_library(prev)
