@@ -67,6 +67,12 @@ const at::Tensor& tensor_of(PyObject* o) {
   return THPVariable_Unpack(o);
 }
 
+const at::Tensor& matrix_of(PyObject* o) {              // as `B, d = x.shape` has it
+  const at::Tensor& x = tensor_of(o);
+  if (x.dim() != 2) { PyErr_Format(PyExc_ValueError, "expected a matrix, got %lld dimension(s)", (long long)x.dim()); throw BadArgs(); }
+  return x;
+}
+
 template <typename T>
 T* ptr(PyObject* o) { return o == Py_None ? nullptr : (T*)tensor_of(o).data_ptr(); }
 
@@ -328,7 +334,7 @@ PyObject* py_dense1_get(PyObject* const* a, Py_ssize_t n) {
 PyObject* py_cross_forward(PyObject* const* a, Py_ssize_t n) {
   need(n, 7);
   Lib* l = lib_of(a[0]);
-  const at::Tensor& x = tensor_of(a[2]);
+  const at::Tensor& x = matrix_of(a[2]);
   const int64_t B = x.size(0), d = x.size(1), S = as_int(a[5]);
   const auto opt = at::TensorOptions().dtype(at::kFloat).device(x.device());
   at::Tensor y = at::empty_like(x), P = at::empty({B}, opt), part;
@@ -345,7 +351,7 @@ PyObject* py_cross_forward(PyObject* const* a, Py_ssize_t n) {
 PyObject* py_cross_backward(PyObject* const* a, Py_ssize_t n) {
   need(n, 6);
   Lib* l = lib_of(a[0]);
-  const at::Tensor& x = tensor_of(a[2]);
+  const at::Tensor& x = matrix_of(a[2]);
   const int64_t B = x.size(0), d = x.size(1);
   const auto opt = at::TensorOptions().dtype(at::kFloat).device(x.device());
   at::Tensor gx0 = at::empty_like(x), gx = at::empty_like(x), gw = at::empty({d}, opt), gb = at::empty({d}, opt);
