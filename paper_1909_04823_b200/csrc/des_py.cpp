@@ -9,6 +9,7 @@
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
 #include <dlfcn.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "des.h"
@@ -126,11 +127,10 @@ PyObject* status(F&& call) {                           // runs without the inter
 template <PyObject* (*F)(PyObject* const*, Py_ssize_t)>
 PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t n) {
   try {
+    HANDLE_TH_ERRORS                                   // (torch's exceptions keep their types: torch.OutOfMemoryError, ...)
     return F(a, n);
+    END_HANDLE_TH_ERRORS
   } catch (const BadArgs&) {
-    return nullptr;
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
     return nullptr;
   }
 }
@@ -164,6 +164,7 @@ PyObject* py_find_or_insert(PyObject* const* a, Py_ssize_t n) {
   des_table_t* t = table_of(a[1]);
   const des_batch_t b = batch_of(a[2]);
   const int insert = PyObject_IsTrue(a[3]);
+  if (insert < 0) throw BadArgs();
   void* st = stream();
   return status([&] { return l->find_or_insert(t, &b, insert, st); });
 }
@@ -338,7 +339,8 @@ PyObject* py_cross_forward(PyObject* const* a, Py_ssize_t n) {
   const int64_t B = x.size(0), d = x.size(1), S = as_int(a[5]);
   const auto opt = at::TensorOptions().dtype(at::kFloat).device(x.device());
   at::Tensor y = at::empty_like(x), P = at::empty({B}, opt), part;
-  const bool want = PyObject_IsTrue(a[6]) == 1;
+  const int want = PyObject_IsTrue(a[6]);
+  if (want < 0) throw BadArgs();
   if (want) part = at::empty({S, B}, opt);
   const int rc = (int)l->cross_forward((int32_t)B, (int32_t)d, (int32_t)S, ptr<float>(a[1]), ptr<float>(a[2]), ptr<float>(a[3]),
                                        ptr<float>(a[4]), want ? (float*)part.data_ptr() : nullptr, (float*)P.data_ptr(),

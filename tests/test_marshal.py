@@ -18,3 +18,13 @@ def test_cross_takes_matrices_only(shape):
         D.cross_forward(x, x, w, w, 1)
     with pytest.raises(ValueError):
         D.cross_backward(x, x, w, torch.zeros(shape[0]), x)
+
+
+@pytest.mark.gpu
+def test_out_of_memory_keeps_its_type():
+    """Result arrays of 2^45 bytes: the allocator refuses, as for torch.empty."""
+    N, lib = D.native()
+    with pytest.raises(torch.OutOfMemoryError):
+        torch.empty(1 << 43, device="cuda")
+    with pytest.raises(torch.OutOfMemoryError):
+        N.dense1_get(lib, None, 1 << 22, 1 << 21)
