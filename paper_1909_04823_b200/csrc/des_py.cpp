@@ -74,8 +74,22 @@ const at::Tensor& matrix_of(PyObject* o) {              // as `B, d = x.shape` h
   return x;
 }
 
+long long method_int(PyObject* o, const char* name) {
+  PyObject* v = PyObject_CallMethod(o, name, nullptr);
+  if (!v) throw BadArgs();
+  const unsigned long long r = PyLong_AsUnsignedLongLong(v);
+  Py_DECREF(v);
+  if (r == ~0ull && PyErr_Occurred()) throw BadArgs();
+  return (long long)r;
+}
+
+// Memory is anything with data_ptr(): a tensor, a subclass that has its own idea of it, a storage, a caller's own class.
 template <typename T>
-T* ptr(PyObject* o) { return o == Py_None ? nullptr : (T*)tensor_of(o).data_ptr(); }
+T* ptr(PyObject* o) {
+  if (o == Py_None) return nullptr;
+  return THPVariable_CheckExact(o) ? (T*)THPVariable_Unpack(o).data_ptr() : (T*)(uintptr_t)method_int(o, "data_ptr");
+}
+int64_t numel_of(PyObject* o) { return THPVariable_CheckExact(o) ? THPVariable_Unpack(o).numel() : method_int(o, "numel"); }
 
 void* stream() { return (void*)c10::cuda::getCurrentCUDAStream().stream(); }
 
@@ -230,7 +244,7 @@ PyObject* py_head(PyObject* const* a, Py_ssize_t n) {
   des_head_t h;
   h.b0 = as_float(a[4]); h.c_lr = as_float(a[5]); h.c_fm = as_float(a[6]);
   h.u = ptr<float>(a[7]); h.b1 = ptr<float>(a[8]); h.q = ptr<float>(a[9]); h.d = ptr<float>(a[10]);
-  h.n_dense = a[10] == Py_None ? 0 : (int32_t)tensor_of(a[10]).numel();
+  h.n_dense = a[10] == Py_None ? 0 : (int32_t)numel_of(a[10]);
   const des_outputs_t o = {ptr<float>(a[11]), ptr<float>(a[12]), ptr<float>(a[13])};
   const float *xd = ptr<float>(a[14]), *y = ptr<float>(a[15]);
   float *logit = ptr<float>(a[16]), *loss = ptr<float>(a[17]);
@@ -244,11 +258,10 @@ PyObject* py_read_rows(PyObject* const* a, Py_ssize_t n) {
   need(n, 4);
   Lib* l = lib_of(a[0]);
   des_table_t* t = table_of(a[1]);
-  const at::Tensor& rows = tensor_of(a[2]);
-  const int64_t m = rows.numel(), k = as_int(a[3]);
+  const uint32_t* r = ptr<uint32_t>(a[2]);
+  const int64_t m = numel_of(a[2]), k = as_int(a[3]);
   const auto opt = at::TensorOptions().dtype(at::kFloat).device(at::kCUDA);
   at::Tensor emb = at::empty({m, k}, opt), lin = at::empty({m}, opt), ae = at::empty({m, k}, opt), al = at::empty({m}, opt);
-  const uint32_t* r = (const uint32_t*)rows.data_ptr();
   void* st = stream();
   int rc;
   Py_BEGIN_ALLOW_THREADS
@@ -263,9 +276,8 @@ PyObject* py_write_rows(PyObject* const* a, Py_ssize_t n) {
   need(n, 7);
   Lib* l = lib_of(a[0]);
   des_table_t* t = table_of(a[1]);
-  const at::Tensor& rows = tensor_of(a[2]);
-  const int64_t m = rows.numel();
-  const uint32_t* r = (const uint32_t*)rows.data_ptr();
+  const uint32_t* r = ptr<uint32_t>(a[2]);
+  const int64_t m = numel_of(a[2]);
   const float *emb = ptr<float>(a[3]), *lin = ptr<float>(a[4]), *ae = ptr<float>(a[5]), *al = ptr<float>(a[6]);
   void* st = stream();
   return status([&] { return l->write_rows(t, r, m, emb, lin, ae, al, st); });

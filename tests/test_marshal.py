@@ -28,3 +28,26 @@ def test_out_of_memory_keeps_its_type():
         torch.empty(1 << 43, device="cuda")
     with pytest.raises(torch.OutOfMemoryError):
         N.dense1_get(lib, None, 1 << 22, 1 << 21)
+
+
+class _Pointer:
+    """Memory that is no tensor: all a call needs is the address (and the length)."""
+
+    def __init__(self, t):
+        self.t = t
+
+    def data_ptr(self):
+        return self.t.data_ptr()
+
+    def numel(self):
+        return self.t.numel()
+
+
+@pytest.mark.gpu
+def test_objects_with_an_address(native):
+    N, lib = native
+    t = torch.zeros(8, dtype=torch.int32)
+    assert N.write_rows(lib, None, _Pointer(t), None, None, None, None) == 1          # a closed table: INVALID_ARG
+    assert N.write_rows(lib, None, t, _Pointer(t), t.untyped_storage(), None, None) == 1
+    with pytest.raises(AttributeError):
+        N.write_rows(lib, None, t, object(), None, None, None)
