@@ -136,7 +136,7 @@ def native():
     if path not in _native:
         load()
         from . import _marshal
-        _native[path] = (_marshal, _marshal.open(path))
+        _native[path] = (_marshal, _marshal.open(path, DeviceBatch))
     return _native[path]
 
 

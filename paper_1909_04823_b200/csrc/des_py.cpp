@@ -3,12 +3,13 @@
 // the small kernels behind it take; here it is about 1 us.)
 //
 // The C ABI is resolved from an already built library by path, so that the product and the checking library
-// can be used side by side: open(path) -> capsule, then every function takes (capsule, table handle, ...).
+// can be used side by side: open(path, batch class) -> capsule, then every function takes (capsule, table handle, ...).
 #include <Python.h>
 
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAStream.h>
 #include <dlfcn.h>
+#include <string.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -114,8 +115,25 @@ long long attr_int(PyObject* o, PyObject* name) {
   return r;
 }
 
+PyObject* batch_type;                                  // binding.DeviceBatch
+
+// A batch of the binding's own class is read by its attributes; one of any other class builds its struct itself (c(), a
+// ctypes structure: 3 us).
 des_batch_t batch_of(PyObject* o) {
   des_batch_t b;
+  if ((PyObject*)Py_TYPE(o) != batch_type) {
+    PyObject* c = PyObject_CallMethod(o, "c", nullptr);
+    if (!c) throw BadArgs();
+    Py_buffer v;
+    const bool ok = PyObject_GetBuffer(c, &v, PyBUF_SIMPLE) == 0;
+    const bool whole = ok && v.len == (Py_ssize_t)sizeof(b);
+    if (whole) memcpy(&b, v.buf, sizeof(b));
+    if (ok) PyBuffer_Release(&v);
+    Py_DECREF(c);
+    if (ok && !whole) PyErr_SetString(PyExc_TypeError, "c() is not a des_batch_t");
+    if (!whole) throw BadArgs();
+    return b;
+  }
   b.batch = (int32_t)attr_int(o, s_batch);
   b.nnz = attr_int(o, s_nnz);
   b.offsets = attr_ptr<int32_t>(o, s_offsets);
@@ -150,7 +168,7 @@ PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 PyObject* py_open(PyObject* const* a, Py_ssize_t n) {
-  need(n, 1);
+  need(n, 2);                                          // (path, class of the binding's batches)
   const char* path = PyUnicode_AsUTF8(a[0]);
   if (!path) throw BadArgs();
   void* h = dlopen(path, RTLD_NOW | RTLD_LOCAL);
@@ -168,6 +186,8 @@ PyObject* py_open(PyObject* const* a, Py_ssize_t n) {
   SYM(cross_backward, "des_cross_backward"); SYM(cross_workspace_floats, "des_cross_workspace_floats");
 #undef SYM
   if (!ok) { delete l; PyErr_SetString(PyExc_OSError, "library lacks a symbol of the C ABI"); throw BadArgs(); }
+  Py_INCREF(a[1]);
+  Py_XSETREF(batch_type, a[1]);
   return PyCapsule_New(l, "des_lib", nullptr);         // lives as long as the process, like the library
 }
 

@@ -51,3 +51,48 @@ def test_objects_with_an_address(native):
     assert N.write_rows(lib, None, t, _Pointer(t), t.untyped_storage(), None, None) == 1
     with pytest.raises(AttributeError):
         N.write_rows(lib, None, t, object(), None, None, None)
+
+
+class _Own(D.DeviceBatch):
+    """A batch that builds its own struct."""
+    made = 0
+
+    def c(self):
+        self.made += 1
+        return super().c()
+
+
+class _Bare:
+    def __init__(self, db):
+        self.db = db
+
+    def c(self):
+        return self.db.c()
+
+
+@pytest.mark.gpu
+def test_batches_that_build_their_own_struct(native):
+    N, lib = native
+    off, ids = torch.zeros(4, dtype=torch.int32), torch.zeros(3, dtype=torch.int64)
+    db = _Own(off, ids, None, 1, device="cpu")
+    assert N.find_or_insert(lib, None, db, True) == 1 and db.made == 1
+    assert N.find_or_insert(lib, None, _Bare(db), True) == 1 and db.made == 2
+    assert N.find_or_insert(lib, None, D.DeviceBatch(off, ids, None, 1, device="cpu"), True) == 1
+
+
+@pytest.mark.gpu
+def test_batch_struct_is_read_as_c():
+    """The same step from a batch of the class itself and from one that builds its own struct."""
+    res = []
+    for cls in (D.DeviceBatch, _Own):
+        t = D.Table(2, 3, 8, max_rows=1000, seed=1, max_nnz=64, max_batch=8)
+        try:
+            off = torch.arange(0, 13, dtype=torch.int32)
+            db = cls(off, torch.arange(12) % 7 + 1, torch.arange(12) + 0.5, 4)
+            t.find_or_insert(db)
+            out = torch.zeros(4, 12, device="cuda")
+            t.forward_fused(D.OP_LR | D.OP_FM, db, out_small=out)
+            res.append((db.rows.clone(), db.uidx.clone(), db.n_uniq.clone(), out))
+        finally:
+            t.close()
+    assert all(torch.equal(a, b) for a, b in zip(*res))
