@@ -372,9 +372,9 @@ class Table:
     def head(self, ops, batch_size, hc, out_small=None, pooled=None, Z=None, xdense=None, y=None, logit=None, loss=None,
              gL=None, gF=None, gE=None, gZ=None):
         """hc: dict(b0, c_lr, c_fm, u, b1, q, d) with device tensors (or None) for the vectors."""
-        self._check(self.N.head(self._lib, self.h.value, ops, batch_size, hc["b0"], hc["c_lr"], hc["c_fm"], hc.get("u"),
-                                hc.get("b1"), hc.get("q"), hc.get("d"), out_small, pooled, Z, xdense, y, logit, loss, gL, gF,
-                                gE, gZ), "des_head")
+        self._check(self.N.head(self._lib, self.h.value, ops, int(batch_size), float(hc["b0"]), float(hc["c_lr"]), float(hc["c_fm"]),
+                                hc.get("u"), hc.get("b1"), hc.get("q"), hc.get("d"), out_small, pooled, Z, xdense, y, logit, loss,
+                                gL, gF, gE, gZ), "des_head")
 
     def evict_keys(self, keys: torch.Tensor) -> int:
         """keys: int64 / uint64 device tensor of ids to remove.  Returns the number of rows removed."""

@@ -1,5 +1,7 @@
 """What the marshalling extension takes and refuses: the same objects, and the same exceptions, as the ctypes calls of the
 other entry points."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -96,3 +98,14 @@ def test_batch_struct_is_read_as_c():
         finally:
             t.close()
     assert all(torch.equal(a, b) for a, b in zip(*res))
+
+
+@pytest.mark.gpu
+def test_head_converts_its_numbers(native):
+    t = object.__new__(D.Table)
+    t.N, t._lib = native
+    t.h = C.c_void_p()
+    for b in (4, 4.0, torch.tensor(4)):
+        with pytest.raises(D.DesError) as e:                # a closed table, not a TypeError
+            t.head(D.OP_LR, b, dict(b0="0.5", c_lr=torch.tensor(1.0), c_fm=1, u=None, b1=None, q=None, d=None))
+        assert e.value.code == 1
