@@ -148,13 +148,15 @@ des_batch_t batch_of(PyObject* o) {
 }
 
 template <typename F>
-PyObject* status(F&& call) {                           // runs without the interpreter lock
+int unlocked(F&& call) {                               // a call of the library, without the interpreter lock
   int rc;
   Py_BEGIN_ALLOW_THREADS
   rc = (int)call();
   Py_END_ALLOW_THREADS
-  return PyLong_FromLong(rc);
+  return rc;
 }
+template <typename F>
+PyObject* status(F&& call) { return PyLong_FromLong(unlocked(call)); }
 
 template <PyObject* (*F)(PyObject* const*, Py_ssize_t)>
 PyObject* guarded(PyObject*, PyObject* const* a, Py_ssize_t n) {
@@ -283,11 +285,8 @@ PyObject* py_read_rows(PyObject* const* a, Py_ssize_t n) {
   const auto opt = at::TensorOptions().dtype(at::kFloat).device(at::kCUDA);
   at::Tensor emb = at::empty({m, k}, opt), lin = at::empty({m}, opt), ae = at::empty({m, k}, opt), al = at::empty({m}, opt);
   void* st = stream();
-  int rc;
-  Py_BEGIN_ALLOW_THREADS
-  rc = (int)l->read_rows(t, r, m, (float*)emb.data_ptr(), (float*)lin.data_ptr(), (float*)ae.data_ptr(),
-                         (float*)al.data_ptr(), st);
-  Py_END_ALLOW_THREADS
+  float *pe = (float*)emb.data_ptr(), *pl = (float*)lin.data_ptr(), *pae = (float*)ae.data_ptr(), *pal = (float*)al.data_ptr();
+  const int rc = unlocked([&] { return l->read_rows(t, r, m, pe, pl, pae, pal, st); });
   return Py_BuildValue("(iNNNN)", rc, THPVariable_Wrap(emb), THPVariable_Wrap(lin), THPVariable_Wrap(ae), THPVariable_Wrap(al));
 }
 
@@ -336,11 +335,10 @@ PyObject* py_step_host_submit(PyObject* const* a, Py_ssize_t n) {
   des_table_t* t = table_of(a[1]);
   const HostStep s = host_step_of(a + 2);
   void* st = stream();
-  int rc;
   int32_t ticket = -1;
-  Py_BEGIN_ALLOW_THREADS
-  rc = (int)l->step_host_submit(t, s.ops, s.batch, s.nnz, s.offsets, s.ids, s.vals, &s.g, s.pooled, s.Z, s.out, st, &ticket);
-  Py_END_ALLOW_THREADS
+  const int rc = unlocked([&] {
+    return l->step_host_submit(t, s.ops, s.batch, s.nnz, s.offsets, s.ids, s.vals, &s.g, s.pooled, s.Z, s.out, st, &ticket);
+  });
   return Py_BuildValue("(ii)", rc, (int)ticket);
 }
 
@@ -359,7 +357,9 @@ PyObject* py_dense1_get(PyObject* const* a, Py_ssize_t n) {
   Lib* l = lib_of(a[0]);
   des_table_t* t = table_of(a[1]);
   at::Tensor w = at::empty({as_int(a[2]), as_int(a[3])}, at::TensorOptions().dtype(at::kFloat).device(at::kCUDA));
-  const int rc = (int)l->dense1_get(t, (float*)w.data_ptr(), stream());
+  float* pw = (float*)w.data_ptr();
+  void* st = stream();
+  const int rc = unlocked([&] { return l->dense1_get(t, pw, st); });
   return Py_BuildValue("(iN)", rc, THPVariable_Wrap(w));
 }
 
@@ -374,9 +374,10 @@ PyObject* py_cross_forward(PyObject* const* a, Py_ssize_t n) {
   const int want = PyObject_IsTrue(a[6]);
   if (want < 0) throw BadArgs();
   if (want) part = at::empty({S, B}, opt);
-  const int rc = (int)l->cross_forward((int32_t)B, (int32_t)d, (int32_t)S, ptr<float>(a[1]), ptr<float>(a[2]), ptr<float>(a[3]),
-                                       ptr<float>(a[4]), want ? (float*)part.data_ptr() : nullptr, (float*)P.data_ptr(),
-                                       (float*)y.data_ptr(), stream());
+  const float *x0 = ptr<float>(a[1]), *px = ptr<float>(a[2]), *pw = ptr<float>(a[3]), *pb = ptr<float>(a[4]);
+  float *pp = want ? (float*)part.data_ptr() : nullptr, *pP = (float*)P.data_ptr(), *py = (float*)y.data_ptr();
+  void* st = stream();
+  const int rc = unlocked([&] { return l->cross_forward((int32_t)B, (int32_t)d, (int32_t)S, x0, px, pw, pb, pp, pP, py, st); });
   if (want) return Py_BuildValue("(iNNN)", rc, THPVariable_Wrap(y), THPVariable_Wrap(P), THPVariable_Wrap(part));
   return Py_BuildValue("(iNNO)", rc, THPVariable_Wrap(y), THPVariable_Wrap(P), Py_None);
 }
@@ -390,9 +391,11 @@ PyObject* py_cross_backward(PyObject* const* a, Py_ssize_t n) {
   const auto opt = at::TensorOptions().dtype(at::kFloat).device(x.device());
   at::Tensor gx0 = at::empty_like(x), gx = at::empty_like(x), gw = at::empty({d}, opt), gb = at::empty({d}, opt);
   at::Tensor ws = at::empty({l->cross_workspace_floats((int32_t)B, (int32_t)d)}, opt);
-  const int rc = (int)l->cross_backward((int32_t)B, (int32_t)d, ptr<float>(a[1]), ptr<float>(a[2]), ptr<float>(a[3]),
-                                        ptr<float>(a[4]), ptr<float>(a[5]), (float*)gx0.data_ptr(), (float*)gx.data_ptr(),
-                                        (float*)gw.data_ptr(), (float*)gb.data_ptr(), (float*)ws.data_ptr(), stream());
+  const float *x0 = ptr<float>(a[1]), *px = ptr<float>(a[2]), *pw = ptr<float>(a[3]), *pP = ptr<float>(a[4]), *pY = ptr<float>(a[5]);
+  float *p0 = (float*)gx0.data_ptr(), *p1 = (float*)gx.data_ptr(), *p2 = (float*)gw.data_ptr(), *p3 = (float*)gb.data_ptr(),
+        *p4 = (float*)ws.data_ptr();
+  void* st = stream();
+  const int rc = unlocked([&] { return l->cross_backward((int32_t)B, (int32_t)d, x0, px, pw, pP, pY, p0, p1, p2, p3, p4, st); });
   return Py_BuildValue("(iNNNN)", rc, THPVariable_Wrap(gx0), THPVariable_Wrap(gx), THPVariable_Wrap(gw), THPVariable_Wrap(gb));
 }
 
