@@ -2,7 +2,6 @@
 // workspace, status, size, export, row read-back (Section 5, "Dynamic Hash
 // Table": the storage behind lookup / insert / update).
 #include <new>
-#include <vector>
 #include <math.h>
 #include <string.h>
 
@@ -199,8 +198,11 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
     p = (typename std::remove_reference<decltype(p)>::type)dalloc(c, bytes);
     if (!p) ok = false;
   };
-  std::vector<DesSlabItem> items;                      // the workspace: one allocation
-  auto A = [&](auto*& p, size_t bytes) { items.push_back({(void**)&p, bytes}); };
+  DesSlabItem items[32];                               // the workspace: one allocation
+  int n_items = 0;
+  auto A = [&](auto*& p, size_t bytes) {
+    if (n_items < (int)(sizeof(items) / sizeof(items[0]))) items[n_items++] = {(void**)&p, bytes}; else ok = false;
+  };
   big(t->slots, slots * sizeof(Slot));
   big(t->W, (rows + 1) * rowbytes);          // one all-zero row behind the table stands for "no row" in gathers
   if (c.optimizer != DES_OPT_SGD || c.lin_optimizer == DES_LIN_FTRL) big(t->A, rows * rowbytes);
@@ -242,7 +244,7 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
     A(t->gemm_ws, t->gemm_ws_bytes);
   }
   if (ok) {
-    t->slab = des_slab_alloc(c, items.data(), (int)items.size());
+    t->slab = des_slab_alloc(c, items, n_items);
     ok = t->slab != nullptr;
   }
   if (!ok) { des_table_destroy(t); return DES_ERR_CUDA; }
