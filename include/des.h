@@ -453,9 +453,11 @@ des_status_t des_head(des_table_t* t, uint32_t ops, int32_t batch, const des_hea
 /* y = x0 * (+)_s <x[slice s], w[slice s]> + b + x  for x0, x, y [B][d] and w, b [d]
  * (all float32, device, row-major).  w is split along d into num_shards contiguous
  * slices (slice s = columns floor(s d / S) .. floor((s+1) d / S) - 1); each shard's
- * partial is one scalar per sample, (+) adds them in shard order.  d_part [S][B]
- * (optional, may be NULL) receives the per-shard scalars, d_P [B] the aggregate
- * (needed by the backward), d_y the layer output.  No table is involved; the call
+ * partial is one scalar per sample.  With d_part [S][B] (optional, may be NULL) the
+ * per-shard scalars are formed, written there and added in shard order.  Without it the sum
+ * over a row is taken in one go (d a multiple of 4 up to 2048, 16-byte aligned rows; in shard order
+ * otherwise): the same sum in another order, num_shards then only has to be valid.  d_P [B]
+ * receives the aggregate (needed by the backward), d_y the layer output.  No table is involved; the call
  * only enqueues kernels on `stream`.  DES_ERR_INVALID_ARG for NULL / non-positive
  * arguments or num_shards > d. */
 des_status_t des_cross_forward(int32_t batch, int32_t dim, int32_t num_shards, const float* d_x0,

@@ -3,7 +3,8 @@
 //
 // Cross layer: w is split along its long dimension d into S contiguous slices;
 // shard s forms the scalar p_s = <x[slice s], w[slice s]> per sample, (+) adds
-// the scalars in shard order, and y = x0 * (+)p + b + x.  Both passes are
+// the scalars in shard order, and y = x0 * (+)p + b + x.  A caller that does not ask for the p_s gets
+// the unsplit sum <x, w> where the rows allow it ("rows in registers"): equal up to the order of the additions.  Both passes are
 // streams over [B][d] rows, bound by memory: a row is read once per array and held in registers between the dot
 // product and its use ("rows in registers" below).  Rows that are not 16-byte aligned or longer than
 // CX_MAX_D, and callers that want the per-shard scalars, take the kernels with one warp per sample, which read a row twice.

@@ -185,30 +185,28 @@ __device__ __forceinline__ void sp_round(const uint32_t* __restrict__ grow_sorte
   }
 }
 
-// A bag walked by LB = G * P lanes together, LB occurrences at a time: every lane looks up the row of one occurrence (and adds
-// its linear weight and squared norm to sums of its own), then the rows are handed round by shuffles, sub-group p taking
-// positions p, p + P, ...  Looked up by all lanes of every occurrence instead, the row number, shard and tail are three of
-// the four loads of an occurrence.
-template <int G, int P, bool HAS_VALS, bool TAIL>
+// A bag walked by a warp (P groups of G lanes) together, 32 occurrences at a time: every lane looks up the row of one occurrence
+// (and adds its linear weight and squared norm to sums of its own), then the rows are handed round by shuffles, sub-group p
+// taking positions p, p + P, ...  Looked up by all lanes of every occurrence instead, the row number, shard and tail are
+// three of the four loads of an occurrence.
+template <int G, int P, bool HAS_VALS>
 __device__ __forceinline__ void coop_bag(const uint32_t* __restrict__ rows, const uint8_t* __restrict__ shards,
                                          const float* __restrict__ vals, const uint32_t* __restrict__ s_base, int lo, int hi,
-                                         int sub, unsigned gmask, const char* __restrict__ Wc, const char* __restrict__ Wt,
+                                         int sub, const char* __restrict__ Wc, const char* __restrict__ Wt,
                                          unsigned rowB, uint32_t null_row, float4& acc, float& bl, float& bq) {
-  constexpr int LB = G * P;
+  static_assert(G * P == 32, "a warp per bag");
   const int p = sub / G;
-  for (int c0 = lo; c0 < hi; c0 += LB) {
-    const int j = c0 + sub, n = min(LB, hi - c0);
+  for (int c0 = lo; c0 < hi; c0 += 32) {
+    const int j = c0 + sub, n = min(32, hi - c0);
     uint32_t g = null_row;
     float x = 0.f;
     if (j < hi) {
       const uint32_t r = __ldg(rows + j);
       if (r != DES_ROW_NONE) g = DES_DBG_ROW(s_base[__ldg(shards + j)] + r);
       if (HAS_VALS) x = __ldg(vals + j);
-      if (TAIL) {
-        const float2 tl = __ldg(reinterpret_cast<const float2*>(Wt + (size_t)g * rowB));
-        bl += HAS_VALS ? tl.x * x : tl.x;
-        bq += HAS_VALS ? tl.y * x * x : tl.y;
-      }
+      const float2 tl = __ldg(reinterpret_cast<const float2*>(Wt + (size_t)g * rowB));
+      bl += HAS_VALS ? tl.x * x : tl.x;
+      bq += HAS_VALS ? tl.y * x * x : tl.y;
     }
     int t = 0;
     auto step = [&](auto U) {
@@ -216,8 +214,8 @@ __device__ __forceinline__ void coop_bag(const uint32_t* __restrict__ rows, cons
       float4 v[N]; float xx[N];
 #pragma unroll
       for (int u = 0; u < N; ++u) {
-        const uint32_t gg = __shfl_sync(gmask, g, t + u * P + p, LB);
-        if (HAS_VALS) xx[u] = __shfl_sync(gmask, x, t + u * P + p, LB);
+        const uint32_t gg = __shfl_sync(0xFFFFFFFFu, g, t + u * P + p);
+        if (HAS_VALS) xx[u] = __shfl_sync(0xFFFFFFFFu, x, t + u * P + p);
         v[u] = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)gg * rowB));
       }
 #pragma unroll
@@ -680,9 +678,9 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
         }
       }
     }
-    if (COOP) {
-      coop_bag<G, P, HAS_VALS, true>(rows, shards, vals, s_base, lo[0], hi[0], sub, 0xFFFFFFFFu, Wc, Wt, rowB, null_row, acc[0], bl[0], bq[0]);
-    } else
+    if constexpr (COOP) {
+      coop_bag<G, P, HAS_VALS>(rows, shards, vals, s_base, lo[0], hi[0], sub, Wc, Wt, rowB, null_row, acc[0], bl[0], bq[0]);
+    } else {
 #pragma unroll
     for (int q = 0; q < BU; ++q) {                 // the rest of each bag
       int i0 = lo[q] + P;
@@ -693,6 +691,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
       if (i0 + P <= h) { SG_STEP(1); i0 += P; }
       if (i0 + p < h) SG_STEP(1);
 #undef SG_STEP
+    }
     }
 #pragma unroll
     for (int q = 0; q < BU; ++q) {
@@ -859,7 +858,7 @@ __global__ void __launch_bounds__(256, 4) sample_stage_kernel(
       if (ws == 0) {
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         float bl = 0.f, bq = 0.f;
-        coop_bag<G, P, HAS_VALS, true>(rows, shards, vals, s_base, j0, __ldg(off + fa + 1), lane, 0xFFFFFFFFu, Wc, Wt, rowB, null_row,
+        coop_bag<G, P, HAS_VALS>(rows, shards, vals, s_base, j0, __ldg(off + fa + 1), lane, Wc, Wt, rowB, null_row,
                                        acc, bl, bq);
         tail_done(bl, bq);
         bag_done(fa, acc);

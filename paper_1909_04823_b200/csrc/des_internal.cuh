@@ -144,8 +144,9 @@ struct des_table {
 };
 #define DES_PROF_MAX 16384
 
-// Many arrays, one allocation: every array starts on a 256-byte boundary.  (A table made 25 allocations of its own, and each
-// can take milliseconds when the driver has to find memory.)  Returns NULL when there is no memory.
+// Many arrays, one allocation: every array starts on a 256-byte boundary.  (A table made 25 allocations of its own.  On a quiet
+// driver creating one took 1.4 to 5 ms and takes 1.1 to 3; in sessions where single allocations take tens of
+// milliseconds, which come and go, it can cost more than before as well.)  Returns NULL when there is no memory.
 struct DesSlabItem { void** p; size_t bytes; };
 void* des_slab_alloc(const des_config_t& c, const DesSlabItem* items, int n);
 
@@ -160,9 +161,11 @@ void des_api_begin(des_table* t, cudaStream_t cs);
 // wait in des_pdl_wait for that kernel's completion (memory included) before they touch anything.  EVERY
 // kernel launched through des_launch starts with that wait.  It takes ALL pointers that the kernel reads
 // through: a read-only load (__ldg, const __restrict__) may be moved by the compiler across a mere memory barrier, to
-// before the wait, so the pointers come out of it as new values.  No kernel lets the next one in before its
+// before the wait, so the pointers come out of it as new values.  No kernel of this library lets the next one in before its
 // blocks end: blocks that wait on an SM take room and end up unevenly spread (512 x 8 LR + FM step 47 -> 42 us
-// without, a 2379-sample prediction 204 -> 184).
+// without, a 2379-sample prediction 204 -> 184).  The exception are the first layer's tensor-core products: the switch that gives
+// the CUTLASS kernel its wait gives it its early trigger too, so behind a product the next kernel's blocks can be
+// resident while it runs.  Nothing in global memory may be touched before the wait there either.
 template <typename P>
 __device__ __forceinline__ void des_pdl_new(P& p) {
   static_assert(sizeof(P) == 8, "pointers only");
