@@ -41,7 +41,7 @@
 
 #define SGF_BU 4                  // short bags of a lane group in flight together (sample_gather_kernel)
 #define SGF_SMEM (24u << 10)      // shared memory a block of the FIELD form takes at most, unless one sample needs more
-#define SGF_ONE (47u << 10)       // and at most for one sample: a launch has 48 KiB, the kernel's own arrays (s_base and the like) included
+#define SGF_ONE ((48u << 10) - DES_MAX_SHARDS * 4)   // and at most for one sample: a launch has 48 KiB, the kernel's own s_base included
 #ifndef POOL_BLOCKS_PER_SM
 #define POOL_BLOCKS_PER_SM 64   // grid cap of the pooling kernel (it strides over the bags)
 #endif

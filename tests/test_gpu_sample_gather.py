@@ -44,7 +44,9 @@ def _setup(D, B, F, k, S, partition, mean, vals, seed):
     (20, 400, 64, 9, 1, 1, False),
     # about the largest sample whose pooled vectors a block holds, and the sizes behind it
     *[(20, F, 64, 9, 1, 1, False) for F in (182, 183, 185, 186, 187)], (20, 360, 32, 7, 1, 1, True), (20, 361, 32, 7, 1, 1, False),
-    (20, 682, 16, 5, 1, 1, False)])
+    (20, 682, 16, 5, 1, 1, False),
+    # long bags under FIELD: a warp per bag
+    (300, 20, 64, 7, 1, 12, False), (40, 30, 16, 4, 1, 20, True), (2500, 8, 32, 8, 1, 10, True)])
 def test_sums_of_a_sample(B, F, k, S, partition, mean, vals):
     from paper_1909_04823_b200 import binding as D
     t, db, bag, v, w, nnz = _setup(D, B, F, k, S, partition, mean, vals, B + F)
