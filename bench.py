@@ -269,8 +269,10 @@ def kernel_bytes(name, st):
         return 2 * row * R
     if name == "update_rows_kernel":
         return U * (2 * row + 2 * row * (1 + state) + 8)
-    if name == "cvt_bf16_kernel":          # one launch per step: gZ and pooled of the backward (the forward's copy of
-        return 6 * (B * F * k + B * st["H"])   # pooled comes out of the pooling kernel)
+    if name == "cvt_bf16_fwd_kernel":      # the pooled block that des_aggregate is given (the fused forward writes its copy itself)
+        return 6 * B * F * k
+    if name == "cvt_bf16_kernel":          # gZ and pooled of the backward, in one launch
+        return 6 * (B * F * k + B * st["H"])
     return None
 
 

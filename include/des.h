@@ -230,7 +230,8 @@ des_status_t des_forward_partials(des_table_t* t, uint32_t ops, const des_batch_
  * runs over the columns of pooled in field order; under the FIELD partition that
  * visits every shard's block once, not shard by shard — inside the 2e-2 bound of
  * bf16 operands) or, when part->part_dense is given, P_s materialised first (K
- * slices in shard order, CUDA-core kernel) and Z = sum_s P_s. */
+ * slices in shard order, CUDA-core kernel) and Z = sum_s P_s.  The pooled block is taken
+ * as it is when the call's kernels run: between the two calls it is the caller's to change. */
 des_status_t des_aggregate(des_table_t* t, uint32_t ops, const des_batch_t* batch,
                            const des_partials_t* part, const des_outputs_t* out, void* stream);
 

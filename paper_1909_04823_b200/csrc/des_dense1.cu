@@ -155,17 +155,8 @@ __global__ void w1_update_kernel(const float* __restrict__ part, int slices, siz
   }
 }
 
-__global__ void cvt_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t n) {
-  size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4, st = (size_t)gridDim.x * blockDim.x * 4;
-  for (; i + 3 < n; i += st) {
-    const float4 v = *reinterpret_cast<const float4*>(src + i);
-    __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-    *reinterpret_cast<uint2*>(dst + i) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
-  }
-}
-
-// two arrays in one launch (the backward's two operands), zeros from n to the padded length; four 16-byte loads of a thread
-// in flight
+// one array, or two in one launch (the backward's two operands), zeros from n to the padded length; four 16-byte loads of a
+// thread in flight
 __global__ void __launch_bounds__(256) cvt_bf16_pair_kernel(const float* __restrict__ s1, __nv_bfloat16* __restrict__ d1, size_t n1,
                                                             size_t pad1, const float* __restrict__ s2,
                                                             __nv_bfloat16* __restrict__ d2, size_t n2, size_t pad2) {
@@ -190,10 +181,9 @@ __global__ void __launch_bounds__(256) cvt_bf16_pair_kernel(const float* __restr
   }
 }
 
-static des_status_t to_bf16(des_table* t, const float* src, __nv_bfloat16* dst, size_t n, cudaStream_t st) {
-  cvt_bf16_kernel<<<t->sm_count * 4, 256, 0, st>>>(src, dst, n);     // n is a multiple of 4 (k and H are)
-  DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
-  return DES_OK;
+static void launch_cvt(const float* s1, __nv_bfloat16* d1, size_t n1, size_t p1, const float* s2, __nv_bfloat16* d2, size_t n2, size_t p2,
+                       cudaStream_t st) {
+  des_launch(cvt_bf16_pair_kernel, (unsigned)(((p1 + p2) / 4 + 1023) / 1024), 256, 0, st, s1, d1, n1, p1, s2, d2, n2, p2);
 }
 
 // a thread per four weights, as far as the chip holds them at once
@@ -204,15 +194,13 @@ static void launch_w1_update(des_table* t, int slices, cudaStream_t st) {
 }
 
 des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float* Z, float* part_dense,
-                                const float* part_pooled, cudaStream_t st) {
+                                const float* part_pooled, bool have_b, cudaStream_t st) {
   if (!part_dense && t->use_tc) {
     const int FK = t->F * t->k;
-    // the pooling kernel of the same forward has usually left the bfloat16 copy already
-    const bool have = t->pooled_b_src == pooled;
-    t->pooled_b_src = nullptr;                         // good for one product only
-    if (!have) {
-      des_status_t e = to_bf16(t, pooled, t->pooled_b, (size_t)B * FK, st);
-      if (e != DES_OK) return e;
+    if (!have_b) {
+      const size_t n = (size_t)B * FK;
+      launch_cvt(pooled, t->pooled_b, n, n, nullptr, nullptr, 0, 0, st);
+      DES_LAUNCH_CHECK(t, "cvt_bf16_fwd_kernel");
     }
     const int rc = des_tc_gemm_fwd(B, t->H, FK, 1, t->pooled_b, t->W1b, Z, Z, 0.f, t->gemm_ws, t->gemm_ws_bytes, st);
     if (rc == 0) { DES_LAUNCH_CHECK(t, "tc_gemm_fwd"); return DES_OK; }
@@ -237,7 +225,6 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
                                  float* gE_work, int B, cudaStream_t st) {
   const int FK = t->F * t->k;
   if (t->use_tc) {
-    t->pooled_b_src = nullptr;
     // The weight gradient has few output tiles (F*k x H) and a long contraction (the batch): the batch is cut into L pieces so
     // that every SM gets a tile (L partial products, added in piece order by w1_update_kernel).  The pieces are of
     // equal length, a multiple of 64 samples; zero rows fill the last one up.
@@ -249,8 +236,7 @@ des_status_t des_dense1_backward(des_table* t, const float* pooled, const float*
     const int piece = L == 1 ? B : ((B + L - 1) / L + 63) / 64 * 64;
     L = (B + piece - 1) / piece;
     const size_t n1 = (size_t)B * t->H, n2 = (size_t)B * FK, p1 = (size_t)piece * L * t->H, p2 = (size_t)piece * L * FK;
-    des_launch(cvt_bf16_pair_kernel, (unsigned)(((p1 + p2) / 4 + 1023) / 1024), 256, 0, st, gZ, t->gZ_b, n1, p1, pooled, t->pooled_b,
-               n2, p2);
+    launch_cvt(gZ, t->gZ_b, n1, p1, pooled, t->pooled_b, n2, p2, st);
     DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
     const int rc1 = des_tc_gemm_dgrad(B, FK, t->H, 1, t->gZ_b, t->W1b, gE ? gE : gE_work, gE_work, gE ? 1.f : 0.f,
                                       t->gemm_ws, t->gemm_ws_bytes, st);

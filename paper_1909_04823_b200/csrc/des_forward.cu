@@ -1004,14 +1004,20 @@ __global__ void reduce_shards_kernel(const float* __restrict__ part, size_t per_
 
 static int group_for(int k) { int K4 = k / 4, G = 1; while (G < K4) G <<= 1; return G; }
 
-static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, float* pooled, cudaStream_t cs);
+static des_status_t launch_single_gather(des_table_t* t, const des_batch_t* b, float* pooled, __nv_bfloat16* pb, cudaStream_t cs);
 static bool sample_gather_fits(const des_table* t) { return (size_t)t->F * (t->k + 2) * 4 <= SGF_ONE; }   // FIELD form, one sample
 static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, bool field, float* pooled,
-                                         float* part_small, float* out_small, cudaStream_t cs);
+                                         __nv_bfloat16* pb, float* part_small, float* out_small, cudaStream_t cs);
+// Where the pooled vectors are left as bfloat16 too, the operand format of the first layer's tensor-core product: only in
+// the call that goes on to that product (des_forward_fused).  Between des_forward_partials and des_aggregate the block is the
+// caller's, who may have changed it, so des_aggregate converts what it is given (16384 x 1248: 15 us of a step of 384).
+static __nv_bfloat16* pooled_copy(const des_table* t, uint32_t ops, bool whole) {
+  return whole && (ops & DES_OP_DENSE1) && t->use_tc ? t->pooled_b : nullptr;
+}
 
-// shared by des_forward_partials (fused_out == NULL) and des_forward_fused
+// shared by des_forward_partials (fused_out == NULL) and des_forward_fused (whole: the aggregation follows in the same call)
 static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t* b, const des_partials_t* part,
-                                 float* fused_out, void* stream) {
+                                 float* fused_out, bool whole, void* stream) {
   des_status_t st = des_check_batch(t, b, 0);
   if (st != DES_OK) return st;
   if (!part || (ops & ~15u) || ops == 0) return DES_ERR_INVALID_ARG;
@@ -1033,8 +1039,8 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
     // FIELD partition with pooling among the operators: one gather pass (pooled vectors + bag tails), then the
     // per-shard sub-operators as sums over each shard's own fields — no routing pass, no second gather.  In one kernel
     // unless a sample's pooled vectors do not fit its shared memory.
-    if (sample_gather_fits(t)) return launch_sample_gather(t, ops, b, true, pl, ps, fused_out, cs);
-    if ((st = launch_single_gather(t, ops, b, pl, cs)) != DES_OK) return st;
+    if (sample_gather_fits(t)) return launch_sample_gather(t, ops, b, true, pl, pooled_copy(t, ops, whole), ps, fused_out, cs);
+    if ((st = launch_single_gather(t, b, pl, pooled_copy(t, ops, whole), cs)) != DES_OK) return st;
     const int grid = (int)(((long long)B * G + 255) / 256);
 #define FP2(GG, FU) des_launch(field_partials_kernel<GG, FU>, grid, 256, 0, cs, (const float*)pl, t->bag_tail, B, (int)t->F, (int)t->S, (int)t->k, ops, ps, fused_out)
 #define FP(GG) do { if (fused_out) FP2(GG, true); else FP2(GG, false); } while (0)
@@ -1072,9 +1078,7 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
     long long blocks = (threads + 255) / 256;
     if (blocks > (long long)t->sm_count * POOL_BLOCKS_PER_SM) blocks = (long long)t->sm_count * POOL_BLOCKS_PER_SM;
     const unsigned grid = (unsigned)blocks;
-    // with the first layer among the operators the pooled vectors are also left as bfloat16, the operand
-    // format of the tensor-core product that follows (one conversion pass less)
-    __nv_bfloat16* pb = ((ops & DES_OP_DENSE1) && t->use_tc && !pp) ? t->pooled_b : nullptr;
+    __nv_bfloat16* pb = pooled_copy(t, ops, whole);      // (whole: no materialised partials)
 #define PK5(GG, PP, HV, MT, BO) des_launch(pool_kernel<GG, PP, HV, MT, BO>, grid, 256, 0, cs, b->offsets, b->vals, grow_csr,    \
         b->shards, nbags, B, (int)t->F, (int)t->k, t->W, (uint32_t)t->total_rows, pl, pp, pb)
 #define PK3(GG, HV, MT, BO) do { if (wide) PK5(GG, 32 / GG, HV, MT, BO); else PK5(GG, 1, HV, MT, BO); } while (0)
@@ -1086,18 +1090,17 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
 #undef PK3
 #undef PK5
     DES_LAUNCH_CHECK(t, "pool_kernel");
-    t->pooled_b_src = pb ? pl : nullptr;
   }
   return DES_OK;
 }
 extern "C" des_status_t des_forward_partials(des_table_t* t, uint32_t ops, const des_batch_t* b,
                                              const des_partials_t* part, void* stream) {
-  return forward_impl(t, ops, b, part, nullptr, stream);
+  return forward_impl(t, ops, b, part, nullptr, false, stream);
 }
 
 // the gather pass of the single-gather forms: pooled vectors (and their bfloat16 copy when the first layer
 // follows) and per-bag sums of the linear weights and squared norms
-static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, float* pooled, cudaStream_t cs) {
+static des_status_t launch_single_gather(des_table_t* t, const des_batch_t* b, float* pooled, __nv_bfloat16* pb, cudaStream_t cs) {
   const int B = b->batch, G = group_for(t->k);
   const long long nbags = (long long)B * t->F;
   const bool wide = b->nnz >= 8 * nbags;
@@ -1105,7 +1108,6 @@ static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des
   long long blocks = (threads + 255) / 256;
   if (blocks > (long long)t->sm_count * POOL_BLOCKS_PER_SM) blocks = (long long)t->sm_count * POOL_BLOCKS_PER_SM;
   const unsigned grid = (unsigned)blocks;
-  __nv_bfloat16* pb = ((ops & DES_OP_DENSE1) && t->use_tc) ? t->pooled_b : nullptr;
 #define SG3(GG, PP, HV) des_launch(single_gather_kernel<GG, PP, HV>, grid, 256, 0, cs, b->offsets, b->vals, b->rows, b->shards, nbags, \
                                    (int)t->S, (int)t->k, t->W, t->meta, (uint32_t)t->total_rows, pooled, t->bag_tail, pb)
 #define SG2(GG, HV) do { if (wide) SG3(GG, 32 / GG, HV); else SG3(GG, 1, HV); } while (0)
@@ -1115,14 +1117,13 @@ static des_status_t launch_single_gather(des_table_t* t, uint32_t ops, const des
 #undef SG2
 #undef SG3
   DES_LAUNCH_CHECK(t, "single_gather_kernel");
-  t->pooled_b_src = pb ? pooled : nullptr;
   return DES_OK;
 }
 
 // Samples per block: one warp per sample once there are samples for the chip, more warps per sample below that (as long as
 // they have bags to take), and always for samples of many long bags, whose lengths differ too much for one warp each.
 static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des_batch_t* b, bool field, float* pooled,
-                                         float* part_small, float* out_small, cudaStream_t cs) {
+                                         __nv_bfloat16* pb, float* part_small, float* out_small, cudaStream_t cs) {
   const int B = b->batch, F = (int)t->F, G = group_for(t->k);
   const bool wide = b->nnz >= 8ll * B * F;
   const int per_warp = wide ? 1 : 32 / G * SGF_BU;      // bags a warp has in flight
@@ -1131,7 +1132,6 @@ static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des
   const size_t per_sample = field ? (size_t)F * (t->k + 2) * 4 : 0;
   while (T > 1 && T * per_sample > SGF_SMEM) T >>= 1;
   const unsigned grid = (unsigned)((B + T - 1) / T);
-  __nv_bfloat16* pb = ((ops & DES_OP_DENSE1) && t->use_tc) ? t->pooled_b : nullptr;
 #define SF4(GG, PP, HV, FD) des_launch(sample_gather_kernel<GG, PP, HV, FD>, grid, 256, T * per_sample, cs, b->offsets, b->vals,     \
                                        b->rows, b->shards, B, F, (int)t->S, (int)t->k, T, ops, t->W, t->meta,                     \
                                        (uint32_t)t->total_rows, pooled, pb, part_small, out_small)
@@ -1146,9 +1146,11 @@ static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des
 #undef SS
 #undef SF4
   DES_LAUNCH_CHECK(t, wide && !field ? "sample_stage_kernel" : "sample_gather_kernel");
-  t->pooled_b_src = pb ? pooled : nullptr;
   return DES_OK;
 }
+
+static des_status_t aggregate_impl(des_table_t* t, uint32_t ops, const des_batch_t* b, const des_partials_t* part,
+                                   const des_outputs_t* out, bool have_b, void* stream);
 
 extern "C" des_status_t des_forward_fused(des_table_t* t, uint32_t ops, const des_batch_t* b,
                                           const des_partials_t* part, const des_outputs_t* out, void* stream) {
@@ -1166,17 +1168,23 @@ extern "C" des_status_t des_forward_fused(des_table_t* t, uint32_t ops, const de
     if (!part->pooled || ((ops & DES_OP_DENSE1) && !t->H)) return DES_ERR_INVALID_ARG;
     des_api_begin(t, (cudaStream_t)stream);
     DES_DBG_ARM(t, (cudaStream_t)stream);
-    st = launch_sample_gather(t, ops, b, false, part->pooled, nullptr, out->out_small, (cudaStream_t)stream);
+    st = launch_sample_gather(t, ops, b, false, part->pooled, pooled_copy(t, ops, true), nullptr, out->out_small, (cudaStream_t)stream);
   } else {
-    st = forward_impl(t, ops, b, part, out->out_small, stream);
+    st = forward_impl(t, ops, b, part, out->out_small, true, stream);
   }
   if (st != DES_OK) return st;
   // what is left of the aggregation: hand the pooled block over and run the first layer
-  return rest ? des_aggregate(t, rest, b, part, out, stream) : DES_OK;
+  return rest ? aggregate_impl(t, rest, b, part, out, pooled_copy(t, ops, true) != nullptr, stream) : DES_OK;
 }
 
 extern "C" des_status_t des_aggregate(des_table_t* t, uint32_t ops, const des_batch_t* b, const des_partials_t* part,
                                       const des_outputs_t* out, void* stream) {
+  return aggregate_impl(t, ops, b, part, out, false, stream);
+}
+
+// have_b: the pooling kernel of this call has left the bfloat16 copy of the pooled block
+static des_status_t aggregate_impl(des_table_t* t, uint32_t ops, const des_batch_t* b, const des_partials_t* part,
+                                   const des_outputs_t* out, bool have_b, void* stream) {
   if (!t || !b || !part || !out || (ops & ~15u) || ops == 0) return DES_ERR_INVALID_ARG;
   if (b->batch <= 0 || b->batch > t->max_batch) return DES_ERR_INVALID_ARG;
   cudaStream_t cs = (cudaStream_t)stream;
@@ -1205,14 +1213,13 @@ extern "C" des_status_t des_aggregate(des_table_t* t, uint32_t ops, const des_ba
       // materialised per-shard pooled partials: aggregate them in shard order
       des_launch(reduce_shards_kernel, t->sm_count * 4, 256, 0, cs, part->part_pooled, n, (int)t->S, out->pooled);
       DES_LAUNCH_CHECK(t, "reduce_shards_kernel");
-      t->pooled_b_src = nullptr;
     } else if (out->pooled != part->pooled) {
       DES_CUDA(cudaMemcpyAsync(out->pooled, part->pooled, n * 4, cudaMemcpyDeviceToDevice, cs));
     }
   }
   if (ops & DES_OP_DENSE1) {
     if (!t->H || !out->Z) return DES_ERR_INVALID_ARG;
-    des_status_t st = des_dense1_forward(t, out->pooled, B, out->Z, part->part_dense, part->part_pooled, cs);
+    des_status_t st = des_dense1_forward(t, out->pooled, B, out->Z, part->part_dense, part->part_pooled, have_b, cs);
     if (st != DES_OK) return st;
     if (part->part_dense) {
       des_launch(reduce_shards_kernel, t->sm_count * 4, 256, 0, cs, part->part_dense, (size_t)B * t->H, (int)t->S, out->Z);

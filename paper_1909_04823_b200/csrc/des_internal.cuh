@@ -122,7 +122,6 @@ struct des_table {
   float* gW1_part; int gw1_splits;   // [splits][F*k][H]
   int use_tc;                        // tensor-core GEMM path usable for this table's shapes
   __nv_bfloat16 *pooled_b, *gZ_b;    // bf16 copies of V [max_batch][F*k] and gZ [max_batch][H]
-  const float* pooled_b_src;         // the pooled array whose bf16 copy the pooling kernel has just left in pooled_b
                                      // (consumed, once, by the first-layer product that follows); NULL otherwise
   void* gemm_ws; size_t gemm_ws_bytes;
   // host-step staging
@@ -370,7 +369,7 @@ __device__ __forceinline__ bool des_dbg_in(unsigned long long i, unsigned long l
 // shared declarations across translation units
 des_status_t des_check_batch(const des_table* t, const des_batch_t* b, int need_dedup);
 des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float* Z, float* part_dense,
-                                const float* part_pooled, cudaStream_t st);
+                                const float* part_pooled, bool have_b, cudaStream_t st);
 des_status_t des_dense1_backward(des_table* t, const float* pooled, const float* gE, const float* gZ,
                                  float* gE_work, int B, cudaStream_t st);
 // Whether the keys that own a large share of the batch are counted instead of scattered in the backward.
