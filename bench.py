@@ -288,11 +288,17 @@ def occurrence_bytes(name, st):
 
 
 def shift_of(nnz):
-    """log2 of the sampling stride of the backward's hot-key count (about 2^20 samples)."""
+    """log2 of the stride that takes about 2^20 samples of a batch, up to 6."""
     shift = 0
     while shift < 6 and (nnz >> shift) > (1 << 20):
         shift += 1
     return shift
+
+
+def count_shift(nnz):
+    """log2 of the sampling stride of the backward's hot-key count as the library takes it: all of up to 2^17 occurrences, one
+    in four of up to 2^20, one in 16 to 64 of more."""
+    return 0 if nnz <= 1 << 17 else 2 if nnz <= 1 << 20 else max(4, shift_of(nnz))
 
 
 def kernel_flops(name, st):
@@ -479,7 +485,7 @@ def run_workload(args, cfg_index, w, ctx, *, steps, warmup, repeats, modes, want
     stats = dict(nnz=batches[0].nnz, B=B, F=F, k=k, S=S, H=H, U=U, ops=w.ops,
                  adagrad=(w.optimizer == synth.OPT_ADAGRAD), rep_rows=0,
                  super=(k > 28 and batches[0].nnz >= (1 << 20) and batches[0].vals is None),
-                 shift=shift_of(batches[0].nnz), new_keys=(w.p_new > 0 or not w.prepopulate))
+                 shift=count_shift(batches[0].nnz), new_keys=(w.p_new > 0 or not w.prepopulate))
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     for mode in modes:
         graphs = None

@@ -49,6 +49,8 @@
 
 // ROUTE_PF batches of 32 occurrences are in flight per warp: eight where a sample has many (2000 occurrences: 267 us, 324 with
 // two), two where it has few (120: 50 us with eight, 41 with two, whose registers let more warps in).
+// Whole forward of 4 M occurrences, k = 64, two against eight: 120 a sample 327 / 339 us, 512 270 / 278, 1024 233 / 241, 2000 292 / 280:
+// the two meet between 1000 and 2000, and are 3 % apart at the line.
 #define ROUTE_LONG 512          // occurrences per sample, on average, from which it is eight
 template <int ROUTE_PF>
 __global__ void __launch_bounds__(256) route_kernel(
@@ -277,7 +279,10 @@ __device__ __forceinline__ void pool_step(const uint32_t* __restrict__ grow_csr,
 // double), and out_small is written directly — the per-shard partials then never
 // touch memory.
 #define SP_U 4
-#define SP_BRIEF 8       // occurrences per (sample, shard) segment, on average, up to which segments are taken one per sub-group
+// Occurrences per (sample, shard) segment, on average, up to which segments are taken one per sub-group.  LR + FM partials of 3 M
+// occurrences, one per sub-group against one per warp, k = 64: 4 a segment 173 / 214 us, 8 142 / 146, 12 150 / 136; k = 16 (four
+// sub-groups more): 8 85 / 132, 16 89 / 99, 32 99 / 80.
+#define SP_BRIEF 8
 #define SP_FLUSH 4
 // (40 registers, six blocks per SM: 776 -> 752 us at 32 M occurrences of k = 64, 32 and eight: 770; FUSED 64, four: 127 -> 118 at
 // 2.5 M of k = 40)

@@ -27,7 +27,11 @@
 
 #include <type_traits>
 
-#define ASSIGN_DEEP_TILES 16   // tiles per SM from which a block of assign_kernel takes four of them
+// Tiles per SM from which a block of assign_kernel takes four of them.  Known keys only, the deep form is the faster one from 0.5 M
+// occurrences on (whole call: 0.5 M 28 / 27 us, 1 M 38 / 35, 2.1 M 59 / 52, 4.2 M 102 / 87); a batch of new keys needs the lane
+// groups of the other (400 k new keys of k = 64: 120 us in small blocks, 190 in a quarter of them), and how many keys are new is
+// not known when the call is enqueued.
+#define ASSIGN_DEEP_TILES 16
 #define IB 1024  // occurrences per block (tile) in every per-occurrence kernel of this file
 
 // A probe may read a slot through L1 although other SMs claim slots meanwhile: a key never changes once
@@ -47,7 +51,10 @@ __device__ __forceinline__ Slot load_slot(const Slot* p) {
 // per distinct key of a warp costs more in match instructions than the cached slot loads it saves).
 #define PROBE_ILP 1
 #define PROBE_MINB 8
-#define PROBE_MERGE_WAVES 24 // waves of resident blocks up to which blocks merge (3.9 M occurrences: 76 against 88 us; 32 M: 350 against 320)
+// Waves of resident blocks up to which blocks merge (24: 7.3 M occurrences).  Whole call, Zipf 1.2, merged against not: 1 M 38 / 76 us,
+// 4 M 87 / 120, 6.3 M 132 / 169, 8.4 M 169 / 200, 16.8 M 327 / 351 (Zipf 1.05: 421 / 427); on the table of 2e8 keys 32 M 350 /
+// 320 for the kernel.  The two meet between 17 and 32 M: the line is on the safe side.
+#define PROBE_MERGE_WAVES 24
 #define PROBE_MERGE 256   // entries of a block's table of first occurrences (= threads per block)
 
 struct SlotGeom {
