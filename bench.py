@@ -211,14 +211,15 @@ class ClockSampler:
 # the table; kernels that touch table rows move fewer DRAM bytes there (U = 1.06 M instead of 1.81 M).
 NCU_DRAM_TRAFFIC = {
     ("cfg5", "grad_scatter_kernel"): 1811e6,
-    ("cfg5", "super_dense_kernel"): 533e6,
-    ("cfg5", "shard_partials_kernel"): 979e6,
-    ("cfg5", "pool_kernel"): 1212e6,
-    ("cfg5", "update_rows_kernel"): 1945e6,
-    ("cfg5", "probe_claim_kernel"): 596e6,
+    ("cfg5", "super_dense_kernel"): 534e6,
+    ("cfg5", "shard_partials_kernel"): 994e6,
+    ("cfg5", "pool_kernel"): 1211e6,
+    ("cfg5", "update_rows_kernel"): 1954e6,
+    ("cfg5", "probe_claim_kernel"): 595e6,
     ("cfg5", "flag_count_kernel"): 565e6,
     ("cfg5", "resolve_kernel"): 421e6,
     ("cfg5", "make_dest_kernel"): 225e6,
+    ("cfg5", "count_kernel"): 136e6,
     ("cfg5", "route_kernel"): 453e6,
     ("cfg5", "sample_stage_kernel"): 1270e6,
 }
