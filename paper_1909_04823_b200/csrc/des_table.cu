@@ -374,16 +374,16 @@ __device__ __forceinline__ float rows_sq(float v) { return v * v; }
 __device__ __forceinline__ float rows_sq(const float4& v) { return v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w; }
 
 template <int G, typename V>
-__global__ void __launch_bounds__(256) read_rows_kernel(const uint32_t* __restrict__ grows, long long n, int k, int stride,
+__global__ void __launch_bounds__(256, 6) read_rows_kernel(const uint32_t* __restrict__ grows, long long n, int k, int stride,
                                                         unsigned long long total_rows, const float* __restrict__ W,
                                                         const float* __restrict__ A, float* __restrict__ emb,
                                                         float* __restrict__ lin, float* __restrict__ acc_emb,
                                                         float* __restrict__ acc_lin) {
   constexpr int VW = sizeof(V) / 4;
-  des_pdl_wait(grows, W, A, emb, lin, acc_emb, acc_lin);
+  const int zero = des_pdl_wait0();
   const int C = k / VW, lane = threadIdx.x % G;
   // a warp's groups take neighbouring rows, its ROWS_U rounds too
-  const long long i0 = ((long long)blockIdx.x * 256 + (threadIdx.x & ~31)) / G * ROWS_U + (threadIdx.x & 31) / G;
+  const long long i0 = ((long long)blockIdx.x * 256 + (threadIdx.x & ~31)) / G * ROWS_U + (threadIdx.x & 31) / G + zero;
   uint32_t g[ROWS_U];
 #pragma unroll
   for (int q = 0; q < ROWS_U; ++q) {
@@ -391,6 +391,17 @@ __global__ void __launch_bounds__(256) read_rows_kernel(const uint32_t* __restri
     g[q] = i < n ? __ldg(grows + i) : DES_ROW_NONE;
     if (g[q] >= total_rows) g[q] = DES_ROW_NONE;
   }
+  // The tails (linear weight and its state word) are fetched with the columns, not behind their stores, and the kernel is kept to 40
+  // registers: six blocks per SM instead of four (1.6 M random rows of k = 64 with state 405 -> 318 us, 0.4 M 143 -> 110, 0.17 M of k = 32
+  // 20 -> 17, 3 k of k = 8 3.2 -> 2.4).
+  float wt[ROWS_U], at[ROWS_U];
+#pragma unroll
+  for (int q = 0; q < ROWS_U; ++q) {
+    const bool ok = lane == 0 && g[q] != DES_ROW_NONE;
+    wt[q] = ok && lin ? __ldg(W + (size_t)g[q] * stride + k) : 0.f;
+    at[q] = ok && acc_lin && A ? __ldg(A + (size_t)g[q] * stride + k) : 0.f;
+  }
+#pragma unroll 1                                         // (unrolled it takes 62 registers; 16-byte columns need one round)
   for (int c = lane; c < C; c += G) {
     V w[ROWS_U], a[ROWS_U];
 #pragma unroll
@@ -409,15 +420,20 @@ __global__ void __launch_bounds__(256) read_rows_kernel(const uint32_t* __restri
       if (acc_emb) __stcs(reinterpret_cast<V*>(acc_emb + i * k) + c, a[q]);
     }
   }
-  if (lane == 0) {
+  // a warp's ROWS_U * 32 / G rows are neighbours: their tails leave in one store each, a lane per row
+  constexpr int NG = 32 / G;
+  const int wl = threadIdx.x & 31;
+  for (int l = wl; l < ROWS_U * NG + (32 - ROWS_U * NG % 32) % 32; l += 32) {   // (whole warps; one round unless G is 1 or 2)
+    float w = 0.f, a = 0.f;
 #pragma unroll
     for (int q = 0; q < ROWS_U; ++q) {
-      const long long i = i0 + q * (32 / G);
-      if (i >= n) continue;
-      const bool ok = g[q] != DES_ROW_NONE;
-      if (lin) lin[i] = ok ? W[(size_t)g[q] * stride + k] : 0.f;
-      if (acc_lin) acc_lin[i] = (ok && A) ? A[(size_t)g[q] * stride + k] : 0.f;
+      const float x = __shfl_sync(0xFFFFFFFFu, wt[q], l % NG * G), y = __shfl_sync(0xFFFFFFFFu, at[q], l % NG * G);
+      if (l / NG == q) { w = x; a = y; }
     }
+    const long long i = i0 - wl / G + l;
+    if (l >= ROWS_U * NG || i >= n) continue;
+    if (lin) lin[i] = w;
+    if (acc_lin) acc_lin[i] = a;
   }
 }
 
