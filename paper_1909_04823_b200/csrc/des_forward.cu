@@ -429,6 +429,27 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16* dst, const float4& v
   *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
 }
 
+// U rows of a lane in flight: positions i, i + P, ... of a list, below hi.
+template <int U, int P, bool HAS_VALS>
+__device__ __forceinline__ void list_round(const uint32_t* list, const float* xs, int i, int hi, const char* __restrict__ Wc,
+                                           unsigned rowB, float4& acc) {
+  float4 v[U]; float x[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const bool in = i + u * P < hi;
+    v[u] = make_float4(0.f, 0.f, 0.f, 0.f); x[u] = 0.f;
+    if (in) {
+      v[u] = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)DES_DBG_ROW(list[i + u * P]) * rowB));
+      if (HAS_VALS) x[u] = __ldg(xs + i + u * P);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (HAS_VALS) { v[u].x *= x[u]; v[u].y *= x[u]; v[u].z *= x[u]; v[u].w *= x[u]; }
+    acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w;
+  }
+}
+
 template <int G, int P, bool HAS_VALS, bool MATERIALISE, bool BF16OUT>
 __global__ void __launch_bounds__(256) pool_kernel(
     const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ grow_csr,
@@ -461,10 +482,15 @@ __global__ void __launch_bounds__(256) pool_kernel(
     int i0 = lo;
 #define POOL_STEP(U) pool_step<U, P, HAS_VALS, MATERIALISE>(grow_csr, vals, shards, i0 + p, Wc, rowB, null_row, part_block, \
                                                            shard_pitch, col, acc)
+    if constexpr (P == 1 && !MATERIALISE) {            // (short bags: whole rounds, the last one masked, are a shorter chain: bags of 4,
+                                                       // k = 64, 3.9 M occurrences 130 -> 120 us, 2 M 69 -> 64)
+      for (; i0 < hi; i0 += 4) list_round<4, 1, HAS_VALS>(grow_csr, vals, i0, hi, Wc, rowB, acc);
+    } else {
     for (; i0 + 4 * P <= hi; i0 += 4 * P) POOL_STEP(4);
     if (i0 + 2 * P <= hi) { POOL_STEP(2); i0 += 2 * P; }
     if (i0 + P <= hi) { POOL_STEP(1); i0 += P; }
     if (i0 + p < hi) POOL_STEP(1);
+    }
 #undef POOL_STEP
 #pragma unroll
     for (int d = G; d < LB; d <<= 1) {                 // combine the bag's sub-groups
