@@ -1,0 +1,29 @@
+"""Hot keys of batches around the sizes where the counting changes its form (one block, many blocks, larger blocks, a sample): keys that own a
+quarter of the batch, hundreds of keys just above and below the threshold, and none at all.  Against sums in double."""
+import pytest
+import torch
+
+from test_gpu_hot_keys_batches import _Step
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,F,n", [(1, 1, 130), (127, 8, 1), (1024, 8, 1), (8193, 1, 1), (2048, 8, 1), (16385, 1, 1), (4095, 16, 1), (4097, 16, 1),
+                                   (5000, 26, 1), (20000, 16, 1)])
+@pytest.mark.parametrize("law", ["heavy", "level", "distinct"])
+def test_sums_per_key(B, F, n, law):
+    from paper_1909_04823_b200 import binding as D
+    g = torch.Generator(device="cuda").manual_seed(B + F)
+    nnz, k = B * F * n, 20
+    t = D.Table(4, F, k, optimizer=D.OPT_SGD, lr=1.0, max_rows=nnz + 5000, seed=3, init_scale=0.0, max_nnz=nnz, max_batch=B)
+    try:
+        s = _Step(D, t, g, B, F, n, k, 1e6)
+        if law == "level":                                 # every key about 128 times
+            s.db.ids.copy_(torch.randint(0, max(1, nnz // 128), (nnz,), generator=g, device="cuda") * 31 + 7)
+        elif law == "distinct":
+            s.db.ids.copy_(torch.randperm(nnz, generator=g, device="cuda") * 31 + 7)
+        for _ in range(2):                                 # (the second: nothing is left behind by the first)
+            s.insert(); s.clear(); s.backward(); s.check((law, nnz))
+        assert t.status() == 0
+    finally:
+        t.close()
