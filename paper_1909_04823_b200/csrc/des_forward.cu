@@ -39,7 +39,13 @@
 
 #include "des_internal.cuh"
 
-#define SGF_BU 4                  // short bags of a lane group in flight together (sample_gather_kernel)
+// Short bags of a lane group in flight together (sample_gather_kernel) and resident blocks: SGF_FEW at three where the chip then holds all
+// bags of the batch at once and what counts is one group's chain of loads; else more warps instead of more rows of a warp, one bag at
+// six, or two at five where a warp has eight groups and more.  (FIELD, 16384 x 39 fields, k = 32: four at three 73 us, two at five 57, one at six
+// 53, one at five 57; 8192 x 26, k = 16: 16.2 / 15.3 / 16.9 / 16.5.  The form without FIELD has sums in double to keep: a block less.)
+#define SGF_FEW 4
+#define SGF_MINB(bags, field) ((bags) == SGF_FEW ? 3 : (bags) == 2 ? ((field) ? 5 : 4) : (field) ? 6 : 5)
+#define SGF_MANY(G) ((G) > 4 ? 1 : 2)
 #define SGF_SMEM (24u << 10)      // shared memory a block of the FIELD form takes at most, unless one sample needs more
 #define SGF_ONE ((48u << 10) - DES_MAX_SHARDS * 4)   // and at most for one sample: a launch has 48 KiB, the kernel's own s_base included
 #ifndef POOL_BLOCKS_PER_SM
@@ -623,7 +629,7 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
 
 // ---- gather and reduce in one pass ---------------------------------------------------------------------
 // The same sums with a sample's bags kept together: WPS = 8 / T warps take a sample, T samples a block.  Every lane group
-// of a warp walks bags of its own, SGF_BU short ones with their first occurrences in flight together (a one-hot
+// of a warp walks bags of its own, a few short ones with their first occurrences in flight together (a one-hot
 // batch is a chain offsets -> row number -> row per bag).
 //  FIELD = false  (the fused form): the groups add their bags in double as they go, and the sample's sums are combined by
 //                 shuffles and, over its warps, in shared memory.  Against a gather and a second pass over its output the
@@ -635,8 +641,8 @@ __global__ void __launch_bounds__(256) single_gather_kernel(
 //                 partials are added in double in shard order and passed through F, as aggregate_small_kernel does.
 //                 (16384 x 39 fields, k = 32: 92 -> 79 us against single_gather + field_partials.)
 // The sums over fields are taken in double in a fixed order that depends on WPS, i.e. on the batch size.
-template <int G, int P, bool HAS_VALS, bool FIELD>
-__global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
+template <int G, int P, bool HAS_VALS, bool FIELD, int BAGS>
+__global__ void __launch_bounds__(256, P > 1 ? 4 : SGF_MINB(BAGS, FIELD)) sample_gather_kernel(
     const int32_t* __restrict__ offsets, const float* __restrict__ vals, const uint32_t* __restrict__ rows,
     const uint8_t* __restrict__ shards, int B, int F, int S, int k, int T, uint32_t ops, const float* __restrict__ W,
     const DevMeta* __restrict__ meta, uint32_t null_row, float* __restrict__ pooled, __nv_bfloat16* __restrict__ pooled_b,
@@ -644,7 +650,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
   constexpr int LB = G * P, GW = 32 / LB;              // lanes per bag, bags per warp
   static_assert(FIELD || P == 1, "long bags of the fused form: sample_stage_kernel");
   constexpr bool COOP = P > 1;
-  constexpr int BU = COOP ? 1 : SGF_BU;                // bags of a group in flight together (long bags: their own rows are)
+  constexpr int BU = COOP ? 1 : BAGS;                  // bags of a group in flight together (long bags: their own rows are)
   extern __shared__ __align__(16) unsigned char sg_smem[];
   __shared__ uint32_t s_base[DES_MAX_SHARDS];
   __shared__ double s_red[FIELD ? 1 : 8][FIELD ? 1 : G][4], s_tail[FIELD ? 1 : 8][2];
@@ -685,7 +691,7 @@ __global__ void __launch_bounds__(256, P > 1 ? 4 : 3) sample_gather_kernel(
       if (f < F) { lo_n[q] = __ldg(off + f); hi_n[q] = __ldg(off + f + 1); }
       acc[q] = make_float4(0.f, 0.f, 0.f, 0.f); bl[q] = 0.f; bq[q] = 0.f;
     }
-    if (BU > 1) {                                      // the bags' first occurrences
+    if constexpr (!COOP) {                             // the bags' first occurrences
       uint32_t g[BU]; float x[BU];
 #pragma unroll
       for (int q = 0; q < BU; ++q) {
@@ -1157,15 +1163,17 @@ static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des
                                          __nv_bfloat16* pb, float* part_small, float* out_small, cudaStream_t cs) {
   const int B = b->batch, F = (int)t->F, G = group_for(t->k);
   const bool wide = b->nnz >= 8ll * B * F;
-  const int per_warp = wide ? 1 : 32 / G * SGF_BU;      // bags a warp has in flight
+  const int bags = wide ? 1 : (long long)B * F > (long long)t->sm_count * 8 * SGF_MINB(SGF_FEW, field) * (32 / G) * SGF_FEW ? SGF_MANY(G) : SGF_FEW;
+  const int per_warp = wide ? 1 : 32 / G * bags;       // bags a warp has in flight
   int T = 8;
   while (T > 1 && (B < t->sm_count * 4 * T || (wide && b->nnz >= 256ll * B)) && F > per_warp * (8 / T)) T >>= 1;
   const size_t per_sample = field ? (size_t)F * (t->k + 2) * 4 : 0;
   while (T > 1 && T * per_sample > SGF_SMEM) T >>= 1;
   const unsigned grid = (unsigned)((B + T - 1) / T);
-#define SF4(GG, PP, HV, FD) des_launch(sample_gather_kernel<GG, PP, HV, FD>, grid, 256, T * per_sample, cs, b->offsets, b->vals,     \
+#define SF5(GG, PP, HV, FD, BU) des_launch(sample_gather_kernel<GG, PP, HV, FD, BU>, grid, 256, T * per_sample, cs, b->offsets, b->vals,     \
                                        b->rows, b->shards, B, F, (int)t->S, (int)t->k, T, ops, t->W, t->meta,                     \
                                        (uint32_t)t->total_rows, pooled, pb, part_small, out_small)
+#define SF4(GG, PP, HV, FD) do { if (PP > 1) SF5(GG, PP, HV, FD, 1); else if (bags == SGF_FEW) SF5(GG, PP, HV, FD, SGF_FEW); else SF5(GG, PP, HV, FD, SGF_MANY(GG)); } while (0)
 #define SS(GG, HV) des_launch(sample_stage_kernel<GG, 32 / GG, HV>, grid, 256, 0, cs, b->offsets, b->vals, b->rows, b->shards, B, F, \
                               (int)t->S, (int)t->k, T, ops, t->W, t->meta, (uint32_t)t->total_rows, pooled, pb, out_small)
 #define SF2(GG, HV) do { if (!wide) { if (field) SF4(GG, 1, HV, true); else SF4(GG, 1, HV, false); }                              \
@@ -1176,6 +1184,7 @@ static des_status_t launch_sample_gather(des_table_t* t, uint32_t ops, const des
 #undef SF2
 #undef SS
 #undef SF4
+#undef SF5
   DES_LAUNCH_CHECK(t, wide && !field ? "sample_stage_kernel" : "sample_gather_kernel");
   return DES_OK;
 }
