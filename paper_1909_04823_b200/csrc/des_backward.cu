@@ -707,39 +707,28 @@ static des_status_t backward_args(const des_table* t, uint32_t ops, const des_ou
   return DES_OK;
 }
 
-extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const des_batch_t* b,
-                                            const des_outputs_t* out, const des_grads_t* gr, void* stream) {
-  des_status_t st = des_check_batch(t, b, 1);
-  if (st != DES_OK) return st;
-  if ((st = backward_args(t, ops, out, gr)) != DES_OK) return st;
-  cudaStream_t cs = (cudaStream_t)stream;
-  des_api_begin(t, cs);
-  DES_DBG_ARM(t, cs);
-  const int B = b->batch;
-  const OptParams opt = des_opt_params(t);
-  if (opt.optimizer == DES_OPT_ADAM) {               // one optimizer step per backward call (Adam's t)
-    adam_tick_kernel<<<1, 1, 0, cs>>>(t->meta, opt.beta1, opt.beta2);
-    DES_LAUNCH_CHECK(t, "adam_tick_kernel");
-  }
-  const float* gE = (ops & DES_OP_POOL) ? gr->gE : nullptr;
-  if (ops & DES_OP_DENSE1) {
-    st = des_dense1_backward(t, out->pooled, gE, gr->gZ, gr->gE_work, B, cs);
-    if (st != DES_OK) return st;
-    gE = gr->gE_work;
-  }
-  if (b->nnz == 0) return DES_OK;
-  const int G = group_for(t->k);
-  const int nnz = (int)b->nnz;
-  const long long nbags = (long long)B * t->F;
-  if ((st = des_count_batch(t, b, cs)) != DES_OK) return st;
-  const bool use_super = des_super_path(t, b);
+// Counts, hot keys and, for a batch of many occurrences, every occurrence's gradient row.
+static DestMap dest_map(const des_table* t, const des_batch_t* b) {
   DestMap dm;
   dm.uidx = b->uidx; dm.hinfo = t->hinfo; dm.hot_rep = t->hot_rep; dm.max_uniq = (uint32_t)t->max_uniq; dm.dest = t->dest;
-  const bool inl = nnz < DEST_INLINE;
-  if (!inl) {
-    des_launch(make_dest_kernel, (nnz + 1023) / 1024, 256, 0, cs, dm, nnz);
-    DES_LAUNCH_CHECK(t, "make_dest_kernel");
-  }
+  return dm;
+}
+static des_status_t backward_dest(des_table* t, const des_batch_t* b, cudaStream_t cs) {
+  const des_status_t st = des_count_batch(t, b, cs);
+  if (st != DES_OK || b->nnz < DEST_INLINE) return st;
+  des_launch(make_dest_kernel, ((int)b->nnz + 1023) / 1024, 256, 0, cs, dest_map(t, b), (int)b->nnz);
+  DES_LAUNCH_CHECK(t, "make_dest_kernel");
+  return DES_OK;
+}
+
+// Scatter into the gradient rows, then the update of the keys.
+static des_status_t backward_rows(des_table* t, uint32_t ops, const des_batch_t* b, const des_outputs_t* out, const des_grads_t* gr,
+                                  const OptParams& opt, cudaStream_t cs) {
+  const int G = group_for(t->k), nnz = (int)b->nnz;
+  const long long nbags = (long long)b->batch * t->F;
+  const float* gE = (ops & DES_OP_DENSE1) ? gr->gE_work : (ops & DES_OP_POOL) ? gr->gE : nullptr;
+  const bool use_super = des_super_path(t, b), inl = nnz < DEST_INLINE;
+  const DestMap dm = dest_map(t, b);
   {
     // long bags: a whole warp per bag (its sub-groups take alternate occurrences); short bags: G lanes per bag
     const bool wide = (long long)nnz >= 8 * nbags;   // (at 4 ids per bag the narrow form measured faster)
@@ -801,6 +790,74 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
     DES_LAUNCH_CHECK(t, "update_rows_kernel");
   }
   return DES_OK;
+}
+
+#define SIDE_MIN (5ll << 20)      // entries of gE from which the backward takes this form
+// The whole backward with a first layer: on the caller's stream the operands' conversion, gE, scatter and update; on the side stream
+// the count and look-up of gradient rows, the weight gradient and, once gE has been formed (it reads the weights' bfloat16 copy),
+// the weights' update.  The caller's stream waits for the side stream before the call's work is over, also when a part fails.
+// Backward, one after the other against this, H = 400, 39 fields, k = 32: 16384 samples 189 / 174 us, 8192 112 / 105, 4096 72 / 65; H = 136, 53
+// fields, k = 8: 16384 109 / 98; H = 256, 26 fields, k = 16: 16384 82 / 79, 8192 51 / 50 — and there the step as a whole loses, 136 -> 144,
+// because kernels behind an event do not overlap the one before.  The line is between the last two.
+static des_status_t backward_beside(des_table* t, uint32_t ops, const des_batch_t* b, const des_outputs_t* out, const des_grads_t* gr,
+                                    const Dense1Plan& p, const OptParams& opt, cudaStream_t cs) {
+  const float* gE = (ops & DES_OP_POOL) ? gr->gE : nullptr;
+  DES_CUDA(cudaEventRecord(t->side_fork, cs));
+  DES_CUDA(cudaStreamWaitEvent(t->side, t->side_fork, 0));
+  int rc = 0;
+  auto parts = [&]() -> des_status_t {
+    des_status_t st;
+    if ((st = backward_dest(t, b, t->side)) != DES_OK) return st;
+    DES_CUDA(cudaEventRecord(t->side_dest, t->side));
+    if ((st = des_dense1_dgrad(t, p, out->pooled, gE, gr->gZ, gr->gE_work, b->batch, &rc, cs)) != DES_OK) return st;
+    if (rc != 0 && (st = des_dense1_backward_plain(t, out->pooled, gE, gr->gZ, gr->gE_work, b->batch, cs)) != DES_OK) return st;
+    if (rc == 0) {                                       // (enqueued first, so that its few large blocks find room beside the scatter's)
+      DES_CUDA(cudaEventRecord(t->side_gE, cs));
+      DES_CUDA(cudaStreamWaitEvent(t->side, t->side_gE, 0));
+      if ((st = des_dense1_wgrad(t, p, t->side)) != DES_OK || (st = des_dense1_update(t, p, t->side)) != DES_OK) return st;
+    }
+    DES_CUDA(cudaStreamWaitEvent(cs, t->side_dest, 0));
+    return backward_rows(t, ops, b, out, gr, opt, cs);
+  };
+  const des_status_t st = parts();
+  const bool joined = cudaEventRecord(t->side_join, t->side) == cudaSuccess && cudaStreamWaitEvent(cs, t->side_join, 0) == cudaSuccess;
+  return st == DES_OK && !joined ? DES_ERR_CUDA : st;
+}
+
+extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const des_batch_t* b,
+                                            const des_outputs_t* out, const des_grads_t* gr, void* stream) {
+  des_status_t st = des_check_batch(t, b, 1);
+  if (st != DES_OK) return st;
+  if ((st = backward_args(t, ops, out, gr)) != DES_OK) return st;
+  cudaStream_t cs = (cudaStream_t)stream;
+  des_api_begin(t, cs);
+  DES_DBG_ARM(t, cs);
+  const int B = b->batch;
+  const OptParams opt = des_opt_params(t);
+  if (opt.optimizer == DES_OPT_ADAM) {               // one optimizer step per backward call (Adam's t)
+    adam_tick_kernel<<<1, 1, 0, cs>>>(t->meta, opt.beta1, opt.beta2);
+    DES_LAUNCH_CHECK(t, "adam_tick_kernel");
+  }
+  if ((ops & DES_OP_DENSE1) && t->use_tc) {
+    const Dense1Plan p = des_dense1_plan(t, B);
+    // What the sparse backward does not wait for goes to the table's side stream: the count and the gradient rows' look-up beside
+    // the product that forms gE, the weight gradient beside the scatter.  (Not while launches are being timed one by one.)
+    if (b->nnz && (long long)B * p.FK >= SIDE_MIN && !t->prof_on) return backward_beside(t, ops, b, out, gr, p, opt, cs);
+    const float* gE = (ops & DES_OP_POOL) ? gr->gE : nullptr;
+    int rc = 0;
+    if ((st = des_dense1_dgrad(t, p, out->pooled, gE, gr->gZ, gr->gE_work, B, &rc, cs)) != DES_OK) return st;
+    if (rc == 0) {
+      if ((st = des_dense1_wgrad(t, p, cs)) != DES_OK || (st = des_dense1_update(t, p, cs)) != DES_OK) return st;
+    } else if ((st = des_dense1_backward_plain(t, out->pooled, gE, gr->gZ, gr->gE_work, B, cs)) != DES_OK) {
+      return st;
+    }
+  } else if (ops & DES_OP_DENSE1) {
+    if ((st = des_dense1_backward_plain(t, out->pooled, (ops & DES_OP_POOL) ? gr->gE : nullptr, gr->gZ, gr->gE_work, B, cs)) != DES_OK)
+      return st;
+  }
+  if (b->nnz == 0) return DES_OK;
+  if ((st = backward_dest(t, b, cs)) != DES_OK) return st;
+  return backward_rows(t, ops, b, out, gr, opt, cs);
 }
 
 // ---- whole step from host buffers ---------------------------------------------

@@ -221,37 +221,60 @@ des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float*
   return DES_OK;
 }
 
-des_status_t des_dense1_backward(des_table* t, const float* pooled, const float* gE, const float* gZ,
-                                 float* gE_work, int B, cudaStream_t st) {
+// The backward on the tensor cores, in parts that des_backward_update orders: what the sparse backward waits for (the operands'
+// conversion, gE) comes first; the weight gradient and its update can run beside the scatter.
+Dense1Plan des_dense1_plan(const des_table* t, int B) {
+  // The weight gradient has few output tiles (F*k x H) and a long contraction (the batch): the batch is cut into L pieces so
+  // that every SM gets a tile (L partial products, added in piece order by w1_update_kernel).  The pieces are of
+  // equal length, a multiple of 64 samples; zero rows fill the last one up.
+  Dense1Plan p;
+  p.FK = (int)(t->F * t->k);
+  p.wide = (long long)p.FK * t->H >= DES_TC_WIDE_WGRAD && B >= DES_TC_WIDE_BATCH;
+  const int tiles = p.wide ? ((p.FK + 255) / 256) * (((int)t->H + 255) / 256) : ((p.FK + 127) / 128) * (((int)t->H + 63) / 64);
+  int L = (p.wide ? t->sm_count / 2 : t->sm_count) / tiles;            // (a wide tile is a pair of SMs')
+  if (L > B / 256) L = B / 256;
+  if (L > t->gw1_splits) L = t->gw1_splits;
+  if (L < 1) L = 1;
+  p.piece = L == 1 ? B : ((B + L - 1) / L + 63) / 64 * 64;
+  p.L = (B + p.piece - 1) / p.piece;
+  return p;
+}
+
+// gE_work = gE + gZ W1^T; both operands of the backward are converted on the way.  *rc: 1 = shapes the products cannot take (nothing
+// has been formed), 0 = done.
+des_status_t des_dense1_dgrad(des_table* t, const Dense1Plan& p, const float* pooled, const float* gE, const float* gZ,
+                              float* gE_work, int B, int* rc, cudaStream_t st) {
+  const size_t n1 = (size_t)B * t->H, n2 = (size_t)B * p.FK, p1 = (size_t)p.piece * p.L * t->H, p2 = (size_t)p.piece * p.L * p.FK;
+  launch_cvt(gZ, t->gZ_b, n1, p1, pooled, t->pooled_b, n2, p2, st);
+  DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
+  *rc = des_tc_gemm_dgrad(B, p.FK, (int)t->H, 1, t->gZ_b, t->W1b, gE ? gE : gE_work, gE_work, gE ? 1.f : 0.f, t->gemm_ws,
+                          t->gemm_ws_bytes / 2, st);
+  if (*rc == 1) return DES_OK;
+  if (*rc != 0) return DES_ERR_CUDA;
+  DES_LAUNCH_CHECK(t, "tc_gemm_dgrad");
+  return DES_OK;
+}
+
+// gW1 = V^T gZ (piece by piece) from the operands that des_dense1_dgrad left.
+des_status_t des_dense1_wgrad(des_table* t, const Dense1Plan& p, cudaStream_t st) {
+  const int rc = des_tc_gemm_wgrad(p.FK, (int)t->H, p.piece, p.L, t->pooled_b, t->gZ_b, t->gW1_part, t->gW1_part, 0.f,
+                                   (char*)t->gemm_ws + t->gemm_ws_bytes / 2, t->gemm_ws_bytes / 2, st);
+  if (rc != 0) return DES_ERR_CUDA;                // same alignment rules as the dgrad: cannot differ
+  DES_LAUNCH_CHECK(t, "tc_gemm_wgrad");
+  return DES_OK;
+}
+
+// The optimizer on W1 and its bfloat16 copy, which des_dense1_dgrad reads.
+des_status_t des_dense1_update(des_table* t, const Dense1Plan& p, cudaStream_t st) {
+  launch_w1_update(t, p.L, st);
+  DES_LAUNCH_CHECK(t, "w1_update_kernel");
+  return DES_OK;
+}
+
+// The backward on the CUDA cores, for shapes that the products cannot take.
+des_status_t des_dense1_backward_plain(des_table* t, const float* pooled, const float* gE, const float* gZ, float* gE_work, int B,
+                                       cudaStream_t st) {
   const int FK = t->F * t->k;
-  if (t->use_tc) {
-    // The weight gradient has few output tiles (F*k x H) and a long contraction (the batch): the batch is cut into L pieces so
-    // that every SM gets a tile (L partial products, added in piece order by w1_update_kernel).  The pieces are of
-    // equal length, a multiple of 64 samples; zero rows fill the last one up.
-    const int tiles = ((FK + 127) / 128) * ((t->H + 63) / 64);
-    int L = t->sm_count / tiles;
-    if (L > B / 256) L = B / 256;
-    if (L > t->gw1_splits) L = t->gw1_splits;
-    if (L < 1) L = 1;
-    const int piece = L == 1 ? B : ((B + L - 1) / L + 63) / 64 * 64;
-    L = (B + piece - 1) / piece;
-    const size_t n1 = (size_t)B * t->H, n2 = (size_t)B * FK, p1 = (size_t)piece * L * t->H, p2 = (size_t)piece * L * FK;
-    launch_cvt(gZ, t->gZ_b, n1, p1, pooled, t->pooled_b, n2, p2, st);
-    DES_LAUNCH_CHECK(t, "cvt_bf16_kernel");
-    const int rc1 = des_tc_gemm_dgrad(B, FK, t->H, 1, t->gZ_b, t->W1b, gE ? gE : gE_work, gE_work, gE ? 1.f : 0.f,
-                                      t->gemm_ws, t->gemm_ws_bytes, st);
-    if (rc1 == 0) {
-      DES_LAUNCH_CHECK(t, "tc_gemm_dgrad");
-      const int rc2 = des_tc_gemm_wgrad(FK, t->H, piece, L, t->pooled_b, t->gZ_b, t->gW1_part, t->gW1_part, 0.f,
-                                        t->gemm_ws, t->gemm_ws_bytes, st);
-      if (rc2 != 0) return DES_ERR_CUDA;           // same alignment rules as the dgrad: cannot differ
-      DES_LAUNCH_CHECK(t, "tc_gemm_wgrad");
-      launch_w1_update(t, L, st);
-      DES_LAUNCH_CHECK(t, "w1_update_kernel");
-      return DES_OK;
-    }
-    if (rc1 != 1) return DES_ERR_CUDA;
-  }
   {  // gE_work = gE + gZ W1^T
     GemmArgs g; memset(&g, 0, sizeof(g));
     g.M = B; g.N = FK; g.K = t->H; g.A32 = gZ; g.Bb = t->W1b; g.add = gE; g.out = gE_work;

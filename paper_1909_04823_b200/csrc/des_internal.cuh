@@ -123,7 +123,9 @@ struct des_table {
   int use_tc;                        // tensor-core GEMM path usable for this table's shapes
   __nv_bfloat16 *pooled_b, *gZ_b;    // bf16 copies of V [max_batch][F*k] and gZ [max_batch][H]
                                      // (consumed, once, by the first-layer product that follows); NULL otherwise
-  void* gemm_ws; size_t gemm_ws_bytes;
+  void* gemm_ws; size_t gemm_ws_bytes;   // halves: the two products of a backward can overlap
+  cudaStream_t side;                 // the part of a backward that nothing of the rest waits for runs here, between two events of the
+  cudaEvent_t side_fork, side_dest, side_gE, side_join;   // caller's stream (NULL: no first layer)
   // host-step staging
   int32_t* st_offsets[2]; unsigned long long* st_ids[2]; float* st_vals[2];   // two input slots (pipelined submit)
   cudaStream_t st_copy_stream; cudaEvent_t st_copied[2], st_done[2]; int st_busy[2]; uint64_t st_next;
@@ -370,8 +372,14 @@ __device__ __forceinline__ bool des_dbg_in(unsigned long long i, unsigned long l
 des_status_t des_check_batch(const des_table* t, const des_batch_t* b, int need_dedup);
 des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float* Z, float* part_dense,
                                 const float* part_pooled, bool have_b, cudaStream_t st);
-des_status_t des_dense1_backward(des_table* t, const float* pooled, const float* gE, const float* gZ,
-                                 float* gE_work, int B, cudaStream_t st);
+struct Dense1Plan { int FK, piece, L; };   // F*k; samples of a piece of the weight gradient's contraction, pieces
+Dense1Plan des_dense1_plan(const des_table* t, int B);
+des_status_t des_dense1_dgrad(des_table* t, const Dense1Plan& p, const float* pooled, const float* gE, const float* gZ,
+                              float* gE_work, int B, int* rc, cudaStream_t st);
+des_status_t des_dense1_wgrad(des_table* t, const Dense1Plan& p, cudaStream_t st);
+des_status_t des_dense1_update(des_table* t, const Dense1Plan& p, cudaStream_t st);
+des_status_t des_dense1_backward_plain(des_table* t, const float* pooled, const float* gE, const float* gZ, float* gE_work, int B,
+                                       cudaStream_t st);
 // Whether the keys that own a large share of the batch are counted instead of scattered in the backward.
 bool des_super_path(const des_table* t, const des_batch_t* b);
 // Counts a batch's occurrences per unique key (a sample of a large batch) and makes the hot list: opens a backward.

@@ -120,6 +120,8 @@ extern "C" des_status_t des_table_destroy(des_table_t* t) {
     for (int s = 0; s < 2; ++s)
       for (cudaEvent_t e : {t->st_copied[s], t->st_done[s], t->st_fwd[s], t->st_out[s]}) if (e) cudaEventDestroy(e);
   }
+  if (t->side) cudaStreamDestroy(t->side);
+  for (cudaEvent_t e : {t->side_fork, t->side_dest, t->side_gE, t->side_join}) if (e) cudaEventDestroy(e);
   if (t->prof_ev) { for (int i = 0; i < DES_PROF_MAX; ++i) cudaEventDestroy(t->prof_ev[i]); delete[] t->prof_ev; }
   delete[] t->prof_name;
   const int own_dev = t->device;
@@ -264,6 +266,9 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
     cu &= cudaMemset(t->W1, 0, FKH * 4) == cudaSuccess;
     cu &= cudaMemset(t->W1b, 0, FKH * 2) == cudaSuccess;
     fill_f32_kernel<<<256, 256>>>(t->accW1, FKH, c.optimizer == DES_OPT_ADAGRAD ? c.init_acc : 0.f);
+    cu &= cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t* e : {&t->side_fork, &t->side_dest, &t->side_gE, &t->side_join})
+      cu &= cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
     if (t->acc2W1) cu &= cudaMemset(t->acc2W1, 0, FKH * 4) == cudaSuccess;
     cu &= cudaGetLastError() == cudaSuccess;
   }
