@@ -229,8 +229,9 @@ Dense1Plan des_dense1_plan(const des_table* t, int B) {
   // equal length, a multiple of 64 samples; zero rows fill the last one up.
   Dense1Plan p;
   p.FK = (int)(t->F * t->k);
-  const int tiles = ((p.FK + 127) / 128) * (((int)t->H + 63) / 64);
-  int L = t->sm_count / tiles;
+  p.wide = (long long)p.FK * t->H >= DES_TC_WIDE_WGRAD && B >= DES_TC_WIDE_BATCH;
+  const int tiles = p.wide ? ((p.FK + 255) / 256) * (((int)t->H + 255) / 256) : ((p.FK + 127) / 128) * (((int)t->H + 63) / 64);
+  int L = (p.wide ? t->sm_count / 2 : t->sm_count) / tiles;            // (a wide tile is a pair of SMs')
   if (L > B / 256) L = B / 256;
   if (L > t->gw1_splits) L = t->gw1_splits;
   if (L < 1) L = 1;
@@ -256,7 +257,7 @@ des_status_t des_dense1_dgrad(des_table* t, const Dense1Plan& p, const float* po
 
 // gW1 = V^T gZ (piece by piece) from the operands that des_dense1_dgrad left.
 des_status_t des_dense1_wgrad(des_table* t, const Dense1Plan& p, cudaStream_t st) {
-  const int rc = des_tc_gemm_wgrad(p.FK, (int)t->H, p.piece, p.L, t->pooled_b, t->gZ_b, t->gW1_part, t->gW1_part, 0.f,
+  const int rc = des_tc_gemm_wgrad(p.wide, p.FK, (int)t->H, p.piece, p.L, t->pooled_b, t->gZ_b, t->gW1_part, t->gW1_part, 0.f,
                                    (char*)t->gemm_ws + t->gemm_ws_bytes / 2, t->gemm_ws_bytes / 2, st);
   if (rc != 0) return DES_ERR_CUDA;                // same alignment rules as the dgrad: cannot differ
   DES_LAUNCH_CHECK(t, "tc_gemm_wgrad");

@@ -372,7 +372,7 @@ __device__ __forceinline__ bool des_dbg_in(unsigned long long i, unsigned long l
 des_status_t des_check_batch(const des_table* t, const des_batch_t* b, int need_dedup);
 des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float* Z, float* part_dense,
                                 const float* part_pooled, bool have_b, cudaStream_t st);
-struct Dense1Plan { int FK, piece, L; };   // F*k; samples of a piece of the weight gradient's contraction, pieces
+struct Dense1Plan { int FK, piece, L; bool wide; };   // F*k; samples of a piece of the weight gradient's contraction, pieces, tile
 Dense1Plan des_dense1_plan(const des_table* t, int B);
 des_status_t des_dense1_dgrad(des_table* t, const Dense1Plan& p, const float* pooled, const float* gE, const float* gZ,
                               float* gE_work, int B, int* rc, cudaStream_t st);

@@ -15,7 +15,10 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
-#define DES_TC_WIDE_OUTPUTS (4ll << 20)   // outputs (M x N) from which a product takes the wide tile
+#define DES_TC_WIDE_FWD (3ll << 19)       // outputs (M x N) from which a product takes the wide tile
+#define DES_TC_WIDE_DGRAD (4ll << 20)
+#define DES_TC_WIDE_WGRAD (1ll << 18)     // (weights; and a batch of DES_TC_WIDE_BATCH samples)
+#define DES_TC_WIDE_BATCH 2048
 
 #if defined(DES_TC_GEMM_DECL_ONLY)
 /* prototypes only */
@@ -29,15 +32,19 @@
 #include "cutlass/epilogue/collective/collective_builder.hpp"
 #include "cutlass/util/packed_stride.hpp"
 
-// TileN: a small product is bound by the latency of its few tiles, so narrow ones (64 columns) spread it over the SMs; a
-// large one by what the tiles read from L2 per product, so wide ones (192).  Measured, 128 columns before: 777 x 1248 x
-// 400 forward 7.1 -> 5.2 us, 16384 x 1248 x 400 backward 49 -> 41, weight gradient 32 -> 29 (64 columns, any size).
-// Around the line, conversion and product, 64 against 192 columns: forward of 1248 x 400 0.8 M outputs 17 / 21 us, 2.5 M 34 / 30, 3.3 M
-// 40 / 40, 4.9 M 53 / 49; of 416 x 256 2.1 M 17 / 19, 4.2 M 26 / 28; backward of 1248 x 400 2.6 M 56 / 55, 10 M 117 / 113.
+// Tiles: a small product is bound by the latency of its few tiles, so narrow ones (128 x 64) spread it over the SMs; a
+// large one by what the tiles read from L2 per product, so wide ones: 256 rows on a pair of SMs (cta_group::2, each CTA loads half of the
+// columns' operand and both multiply by it) by 256 columns, 192 where the result is wide.  Measured, products alone, 128 x 64 / 128 x 192
+// / the pair's tile:
+//   forward          16384 x 1248 x 400 (6.6 M outputs) 38 / 34 / 26 us, 16384 x 1696 x 400 46 / 40 / 30, 5000 x 1000 x 296 (1.5 M) 19 / 17 /
+//                    17, 8192 x 416 x 256 (2.1 M) 11 / 11 / 11, 777 x 1248 x 400 (0.3 M) 11 / 15 / 15
+//   backward         16384 x 400 x 1248 (20 M) 56 / 46 / 44, 5000 x 296 x 1000 (5 M) 24 / 22 / 20, 8192 x 256 x 416 (3.4 M) 17 / 17 / 17
+//   weight gradient  1248 x 400 over 16384 (two pieces / four / seven) 34 / 32 / 24, 1696 x 400 (three / seven / five) 40 / 36 / 30, 1000 x 296
+//                    over 5000 20 / 15 / 17, 416 x 256 over 8192 (ten pieces) 13 / 13 / 13, 1248 x 400 over 777 11 / 11 / 11
 
 // LayoutA: RowMajor = K contiguous, ColumnMajor = M contiguous.
 // LayoutB: ColumnMajor = K contiguous, RowMajor = N contiguous.
-#define DES_DEFINE_TC_GEMM(NAME, LayoutA, LayoutB, TileN)                                                              \
+#define DES_DEFINE_TC_GEMM(NAME, LayoutA, LayoutB, TileM, TileN)                                                       \
   struct NAME {                                                                                                       \
     using ElementA = cutlass::bfloat16_t;                                                                             \
     using ElementB = cutlass::bfloat16_t;                                                                             \
@@ -46,8 +53,8 @@
     using ElementAccumulator = float;                                                                                 \
     using ArchTag = cutlass::arch::Sm100;                                                                             \
     using OperatorClass = cutlass::arch::OpClassTensorOp;                                                             \
-    using MmaTileShape = cute::Shape<cute::_128, cute::Int<TileN>, cute::_64>;                                            \
-    using ClusterShape = cute::Shape<cute::_1, cute::_1, cute::_1>; /* one CTA per tile, plain (non-cluster) TMA loads */        \
+    using MmaTileShape = cute::Shape<cute::Int<TileM>, cute::Int<TileN>, cute::_64>;                                  \
+    using ClusterShape = cute::Shape<cute::Int<(TileM) / 128>, cute::_1, cute::_1>; /* a CTA, or a pair, per tile: no multicast */ \
     using CollectiveEpilogue = cutlass::epilogue::collective::CollectiveBuilder<                                      \
         ArchTag, OperatorClass, MmaTileShape, ClusterShape, cutlass::epilogue::collective::EpilogueTileAuto,          \
         ElementAccumulator, ElementAccumulator, ElementC, LayoutC, 4, ElementC, LayoutC, 4,                           \
@@ -84,7 +91,7 @@
   };
 #define DES_TC_GEMM_BODY(NAME) return NAME::run(M, N, K, L, A, B, C, D, beta, ws, ws_bytes, stream);
 #else
-#define DES_DEFINE_TC_GEMM(NAME, LayoutA, LayoutB, TileN)
+#define DES_DEFINE_TC_GEMM(NAME, LayoutA, LayoutB, TileM, TileN)
 #define DES_TC_GEMM_BODY(NAME) return 1;   /* built without the CUTLASS headers: CUDA-core fallback only */
 #endif
 
@@ -96,5 +103,5 @@ int des_tc_gemm_dgrad(int M, int N, int K, int L, const void* A, const void* B, 
                       size_t ws_bytes, cudaStream_t stream);
 // gW1 = V^T gZ: A = pooled bf16 [B][F*k] read as (M = F*k, K = B), M contiguous; B = gZ bf16 [B][H] (N contiguous);
 // L > 1 cuts the batch into L pieces (K = B / L samples each) whose partial products the caller adds
-int des_tc_gemm_wgrad(int M, int N, int K, int L, const void* A, const void* B, const float* C, float* D, float beta, void* ws,
-                      size_t ws_bytes, cudaStream_t stream);
+int des_tc_gemm_wgrad(bool wide, int M, int N, int K, int L, const void* A, const void* B, const float* C, float* D, float beta,
+                      void* ws, size_t ws_bytes, cudaStream_t stream);

@@ -1,9 +1,9 @@
 // tcgen05 GEMM, operand layout "dgrad" (see des_tc_gemm.cuh).
 #include "des_tc_gemm.cuh"
-DES_DEFINE_TC_GEMM(TcGemm_dgrad, cutlass::layout::RowMajor, cutlass::layout::ColumnMajor, 64)
-DES_DEFINE_TC_GEMM(TcGemm_dgrad_wide, cutlass::layout::RowMajor, cutlass::layout::ColumnMajor, 192)
+DES_DEFINE_TC_GEMM(TcGemm_dgrad, cutlass::layout::RowMajor, cutlass::layout::ColumnMajor, 128, 64)
+DES_DEFINE_TC_GEMM(TcGemm_dgrad_wide, cutlass::layout::RowMajor, cutlass::layout::ColumnMajor, 256, 192)
 int des_tc_gemm_dgrad(int M, int N, int K, int L, const void* A, const void* B, const float* C, float* D, float beta, void* ws,
                    size_t ws_bytes, cudaStream_t stream) {
-  if ((long long)M * N >= DES_TC_WIDE_OUTPUTS) { DES_TC_GEMM_BODY(TcGemm_dgrad_wide) }
+  if ((long long)M * N >= DES_TC_WIDE_DGRAD) { DES_TC_GEMM_BODY(TcGemm_dgrad_wide) }
   DES_TC_GEMM_BODY(TcGemm_dgrad)
 }

@@ -1,9 +1,9 @@
 // tcgen05 GEMM, operand layout "fwd" (see des_tc_gemm.cuh).
 #include "des_tc_gemm.cuh"
-DES_DEFINE_TC_GEMM(TcGemm_fwd, cutlass::layout::RowMajor, cutlass::layout::RowMajor, 64)
-DES_DEFINE_TC_GEMM(TcGemm_fwd_wide, cutlass::layout::RowMajor, cutlass::layout::RowMajor, 192)
+DES_DEFINE_TC_GEMM(TcGemm_fwd, cutlass::layout::RowMajor, cutlass::layout::RowMajor, 128, 64)
+DES_DEFINE_TC_GEMM(TcGemm_fwd_wide, cutlass::layout::RowMajor, cutlass::layout::RowMajor, 256, 256)
 int des_tc_gemm_fwd(int M, int N, int K, int L, const void* A, const void* B, const float* C, float* D, float beta, void* ws,
                    size_t ws_bytes, cudaStream_t stream) {
-  if ((long long)M * N >= DES_TC_WIDE_OUTPUTS) { DES_TC_GEMM_BODY(TcGemm_fwd_wide) }
+  if ((long long)M * N >= DES_TC_WIDE_FWD) { DES_TC_GEMM_BODY(TcGemm_fwd_wide) }
   DES_TC_GEMM_BODY(TcGemm_fwd)
 }
