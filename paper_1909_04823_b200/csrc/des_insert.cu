@@ -48,7 +48,9 @@ __device__ __forceinline__ Slot load_slot(const Slot* p) {
 
 // Occurrences per thread and resident blocks per SM: one probe chain per thread at full occupancy
 // measured fastest (more chains per thread cost registers, hence warps in flight; electing one lane
-// per distinct key of a warp costs more in match instructions than the cached slot loads it saves).
+// per distinct key of a warp costs more in match instructions than the cached slot loads it saves, and finding
+// the distinct keys of 2048 or 4096 occurrences in shared memory first costs more than the rest saves: 32 M occurrences 690 -> 900 us
+// for the whole call, a look-up of 8.2 M 74 -> 111).
 #define PROBE_ILP 1
 #define PROBE_MINB 8
 // Waves of resident blocks up to which blocks merge (24: 7.3 M occurrences).  Whole call, Zipf 1.2, merged against not: 1 M 38 / 76 us,
@@ -62,13 +64,104 @@ struct SlotGeom {
   uint32_t mod_M, mod_two32;        // constants of the division-free mod S (des_mod_consts)
 };   // kernel parameter: constant-bank reads
 
+// Start of an occurrence's probe chain: its shard, and the slot it looks at first inside [lo, hi), the shard's region
+// (cur = DES_SLOT_NONE: a reserved key, or a shard of another process).
+struct ProbeArgs {
+  const int32_t* offsets;
+  int nnz, nbags, S, F, partition, insert;
+  uint32_t world, rank;
+  Slot* slots;
+  DevMeta* meta;
+  uint32_t mod_M, mod_two32;        // as in SlotGeom
+};
+__device__ __forceinline__ uint32_t probe_home(const ProbeArgs& a, unsigned long long id, int j, const uint32_t* s_base,
+                                               uint32_t& cur, uint32_t& lo, uint32_t& hi) {
+  const unsigned long long h = des_mix64(id);
+  uint32_t s;
+  if (a.partition == DES_PART_HASH) s = des_mod_small(h, (uint32_t)a.S, a.mod_M, a.mod_two32);
+  else s = (uint32_t)(des_bag_near(a.offsets, a.nbags, a.nnz, j) % a.F) % (unsigned)a.S;
+  if (id == DES_KEY_EMPTY) {
+    des_raise(a.meta, DES_ERR_RESERVED_KEY);
+  } else if (a.world > 1 && s % a.world != a.rank) {
+    // another process holds this shard: the occurrence has no row here
+  } else {
+    lo = s_base[s];
+    hi = s_base[s + 1];
+    // position inside the region: the top bits of an odd multiple of the same mixed word (the shard is its
+    // residue mod S; a second full mixing round bought nothing measurable in probe lengths)
+    cur = des_slot_home(h, lo, hi - lo);
+  }
+  return s;
+}
+// The chains of a thread's occurrences: the slot of the key, found or claimed, with the row and the scratch word it showed.
+template <int ILP>
+__device__ __forceinline__ void probe_chain(const ProbeArgs& a, const unsigned long long (&id)[ILP], uint32_t (&cur)[ILP],
+                                            const uint32_t (&lo)[ILP], const uint32_t (&hi)[ILP], uint32_t (&found)[ILP],
+                                            uint32_t (&row)[ILP], uint32_t (&seen_fo)[ILP]) {
+  uint32_t nmax = 0;
+#pragma unroll
+  for (int q = 0; q < ILP; ++q) if (cur[q] != DES_SLOT_NONE) nmax = max(nmax, hi[q] - lo[q]);
+  for (uint32_t probe = 0; probe < nmax; ++probe) {
+    Slot sl[ILP];
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < ILP; ++q) {
+      if (cur[q] != DES_SLOT_NONE && !DES_DBG_SLOT_OK(cur[q])) cur[q] = DES_SLOT_NONE;   // (checking build)
+      if (cur[q] != DES_SLOT_NONE) { sl[q] = load_slot(a.slots + cur[q]); any = true; }
+    }
+    if (!any) break;
+#pragma unroll
+    for (int q = 0; q < ILP; ++q) {
+      if (cur[q] == DES_SLOT_NONE) continue;
+      bool done = false;
+      if (sl[q].key == id[q]) {
+        found[q] = cur[q]; row[q] = sl[q].row; seen_fo[q] = sl[q].first_occ;
+        done = true;
+      } else if (sl[q].key == DES_KEY_EMPTY) {
+        if (!a.insert) {
+          done = true;
+        } else {
+          const unsigned long long old = atomicCAS(&a.slots[cur[q]].key, DES_KEY_EMPTY, id[q]);
+          if (old == DES_KEY_EMPTY || old == id[q]) { found[q] = cur[q]; done = true; }
+        }
+      }
+      if (!done && probe + 1 >= hi[q] - lo[q]) {       // region is full
+        done = true;
+        if (a.insert) des_raise(a.meta, DES_ERR_CAPACITY);
+      }
+      cur[q] = done ? DES_SLOT_NONE : (cur[q] + 1 == hi[q] ? lo[q] : cur[q] + 1);
+    }
+  }
+}
+
+// Look-up without insertion: one probe chain per thread, and where there are more occurrences than threads the next key is fetched while
+// this one is looked for.  (8.2 M occurrences 74 -> 69 us.  With insertion the same costs more than it gives: 32 M 323 -> 335.)
+__global__ void __launch_bounds__(256, PROBE_MINB) lookup_kernel(const unsigned long long* __restrict__ ids, ProbeArgs pa,
+                                                                 const __grid_constant__ SlotGeom geom, uint8_t* __restrict__ shards,
+                                                                 uint32_t* __restrict__ rows) {
+  __shared__ uint32_t s_base[DES_MAX_SHARDS + 1];
+  if (threadIdx.x <= (unsigned)pa.S) s_base[threadIdx.x] = (uint32_t)geom.slot_base[threadIdx.x];
+  des_pdl_wait(ids, pa.offsets, pa.slots, pa.meta, shards, rows);
+  const uint32_t nnz = (uint32_t)pa.nnz, step = gridDim.x * 256u;
+  uint32_t j = blockIdx.x * 256u + threadIdx.x;
+  unsigned long long next = j < nnz ? ids[j] : 0ull;
+  __syncthreads();
+  for (; j < nnz; j += step) {
+    const unsigned long long id[1] = {next};
+    uint32_t cur[1] = {DES_SLOT_NONE}, lo[1] = {0}, hi[1] = {0}, found[1] = {DES_SLOT_NONE}, row[1] = {DES_ROW_NONE}, fo[1] = {0};
+    if (j + step < nnz) next = ids[j + step];
+    shards[j] = (uint8_t)probe_home(pa, id[0], (int)j, s_base, cur[0], lo[0], hi[0]);
+    probe_chain<1>(pa, id, cur, lo, hi, found, row, fo);
+    rows[j] = row[0];
+  }
+}
+
 // MERGE: the block merges its occurrences before the atomics (see the end of the kernel).
 template <bool MERGE>
 __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
     const unsigned long long* __restrict__ ids, const int32_t* __restrict__ offsets, int nnz, int nbags,
-    int S, int F, int partition, int insert, uint32_t world, uint32_t rank, Slot* slots, DevMeta* meta,
-    const __grid_constant__ SlotGeom geom, uint32_t* __restrict__ slot_of, uint8_t* __restrict__ shards,
-    uint32_t* __restrict__ rows) {
+    int S, int F, int partition, uint32_t world, uint32_t rank, Slot* slots, DevMeta* meta,
+    const __grid_constant__ SlotGeom geom, uint32_t* __restrict__ slot_of, uint8_t* __restrict__ shards) {
   // occurrence j = tile * (256 * PROBE_ILP) + q * 256 + thread: every access of a warp is contiguous.
   // Per occurrence the probe keeps its key, the table-global slot it looks at (DES_SLOT_NONE once it
   // is done) and the bounds of the owning shard's slot region: all 32-bit but the key.
@@ -77,18 +170,18 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
   __shared__ uint32_t s_base[DES_MAX_SHARDS + 1];
   __shared__ uint32_t m_slot[PROBE_MERGE], m_occ[PROBE_MERGE];
   if (MERGE) { m_slot[threadIdx.x] = DES_SLOT_NONE; m_occ[threadIdx.x] = DES_ROW_NONE; }
-  des_pdl_wait(ids, offsets, slots, meta, slot_of, shards, rows);
+  des_pdl_wait(ids, offsets, slots, meta, slot_of, shards);
   if (threadIdx.x <= (unsigned)S) s_base[threadIdx.x] = (uint32_t)geom.slot_base[threadIdx.x];
   __syncthreads();
   const uint32_t base = meta->scratch_base - (uint32_t)nnz;   // this call's scratch range (Slot::first_occ)
   const int j0 = blockIdx.x * (256 * PROBE_ILP) + threadIdx.x;
   unsigned long long id[PROBE_ILP];
-  uint32_t cur[PROBE_ILP], lo[PROBE_ILP], hi[PROBE_ILP], found[PROBE_ILP], row[PROBE_ILP], seen_fo[PROBE_ILP];
+  uint32_t cur[PROBE_ILP], lo[PROBE_ILP], hi[PROBE_ILP], found[PROBE_ILP], seen_fo[PROBE_ILP];
   uint32_t nmax = 0;
 #pragma unroll
   for (int q = 0; q < PROBE_ILP; ++q) {
     const int j = j0 + q * 256;
-    cur[q] = DES_SLOT_NONE; found[q] = DES_SLOT_NONE; row[q] = DES_ROW_NONE; seen_fo[q] = DES_ROW_NONE;
+    cur[q] = DES_SLOT_NONE; found[q] = DES_SLOT_NONE; seen_fo[q] = DES_ROW_NONE;
     id[q] = 0; lo[q] = 0; hi[q] = 0;
     if (j < nnz) {
       id[q] = ids[j];
@@ -126,19 +219,15 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
       if (cur[q] == DES_SLOT_NONE) continue;
       bool done = false;
       if (sl[q].key == id[q]) {
-        found[q] = cur[q]; row[q] = sl[q].row; seen_fo[q] = sl[q].first_occ;
+        found[q] = cur[q]; seen_fo[q] = sl[q].first_occ;
         done = true;
       } else if (sl[q].key == DES_KEY_EMPTY) {
-        if (!insert) {
-          done = true;
-        } else {
-          const unsigned long long old = atomicCAS(&slots[cur[q]].key, DES_KEY_EMPTY, id[q]);
-          if (old == DES_KEY_EMPTY || old == id[q]) { found[q] = cur[q]; done = true; }
-        }
+        const unsigned long long old = atomicCAS(&slots[cur[q]].key, DES_KEY_EMPTY, id[q]);
+        if (old == DES_KEY_EMPTY || old == id[q]) { found[q] = cur[q]; done = true; }
       }
       if (!done && probe + 1 >= hi[q] - lo[q]) {       // region is full
         done = true;
-        if (insert) des_raise(meta, DES_ERR_CAPACITY);
+        des_raise(meta, DES_ERR_CAPACITY);
       }
       cur[q] = done ? DES_SLOT_NONE : (cur[q] + 1 == hi[q] ? lo[q] : cur[q] + 1);
     }
@@ -153,16 +242,15 @@ __global__ void __launch_bounds__(256, PROBE_MINB) probe_claim_kernel(
   for (int q = 0; q < PROBE_ILP; ++q) {
     const int j = j0 + q * 256;
     if (j >= nnz) continue;
-    if (found[q] != DES_SLOT_NONE && insert && seen_fo[q] > base + (uint32_t)j) {
+    if (found[q] != DES_SLOT_NONE && seen_fo[q] > base + (uint32_t)j) {
       const uint32_t e = (found[q] * 0x9E3779B1u) >> 24;
       const uint32_t old = MERGE ? atomicCAS(&m_slot[e], DES_SLOT_NONE, found[q]) : 0u;
       if (MERGE && (old == DES_SLOT_NONE || old == found[q])) atomicMin(&m_occ[e], base + (uint32_t)j);
       else atomicMin(&slots[found[q]].first_occ, base + (uint32_t)j);
     }
-    if (insert) slot_of[j] = found[q];
-    else rows[j] = row[q];
+    slot_of[j] = found[q];
   }
-  if (!MERGE || !insert) return;
+  if (!MERGE) return;
   __syncthreads();
   if (m_slot[threadIdx.x] != DES_SLOT_NONE) atomicMin(&slots[m_slot[threadIdx.x]].first_occ, m_occ[threadIdx.x]);
 }
@@ -232,9 +320,108 @@ __device__ __forceinline__ uint32_t tile_offset_part(const uint32_t* __restrict_
   const int sup = tile / (int)SUP_TILES;
   uint32_t v = 0;
   for (int x = i; x < sup; x += n) v += __ldg(sup_cnt + (size_t)x * step);
-#pragma unroll 4
+#pragma unroll 8
   for (int x = sup * (int)SUP_TILES + i; x < tile; x += n) v += __ldg(blk_cnt + (size_t)x * step);
   return v;
+}
+
+// What a block of NT threads needs to rank and fill a list of up to CAP new keys.
+template <int NT, int CAP = IB>
+struct NewShared {
+  uint32_t n_base[DES_MAX_SHARDS], s_cap[DES_MAX_SHARDS], s_row[DES_MAX_SHARDS];
+  uint16_t n_warp[NT / 32][DES_MAX_SHARDS];             // new keys per list part and shard, then running ranks
+  uint16_t l_off[CAP];                                  // listed new keys: occurrence within the block's range, ...
+  uint8_t l_shard[CAP];
+  uint32_t l_slot[CAP];
+  uint32_t l_grow[CAP];                                  // ... batch-unique index, then table-global row
+};
+struct NewArgs {
+  const unsigned long long* ids;
+  uint32_t *rows, *uidx, *uniq_rows;
+  Slot* slots;
+  DevMeta* meta;
+  int S, k, stride;
+  float *W, *A, *A2;
+  unsigned long long seed;
+  float init_scale, state_init, lin_state_init;
+};
+// The n listed new keys of the occurrences from jb on, ranked per shard by the block's warps, each over a consecutive part
+// of the list, on top of n_base; then lane groups fill their rows: weights from the counter-based generator keyed on the id,
+// optimizer state at its start value.  The whole block, list and n_base in place (the first barrier is in here).
+template <int G, int NT, int CAP>
+__device__ __forceinline__ void new_keys(NewShared<NT, CAP>& sh, const NewArgs& a, int n, int jb) {
+  constexpr int NW = NT / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int K4 = a.k >> 2, c4 = tid % G;
+  const float stamp = des_stamp_bits(a.meta->clock + 1ull);   // the clock value this call ends with
+  for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&sh.n_warp[0][0])[i] = 0;
+  __syncthreads();
+  const int per = ((n + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min(n, lo + per);
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i0 = lo; i0 < hi; i0 += 32) {
+      const int i = i0 + lane;
+      const int key = i < hi ? (int)sh.l_shard[i] : -1;
+      const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+      const uint32_t at = i < hi ? sh.n_warp[warp][key] : 0u;
+      __syncwarp();
+      if (i < hi && (same >> lane) == 1u) sh.n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
+      if (pass == 1 && i < hi) {
+        uint32_t local = sh.n_base[key] + at + __popc(same & ((1u << lane) - 1u));
+        if (local >= sh.s_cap[key]) { local = DES_ROW_NONE; a.meta->rowless[key] = 1u; des_raise(a.meta, DES_ERR_CAPACITY); }
+        const int j = jb + sh.l_off[i];
+        const uint32_t uu = sh.l_grow[i];
+        const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : sh.s_row[key] + local;
+        if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(sh.l_slot[i])) a.slots[sh.l_slot[i]].row = local;
+        a.rows[j] = local;
+        a.uidx[j] = local == DES_ROW_NONE ? DES_ROW_NONE : uu;
+        a.uniq_rows[uu] = grow;
+        sh.l_grow[i] = grow;
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    if (pass == 0) {                                   // counts of the list parts -> where each part starts
+      if (tid < a.S) {
+        uint32_t run = 0;
+        for (int i = 0; i < NW; ++i) { const uint16_t v = sh.n_warp[i][tid]; sh.n_warp[i][tid] = (uint16_t)run; run += v; }
+      }
+      __syncthreads();
+    }
+  }
+  // ---- their rows: G lanes per row, every lane of a warp runs the same rounds (the squared norm is a warp-level sum)
+  constexpr int U = 4;                                  // rows of a group whose ids are in flight together
+  for (int i0 = 0; i0 < n; i0 += NT / G * U) {
+    uint32_t grow[U];
+    unsigned long long id[U];
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      const int i = i0 + q * (NT / G) + tid / G;
+      grow[q] = i < n ? sh.l_grow[i] : DES_ROW_NONE;
+      id[q] = i < n ? __ldg(a.ids + jb + sh.l_off[i]) : 0ull;
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c4 < K4) v = des_init4(a.seed, id[q], (uint32_t)c4, a.init_scale);
+      float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+      for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
+      if (grow[q] == DES_ROW_NONE || DES_DBG_ROW(grow[q]) != grow[q]) continue;
+      float4* wr = reinterpret_cast<float4*>(a.W + (size_t)grow[q] * a.stride);
+      if (c4 < K4) wr[c4] = v;
+      if (c4 == 0) wr[K4] = make_float4(0.f, n2, stamp, 0.f);   // linear weight, squared norm, age stamp
+      if (a.A) {
+        float4* ar = reinterpret_cast<float4*>(a.A + (size_t)grow[q] * a.stride);
+        if (c4 < K4) ar[c4] = make_float4(a.state_init, a.state_init, a.state_init, a.state_init);
+        if (c4 == 0) ar[K4] = make_float4(a.lin_state_init, 0.f, 0.f, 0.f);
+      }
+      if (a.A2) {
+        float4* a2 = reinterpret_cast<float4*>(a.A2 + (size_t)grow[q] * a.stride);
+        if (c4 < K4) a2[c4] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c4 == 0) a2[K4] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  }
 }
 
 // PER consecutive occurrences per thread: a block covers M = 512 PER / IB counting tiles.  First
@@ -247,29 +434,24 @@ __device__ __forceinline__ uint32_t tile_offset_part(const uint32_t* __restrict_
 // occurrences once every SM has several blocks (32 M occurrences: 212 -> 70 us).
 template <int G, int PER>
 __global__ void __launch_bounds__(512, 3) assign_kernel(
-    int nnz, int ntiles, int S, DevMeta* meta, const unsigned long long* __restrict__ ids, const uint8_t* __restrict__ shards,
-    const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
-    int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx,
-    uint32_t* __restrict__ uniq_rows, uint32_t* __restrict__ n_uniq_out, Slot* slots, unsigned long long total_slots,
-    uint32_t max_nnz, int k, int stride, float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2,
-    unsigned long long seed, float init_scale, float state_init, float lin_state_init) {
+    int nnz, int ntiles, int S, DevMeta* meta, const uint8_t* __restrict__ shards, const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
+    int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* __restrict__ n_uniq_out,
+    unsigned long long total_slots, uint32_t max_nnz, NewArgs na) {
   constexpr int NT = 512, NW = NT / 32, M = NT * PER / IB;
   constexpr bool DEEP = PER > 2;
   __shared__ uint16_t s_first[DEEP ? NT * PER : 1];     // DEEP: the block's first occurrences in order (bit 15: new key)
-  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW], n_base[DES_MAX_SHARDS], s_cap[DES_MAX_SHARDS], s_row[DES_MAX_SHARDS];
-  __shared__ uint16_t n_warp[NW][DES_MAX_SHARDS];       // new keys per list part and shard, then running ranks
-  __shared__ uint16_t l_off[IB];                        // listed new keys: occurrence within the block's range, ...
-  __shared__ uint8_t l_shard[IB];
-  __shared__ uint32_t l_slot[IB];
-  __shared__ uint32_t l_grow[IB];                       // ... batch-unique index, then table-global row
+  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW];
+  __shared__ NewShared<NT> sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile0 = blockIdx.x * M, jb = tile0 * IB, j0 = jb + tid * PER;
-  des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2);
+  des_pdl_wait(meta, shards, flags, blk_cnt, sup_cnt, slot_of, n_uniq_out, na.ids, na.rows, na.uidx, na.uniq_rows, na.slots, na.W, na.A, na.A2);
+  na.meta = meta;
+  uint32_t *rows = na.rows, *uidx = na.uidx, *uniq_rows = na.uniq_rows;
   // The slots' scratch range ends with this call (see Slot::first_occ; resolve_kernel then starts a new one): nothing
   // reads the scratch words after flag_count_kernel, so they are all cleared here, once every few billion occurrences.
   if (meta->scratch_base - (uint32_t)nnz < max_nnz)
     for (unsigned long long i = (unsigned long long)blockIdx.x * NT + tid; i < total_slots; i += (unsigned long long)gridDim.x * NT)
-      slots[i].first_occ = DES_ROW_NONE;
+      na.slots[i].first_occ = DES_ROW_NONE;
   typedef typename std::conditional<PER == 8, unsigned long long, uint16_t>::type flags_t;
   unsigned long long w = 0;
   if (j0 + PER <= nnz) w = __ldg(reinterpret_cast<const flags_t*>(flags + j0));
@@ -279,14 +461,14 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
   auto first = [&](int q) { return (w >> (8 * q)) & 1ull; };
   auto fresh = [&](int q) { return (w >> (8 * q)) & 2ull; };
   // PER = 2: what the first occurrences need, in flight while the ranks are formed
-  uint32_t r[DEEP ? 1 : PER], sh[DEEP ? 1 : PER];
+  uint32_t r[DEEP ? 1 : PER], sd[DEEP ? 1 : PER];
   if (!DEEP)
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       r[q] = first(q) ? rows[j0 + q] : DES_ROW_NONE;
-      sh[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
+      sd[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
     }
-  if (tid < S) s_row[tid] = (uint32_t)meta->row_base[tid];
+  if (tid < S) sh.s_row[tid] = (uint32_t)meta->row_base[tid];
   uint32_t incl = cf | cn << 16;                        // (at most 4096 of each in a block)
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -322,7 +504,7 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
       if (e & 0x8000u) continue;
       const uint32_t row = rows[jb + e], sd = __ldg(shards + jb + e);
       uidx[jb + e] = row == DES_ROW_NONE ? DES_ROW_NONE : u0 + i;
-      uniq_rows[u0 + i] = row == DES_ROW_NONE ? DES_ROW_NONE : s_row[sd] + row;
+      uniq_rows[u0 + i] = row == DES_ROW_NONE ? DES_ROW_NONE : sh.s_row[sd] + row;
     }
   } else {
     uint32_t uu = u;
@@ -331,22 +513,19 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
       if (!first(q)) continue;
       if (!fresh(q)) {
         uidx[j0 + q] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : uu;
-        uniq_rows[uu] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : s_row[sh[q]] + r[q];
+        uniq_rows[uu] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : sh.s_row[sd[q]] + r[q];
       }
       ++uu;
     }
   }
   if (n_new == 0) return;                               // (whole block) the steady state of a populated table
   // ---- new keys: rank among the shard's new keys, on top of the shard's size
-  if (tid < S) { n_base[tid] = meta->n_rows[tid]; s_cap[tid] = meta->row_cap[tid]; }
+  if (tid < S) { sh.n_base[tid] = meta->n_rows[tid]; sh.s_cap[tid] = meta->row_cap[tid]; }
   __syncthreads();
-  for (int i = tid; i < S * (NT / DES_MAX_SHARDS); i += NT) {
-    const uint32_t v = tile_offset_part(blk_cnt + nblk_max + i % S, sup_cnt + nsup_max + i % S, S, tile0, i / S,
-                                        NT / DES_MAX_SHARDS);
-    if (v) atomicAdd(&n_base[i % S], v);
+  if (const int per = NT / S; tid < per * S) {          // as many threads a shard as there are
+    const uint32_t v = tile_offset_part(blk_cnt + nblk_max + tid % S, sup_cnt + nsup_max + tid % S, S, tile0, tid / S, per);
+    if (v) atomicAdd(&sh.n_base[tid % S], v);
   }
-  const int K4 = k >> 2, c4 = tid % G;
-  const float stamp = des_stamp_bits(meta->clock + 1ull);   // the clock value this call ends with
   for (uint32_t win = 0; win < n_new; win += IB) {      // (one round unless PER = 8 and most keys are new)
     const int n = (int)min(n_new - win, (uint32_t)IB);
     {
@@ -356,86 +535,22 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
         if (!first(q)) continue;
         if (fresh(q)) {
           if (rank < (uint32_t)n) {                     // (unsigned: earlier windows are out of range too)
-            l_off[rank] = (uint16_t)(tid * PER + q); l_grow[rank] = uu;
+            sh.l_off[rank] = (uint16_t)(tid * PER + q); sh.l_grow[rank] = uu;
           }
           ++rank;
         }
         ++uu;
       }
     }
-    for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&n_warp[0][0])[i] = 0;
     __syncthreads();
-    for (int i = tid; i < n; i += NT) { l_shard[i] = __ldg(shards + jb + l_off[i]); l_slot[i] = __ldg(slot_of + jb + l_off[i]); }
-    __syncthreads();
-    const int per = ((n + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min(n, lo + per);
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int i0 = lo; i0 < hi; i0 += 32) {
-        const int i = i0 + lane;
-        const int key = i < hi ? (int)l_shard[i] : -1;
-        const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
-        const uint32_t at = i < hi ? n_warp[warp][key] : 0u;
-        __syncwarp();
-        if (i < hi && (same >> lane) == 1u) n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
-        if (pass == 1 && i < hi) {
-          uint32_t local = n_base[key] + at + __popc(same & ((1u << lane) - 1u));
-          if (local >= s_cap[key]) { local = DES_ROW_NONE; meta->rowless[key] = 1u; des_raise(meta, DES_ERR_CAPACITY); }
-          const int j = jb + l_off[i];
-          const uint32_t uu = l_grow[i];
-          const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : s_row[key] + local;
-          if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(l_slot[i])) slots[l_slot[i]].row = local;
-          rows[j] = local;
-          uidx[j] = local == DES_ROW_NONE ? DES_ROW_NONE : uu;
-          uniq_rows[uu] = grow;
-          l_grow[i] = grow;
-        }
-        __syncwarp();
-      }
-      __syncthreads();
-      if (pass == 0) {                                   // counts of the list parts -> where each part starts
-        if (tid < S) {
-          uint32_t run = 0;
-          for (int i = 0; i < NW; ++i) { const uint16_t v = n_warp[i][tid]; n_warp[i][tid] = (uint16_t)run; run += v; }
-        }
-        __syncthreads();
-      }
+    for (int i = tid; i < n; i += NT) {
+      sh.l_shard[i] = __ldg(shards + jb + sh.l_off[i]);
+      sh.l_slot[i] = __ldg(slot_of + jb + sh.l_off[i]);
     }
-    // ---- their rows: G lanes per row, every lane of a warp runs the same rounds (the squared norm is a warp-level sum)
-    constexpr int U = 4;                                // rows of a group whose ids are in flight together
-    for (int i0 = 0; i0 < n; i0 += NT / G * U) {
-      uint32_t grow[U];
-      unsigned long long id[U];
-#pragma unroll
-      for (int q = 0; q < U; ++q) {
-        const int i = i0 + q * (NT / G) + tid / G;
-        grow[q] = i < n ? l_grow[i] : DES_ROW_NONE;
-        id[q] = i < n ? __ldg(ids + jb + l_off[i]) : 0ull;
-      }
-#pragma unroll
-      for (int q = 0; q < U; ++q) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c4 < K4) v = des_init4(seed, id[q], (uint32_t)c4, init_scale);
-        float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-#pragma unroll
-        for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
-        if (grow[q] == DES_ROW_NONE || DES_DBG_ROW(grow[q]) != grow[q]) continue;
-        float4* wr = reinterpret_cast<float4*>(W + (size_t)grow[q] * stride);
-        if (c4 < K4) wr[c4] = v;
-        if (c4 == 0) wr[K4] = make_float4(0.f, n2, stamp, 0.f);   // linear weight, squared norm, age stamp
-        if (A) {
-          float4* a = reinterpret_cast<float4*>(A + (size_t)grow[q] * stride);
-          if (c4 < K4) a[c4] = make_float4(state_init, state_init, state_init, state_init);
-          if (c4 == 0) a[K4] = make_float4(lin_state_init, 0.f, 0.f, 0.f);
-        }
-        if (A2) {
-          float4* a2 = reinterpret_cast<float4*>(A2 + (size_t)grow[q] * stride);
-          if (c4 < K4) a2[c4] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (c4 == 0) a2[K4] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
-    }
+    new_keys<G>(sh, na, n, jb);
     if (win + IB < n_new) {                             // another window: the list and the counts are reused
       __syncthreads();
-      if (tid < S) n_base[tid] += n_warp[NW - 1][tid];
+      if (tid < S) sh.n_base[tid] += sh.n_warp[NW - 1][tid];
       __syncthreads();
     }
   }
@@ -671,29 +786,39 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
   const int ntiles = (nnz + IB - 1) / IB, nsup_max = (int)(t->nblk_max / SUP_TILES) + 1;
   SlotGeom geom;
   for (uint32_t s = 0; s <= t->S; ++s) geom.slot_base[s] = t->h_slot_base[s];
+  ProbeArgs pa;
+  pa.offsets = b->offsets; pa.nnz = nnz; pa.nbags = nbags; pa.S = (int)t->S; pa.F = (int)t->F; pa.partition = (int)t->cfg.partition;
+  pa.insert = insert; pa.world = t->cfg.shard_world; pa.rank = t->cfg.shard_rank; pa.slots = t->slots; pa.meta = t->meta;
   des_mod_consts(t->S, &geom.mod_M, &geom.mod_two32);
+  pa.mod_M = geom.mod_M; pa.mod_two32 = geom.mod_two32;
+  NewArgs na;
+  na.ids = (const unsigned long long*)b->ids; na.rows = b->rows; na.uidx = b->uidx; na.uniq_rows = b->uniq_rows; na.slots = t->slots;
+  na.meta = t->meta; na.S = (int)t->S; na.k = (int)t->k; na.stride = (int)t->stride; na.W = t->W; na.A = t->A; na.A2 = t->A2;
+  na.seed = t->cfg.seed; na.init_scale = t->cfg.init_scale;
+  na.state_init = t->cfg.optimizer == DES_OPT_ADAGRAD ? t->cfg.init_acc : 0.f;
+  na.lin_state_init = (t->cfg.lin_optimizer == DES_LIN_FTRL || t->cfg.optimizer != DES_OPT_ADAGRAD) ? 0.f : t->cfg.init_acc;
+  int G = 1;
+  while (G < (int)t->k / 4) G <<= 1;
+  if (!insert) {
+    const int blocks = (nnz + 255) / 256, most = t->sm_count * PROBE_MINB;
+    des_launch(lookup_kernel, blocks < most ? blocks : most, 256, 0, cs, na.ids, pa, geom, b->shards, b->rows);
+    DES_LAUNCH_CHECK(t, "lookup_kernel");
+    return DES_OK;
+  }
   const bool merge = nnz <= PROBE_MERGE_WAVES * t->sm_count * PROBE_MINB * 256;
-  des_launch(merge ? probe_claim_kernel<true> : probe_claim_kernel<false>, (nnz + 256 * PROBE_ILP - 1) / (256 * PROBE_ILP), 256, 0, cs, (const unsigned long long*)b->ids,
-             b->offsets, nnz, nbags, (int)t->S, (int)t->F, (int)t->cfg.partition, insert, t->cfg.shard_world, t->cfg.shard_rank,
-             t->slots, t->meta, geom, t->slot_of, b->shards, b->rows);
+  des_launch(merge ? probe_claim_kernel<true> : probe_claim_kernel<false>, (nnz + 256 * PROBE_ILP - 1) / (256 * PROBE_ILP), 256, 0, cs,
+             na.ids, b->offsets, nnz, nbags, (int)t->S, (int)t->F, (int)t->cfg.partition, t->cfg.shard_world, t->cfg.shard_rank, t->slots,
+             t->meta, geom, t->slot_of, b->shards);
   DES_LAUNCH_CHECK(t, "probe_claim_kernel");
-  if (!insert) return DES_OK;
   uint32_t* first_of = t->uslot;
   des_launch(flag_count_kernel, ntiles, IB / 4, 0, cs, nnz, (int)t->S, t->slots, t->meta, t->slot_of, b->shards, t->flags,
              b->rows, first_of, t->blk_cnt, t->sup_cnt, (int)t->nblk_max, nsup_max, &t->meta->any_new);
   DES_LAUNCH_CHECK(t, "flag_count_kernel");
   {
-    const float state_init = t->cfg.optimizer == DES_OPT_ADAGRAD ? t->cfg.init_acc : 0.f;
-    const float lin_state_init =
-        (t->cfg.lin_optimizer == DES_LIN_FTRL || t->cfg.optimizer != DES_OPT_ADAGRAD) ? 0.f : t->cfg.init_acc;
-    int G = 1;
-    while (G < (int)t->k / 4) G <<= 1;
     const bool deep = ntiles >= ASSIGN_DEEP_TILES * t->sm_count;
 #define ASSIGN2(GG, PP) des_launch(assign_kernel<GG, PP>, (ntiles * IB + 512 * PP - 1) / (512 * PP), 512, 0, cs, nnz, ntiles,   \
-        (int)t->S, t->meta, (const unsigned long long*)b->ids, b->shards, t->flags, t->blk_cnt, t->sup_cnt,               \
-        (int)t->nblk_max, nsup_max, t->slot_of, b->rows, b->uidx, b->uniq_rows, b->n_uniq, t->slots, t->total_slots,     \
-        (uint32_t)t->max_nnz, (int)t->k, (int)t->stride, t->W, t->A, t->A2, t->cfg.seed, t->cfg.init_scale, state_init,  \
-        lin_state_init)
+        (int)t->S, t->meta, b->shards, t->flags, t->blk_cnt, t->sup_cnt, (int)t->nblk_max, nsup_max, t->slot_of, b->n_uniq,      \
+        t->total_slots, (uint32_t)t->max_nnz, na)
 #define ASSIGN(GG) do { if (deep) ASSIGN2(GG, 8); else ASSIGN2(GG, 2); } while (0)
     switch (G) { case 1: ASSIGN(1); break; case 2: ASSIGN(2); break; case 4: ASSIGN(4); break; case 8: ASSIGN(8); break;
                  default: ASSIGN(16); }
