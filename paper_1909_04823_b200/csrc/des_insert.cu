@@ -622,6 +622,238 @@ __global__ void __launch_bounds__(IB / 4) resolve_kernel(int nnz, int ntiles, in
   }
 }
 
+// ---- small batches: the call as one cluster ----------------------------------------------------------------------------
+// A batch of at most ONCE_BLOCKS tiles of ONCE_TILE occurrences is one thread block cluster, a tile per block: the passes above with a
+// barrier of the cluster where they have a launch, and with everything that an occurrence hands from pass to pass (slot, row, first
+// occurrence, shard) in its thread's registers.  Per tile the blocks exchange the bits of the first occurrences with running
+// counts and the numbers of firsts and new keys, so that any occurrence finds the unique index of its key's first one from the prefix
+// of the tiles' counts, its word and a population count: no index array is read back, and without new keys two barriers do.
+// (Over the whole grid of a cooperative launch instead: 10 k occurrences 12.8 -> 10.9 us of kernels, but such a launch does not
+// overlap the kernel before it, and the step gained nothing; 0.2 M 19 -> 21.)
+#define ONCE_BLOCKS 16
+#define ONCE_TILE 1024
+struct OnceArgs {
+  uint2* words;                 // [tile][32] first-occurrence bits, first occurrences of the tile before them
+  uint32_t* new_cnt;            // [tile][S] new keys per shard, where a tile has any
+  uint32_t* n_uniq_out;
+  unsigned long long total_slots;
+  uint32_t max_nnz;
+};
+__device__ __forceinline__ void cluster_barrier() {      // all threads of the cluster; what they wrote before it is seen behind it
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int G>
+__global__ void __launch_bounds__(ONCE_TILE / 2, 1) insert_once_kernel(ProbeArgs pa, const __grid_constant__ SlotGeom geom, NewArgs na, OnceArgs oa,
+                                                            uint8_t* shards) {
+  constexpr int PER = 2, TILE = ONCE_TILE, NT = TILE / PER, NW = NT / 32, WORDS = TILE / 32, E = TILE;   // E: entries of the block's table of first occurrences
+  typedef NewShared<NT, TILE> New;
+  __shared__ uint32_t s_base[DES_MAX_SHARDS + 1], s_tile[32], s_cnt[WORDS], s_pre[WORDS], s_new[WORDS], s_npre[WORDS];
+  __shared__ uint32_t s_own, s_all[ONCE_BLOCKS], s_shard_new[DES_MAX_SHARDS];   // (s_all: first occurrences | new keys << 16 per tile)
+  union Scratch { uint32_t merge[2][E]; New nw; };
+  __shared__ Scratch sx;
+  New& sh = sx.nw;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tile = (int)blockIdx.x;
+  for (int i = tid; i < 2 * E; i += NT) (&sx.merge[0][0])[i] = DES_ROW_NONE;     // (DES_SLOT_NONE is the same word)
+  if (tid < DES_MAX_SHARDS) s_shard_new[tid] = 0u;
+  if (tid <= pa.S) s_base[tid] = (uint32_t)geom.slot_base[tid];
+  des_pdl_wait(pa.offsets, pa.slots, pa.meta, shards, na.ids, na.rows, na.uidx, na.uniq_rows, na.W, na.A, na.A2, oa.words,
+               oa.new_cnt, oa.n_uniq_out);
+  DevMeta* meta = pa.meta;
+  na.meta = meta; na.slots = pa.slots;
+  Slot* slots = pa.slots;
+  uint32_t *rows = na.rows, *uidx = na.uidx, *uniq_rows = na.uniq_rows;
+  const int nnz = pa.nnz, S = pa.S, jb = tile * TILE, ntiles = (nnz + TILE - 1) / TILE;   // (a cluster may have blocks without a tile)
+  const uint32_t base = meta->scratch_base - (uint32_t)nnz;
+  uint32_t found[PER], row[PER], fo[PER], sd[PER];
+  {
+    unsigned long long id[PER];
+    uint32_t cur[PER], lo[PER], hi[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int j = jb + q * NT + tid;
+      cur[q] = DES_SLOT_NONE; found[q] = DES_SLOT_NONE; row[q] = DES_ROW_NONE; fo[q] = DES_ROW_NONE; sd[q] = 0;
+      id[q] = j < nnz ? __ldg(na.ids + j) : 0ull;
+      lo[q] = 0; hi[q] = 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int j = jb + q * NT + tid;
+      if (j < nnz) { sd[q] = probe_home(pa, id[q], j, s_base, cur[q], lo[q], hi[q]); shards[j] = (uint8_t)sd[q]; }
+    }
+    probe_chain<PER>(pa, id, cur, lo, hi, found, row, fo);
+  }
+  // The smallest occurrence of every slot, merged in the block first (20 k occurrences of one key: 27 us of atomics on one address); an
+  // entry taken by another slot sends the atomic straight on.
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const uint32_t v = base + (uint32_t)(jb + q * NT + tid);
+    if (found[q] == DES_SLOT_NONE || fo[q] <= v) continue;
+    const uint32_t e = (found[q] * 0x9E3779B1u) >> 16 & (E - 1);
+    const uint32_t old = atomicCAS(&sx.merge[0][e], DES_SLOT_NONE, found[q]);
+    if (old == DES_SLOT_NONE || old == found[q]) atomicMin(&sx.merge[1][e], v);
+    else atomicMin(&slots[found[q]].first_occ, v);
+  }
+  __syncthreads();
+  for (int i = tid; i < E; i += NT)
+    if (sx.merge[0][i] != DES_SLOT_NONE) atomicMin(&slots[sx.merge[0][i]].first_occ, sx.merge[1][i]);
+  cluster_barrier();
+  // ---- first occurrences and new keys of the tile
+  uint32_t isf = 0, isn = 0;                            // bit q
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    uint2 rf = make_uint2(DES_ROW_NONE, DES_ROW_NONE);
+    if (found[q] != DES_SLOT_NONE) rf = __ldcg(reinterpret_cast<const uint2*>(slots + found[q]) + 1);   // (L1 holds what the probe saw)
+    row[q] = rf.x; fo[q] = rf.y;
+  }
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const uint32_t v = base + (uint32_t)(jb + q * NT + tid);
+    const bool f = found[q] != DES_SLOT_NONE && fo[q] == v, n = f && row[q] == DES_ROW_NONE;
+    const unsigned fb = __ballot_sync(0xFFFFFFFFu, f), nb = __ballot_sync(0xFFFFFFFFu, n);
+    if (lane == 0) { s_cnt[q * NW + warp] = fb; s_new[q * NW + warp] = nb; }
+    if (n) atomicAdd(&s_shard_new[sd[q]], 1u);
+    isf |= (uint32_t)f << q; isn |= (uint32_t)n << q;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    constexpr int C = WORDS / 32;                       // words of a lane
+    uint32_t c[C], sum = 0;
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      c[i] = sum;
+      sum += (uint32_t)__popc(s_cnt[lane * C + i]) | (uint32_t)__popc(s_new[lane * C + i]) << 16;
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+      if (lane >= d) incl += v;
+    }
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      const uint32_t pre = incl - sum + c[i];
+      s_pre[lane * C + i] = pre & 0xFFFFu; s_npre[lane * C + i] = pre >> 16;
+      oa.words[tile * WORDS + lane * C + i] = make_uint2(s_cnt[lane * C + i], pre & 0xFFFFu);
+    }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    if (lane == 0) s_own = total >> 16;
+    if (lane < (int)gridDim.x) {                        // into every block's shared memory
+      uint32_t at;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_all[tile])), "r"(lane));
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(total) : "memory");
+    }
+  }
+  __syncthreads();
+  const int n_own = (int)s_own;                         // this tile's new keys
+  if (n_own && tid < S) oa.new_cnt[(size_t)tile * S + tid] = s_shard_new[tid];
+  cluster_barrier();
+  // ---- unique indices: prefix of the tiles' counts (every warp for itself)
+  const uint32_t tw = lane < ntiles ? s_all[lane] : 0u;
+  const unsigned has = __ballot_sync(0xFFFFFFFFu, tw >> 16);   // tiles with new keys: the same in all blocks
+  uint32_t incl = tw & 0xFFFFu;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+    if (lane >= d) incl += v;
+  }
+  if (warp == 0) s_tile[lane] = incl - (tw & 0xFFFFu);
+  if (tile == 0 && tid == 31) { meta->n_uniq = incl; *oa.n_uniq_out = incl; }
+  if (tid < S) sh.s_row[tid] = (uint32_t)meta->row_base[tid];
+  __syncthreads();
+  uint32_t wait = 0;                                     // occurrences whose key is new, but not their own
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int j = jb + q * NT + tid;
+    if (j >= nnz || ((isn >> q) & 1u)) continue;
+    uint32_t u = DES_ROW_NONE, r = row[q];
+    if (found[q] != DES_SLOT_NONE) {
+      const uint32_t f = fo[q] - base;
+      if (f >= (uint32_t)nnz) { des_raise(meta, DES_ERR_CUDA); r = DES_ROW_NONE; }   // (a broken scratch word)
+      else if (r == DES_ROW_NONE) { wait |= 1u << q; continue; }
+      else {
+        const uint2 wd = __ldcg(oa.words + (f >> 5));
+        u = s_tile[f / TILE] + wd.y + (uint32_t)__popc(wd.x & ((1u << (f & 31)) - 1u));
+        if ((isf >> q) & 1u) uniq_rows[u] = sh.s_row[sd[q]] + r;
+      }
+    }
+    rows[j] = r;
+    uidx[j] = u;
+  }
+  // The slots' scratch range ends with this call (Slot::first_occ): nothing reads the scratch words any more.
+  if (base < oa.max_nnz)
+    for (unsigned long long i = (unsigned long long)tile * NT + tid; i < oa.total_slots; i += (unsigned long long)gridDim.x * NT)
+      slots[i].first_occ = DES_ROW_NONE;
+  const bool last = tile == ntiles - 1;                  // the block that ends the call
+  if (has) {
+    if (n_own || last) {
+      if (tid < S) { sh.n_base[tid] = meta->n_rows[tid]; sh.s_cap[tid] = meta->row_cap[tid]; }
+      __syncthreads();
+      for (int i = tid; i < S * tile; i += NT)           // the new keys of the tiles before
+        if ((has >> (i / S)) & 1u) {
+          const uint32_t v = __ldcg(oa.new_cnt + i);
+          if (v) atomicAdd(&sh.n_base[i % S], v);
+        }
+#pragma unroll
+      for (int q = 0; q < PER; ++q)
+        if ((isn >> q) & 1u) {
+          const int w = q * NW + warp;
+          const unsigned lt = (1u << lane) - 1u;
+          const uint32_t at = s_npre[w] + __popc(s_new[w] & lt);
+          sh.l_off[at] = (uint16_t)(q * NT + tid); sh.l_shard[at] = (uint8_t)sd[q]; sh.l_slot[at] = found[q];
+          sh.l_grow[at] = s_tile[tile] + s_pre[w] + __popc(s_cnt[w] & lt);
+        }
+      new_keys<G>(sh, na, n_own, jb);
+    }
+    cluster_barrier();
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if ((wait >> q) & 1u) {
+        const int j = jb + q * NT + tid;
+        const uint32_t f = fo[q] - base;
+        rows[j] = __ldcg(rows + f);
+        uidx[j] = __ldcg(uidx + f);
+      }
+    if (last && tid < S) meta->n_rows[tid] = min(sh.n_base[tid] + s_shard_new[tid], sh.s_cap[tid]);
+  }
+  if (last && tid == 0) { meta->clock += 1ull; meta->scratch_base = base < oa.max_nnz ? 0xFFFFFFFFu : base; }
+}
+
+// Blocks of such a cluster on the table's device: 16 where it takes clusters of more than the portable 8.
+int des_insert_once_blocks() {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ONCE_BLOCKS; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.gridDim = ONCE_BLOCKS; cfg.blockDim = ONCE_TILE / 2; cfg.attrs = &at; cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(insert_once_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, insert_once_kernel<16>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+  return n > 0 ? ONCE_BLOCKS : 8;
+}
+template <int G>
+static des_status_t insert_once(des_table* t, const des_batch_t* b, const ProbeArgs& pa, const SlotGeom& geom, const NewArgs& na,
+                                const OnceArgs& oa, cudaStream_t cs) {
+  const int ntiles = (pa.nnz + ONCE_TILE - 1) / ONCE_TILE;
+  int n = 1;
+  while (n < ntiles) n <<= 1;
+  // (an attribute of the function on the current device, not a stream operation: legal under capture)
+  if (n > 8 && cudaFuncSetAttribute(insert_once_kernel<G>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return DES_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = n; cfg.blockDim = ONCE_TILE / 2; cfg.stream = cs;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = n; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  cudaLaunchKernelEx(&cfg, insert_once_kernel<G>, pa, geom, na, oa, b->shards);
+  DES_LAUNCH_CHECK(t, "insert_once_kernel");
+  return DES_OK;
+}
+
 // ---- counting ------------------------------------------------------------------------------------------------------
 // hinfo[u] += occurrences of key u among a 1 / 2^shift sample.  A hot key would draw tens of thousands of atomics on one
 // word, which L2 serialises, so counts are merged per warp (lanes holding the same key), then per block in a small
@@ -799,6 +1031,14 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
   na.lin_state_init = (t->cfg.lin_optimizer == DES_LIN_FTRL || t->cfg.optimizer != DES_OPT_ADAGRAD) ? 0.f : t->cfg.init_acc;
   int G = 1;
   while (G < (int)t->k / 4) G <<= 1;
+  if (insert && nnz <= t->once_blocks * ONCE_TILE) {
+    OnceArgs oa;
+    oa.words = t->once_words; oa.new_cnt = t->once_new; oa.n_uniq_out = b->n_uniq;
+    oa.total_slots = t->total_slots; oa.max_nnz = (uint32_t)t->max_nnz;
+#define ONCE(GG) return insert_once<GG>(t, b, pa, geom, na, oa, cs)
+    switch (G) { case 1: ONCE(1); case 2: ONCE(2); case 4: ONCE(4); case 8: ONCE(8); default: ONCE(16); }
+#undef ONCE
+  }
   if (!insert) {
     const int blocks = (nnz + 255) / 256, most = t->sm_count * PROBE_MINB;
     des_launch(lookup_kernel, blocks < most ? blocks : most, 256, 0, cs, na.ids, pa, geom, b->shards, b->rows);

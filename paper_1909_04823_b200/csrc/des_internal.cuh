@@ -100,6 +100,9 @@ struct des_table {
   uint32_t* uslot;                   // [max_nnz]
   uint32_t* blk_cnt;                 // per tile: first occurrences [nblk_max], then new keys per shard [nblk_max][S]
   uint32_t* sup_cnt;                 // the same per SUP_TILES tiles; zero between calls
+  uint2* once_words;                 // [once_blocks][32] the one-cluster form's words of first occurrences
+  uint32_t* once_new;                // [once_blocks][S] and its new keys per tile and shard
+  int once_blocks;                   // blocks that form has at most
   int32_t* seg_off;                  // [max_batch][S+1] forward routing: (sample, shard) segment bounds
   // backward workspace
   float* Gbuf;                       // [max_uniq + rep_max][stride]: per-unique gradient rows, then
@@ -382,5 +385,6 @@ des_status_t des_dense1_backward_plain(des_table* t, const float* pooled, const 
                                        cudaStream_t st);
 // Whether the keys that own a large share of the batch are counted instead of scattered in the backward.
 bool des_super_path(const des_table* t, const des_batch_t* b);
+int des_insert_once_blocks();
 // Counts a batch's occurrences per unique key (a sample of a large batch) and makes the hot list: opens a backward.
 des_status_t des_count_batch(des_table* t, const des_batch_t* b, cudaStream_t cs);

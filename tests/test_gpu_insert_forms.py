@@ -1,0 +1,150 @@
+"""find_or_insert in its three forms (one cluster; tiles of 2048 and of 4096 occurrences) at the sizes where the form or the
+number of tiles changes: numbering of unique keys and of new rows in order of first occurrence, look-ups of unknown and known keys, both
+partitions, keys that appear once or thousands of times, a shard that runs full.  Against a sort of the batch."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+M = (1 << 64) - 1
+
+
+def _mix64(x):
+    x = x.astype(np.uint64)
+    x = (x ^ (x >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+    x = (x ^ (x >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    return x ^ (x >> np.uint64(31))
+
+
+class _Model:
+    """Rows by (shard, id), numbered as they come; one entry per known key, kept sorted."""
+
+    def __init__(self, S):
+        self.S, self.size = S, np.zeros(S, np.int64)
+        self.rows = {}
+
+    def call(self, ids, shards, insert=True):
+        key = np.stack([shards.astype(np.uint64), ids.astype(np.uint64)], 1)
+        _, first, inv = np.unique(key, axis=0, return_index=True, return_inverse=True)
+        inv = inv.reshape(-1)
+        order = np.argsort(first, kind="stable")
+        row_of = np.full(len(first), -1, np.int64)
+        for u in order:
+            s, i = int(shards[first[u]]), int(ids[first[u]])
+            r = self.rows.get((s, i), -1)
+            if r < 0 and insert:
+                r = self.size[s]
+                self.size[s] += 1
+                self.rows[(s, i)] = r
+            row_of[u] = r
+        rank = np.empty(len(first), np.int64)
+        rank[order] = np.arange(len(first))
+        return row_of[inv], rank[inv], row_of[order], shards[first[order]]
+
+
+def _check(t, db, model, base, ids, shards, insert, what):
+    rows, uidx, urow, ush = model.call(ids, shards, insert)
+    n = len(ids)
+    assert np.array_equal(db.shards[:n].cpu().numpy(), shards), what
+    assert np.array_equal(db.rows[:n].cpu().numpy().astype(np.int64), rows), what
+    if not insert:
+        return
+    assert int(db.n_uniq) == len(urow), what
+    assert np.array_equal(db.uidx[:n].cpu().numpy().astype(np.int64), uidx), what
+    assert np.array_equal(db.uniq_rows[:len(urow)].cpu().numpy().astype(np.int64), base[ush] + urow), what
+    assert np.array_equal(np.array(t.size()), model.size), what
+
+
+@pytest.mark.parametrize("partition", [0, 1])
+@pytest.mark.parametrize("nnz", [1, 31, 1024, 1025, 8192, 8193, 16384, 16385, 32768, 32769, 34815, 34816, 65537, 270001])
+def test_numbering(partition, nnz):
+    from paper_1909_04823_b200 import binding as D
+    rng = np.random.default_rng(nnz + partition)
+    S, F, k = (5, 7, 12) if nnz % 2 else (64, 3, 64)
+    B = (nnz + F - 1) // F
+    off = np.minimum(np.arange(B * F + 1), nnz)             # one-hot bags, the last ones empty
+    if nnz % 4 == 1:                                       # ragged bags
+        off = np.sort(np.concatenate([[0, nnz], rng.integers(0, nnz + 1, B * F - 1)]))
+    field = (np.searchsorted(off, np.arange(nnz), side="right") - 1) % F
+
+    def batch(lo, hi, hot):
+        ids = rng.integers(lo, hi, nnz).astype(np.uint64)
+        ids[rng.random(nnz) < hot] = lo + 3                # one key thousands of times
+        return ids * np.uint64(0x9E3779B97F4A7C15)         # (any 64-bit words but the reserved one)
+
+    cap = 2 * nnz + 300
+    t = D.Table(S, F, k, partition=partition, optimizer=D.OPT_ADAGRAD, max_rows=S * cap, rows_per_shard=[cap] * S, seed=3, max_nnz=nnz + 5,
+                max_batch=B)
+    try:
+        model, base = _Model(S), np.array(t.row_base(), np.int64)
+        # all new; half known, half new; all known; unknown and known keys looked up; new again
+        for step, (lo, hi, hot, insert) in enumerate([(10, 10 + nnz, 0.1, True), (10 + nnz // 2, 10 + 2 * nnz, 0.3, True),
+                                                      (10 + nnz // 2, 11 + nnz, 0.0, True), (10, 20 + 4 * nnz, 0.1, False),
+                                                      (10, 40 + 3 * nnz, 0.0, True)]):
+            ids = batch(lo, hi, hot)
+            shards = (field % S if partition else _mix64(ids) % np.uint64(S)).astype(np.uint8)
+            db = D.DeviceBatch(torch.from_numpy(off).cuda(), torch.from_numpy(ids.view(np.int64)).cuda(), None, B)
+            t.find_or_insert(db, insert=insert)
+            if model.size.max(initial=0) + nnz > cap and step == 4:
+                continue
+            _check(t, db, model, base, ids, shards, insert, (step, nnz))
+        got = t.read_rows(db.uniq_rows[:int(db.n_uniq)])
+        assert bool(torch.isfinite(got["emb"]).all())
+    finally:
+        t.close()
+
+
+@pytest.mark.parametrize("nnz", [(4 << 20) - 1, (4 << 20) + 4097])
+def test_large_tiles(nnz):
+    """The two tile sizes on a skewed batch: the same integers as a stable sort gives."""
+    from paper_1909_04823_b200 import binding as D
+    S, F, B = 9, 4, 1024
+    g = torch.Generator(device="cuda").manual_seed(nnz)
+    off = torch.sort(torch.randint(0, nnz + 1, (B * F - 1,), generator=g, device="cuda")).values
+    off = torch.cat([torch.zeros(1, dtype=torch.int64, device="cuda"), off, torch.full((1,), nnz, device="cuda")])
+    t = D.Table(S, F, 4, max_rows=3_000_000, seed=3, max_nnz=nnz, max_batch=B)
+    try:
+        sizes = torch.zeros(S, dtype=torch.int64, device="cuda")
+        known = torch.empty(0, dtype=torch.int64, device="cuda")
+        for step in range(2):
+            u = torch.rand(nnz, generator=g, device="cuda", dtype=torch.float64)
+            ids = (u.pow(-3.0 - step).clamp(max=4e5).long() * 7919 + 11) * (2 * step + 1)
+            db = D.DeviceBatch(off, ids, None, B)
+            t.find_or_insert(db)
+            uq, inv = torch.unique(ids, return_inverse=True)
+            first = torch.full((uq.numel(),), nnz, device="cuda").scatter_reduce_(0, inv, torch.arange(nnz, device="cuda"), "amin")
+            order = torch.argsort(first)
+            rank = torch.empty_like(order)
+            rank[order] = torch.arange(order.numel(), device="cuda")
+            assert int(db.n_uniq) == uq.numel()
+            assert torch.equal(db.uidx[:nnz].long(), rank[inv])
+            sh = db.shards[:nnz][first[order]].long()
+            new = ~torch.isin(uq[order], known)
+            urow = db.uniq_rows[:uq.numel()].long() - torch.tensor(t.row_base(), device="cuda")[sh]
+            for s in range(S):                             # a shard's new rows: consecutive, in order of first occurrence
+                m = new & (sh == s)
+                assert torch.equal(urow[m], sizes[s] + torch.arange(int(m.sum()), device="cuda"))
+                sizes[s] += int(m.sum())
+            assert torch.equal(db.rows[:nnz].long(), urow[rank[inv]])
+            known = torch.cat([known, uq])
+        assert t.size() == sizes.tolist() and t.status() == 0
+    finally:
+        t.close()
+
+
+@pytest.mark.parametrize("nnz", [3000, 30000, 70000])
+def test_full_shard(nnz):
+    """A shard without room: the keys that came first have rows, the others none, and the status says so."""
+    from paper_1909_04823_b200 import binding as D
+    t = D.Table(1, 1, 8, max_rows=nnz // 2, rows_per_shard=[nnz // 2], seed=3, max_nnz=nnz, max_batch=nnz, max_load=0.3)
+    try:
+        ids = torch.arange(nnz, device="cuda") * 3 + 1
+        db = D.DeviceBatch(torch.arange(nnz + 1, device="cuda"), ids, None, nnz)
+        t.find_or_insert(db)
+        want = torch.arange(nnz, device="cuda")
+        want[nnz // 2:] = -1
+        assert torch.equal(db.rows[:nnz].long(), want)
+        assert torch.equal(db.uidx[:nnz].long(), want)
+        assert t.size() == [nnz // 2] and t.status() != 0
+    finally:
+        t.close()
