@@ -164,16 +164,16 @@ __global__ void __launch_bounds__(256) route_kernel(
 
 // One round of a (sample, shard) segment: U rows per lane in flight, occurrences i, i + P, ... below `hi`;
 // positions past the segment's end read the all-zero row behind the table, so a round has no branch.
-template <int U, int P, bool HAS_VALS>
-__device__ __forceinline__ void sp_round(const uint32_t* __restrict__ grow_sorted, const float* __restrict__ x_sorted,
-                                         int i, int hi, uint32_t null_row, const char* __restrict__ Wc,
+// LOCAL: the lists were written by the block itself, to shared or global memory (plain loads).
+template <int U, int P, bool HAS_VALS, bool LOCAL = false>
+__device__ __forceinline__ void sp_round(const uint32_t* grow_sorted, const float* x_sorted, int i, int hi, uint32_t null_row, const char* __restrict__ Wc,
                                          const char* __restrict__ Wt, unsigned rowB, float4& acc, float& m1lr, float& m2) {
   float4 v[U]; float2 tl[U]; float x[U]; uint32_t g[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const bool in = i + u * P < hi;
-    g[u] = in ? __ldg(grow_sorted + i + u * P) : null_row;
-    if (HAS_VALS) x[u] = in ? __ldg(x_sorted + i + u * P) : 0.f;
+    g[u] = !in ? null_row : LOCAL ? grow_sorted[i + u * P] : __ldg(grow_sorted + i + u * P);
+    if (HAS_VALS) x[u] = !in ? 0.f : LOCAL ? x_sorted[i + u * P] : __ldg(x_sorted + i + u * P);
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -508,6 +508,252 @@ __global__ void __launch_bounds__(256) pool_kernel(
       if (BF16OUT) store_bf16x4(pooled_b + bag * k + c4 * 4, acc);    // operand of the first-layer product
     }
   }
+}
+
+// ---- routing, per-shard partials and pooling in one kernel ------------------------------------------------------------
+// The three kernels above for batches of few samples, which leave the chip idle there (a warp per sample): 8 / T warps take a sample, T
+// samples a block.  The sample's rows are looked up once and left in CSR order in shared memory, then placed in shard-major order by
+// the same stable counting sort (a warp counts and places a consecutive part of the sample, so the order does not depend on
+// T), and both lists are walked from there: segments first, then bags, handed to the sample's warps one by one.  With
+// out_small (fused) the partials also stay in shared memory and are added in double in shard order at the end.
+// Sums are formed exactly as there (same order, same grouping): the same bits.  A sample longer than `cap` keeps its lists
+// in the arrays of the three-kernel form.
+struct RouteArgs {
+  const int32_t* offsets;
+  const float* vals;
+  const uint32_t* rows;
+  const uint8_t* shards;
+  int B, F, S, k, T, cap;
+  uint32_t part_at;                 // where a block's partials start in shared memory (fused)
+  uint32_t ops;
+  bool brief, wide;                 // segments one per sub-group; bags one per warp
+  const float* W;
+  const DevMeta* meta;
+  uint32_t null_row;
+  float *part_small, *out_small, *pooled;
+  __nv_bfloat16* pooled_b;
+  uint32_t *grow_csr, *grow_sorted; // lists of samples longer than cap
+  float* x_sorted;
+};
+
+// One sample (its bounds, its place in the block, its warps).  BIG: the lists are in global memory; a template, so that the others'
+// are known to be in shared memory (through pointers that may be either, 40 samples of 2000 occurrences took 52 us instead of 43).
+struct RouteShared {
+  uint32_t base[DES_MAX_SHARDS];
+  int cnt[8][DES_MAX_SHARDS], cur[8][DES_MAX_SHARDS], seg[8][DES_MAX_SHARDS + 1], next[8];
+};
+template <int G, bool HAS_VALS, bool PART, bool BIG>
+__device__ __forceinline__ void route_sample(const RouteArgs& ra, RouteShared& sh, unsigned char* smem, int b, int lo, int n, int st, int ws,
+                                             int wps) {
+  constexpr int P = 32 / G;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c4 = lane % G, p = lane / G;
+  const int S = ra.S, F = ra.F, k = ra.k, K4 = k >> 2, stride = k + 4, cap = ra.cap;
+  const uint32_t null_row = ra.null_row;
+  auto team_sync = [&]() {                               // the sample's warps
+    if (wps == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(st + 1), "r"(wps * 32) : "memory");
+  };
+  // the sample's lists: rows in CSR order and in shard-major order, shards, values in shard-major order
+  uint32_t* csr = BIG ? ra.grow_csr + lo : reinterpret_cast<uint32_t*>(smem) + st * cap;
+  uint32_t* srt = BIG ? ra.grow_sorted + lo : reinterpret_cast<uint32_t*>(smem) + (ra.T + st) * cap;
+  float* xs = !HAS_VALS ? nullptr : BIG ? ra.x_sorted + lo : reinterpret_cast<float*>(smem) + (2 * ra.T + st) * cap;
+  uint8_t* s_sh = smem + ra.T * cap * (HAS_VALS ? 12 : 8) + st * cap;
+  const uint8_t* shl = BIG ? ra.shards + lo : s_sh;
+  const int chunk = ((n + wps - 1) / wps + 31) / 32 * 32, a0 = min(n, ws * chunk), a1 = min(n, a0 + chunk);
+  // ---- look-up and occurrences per shard
+  for (int i0 = a0; i0 < a1; i0 += 4 * 32) {             // four look-ups of a lane in flight
+    uint32_t r[4]; int sd[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = i0 + q * 32 + lane;
+      r[q] = DES_ROW_NONE; sd[q] = 0;
+      if (i < a1) { r[q] = __ldg(ra.rows + lo + i); sd[q] = __ldg(ra.shards + lo + i); }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = i0 + q * 32 + lane;
+      if (i >= a1) continue;
+      csr[i] = r[q] == DES_ROW_NONE ? null_row : sh.base[sd[q]] + r[q];
+      if (!BIG) s_sh[i] = (uint8_t)sd[q];
+      if (r[q] != DES_ROW_NONE) atomicAdd(&sh.cnt[warp][sd[q]], 1);   // counting only: order does not matter here
+    }
+  }
+  team_sync();
+  // ---- segment starts (two shards per lane, S <= 64), and where this warp's part of each segment starts
+  {
+    static_assert(DES_MAX_SHARDS <= 64, "two counters per lane");
+    int t0 = 0, t1 = 0, b0 = 0, b1 = 0;
+    for (int w = 0; w < wps; ++w) {
+      const int* c = sh.cnt[st * wps + w];
+      const int x0 = lane < S ? c[lane] : 0, x1 = lane + 32 < S ? c[lane + 32] : 0;
+      t0 += x0; t1 += x1;
+      if (w < ws) { b0 += x0; b1 += x1; }
+    }
+    int i0 = t0, i1 = t1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v0 = __shfl_up_sync(0xFFFFFFFFu, i0, d), v1 = __shfl_up_sync(0xFFFFFFFFu, i1, d);
+      if (lane >= d) { i0 += v0; i1 += v1; }
+    }
+    const int e0 = __shfl_sync(0xFFFFFFFFu, i0, 31), e1 = __shfl_sync(0xFFFFFFFFu, i1, 31);
+    i0 -= t0; i1 += e0 - t1;
+    if (lane < S) sh.cur[warp][lane] = i0 + b0;
+    if (lane + 32 < S) sh.cur[warp][lane + 32] = i1 + b1;
+    if (ws == 0) {
+      if (lane < S) sh.seg[st][lane] = i0;
+      if (lane + 32 < S) sh.seg[st][lane + 32] = i1;
+      if (lane == 0) sh.seg[st][S] = e0 + e1;
+    }
+  }
+  __syncwarp();
+  // ---- stable placement: the first lane of every group of equal shards advances the shard's cursor and hands the old value
+  // to its group (a warp's shared-memory atomics execute in program order)
+  for (int i0 = a0; i0 < a1; i0 += 32) {
+    const int i = i0 + lane;
+    int key = -1 - lane; uint32_t g = 0; float x = 1.f;
+    if (i < a1) {
+      g = csr[i];
+      if (g != null_row) key = shl[i];
+      if (HAS_VALS) x = __ldg(ra.vals + lo + i);
+    }
+    const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+    const int leader = __ffs(same) - 1;
+    int first = 0;
+    if (key >= 0 && lane == leader) first = atomicAdd(&sh.cur[warp][key], __popc(same));
+    first = __shfl_sync(0xFFFFFFFFu, first, leader);
+    if (key >= 0) {
+      const int pos = first + __popc(same & ((1u << lane) - 1u));
+      srt[pos] = g;
+      if (HAS_VALS) xs[pos] = x;
+    }
+  }
+  team_sync();
+  // ---- segments, then bags
+  const bool col = c4 < K4, lr = ra.ops & DES_OP_LR, fm = ra.ops & DES_OP_FM;
+  const unsigned rowB = (unsigned)stride * 4u;
+  const char* Wc = reinterpret_cast<const char*>(ra.W) + (col ? c4 : 0) * 16;
+  const char* Wt = reinterpret_cast<const char*>(ra.W + k);
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  float* part = PART ? reinterpret_cast<float*>(smem + ra.part_at) + st * S * stride : nullptr;   // [S][stride]
+  // sums of a segment: two levels, as in shard_partials_kernel
+  auto seg_sum = [&](auto PP, int i, int hi, float4& acc, float& m1lr, float& m2) {
+    constexpr int N = decltype(PP)::value;
+    float4 up = zero4;
+    float up_l = 0.f, up_q = 0.f;
+    acc = zero4; m1lr = 0.f; m2 = 0.f;
+    int round = 0;
+    const int off = N > 1 ? p : 0;
+    for (; i < hi; i += SP_U * N) {
+      sp_round<SP_U, N, HAS_VALS, true>(srt, xs, i + off, hi, null_row, Wc, Wt, rowB, acc, m1lr, m2);
+      if ((++round & (SP_FLUSH - 1)) == 0) {
+        up.x += acc.x; up.y += acc.y; up.z += acc.z; up.w += acc.w; up_l += m1lr; up_q += m2;
+        acc = zero4; m1lr = 0.f; m2 = 0.f;
+      }
+    }
+    acc.x += up.x; acc.y += up.y; acc.z += up.z; acc.w += up.w; m1lr += up_l; m2 += up_q;
+  };
+  auto seg_done = [&](int s, bool mine, float4& acc, float& m1lr, float& m2) {
+    if (!fm) { acc = zero4; m2 = 0.f; }
+    if (!lr) m1lr = 0.f;
+    if (!mine) return;
+    if (ra.part_small) {
+      float4* dst = reinterpret_cast<float4*>(ra.part_small + ((size_t)s * ra.B + b) * stride);
+      if (col) dst[c4] = acc;
+      if (c4 == 0) dst[K4] = make_float4(m1lr, m2, 0.f, 0.f);
+    }
+    if (PART) {
+      float4* dst = reinterpret_cast<float4*>(part + (size_t)s * stride);
+      if (col) dst[c4] = acc;
+      if (c4 == 0) dst[K4] = make_float4(m1lr, m2, 0.f, 0.f);
+    }
+  };
+  const int nseg = !(lr || fm) ? 0 : ra.brief ? (S + P - 1) / P : S;
+  const int nbag = !ra.pooled ? 0 : ra.wide ? F : (F + P - 1) / P;
+  for (int item = -1;;) {
+    if (wps == 1) ++item;
+    else {
+      if (lane == 0) item = atomicAdd(&sh.next[st], 1);
+      item = __shfl_sync(0xFFFFFFFFu, item, 0);
+    }
+    if (item >= nseg + nbag) break;
+    if (item < nseg) {
+      float4 acc; float m1lr, m2;
+      if (ra.brief) {                                    // a segment per sub-group
+        const int s = item * P + p;
+        const int i = s < S ? sh.seg[st][s] : 0, hi = s < S ? sh.seg[st][s + 1] : 0;
+        seg_sum(std::integral_constant<int, 1>(), i, hi, acc, m1lr, m2);
+        __syncwarp();
+        seg_done(s, s < S, acc, m1lr, m2);
+      } else {                                           // a segment per warp, its sub-groups combined by a butterfly
+        seg_sum(std::integral_constant<int, P>(), sh.seg[st][item], sh.seg[st][item + 1], acc, m1lr, m2);
+#pragma unroll
+        for (int d = G; d < 32; d <<= 1) {
+          acc.x += __shfl_xor_sync(0xFFFFFFFFu, acc.x, d); acc.y += __shfl_xor_sync(0xFFFFFFFFu, acc.y, d);
+          acc.z += __shfl_xor_sync(0xFFFFFFFFu, acc.z, d); acc.w += __shfl_xor_sync(0xFFFFFFFFu, acc.w, d);
+          m1lr += __shfl_xor_sync(0xFFFFFFFFu, m1lr, d); m2 += __shfl_xor_sync(0xFFFFFFFFu, m2, d);
+        }
+        seg_done(item, p == 0, acc, m1lr, m2);
+      }
+    } else {
+      const int f = ra.wide ? item - nseg : (item - nseg) * P + p;
+      float4 acc = zero4;
+      if (f < F) {                                       // (wide: the whole warp)
+        const int32_t* o = ra.offsets + (size_t)b * F + f;
+        const int i = __ldg(o) - lo, hi = __ldg(o + 1) - lo;
+        const float* xv = HAS_VALS ? ra.vals + lo : nullptr;
+        if (ra.wide) for (int j = i + p; j < hi; j += 4 * P) list_round<4, P, HAS_VALS>(csr, xv, j, hi, Wc, rowB, acc);
+        else for (int j = i; j < hi; j += 4) list_round<4, 1, HAS_VALS>(csr, xv, j, hi, Wc, rowB, acc);
+      }
+      if (ra.wide) {
+        __syncwarp();
+#pragma unroll
+        for (int d = G; d < 32; d <<= 1) {
+          acc.x += __shfl_xor_sync(0xFFFFFFFFu, acc.x, d); acc.y += __shfl_xor_sync(0xFFFFFFFFu, acc.y, d);
+          acc.z += __shfl_xor_sync(0xFFFFFFFFu, acc.z, d); acc.w += __shfl_xor_sync(0xFFFFFFFFu, acc.w, d);
+        }
+      }
+      if (f < F && col && (!ra.wide || p == 0)) {
+        const size_t o = ((size_t)b * F + f) * K4 + c4;
+        reinterpret_cast<float4*>(ra.pooled)[o] = acc;
+        if (ra.pooled_b) store_bf16x4(ra.pooled_b + o * 4, acc);
+      }
+    }
+  }
+  if (!PART) return;
+  team_sync();
+  if (ws != 0) return;                                   // whole warp; its first lane group has a column each
+  double Ax = 0.0, Ay = 0.0, Az = 0.0, Aw = 0.0, R = 0.0, Q = 0.0;   // (+)M_1, (+)M_1^lr, (+)M_2
+  if (p == 0)
+#pragma unroll 4
+    for (int s = 0; s < S; ++s) {
+      const float4* src = reinterpret_cast<const float4*>(part + (size_t)s * stride);
+      if (col) { const float4 v = src[c4]; Ax += (double)v.x; Ay += (double)v.y; Az += (double)v.z; Aw += (double)v.w; }
+      if (c4 == 0) { const float4 v = src[K4]; R += (double)v.x; Q += (double)v.y; }
+    }
+  __syncwarp();
+  double aa = Ax * Ax + Ay * Ay + Az * Az + Aw * Aw;
+#pragma unroll
+  for (int d = 1; d < G; d <<= 1) aa += __shfl_xor_sync(0xFFFFFFFFu, aa, d);
+  float4* o = reinterpret_cast<float4*>(ra.out_small + (size_t)b * stride);
+  if (p == 0 && col) o[c4] = make_float4((float)Ax, (float)Ay, (float)Az, (float)Aw);
+  if (lane == 0) o[K4] = make_float4((float)R, fm ? (float)(0.5 * aa - 0.5 * Q) : 0.f, (float)Q, 0.f);
+}
+
+template <int G, bool HAS_VALS, bool PART>
+__global__ void __launch_bounds__(256, HAS_VALS ? 4 : 5) sample_route_kernel(const RouteArgs ra) {
+  extern __shared__ __align__(16) unsigned char sr_smem[];
+  __shared__ RouteShared sh;
+  const int zero = des_pdl_wait0();
+  const int wps = 8 / ra.T, warp = threadIdx.x >> 5, st = warp / wps, ws = warp % wps;   // sample within the block, warp within the sample
+  const int b = blockIdx.x * ra.T + st + zero;
+  if (threadIdx.x < ra.S) sh.base[threadIdx.x] = (uint32_t)ra.meta->row_base[threadIdx.x + zero];
+  if (threadIdx.x < 8) sh.next[threadIdx.x] = 0;
+  for (int s = threadIdx.x & 31; s < ra.S; s += 32) sh.cnt[warp][s] = 0;
+  __syncthreads();
+  if (b >= ra.B) return;                                 // (all warps of the sample; no barrier of the block follows)
+  const int lo = __ldg(ra.offsets + (size_t)b * ra.F), n = __ldg(ra.offsets + (size_t)(b + 1) * ra.F) - lo;
+  if (n > ra.cap) route_sample<G, HAS_VALS, PART, true>(ra, sh, sr_smem, b, lo, n, st, ws, wps);
+  else route_sample<G, HAS_VALS, PART, false>(ra, sh, sr_smem, b, lo, n, st, ws, wps);
 }
 
 // (+) over shards and F.  G lanes per sample, one float4 column each; lane 0 of
@@ -1052,6 +1298,31 @@ static __nv_bfloat16* pooled_copy(const des_table* t, uint32_t ops, bool whole) 
   return whole && (ops & DES_OP_DENSE1) && t->use_tc ? t->pooled_b : nullptr;
 }
 
+// Samples per block and list capacity of the one-kernel form (sample_route_kernel); false: the three kernels.
+// Whole des_forward_partials, three kernels against one: k = 64, S = 64, bags of 20 (2000 occurrences a sample): 2 samples 149 / 37 us, 200
+// 214 / 61, 800 293 / 122, 3200 404 / 341, 16384 1548 / 1615; k = 32, S = 16, 400 a sample: 200 44 / 12, 1000 52 / 28, 4000 93 / 85, 16000
+// 262 / 276; k = 64, S = 32, bags of 4 (120 a sample): 41 24 / 11, 666 28 / 14, 3333 47 / 45, 6666 89 / 93; k = 16, 20 a sample: 250 12 / 5,
+// 4000 12 / 7, 10000 16 / 16.  Fused, where the partials take shared memory too: 120 a sample 666 26 / 17, 3333 43 / 56; 400 a sample 2000
+// 59 / 49; 2000 a sample 1600 334 / 202.  The three kernels' warp per sample fills the chip from about SR_MANY samples per SM on.
+#define SR_MANY(fused) ((fused) ? 14 : 28)
+#define SR_SMEM (41u << 10)       // shared memory of a block's lists and partials at most, ...
+#define SR_BLOCK (24u << 10)      // ... and where it holds several samples
+static bool route_plan(const des_table* t, const des_batch_t* b, bool fused, RouteArgs* ra) {
+  const int64_t avg = b->nnz / b->batch;
+  if ((int64_t)b->batch > (int64_t)t->sm_count * SR_MANY(fused)) return false;
+  const int64_t per = b->vals ? 13 : 9, part = fused ? (int64_t)t->S * t->stride * 4 : 0;
+  int64_t cap = (avg + avg / 4 + 64 + 31) / 32 * 32;     // (a geometric bag-length law: 99.8 % of samples of 100 bags of 20)
+  int T = 8;
+  while (T > 1 && T * (cap * per + part) > (int64_t)SR_BLOCK) T >>= 1;
+  if (T * (cap * per + part) > (int64_t)SR_SMEM) cap = ((int64_t)SR_SMEM - part) / per / 32 * 32;
+  while (T > 1 && (int64_t)b->batch * (8 / T) < (int64_t)t->sm_count * 24 && avg >= 32 * (8 / T)) T >>= 1;
+  ra->T = T; ra->cap = (int)cap;
+  ra->part_at = (uint32_t)((T * cap * per + 15) / 16 * 16);
+  ra->brief = b->nnz <= (int64_t)SP_BRIEF * b->batch * t->S;
+  ra->wide = b->nnz >= 8ll * b->batch * t->F;
+  return true;
+}
+
 // shared by des_forward_partials (fused_out == NULL) and des_forward_fused (whole: the aggregation follows in the same call)
 static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t* b, const des_partials_t* part,
                                  float* fused_out, bool whole, void* stream) {
@@ -1092,6 +1363,25 @@ static des_status_t forward_impl(des_table_t* t, uint32_t ops, const des_batch_t
   uint32_t* grow_sorted = t->slot_of;
   float* x_sorted = t->x_sorted;
   uint32_t* grow_csr = t->uslot;
+  if (!pp) {
+    RouteArgs ra;
+    if (route_plan(t, b, fused_out != nullptr, &ra)) {
+      ra.offsets = b->offsets; ra.vals = b->vals; ra.rows = b->rows; ra.shards = b->shards; ra.B = B; ra.F = (int)t->F; ra.S = (int)t->S;
+      ra.k = (int)t->k; ra.ops = ops; ra.W = t->W; ra.meta = t->meta; ra.null_row = (uint32_t)t->total_rows;
+      ra.part_small = ps; ra.out_small = fused_out; ra.pooled = pl; ra.pooled_b = pl ? pooled_copy(t, ops, whole) : nullptr;
+      ra.grow_csr = grow_csr; ra.grow_sorted = grow_sorted; ra.x_sorted = x_sorted;
+      const unsigned grid = (unsigned)((B + ra.T - 1) / ra.T);
+      const size_t smem = ra.part_at + (fused_out ? (size_t)ra.T * t->S * t->stride * 4 : 0);
+#define SR2(GG, HV) do { if (fused_out) des_launch(sample_route_kernel<GG, HV, true>, grid, 256, smem, cs, ra);   \
+                         else des_launch(sample_route_kernel<GG, HV, false>, grid, 256, smem, cs, ra); } while (0)
+#define SR(GG) do { if (b->vals) SR2(GG, true); else SR2(GG, false); } while (0)
+      switch (G) { case 1: SR(1); break; case 2: SR(2); break; case 4: SR(4); break; case 8: SR(8); break; default: SR(16); }
+#undef SR
+#undef SR2
+      DES_LAUNCH_CHECK(t, "sample_route_kernel");
+      return DES_OK;
+    }
+  }
   des_launch(b->nnz >= (int64_t)ROUTE_LONG * B ? route_kernel<8> : route_kernel<2>, (B + 7) / 8 < t->sm_count * 8 ? (B + 7) / 8 : t->sm_count * 8, 256, 0, cs, b->offsets, b->vals, b->rows,
              b->shards, B, (int)t->F, (int)t->S, t->meta, (uint32_t)t->total_rows, grow_csr, grow_sorted, x_sorted, t->seg_off);
   DES_LAUNCH_CHECK(t, "route_kernel");

@@ -1,0 +1,77 @@
+"""Routing, per-shard partials and pooling in one kernel: one to eight warps per sample, short and long segments and bags, empty bags
+and samples, samples longer than the lists in shared memory, occurrences without a row, feature values.  Against sums in
+double of the rows the table holds; the fused form in shard order gives the same bits."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,F,k,S,mean,vals,spike", [
+    (1, 1, 4, 1, 1, False, 0), (500, 8, 8, 4, 2.5, False, 0), (300, 17, 20, 7, 4, True, 900), (5000, 6, 12, 64, 3, False, 0),
+    (40, 100, 64, 64, 20, False, 0), (40, 100, 64, 64, 20, True, 6000), (9, 30, 32, 3, 30, False, 20000), (2500, 20, 16, 16, 12, True, 3000),
+    (700, 50, 64, 5, 8, False, 5000), (150, 3, 28, 33, 0.5, False, 0)])
+def test_partials_and_pools(B, F, k, S, mean, vals, spike):
+    from paper_1909_04823_b200 import binding as D
+    g = torch.Generator(device="cuda").manual_seed(B + F + spike)
+    lens = torch.poisson(torch.full((B * F,), float(mean), device="cuda"), generator=g).long()
+    if spike:
+        lens[(B // 2) * F] = spike                         # one sample far longer than the others
+    if B > 2:
+        lens[F:2 * F] = 0                                  # a sample without occurrences
+    off = torch.zeros(B * F + 1, dtype=torch.int64, device="cuda")
+    off[1:] = torch.cumsum(lens, 0)
+    nnz = int(off[-1])
+    bag = torch.repeat_interleave(torch.arange(B * F, device="cuda"), lens)
+    ids = torch.rand(nnz, generator=g, device="cuda").pow(3).mul(4000).long() * 977 + 5       # some ids many times in a sample
+    x = torch.rand(nnz, generator=g, device="cuda") + 0.5 if vals else None
+    t = D.Table(S, F, k, max_rows=8000 + 64 * S, seed=3, init_scale=0.1, max_nnz=nnz + 64, max_batch=B)
+    try:
+        known = torch.unique(ids)
+        known = known[torch.rand(known.numel(), generator=g, device="cuda") < 0.9]           # the others look up as "no row"
+        for lo in range(0, known.numel(), nnz):
+            part = known[lo:lo + nnz]
+            o = torch.arange(B * F + 1, device="cuda").clamp(max=part.numel())
+            o[-1] = part.numel()
+            first = D.DeviceBatch(o, part, None, B)
+            t.find_or_insert(first)
+            n = int(first.n_uniq)
+            t.write_rows(first.uniq_rows[:n], lin=torch.randn(n, generator=g, device="cuda"))
+        db = D.DeviceBatch(off, ids, x, B)
+        t.find_or_insert(db, insert=False)
+        base = torch.tensor(t.row_base(), device="cuda")
+        found = db.rows[:nnz] != -1
+        assert bool(found.any()) and (nnz < 50 or not bool(found.all()))
+        r = t.read_rows(torch.where(found, base[db.shards[:nnz].long()] + db.rows[:nnz].long(), -1).to(torch.int32))
+        xx = torch.ones(nnz, device="cuda", dtype=torch.float64) if x is None else x.double()
+        v, w = r["emb"].double() * xx[:, None], r["lin"].double() * xx
+        samp, sh = bag // F, db.shards[:nnz].long()
+        z = lambda *s: torch.zeros(*s, dtype=torch.float64, device="cuda")
+        seg = sh * B + samp
+        ref = {"M1": z(S * B, k).index_add_(0, seg, v), "LR": z(S * B).index_add_(0, seg, w), "M2": z(S * B).index_add_(0, seg, (v * v).sum(1)),
+               "pool": z(B * F, k).index_add_(0, bag, v)}
+        mag = {"M1": z(S * B, k).index_add_(0, seg, v.abs()), "LR": z(S * B).index_add_(0, seg, w.abs()), "M2": ref["M2"],
+               "pool": z(B * F, k).index_add_(0, bag, v.abs())}
+
+        def close(got, what):   # float32 sums, at most a few dozen terms per accumulator (bags: their length / 2)
+            rel = 2e-6 + (1.2e-7 * float(lens.max()) ** 0.5 if what == "pool" else 0.0)
+            err = (got.double() - ref[what]).abs()
+            assert bool((err <= 1e-6 * ref[what].abs() + rel * mag[what] + 1e-12).all()), (what, float(err.max()))
+
+        for ops in (D.OP_LR | D.OP_FM | D.OP_POOL, D.OP_LR | D.OP_FM, D.OP_POOL):
+            part, pl = torch.full((S, B, k + 4), 9.0, device="cuda"), torch.full((B, F * k), 9.0, device="cuda")
+            small = ops & (D.OP_LR | D.OP_FM)
+            t.forward_partials(ops, db, part if small else None, pl if ops & D.OP_POOL else None)
+            if small:
+                p = part.view(S * B, k + 4)
+                close(p[:, :k], "M1"); close(p[:, k], "LR"); close(p[:, k + 1], "M2")
+                assert bool((p[:, k + 2:] == 0).all())
+                out, out2 = torch.full((B, k + 4), 9.0, device="cuda"), torch.full((B, k + 4), 9.0, device="cuda")
+                t.aggregate(small, db, part, None, out_small=out)
+                t.forward_fused(ops | (D.FUSED_SHARD_ORDER if ops & D.OP_POOL else 0), db, pooled=pl, out_small=out2)
+                assert torch.equal(out, out2)
+            if ops & D.OP_POOL:
+                close(pl.view(B * F, k), "pool")
+        assert t.status() == 0
+    finally:
+        t.close()
