@@ -15,7 +15,7 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
-#define DES_TC_WIDE_FWD (3ll << 19)       // outputs (M x N) from which a product takes the wide tile
+#define DES_TC_WIDE_FWD (4ll << 20)       // outputs (M x N) from which a product takes the wide tile
 #define DES_TC_WIDE_DGRAD (4ll << 20)
 #define DES_TC_WIDE_WGRAD (1ll << 18)     // (weights; and a batch of DES_TC_WIDE_BATCH samples)
 #define DES_TC_WIDE_BATCH 2048
