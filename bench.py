@@ -235,6 +235,8 @@ def kernel_bytes(name, st):
     pool = bool(st["ops"] & (OP_POOL | OP_DENSE1))
     if name == "probe_claim_kernel":
         return 8 * nnz + 16 * U + 4 * nnz + nnz
+    if name == "insert_once_kernel":     # ids, unique slots; shard, row and unique index out, rows of the unique keys
+        return 8 * nnz + 16 * U + 9 * nnz + 4 * U
     if name == "flag_count_kernel":      # slot index and shard in; the slot's (row, scratch); flag, row, first occurrence out
         return 4 * nnz + nnz + 8 * U + nnz + 4 * nnz + 4 * nnz
     if name == "assign_kernel":          # exits at once when the batch has no new key (a populated table)
@@ -245,6 +247,8 @@ def kernel_bytes(name, st):
         return 8 * B + 2 * 5 * nnz + 8 * nnz + 4 * B * (S + 1)
     if name == "shard_partials_kernel":
         return 4 * B * (S + 1) + 4 * nnz + row * U + 4 * S * B * (k + 4)
+    if name == "sample_route_kernel":    # rows + shards in, every unique row once, per-shard partials (and pooled vectors) out
+        return 4 * (B * F + 1) + 5 * nnz + row * U + 4 * S * B * (k + 4) + (4 * B * F * k if pool else 0)
     if name == "pool_kernel":
         return 4 * (B * F + 1) + 4 * nnz + 4 * k * U + 4 * B * F * k
     if name in ("sample_gather_kernel", "sample_stage_kernel"):   # rows + shards in, every unique row once, pooled + aggregates out
@@ -283,7 +287,7 @@ def occurrence_bytes(name, st):
     nnz, k = st["nnz"], st["k"]
     if name == "pool_kernel":
         return 4 * k * nnz
-    if name in ("shard_partials_kernel", "single_gather_kernel", "sample_gather_kernel", "sample_stage_kernel"):
+    if name in ("shard_partials_kernel", "single_gather_kernel", "sample_gather_kernel", "sample_stage_kernel", "sample_route_kernel"):
         return (4 * k + 32) * nnz          # the vector and the 32-byte sector that holds the row's tail
     return None
 

@@ -35,7 +35,9 @@
  *   are HOST pointers.  The library owns only what des_table_create allocates
  *   and frees it in des_table_destroy.
  * - All device work is enqueued on the caller's stream (a cudaStream_t passed
- *   as void*; NULL = the legacy default stream).  Only des_table_status,
+ *   as void*; NULL = the legacy default stream); where a call uses a stream of
+ *   the table's own beside it, that work is forked from and joined to the
+ *   caller's stream inside the call.  Only des_table_status,
  *   des_table_size, des_table_export, des_dense1_get/set on host pointers,
  *   des_step_host and des_step_host_wait synchronise.
  * - One table, one order: every call on a table reuses workspace that the table

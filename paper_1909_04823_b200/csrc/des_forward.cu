@@ -23,6 +23,7 @@
 //  pool_kernel    one group per bag: sum pooling of the latent vectors in
 //                 registers.  The per-shard pooled partial [S][B][F*k] is only
 //                 materialised (with atomics) when the caller asks for it.
+//  sample_route_kernel   the three in one for batches of few samples: up to eight warps a sample, its lists in shared memory.
 //
 // FIELD partition (field f on shard f mod S): a bag belongs to one shard, so when pooling is among the
 // operators one gather pass (sample_gather_kernel: pooled vectors and per-bag sums of the linear weights and

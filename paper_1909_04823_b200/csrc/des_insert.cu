@@ -22,7 +22,9 @@
 //                 the counter-based generator (a lane group per row).
 //   resolve       every other occurrence takes row and unique index from its
 //                 key's first occurrence; shard sizes advance, the call's scratch range is retired.
-// A fifth kernel (count_kernel) is the backward's: it counts the occurrences per unique key and lists the hot keys.
+// Batches of up to 16 k occurrences take the same passes in one kernel, a thread block cluster (insert_once_kernel); a look-up without
+// insertion has a kernel of its own (lookup_kernel).
+// A further kernel (count_kernel) is the backward's: it counts the occurrences per unique key and lists the hot keys.
 #include "des_internal.cuh"
 
 #include <type_traits>
