@@ -322,7 +322,7 @@ __device__ __forceinline__ uint32_t tile_offset_part(const uint32_t* __restrict_
   const int sup = tile / (int)SUP_TILES;
   uint32_t v = 0;
   for (int x = i; x < sup; x += n) v += __ldg(sup_cnt + (size_t)x * step);
-#pragma unroll 8
+#pragma unroll 4
   for (int x = sup * (int)SUP_TILES + i; x < tile; x += n) v += __ldg(blk_cnt + (size_t)x * step);
   return v;
 }
@@ -347,6 +347,7 @@ struct NewArgs {
   unsigned long long seed;
   float init_scale, state_init, lin_state_init;
 };
+// (assign_kernel has the same steps in its own body: through this function its registers spill, 80.4 -> 83.2 us at 32 M occurrences.)
 // The n listed new keys of the occurrences from jb on, ranked per shard by the block's warps, each over a consecutive part
 // of the list, on top of n_base; then lane groups fill their rows: weights from the counter-based generator keyed on the id,
 // optimizer state at its start value.  The whole block, list and n_base in place (the first barrier is in here).
@@ -436,24 +437,29 @@ __device__ __forceinline__ void new_keys(NewShared<NT, CAP>& sh, const NewArgs& 
 // occurrences once every SM has several blocks (32 M occurrences: 212 -> 70 us).
 template <int G, int PER>
 __global__ void __launch_bounds__(512, 3) assign_kernel(
-    int nnz, int ntiles, int S, DevMeta* meta, const uint8_t* __restrict__ shards, const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
-    int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* __restrict__ n_uniq_out,
-    unsigned long long total_slots, uint32_t max_nnz, NewArgs na) {
+    int nnz, int ntiles, int S, DevMeta* meta, const unsigned long long* __restrict__ ids, const uint8_t* __restrict__ shards,
+    const uint8_t* __restrict__ flags, const uint32_t* __restrict__ blk_cnt, const uint32_t* __restrict__ sup_cnt,
+    int nblk_max, int nsup_max, const uint32_t* __restrict__ slot_of, uint32_t* rows, uint32_t* __restrict__ uidx,
+    uint32_t* __restrict__ uniq_rows, uint32_t* __restrict__ n_uniq_out, Slot* slots, unsigned long long total_slots,
+    uint32_t max_nnz, int k, int stride, float* __restrict__ W, float* __restrict__ A, float* __restrict__ A2,
+    unsigned long long seed, float init_scale, float state_init, float lin_state_init) {
   constexpr int NT = 512, NW = NT / 32, M = NT * PER / IB;
   constexpr bool DEEP = PER > 2;
   __shared__ uint16_t s_first[DEEP ? NT * PER : 1];     // DEEP: the block's first occurrences in order (bit 15: new key)
-  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW];
-  __shared__ NewShared<NT> sh;
+  __shared__ uint32_t wsum[NW], wnew[NW], wbase[NW], n_base[DES_MAX_SHARDS], s_cap[DES_MAX_SHARDS], s_row[DES_MAX_SHARDS];
+  __shared__ uint16_t n_warp[NW][DES_MAX_SHARDS];       // new keys per list part and shard, then running ranks
+  __shared__ uint16_t l_off[IB];                        // listed new keys: occurrence within the block's range, ...
+  __shared__ uint8_t l_shard[IB];
+  __shared__ uint32_t l_slot[IB];
+  __shared__ uint32_t l_grow[IB];                       // ... batch-unique index, then table-global row
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile0 = blockIdx.x * M, jb = tile0 * IB, j0 = jb + tid * PER;
-  des_pdl_wait(meta, shards, flags, blk_cnt, sup_cnt, slot_of, n_uniq_out, na.ids, na.rows, na.uidx, na.uniq_rows, na.slots, na.W, na.A, na.A2);
-  na.meta = meta;
-  uint32_t *rows = na.rows, *uidx = na.uidx, *uniq_rows = na.uniq_rows;
+  des_pdl_wait(meta, ids, shards, flags, blk_cnt, sup_cnt, slot_of, rows, uidx, uniq_rows, n_uniq_out, slots, W, A, A2);
   // The slots' scratch range ends with this call (see Slot::first_occ; resolve_kernel then starts a new one): nothing
   // reads the scratch words after flag_count_kernel, so they are all cleared here, once every few billion occurrences.
   if (meta->scratch_base - (uint32_t)nnz < max_nnz)
     for (unsigned long long i = (unsigned long long)blockIdx.x * NT + tid; i < total_slots; i += (unsigned long long)gridDim.x * NT)
-      na.slots[i].first_occ = DES_ROW_NONE;
+      slots[i].first_occ = DES_ROW_NONE;
   typedef typename std::conditional<PER == 8, unsigned long long, uint16_t>::type flags_t;
   unsigned long long w = 0;
   if (j0 + PER <= nnz) w = __ldg(reinterpret_cast<const flags_t*>(flags + j0));
@@ -463,14 +469,14 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
   auto first = [&](int q) { return (w >> (8 * q)) & 1ull; };
   auto fresh = [&](int q) { return (w >> (8 * q)) & 2ull; };
   // PER = 2: what the first occurrences need, in flight while the ranks are formed
-  uint32_t r[DEEP ? 1 : PER], sd[DEEP ? 1 : PER];
+  uint32_t r[DEEP ? 1 : PER], sh[DEEP ? 1 : PER];
   if (!DEEP)
 #pragma unroll
     for (int q = 0; q < PER; ++q) {
       r[q] = first(q) ? rows[j0 + q] : DES_ROW_NONE;
-      sd[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
+      sh[q] = first(q) ? __ldg(shards + j0 + q) : 0u;
     }
-  if (tid < S) sh.s_row[tid] = (uint32_t)meta->row_base[tid];
+  if (tid < S) s_row[tid] = (uint32_t)meta->row_base[tid];
   uint32_t incl = cf | cn << 16;                        // (at most 4096 of each in a block)
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -506,7 +512,7 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
       if (e & 0x8000u) continue;
       const uint32_t row = rows[jb + e], sd = __ldg(shards + jb + e);
       uidx[jb + e] = row == DES_ROW_NONE ? DES_ROW_NONE : u0 + i;
-      uniq_rows[u0 + i] = row == DES_ROW_NONE ? DES_ROW_NONE : sh.s_row[sd] + row;
+      uniq_rows[u0 + i] = row == DES_ROW_NONE ? DES_ROW_NONE : s_row[sd] + row;
     }
   } else {
     uint32_t uu = u;
@@ -515,19 +521,22 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
       if (!first(q)) continue;
       if (!fresh(q)) {
         uidx[j0 + q] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : uu;
-        uniq_rows[uu] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : sh.s_row[sd[q]] + r[q];
+        uniq_rows[uu] = r[q] == DES_ROW_NONE ? DES_ROW_NONE : s_row[sh[q]] + r[q];
       }
       ++uu;
     }
   }
   if (n_new == 0) return;                               // (whole block) the steady state of a populated table
   // ---- new keys: rank among the shard's new keys, on top of the shard's size
-  if (tid < S) { sh.n_base[tid] = meta->n_rows[tid]; sh.s_cap[tid] = meta->row_cap[tid]; }
+  if (tid < S) { n_base[tid] = meta->n_rows[tid]; s_cap[tid] = meta->row_cap[tid]; }
   __syncthreads();
-  if (const int per = NT / S; tid < per * S) {          // as many threads a shard as there are
-    const uint32_t v = tile_offset_part(blk_cnt + nblk_max + tid % S, sup_cnt + nsup_max + tid % S, S, tile0, tid / S, per);
-    if (v) atomicAdd(&sh.n_base[tid % S], v);
+  for (int i = tid; i < S * (NT / DES_MAX_SHARDS); i += NT) {
+    const uint32_t v = tile_offset_part(blk_cnt + nblk_max + i % S, sup_cnt + nsup_max + i % S, S, tile0, i / S,
+                                        NT / DES_MAX_SHARDS);
+    if (v) atomicAdd(&n_base[i % S], v);
   }
+  const int K4 = k >> 2, c4 = tid % G;
+  const float stamp = des_stamp_bits(meta->clock + 1ull);   // the clock value this call ends with
   for (uint32_t win = 0; win < n_new; win += IB) {      // (one round unless PER = 8 and most keys are new)
     const int n = (int)min(n_new - win, (uint32_t)IB);
     {
@@ -537,22 +546,86 @@ __global__ void __launch_bounds__(512, 3) assign_kernel(
         if (!first(q)) continue;
         if (fresh(q)) {
           if (rank < (uint32_t)n) {                     // (unsigned: earlier windows are out of range too)
-            sh.l_off[rank] = (uint16_t)(tid * PER + q); sh.l_grow[rank] = uu;
+            l_off[rank] = (uint16_t)(tid * PER + q); l_grow[rank] = uu;
           }
           ++rank;
         }
         ++uu;
       }
     }
+    for (int i = tid; i < NW * DES_MAX_SHARDS; i += NT) (&n_warp[0][0])[i] = 0;
     __syncthreads();
-    for (int i = tid; i < n; i += NT) {
-      sh.l_shard[i] = __ldg(shards + jb + sh.l_off[i]);
-      sh.l_slot[i] = __ldg(slot_of + jb + sh.l_off[i]);
+    for (int i = tid; i < n; i += NT) { l_shard[i] = __ldg(shards + jb + l_off[i]); l_slot[i] = __ldg(slot_of + jb + l_off[i]); }
+    __syncthreads();
+    const int per = ((n + NW - 1) / NW + 31) / 32 * 32, lo = warp * per, hi = min(n, lo + per);
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int i0 = lo; i0 < hi; i0 += 32) {
+        const int i = i0 + lane;
+        const int key = i < hi ? (int)l_shard[i] : -1;
+        const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+        const uint32_t at = i < hi ? n_warp[warp][key] : 0u;
+        __syncwarp();
+        if (i < hi && (same >> lane) == 1u) n_warp[warp][key] = (uint16_t)(at + __popc(same));   // the group's last lane
+        if (pass == 1 && i < hi) {
+          uint32_t local = n_base[key] + at + __popc(same & ((1u << lane) - 1u));
+          if (local >= s_cap[key]) { local = DES_ROW_NONE; meta->rowless[key] = 1u; des_raise(meta, DES_ERR_CAPACITY); }
+          const int j = jb + l_off[i];
+          const uint32_t uu = l_grow[i];
+          const uint32_t grow = local == DES_ROW_NONE ? DES_ROW_NONE : s_row[key] + local;
+          if (local != DES_ROW_NONE && DES_DBG_SLOT_OK(l_slot[i])) slots[l_slot[i]].row = local;
+          rows[j] = local;
+          uidx[j] = local == DES_ROW_NONE ? DES_ROW_NONE : uu;
+          uniq_rows[uu] = grow;
+          l_grow[i] = grow;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      if (pass == 0) {                                   // counts of the list parts -> where each part starts
+        if (tid < S) {
+          uint32_t run = 0;
+          for (int i = 0; i < NW; ++i) { const uint16_t v = n_warp[i][tid]; n_warp[i][tid] = (uint16_t)run; run += v; }
+        }
+        __syncthreads();
+      }
     }
-    new_keys<G>(sh, na, n, jb);
+    // ---- their rows: G lanes per row, every lane of a warp runs the same rounds (the squared norm is a warp-level sum)
+    constexpr int U = 4;                                // rows of a group whose ids are in flight together
+    for (int i0 = 0; i0 < n; i0 += NT / G * U) {
+      uint32_t grow[U];
+      unsigned long long id[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int i = i0 + q * (NT / G) + tid / G;
+        grow[q] = i < n ? l_grow[i] : DES_ROW_NONE;
+        id[q] = i < n ? __ldg(ids + jb + l_off[i]) : 0ull;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c4 < K4) v = des_init4(seed, id[q], (uint32_t)c4, init_scale);
+        float n2 = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+#pragma unroll
+        for (int d = 1; d < G; d <<= 1) n2 += __shfl_xor_sync(0xFFFFFFFFu, n2, d);
+        if (grow[q] == DES_ROW_NONE || DES_DBG_ROW(grow[q]) != grow[q]) continue;
+        float4* wr = reinterpret_cast<float4*>(W + (size_t)grow[q] * stride);
+        if (c4 < K4) wr[c4] = v;
+        if (c4 == 0) wr[K4] = make_float4(0.f, n2, stamp, 0.f);   // linear weight, squared norm, age stamp
+        if (A) {
+          float4* a = reinterpret_cast<float4*>(A + (size_t)grow[q] * stride);
+          if (c4 < K4) a[c4] = make_float4(state_init, state_init, state_init, state_init);
+          if (c4 == 0) a[K4] = make_float4(lin_state_init, 0.f, 0.f, 0.f);
+        }
+        if (A2) {
+          float4* a2 = reinterpret_cast<float4*>(A2 + (size_t)grow[q] * stride);
+          if (c4 < K4) a2[c4] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (c4 == 0) a2[K4] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+    }
     if (win + IB < n_new) {                             // another window: the list and the counts are reused
       __syncthreads();
-      if (tid < S) sh.n_base[tid] += sh.n_warp[NW - 1][tid];
+      if (tid < S) n_base[tid] += n_warp[NW - 1][tid];
       __syncthreads();
     }
   }
@@ -1059,8 +1132,9 @@ extern "C" des_status_t des_find_or_insert(des_table_t* t, const des_batch_t* b,
   {
     const bool deep = ntiles >= ASSIGN_DEEP_TILES * t->sm_count;
 #define ASSIGN2(GG, PP) des_launch(assign_kernel<GG, PP>, (ntiles * IB + 512 * PP - 1) / (512 * PP), 512, 0, cs, nnz, ntiles,   \
-        (int)t->S, t->meta, b->shards, t->flags, t->blk_cnt, t->sup_cnt, (int)t->nblk_max, nsup_max, t->slot_of, b->n_uniq,      \
-        t->total_slots, (uint32_t)t->max_nnz, na)
+        (int)t->S, t->meta, na.ids, b->shards, t->flags, t->blk_cnt, t->sup_cnt, (int)t->nblk_max, nsup_max, t->slot_of, b->rows,  \
+        b->uidx, b->uniq_rows, b->n_uniq, t->slots, t->total_slots, (uint32_t)t->max_nnz, (int)t->k, (int)t->stride, t->W, t->A,   \
+        t->A2, na.seed, na.init_scale, na.state_init, na.lin_state_init)
 #define ASSIGN(GG) do { if (deep) ASSIGN2(GG, 8); else ASSIGN2(GG, 2); } while (0)
     switch (G) { case 1: ASSIGN(1); break; case 2: ASSIGN(2); break; case 4: ASSIGN(4); break; case 8: ASSIGN(8); break;
                  default: ASSIGN(16); }
