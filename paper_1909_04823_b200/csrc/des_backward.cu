@@ -792,7 +792,6 @@ static des_status_t backward_rows(des_table* t, uint32_t ops, const des_batch_t*
   return DES_OK;
 }
 
-#define SIDE_MIN (5ll << 20)      // entries of gE from which the backward takes this form
 // The whole backward with a first layer: on the caller's stream the operands' conversion, gE, scatter and update; on the side stream
 // the count and look-up of gradient rows, the weight gradient and, once gE has been formed (it reads the weights' bfloat16 copy),
 // the weights' update.  The caller's stream waits for the side stream before the call's work is over, also when a part fails.
@@ -842,7 +841,7 @@ extern "C" des_status_t des_backward_update(des_table_t* t, uint32_t ops, const 
     const Dense1Plan p = des_dense1_plan(t, B);
     // What the sparse backward does not wait for goes to the table's side stream: the count and the gradient rows' look-up beside
     // the product that forms gE, the weight gradient beside the scatter.  (Not while launches are being timed one by one.)
-    if (b->nnz && (long long)B * p.FK >= SIDE_MIN && !t->prof_on) return backward_beside(t, ops, b, out, gr, p, opt, cs);
+    if (b->nnz && t->side && (long long)B * p.FK >= DES_SIDE_MIN && !t->prof_on) return backward_beside(t, ops, b, out, gr, p, opt, cs);
     const float* gE = (ops & DES_OP_POOL) ? gr->gE : nullptr;
     int rc = 0;
     if ((st = des_dense1_dgrad(t, p, out->pooled, gE, gr->gZ, gr->gE_work, B, &rc, cs)) != DES_OK) return st;

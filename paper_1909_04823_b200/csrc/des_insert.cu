@@ -27,6 +27,7 @@
 // A further kernel (count_kernel) is the backward's: it counts the occurrences per unique key and lists the hot keys.
 #include "des_internal.cuh"
 
+#include <atomic>
 #include <type_traits>
 
 // Tiles per SM from which a block of assign_kernel takes four of them.  Known keys only, the deep form is the faster one from 0.5 M
@@ -895,8 +896,12 @@ __global__ void __launch_bounds__(ONCE_TILE / 2, 1) insert_once_kernel(ProbeArgs
   if (last && tid == 0) { meta->clock += 1ull; meta->scratch_base = base < oa.max_nnz ? 0xFFFFFFFFu : base; }
 }
 
-// Blocks of such a cluster on the table's device: 16 where it takes clusters of more than the portable 8.
-int des_insert_once_blocks() {
+// Blocks of such a cluster on the current device: 16 where it takes clusters of more than the portable 8.  A property of the device, asked
+// once (the question takes milliseconds); threads that ask at the same time store the same answer.
+int des_insert_once_blocks(int device) {
+  static std::atomic<int> known[64];
+  std::atomic<int>* k = device >= 0 && device < 64 ? &known[device] : nullptr;
+  if (k && k->load(std::memory_order_relaxed)) return k->load(std::memory_order_relaxed);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
@@ -905,7 +910,9 @@ int des_insert_once_blocks() {
   int n = 0;
   if (cudaFuncSetAttribute(insert_once_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
       cudaOccupancyMaxActiveClusters(&n, insert_once_kernel<16>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-  return n > 0 ? ONCE_BLOCKS : 8;
+  n = n > 0 ? ONCE_BLOCKS : 8;
+  if (k) k->store(n, std::memory_order_relaxed);
+  return n;
 }
 template <int G>
 static des_status_t insert_once(des_table* t, const des_batch_t* b, const ProbeArgs& pa, const SlotGeom& geom, const NewArgs& na,

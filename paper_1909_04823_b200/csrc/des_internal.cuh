@@ -128,7 +128,7 @@ struct des_table {
                                      // (consumed, once, by the first-layer product that follows); NULL otherwise
   void* gemm_ws; size_t gemm_ws_bytes;   // halves: the two products of a backward can overlap
   cudaStream_t side;                 // the part of a backward that nothing of the rest waits for runs here, between two events of the
-  cudaEvent_t side_fork, side_dest, side_gE, side_join;   // caller's stream (NULL: no first layer)
+  cudaEvent_t side_fork, side_dest, side_gE, side_join;   // caller's stream (NULL: no first layer of that size)
   // host-step staging
   int32_t* st_offsets[2]; unsigned long long* st_ids[2]; float* st_vals[2];   // two input slots (pipelined submit)
   cudaStream_t st_copy_stream; cudaEvent_t st_copied[2], st_done[2]; int st_busy[2]; uint64_t st_next;
@@ -372,6 +372,7 @@ __device__ __forceinline__ bool des_dbg_in(unsigned long long i, unsigned long l
 #endif
 
 // shared declarations across translation units
+#define DES_SIDE_MIN (5ll << 20)   // entries of gE from which a backward uses the side stream (figures at backward_beside)
 des_status_t des_check_batch(const des_table* t, const des_batch_t* b, int need_dedup);
 des_status_t des_dense1_forward(des_table* t, const float* pooled, int B, float* Z, float* part_dense,
                                 const float* part_pooled, bool have_b, cudaStream_t st);
@@ -385,6 +386,6 @@ des_status_t des_dense1_backward_plain(des_table* t, const float* pooled, const 
                                        cudaStream_t st);
 // Whether the keys that own a large share of the batch are counted instead of scattered in the backward.
 bool des_super_path(const des_table* t, const des_batch_t* b);
-int des_insert_once_blocks();
+int des_insert_once_blocks(int device);
 // Counts a batch's occurrences per unique key (a sample of a large batch) and makes the hot list: opens a backward.
 des_status_t des_count_batch(des_table* t, const des_batch_t* b, cudaStream_t cs);

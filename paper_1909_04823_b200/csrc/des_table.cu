@@ -216,7 +216,7 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
   A(t->blk_cnt, (size_t)(t->S + 1) * t->nblk_max * 4);
   const size_t sup_bytes = (size_t)(t->S + 1) * (t->nblk_max / SUP_TILES + 1) * 4;
   A(t->sup_cnt, sup_bytes);
-  t->once_blocks = des_insert_once_blocks();
+  t->once_blocks = des_insert_once_blocks(dev);
   A(t->once_words, (size_t)t->once_blocks * 32 * sizeof(uint2));
   A(t->once_new, (size_t)t->once_blocks * t->S * 4);
   A(t->seg_off, (size_t)t->max_batch * (t->S + 1) * 4);
@@ -269,9 +269,11 @@ extern "C" des_status_t des_table_create(const des_config_t* cfg, des_table_t** 
     cu &= cudaMemset(t->W1, 0, FKH * 4) == cudaSuccess;
     cu &= cudaMemset(t->W1b, 0, FKH * 2) == cudaSuccess;
     fill_f32_kernel<<<256, 256>>>(t->accW1, FKH, c.optimizer == DES_OPT_ADAGRAD ? c.init_acc : 0.f);
-    cu &= cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking) == cudaSuccess;
-    for (cudaEvent_t* e : {&t->side_fork, &t->side_dest, &t->side_gE, &t->side_join})
-      cu &= cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    if ((long long)t->max_batch * t->F * t->k >= DES_SIDE_MIN) {
+      cu &= cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking) == cudaSuccess;
+      for (cudaEvent_t* e : {&t->side_fork, &t->side_dest, &t->side_gE, &t->side_join})
+        cu &= cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    }
     if (t->acc2W1) cu &= cudaMemset(t->acc2W1, 0, FKH * 4) == cudaSuccess;
     cu &= cudaGetLastError() == cudaSuccess;
   }
